@@ -172,6 +172,125 @@ def run(s):
     return out
 
 
+# ------------------------------------------------------------------------------------------------- the same in 64 bits
+def _layers(w, p, X):
+    """One function (state, parameters) -> (next state, diagonal of the residual Jacobian) per residual step, with the parameters it
+    takes: (function, {gradient name: (tensor, index of its slice or None)})."""
+    F = torch.nn.functional
+
+    def mlp(x, W1, W2):
+        return F.gelu(x @ W1.T) @ W2.T
+
+    def norm(x):
+        return F.layer_norm(x, x.shape[-1:], eps=w.ln_eps)
+
+    def attention(x, Wq, Wk, Wv, Wo):
+        y = norm(x).view(w.batch, w.seq, w.d)
+        q, k, v = ((y @ W.T).view(w.batch, w.seq, w.n_heads, w.head_dim).transpose(1, 2) for W in (Wq, Wk, Wv))
+        future = torch.ones(w.seq, w.seq, dtype=torch.bool, device=x.device).triu(1)
+        s = (q @ k.transpose(2, 3) / math.sqrt(w.head_dim)).masked_fill(future, -math.inf)
+        return (s.softmax(-1) @ v).transpose(1, 2).reshape(x.shape) @ Wo.T
+
+    def rnn(xt):
+        return lambda x, W, U, a: (a * x + torch.tanh(x @ W.T + xt @ U.T), a)
+
+    def gru(xt):
+        def step(x, W, U):
+            (ur, uz, un), (wr, wz, wn) = (xt @ U.T).chunk(3, -1), (x @ W.T).chunk(3, -1)
+            z = torch.sigmoid(uz + wz)
+            return z * x + (1 - z) * torch.tanh(un + torch.sigmoid(ur + wr) * wn), z
+        return step
+
+    def lstm(xt):
+        def step(x, W, U):
+            c, h = x.chunk(2, -1)
+            i, f, g, o = (xt @ U.T + h @ W.T).chunk(4, -1)
+            c = torch.sigmoid(f) * c + torch.sigmoid(i) * torch.tanh(g)
+            return torch.cat([c, torch.sigmoid(o) * torch.tanh(c)], -1), torch.cat([torch.sigmoid(f), torch.zeros_like(f)], -1)
+        return step
+
+    def post(x, W1, W2):
+        y = x + mlp(x, W1, W2)
+        return norm(y), (1 - w.gamma) / (y.var(-1, unbiased=False, keepdim=True) + w.ln_eps).sqrt()
+
+    if w.block in ("rnn_tanh", "gru", "lstm"):
+        of = {"rnn_tanh": rnn, "gru": gru, "lstm": lstm}[w.block]
+        return [(of(X[t].double()), {n: (p[n].double(), None) for n in p}) for t in range(w.L)]
+    out = []
+    for b in range(w.L):
+        if w.block == "preln_transformer":
+            out.append((lambda x, *W: (x + attention(x, *W), 1.0), {n: (p[n][b], b) for n in ("Wq", "Wk", "Wv", "Wo")}))
+        whole = {"mlp": lambda x, *W: (x + mlp(x, *W), 1.0), "postln_mlp": post}.get(w.block, lambda x, *W: (x + mlp(norm(x), *W), 1.0))
+        out.append((whole, {n: (p[n][b], b) for n in ("W1", "W2")}))
+    return out
+
+
+def exact(case, seed):
+    """What `run` returns, from the same inputs, with every operation in 64 bits: each layer's vector-Jacobian product is
+    automatic differentiation of the layer less its residual part, and the scan is its recurrence."""
+    if case["do"] == "scan":
+        s = prepare(case, seed)
+        delta, every, L = s["delta"].double(), case["loss"] == "every_mse", case["L"]
+        g = torch.empty(s["g"].shape, dtype=torch.float64, device="cuda")
+        g[L] = delta[L] if every else delta
+        for l in range(L - 1, -1, -1):
+            a = 1.0 if s["a"] is None else (s["a"] if s["a"].dim() == 1 else s["a"][l]).double()
+            g[l] = a * g[l + 1] + s["u"][l].double() + (delta[l] if every else 0.0)
+        return g
+    w = _workload(case, seed)
+    inp = make_inputs(w, "cuda")
+    params = harness.params_for(w, inp)
+    layers = _layers(w, params, inp.get("X"))
+    n = len(layers)
+    x = torch.empty((n + 1, w.tokens, w.d), dtype=torch.float64, device="cuda")
+    x[0] = inp["x0"].double()
+    keep = []  # diagonals of the residual Jacobians, None where they are one
+    with torch.no_grad():
+        for l, (f, p) in enumerate(layers):
+            x[l + 1], a = f(x[l], *(t.double() for t, _ in p.values()))
+            keep.append(a)
+    if case["do"] == "forward":
+        return x
+    delta = torch.zeros_like(x)
+    if w.loss == "every_mse":
+        delta[1:] = (x[1:] - inp["Y"].double()) * (2.0 / (w.L * w.batch * w.d))
+    else:
+        delta[n] = (x[n] - inp["y"].double()) * (1.0 if w.loss == "final_half_sse" else 2.0 / (w.tokens * w.d))
+    grads = {"d" + name: torch.zeros(t.shape, dtype=torch.float64, device="cuda") for name, t in params.items()}
+
+    def vjp(l, v, state=True, weights=False):
+        f, p = layers[l]
+        at = x[l].clone().requires_grad_(state)
+        ws = [t.double().clone().requires_grad_(weights) for t, _ in p.values()]
+        got = list(torch.autograd.grad(f(at, *ws)[0], ([at] if state else []) + (ws if weights else []), v))
+        back = got.pop(0) if state else None
+        for (name, (_, i)), t in zip(p.items(), got):
+            (grads["d" + name] if i is None else grads["d" + name][i]).add_(t)
+        return back
+
+    g = torch.empty_like(x)
+    g[n] = delta[n]
+    if case["do"] == "exact":
+        for l in range(n - 1, -1, -1):
+            g[l] = delta[l] + vjp(l, g[l + 1], weights=True)
+    else:
+        for l in range(n - 1, -1, -1):
+            g[l] = delta[l] + keep[l] * g[l + 1]
+        for _ in range(min(case["k"], n)):
+            new = delta[n]
+            for l in range(n):  # the products of the old estimate first: g[l] is not read again
+                g[l] = vjp(l, g[l + 1]) - keep[l] * g[l + 1]
+            for l in range(n - 1, -1, -1):
+                new = delta[l] + keep[l] * new + g[l]
+                g[l] = new
+        for l in range(n):
+            vjp(l, g[l + 1], state=False, weights=True)
+    out = {"g": g, "grads": grads}
+    if case["do"] == "train":
+        out["x"] = x
+    return out
+
+
 # ------------------------------------------------------------------------------------------------- what a pass cannot do without
 def work(case):
     es = 4 if case["dtype"] == "f32" else 2
