@@ -71,6 +71,7 @@ struct hbp_ctx {
   // post-LN layers: GM holds LayerNorm-backward of g_{l+1} (what the block is differentiated against), CB the part of
   // the layer's VJP that is not the block's, rstd [L][N] is the scan's row gate
   char* CB = nullptr;
+  char* pack = nullptr;    // recurrent kinds: the weights in the order of the one-launch recurrences (cell_pack_bytes)
   char* scan_scratch = nullptr;
   size_t scan_scratch_bytes = 0;
   float* partial = nullptr;  // split-K / gate-gradient partial sums
@@ -149,6 +150,12 @@ size_t carve(hbp_ctx* c, char* base) {
   const bool recurrent = f.block == HBP_BLOCK_RNN_TANH || f.block == HBP_BLOCK_GRU || f.block == HBP_BLOCK_LSTM;
   if (f.dtype == HBP_BF16 && !recurrent) c->xres = (float*)take(N * d * 4);
   c->partial_floats = (size_t)kGateBlocks * d;
+  if (recurrent) {
+    size_t pb = cell_pack_bytes(f.block, f.block == HBP_BLOCK_LSTM ? f.d / 2 : f.d, f.in_dim);
+    const size_t rb = f.block == HBP_BLOCK_RNN_TANH ? rnn_cluster_pack_bytes(f.d, f.in_dim) : 0;
+    if (rb > pb) pb = rb;
+    if (pb) c->pack = take(pb);
+  }
   if (f.block == HBP_BLOCK_LSTM) {
     const size_t in = (size_t)f.in_dim, u = d / 2, rows = steps * N;
     c->Fg = take(rows * d * es);
@@ -912,8 +919,11 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
   if (f.block == HBP_BLOCK_LSTM) {
     const int T = f.L;
     const int64_t u = d / 2;
-    convert_to_f64(r.lc, f.dtype, x0, ctx->hres, state);
-    for (int t = 0; t < T; ++t) {
+    // all T steps in one launch where that form applies, else one launch per step (likewise below)
+    const bool one_launch = !ctx->force_simt && cell_forward_cluster(r.lc, f.dtype, f.block, params->W, params->U, inputs, nullptr, x0, xa,
+                                                                     ctx->Fg, ctx->C5, T, (int)N, (int)u, f.in_dim, ctx->pack, ctx->status);
+    if (!one_launch) convert_to_f64(r.lc, f.dtype, x0, ctx->hres, state);
+    for (int t = 0; t < T && !one_launch; ++t) {
       const double* sin = ctx->hres + (int64_t)(t & 1) * state;
       double* sout = ctx->hres + (int64_t)((t + 1) & 1) * state;
       lstm_forward_step(r.lc, f.dtype, params->W, params->U, r.at(inputs, (int64_t)t * N * f.in_dim), sin, sout,
@@ -927,8 +937,10 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
     }
   } else if (f.block == HBP_BLOCK_GRU) {
     const int T = f.L;
-    convert_to_f64(r.lc, f.dtype, x0, ctx->hres, state);
-    for (int t = 0; t < T; ++t) {
+    const bool one_launch = !ctx->force_simt && cell_forward_cluster(r.lc, f.dtype, f.block, params->W, params->U, inputs, nullptr, x0, xa,
+                                                                     ctx->Zc, ctx->C4, T, (int)N, (int)d, f.in_dim, ctx->pack, ctx->status);
+    if (!one_launch) convert_to_f64(r.lc, f.dtype, x0, ctx->hres, state);
+    for (int t = 0; t < T && !one_launch; ++t) {
       const double* hin = ctx->hres + (int64_t)(t & 1) * state;
       double* hout = ctx->hres + (int64_t)((t + 1) & 1) * state;
       gru_forward_step(r.lc, f.dtype, params->W, params->U, r.at(inputs, (int64_t)t * N * f.in_dim), hin, hout,
@@ -942,10 +954,19 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
     }
   } else if (f.block == HBP_BLOCK_RNN_TANH) {
     const int T = f.L;
-    // all T steps in one launch where that form applies, else one launch per step
-    const bool one_launch = ctx->Pd && !ctx->force_simt &&
-                            rnn_forward_persistent(r.lc, f.dtype, params->W, params->U, inputs, r.gate_ptr(0), x0, ctx->Pd, xa,
-                                                   ctx->C, T, (int)N, (int)d, f.in_dim, ctx->status);
+    // All T steps in one launch where that form applies, else one launch per step.  Of the two one-launch forms the one
+    // with 4 rows per cluster has the shorter step (512 units, 8 rows, 16 inputs: 2.4 us against 2.7) as long as its clusters run at once;
+    // with more rows they queue (32 rows, 256 inputs: 5.5 us against 3.2).
+    const bool one_form = !ctx->force_simt && f.gate != HBP_GATE_CHANNEL_PER_STEP;
+    auto four_rows = [&]() {
+      return ctx->Pd && rnn_forward_persistent(r.lc, f.dtype, params->W, params->U, inputs, r.gate_ptr(0), x0, ctx->Pd, xa, ctx->C, T,
+                                               (int)N, (int)d, f.in_dim, ctx->status);
+    };
+    const bool at_once = one_form && ctx->Pd && rnn_persistent_at_once(f.dtype, false, (int)N, (int)d);
+    const bool one_launch = one_form && ((at_once && four_rows()) ||
+                                         rnn_forward_cluster(r.lc, f.dtype, params->W, params->U, inputs, r.gate_ptr(0), x0, ctx->Pd, xa,
+                                                             ctx->C, T, (int)N, (int)d, f.in_dim, ctx->pack, ctx->status) ||
+                                         four_rows());
     if (!one_launch) {
       convert_to_f64(r.lc, f.dtype, x0, ctx->hres, state);
       for (int t = 0; t < T; ++t) {
@@ -1090,10 +1111,17 @@ static hbp_status backward_common(hbp_ctx* ctx, const hbp_params* params, int32_
     if (rnn) {
       // the sequential recurrence is carried in double beside the stored float gradients: one launch over all
       // steps where that form applies, else one launch per step
-      const bool one_launch = ctx->Pd && !ctx->force_simt &&
-                              rnn_backward_persistent(r.lc, f.dtype, params->W, r.gate_ptr(0), ctx->C,
-                                                      f.loss == HBP_LOSS_EVERY_STEP ? r.delta : nullptr, r.g, steps,
-                                                      (int)r.N, (int)r.d, ctx->status);
+      const bool one_form = !ctx->force_simt && f.gate != HBP_GATE_CHANNEL_PER_STEP;
+      const void* per_step = f.loss == HBP_LOSS_EVERY_STEP ? r.delta : nullptr;
+      auto four_rows = [&]() {
+        return ctx->Pd && rnn_backward_persistent(r.lc, f.dtype, params->W, r.gate_ptr(0), ctx->C, per_step, r.g, steps, (int)r.N, (int)r.d,
+                                                  ctx->status);
+      };
+      const bool at_once = one_form && ctx->Pd && rnn_persistent_at_once(f.dtype, true, (int)r.N, (int)r.d);
+      const bool one_launch = one_form && ((at_once && four_rows()) ||
+                                           cell_backward_cluster(r.lc, f.dtype, f.block, params->W, r.gate_ptr(0), nullptr, ctx->C, per_step,
+                                                                 r.g, steps, (int)r.N, (int)r.d, ctx->pack, ctx->status) ||
+                                           four_rows());
       if (!one_launch) {
         convert_to_f64(r.lc, f.dtype, r.at(r.g, (int64_t)steps * r.state), ctx->hres, r.state);
         for (int t = steps - 1; t >= 0; --t) {
@@ -1106,8 +1134,11 @@ static hbp_status backward_common(hbp_ctx* ctx, const hbp_params* params, int32_
       }
       if (grads) r.rnn_wgrad(grads);
     } else if (gru) {
-      convert_to_f64(r.lc, f.dtype, r.at(r.g, (int64_t)steps * r.state), ctx->hres, r.state);
-      for (int t = steps - 1; t >= 0; --t) {
+      const bool one_launch = !ctx->force_simt && cell_backward_cluster(r.lc, f.dtype, f.block, params->W, nullptr, ctx->Zc, ctx->C4,
+                                                                        f.loss == HBP_LOSS_EVERY_STEP ? r.delta : nullptr, r.g, steps,
+                                                                        (int)r.N, (int)r.d, ctx->pack, ctx->status);
+      if (!one_launch) convert_to_f64(r.lc, f.dtype, r.at(r.g, (int64_t)steps * r.state), ctx->hres, r.state);
+      for (int t = steps - 1; t >= 0 && !one_launch; --t) {
         const double* gin = ctx->hres + (int64_t)((steps - 1 - t) & 1) * r.state;
         double* gout = ctx->hres + (int64_t)((steps - t) & 1) * r.state;
         gru_backward_step(r.lc, f.dtype, params->W, r.at(ctx->Zc, (int64_t)t * r.state),
@@ -1117,8 +1148,11 @@ static hbp_status backward_common(hbp_ctx* ctx, const hbp_params* params, int32_
       }
       if (grads) r.gru_wgrad(grads);
     } else if (f.block == HBP_BLOCK_LSTM) {
-      convert_to_f64(r.lc, f.dtype, r.at(r.g, (int64_t)steps * r.state), ctx->hres, r.state);
-      for (int t = steps - 1; t >= 0; --t) {
+      const bool one_launch = !ctx->force_simt && cell_backward_cluster(r.lc, f.dtype, f.block, params->W, nullptr, ctx->Fg, ctx->C5,
+                                                                        f.loss == HBP_LOSS_EVERY_STEP ? r.delta : nullptr, r.g, steps,
+                                                                        (int)r.N, (int)(r.d / 2), ctx->pack, ctx->status);
+      if (!one_launch) convert_to_f64(r.lc, f.dtype, r.at(r.g, (int64_t)steps * r.state), ctx->hres, r.state);
+      for (int t = steps - 1; t >= 0 && !one_launch; --t) {
         const double* gin = ctx->hres + (int64_t)((steps - 1 - t) & 1) * r.state;
         double* gout = ctx->hres + (int64_t)((steps - t) & 1) * r.state;
         lstm_backward_step(r.lc, f.dtype, params->W, r.at(ctx->Fg, (int64_t)t * r.state),

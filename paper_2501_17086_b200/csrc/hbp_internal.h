@@ -200,6 +200,32 @@ bool rnn_forward_persistent(Launcher& lc, int dtype, const void* W, const void* 
 bool rnn_backward_persistent(Launcher& lc, int dtype, const void* W, const void* gate, const void* deriv,
                              const void* delta, void* g_all, int T, int B, int d, int* status);
 
+// U x_t of every step as one product, M = T * B rows.
+void rnn_project(Launcher& lc, int dtype, const void* X, const void* U, double* P, int64_t M, int d, int in_dim);
+// Whether the one-launch form above would run all its clusters of 4 rows at once (more rows queue behind them).
+bool rnn_persistent_at_once(int dtype, bool backward, int B, int d);
+// Whether rnn_forward_step uses its staged kernel at these widths.
+bool rnn_step_is_staged(int d, int in_dim);
+// The forward recurrence for any number of rows and units, one launch, sums in the order of the two forms above
+// (rnn_cluster.cu): bit for bit their states.  pack: scratch of rnn_cluster_pack_bytes bytes; P as above (128, 256 or 512
+// units only).  false when nothing was done for the recurrence.
+size_t rnn_cluster_pack_bytes(int u, int in_dim);
+bool rnn_forward_cluster(Launcher& lc, int dtype, const void* W, const void* U, const void* X, const void* gate, const void* x0,
+                         double* P, void* x_all, void* deriv, int T, int B, int u, int in_dim, void* pack, int* status);
+
+// ---------------------------------------------------------------- recurrences of the gated cells (cell_cluster.cu)
+// Forward pass (GRU, LSTM) and exact backpropagation (tanh RNN, GRU, LSTM; block = an hbp_block value) as one launch over
+// all T steps: clusters of up to 16 CTAs own 8 to 24 batch rows, contractions on the FP64 matrix instruction.  u = units
+// (LSTM states are 2u wide); keep = the GRU's z or the LSTM's [f | 0]; coef = tanh', C4 or C5; delta may be null.
+// pack: scratch of cell_pack_bytes bytes for the weights in the kernels' order (0 = more units than this form takes).
+// false when nothing was launched (more than 1536 units, unaligned pointers, clusters that cannot be scheduled): the
+// caller then runs the per-step kernels.
+size_t cell_pack_bytes(int block, int u, int in_dim);
+bool cell_forward_cluster(Launcher& lc, int dtype, int block, const void* W, const void* U, const void* X, const void* gate,
+                          const void* x0, void* x_all, void* keep, void* coef, int T, int B, int u, int in_dim, void* pack, int* status);
+bool cell_backward_cluster(Launcher& lc, int dtype, int block, const void* W, const void* gate, const void* keep, const void* coef,
+                           const void* delta, void* g_all, int T, int B, int u, void* pack, int* status);
+
 // ---------------------------------------------------------------- diagnostics (diag.cu)
 // out[seg][4] = {<a,b>, |a|^2, |b|^2, |a-b|^2} over `elems` elements per segment; scratch holds
 // compare_scratch_bytes(segments) bytes.

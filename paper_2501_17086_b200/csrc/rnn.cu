@@ -241,6 +241,8 @@ __global__ void to_f64_kernel(const T* __restrict__ src, double* __restrict__ ds
 
 }  // namespace
 
+bool rnn_step_is_staged(int d, int in_dim) { return staged_bytes(d + in_dim, d + in_dim) <= kStagedSmemLimit; }
+
 void rnn_forward_step(Launcher& lc, int dtype, const void* W, const void* U, const void* x_t, const void* gate,
                       const double* h_in, double* h_out, void* deriv, void* state_out, int B, int d, int in_dim) {
   const size_t staged = staged_bytes(d + in_dim, d + in_dim);

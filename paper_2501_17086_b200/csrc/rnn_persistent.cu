@@ -17,7 +17,7 @@
 // The recurrence is carried in double like the per-step kernels of rnn.cu (a float carry drifts from the fp64
 // reference over thousands of steps).  The input projection U x_t of all steps has no dependence on h and is
 // formed beforehand by one FP64 GEMM (proj_f64_kernel).
-#include "hbp_internal.h"
+#include "cell_common.cuh"
 
 namespace hbp {
 
@@ -247,53 +247,67 @@ __global__ void __launch_bounds__(NW * kKP / kCS * kKP, 1) rnn_persistent_kernel
   cluster_barrier();  // no CTA ends while a peer may still address its shared memory
 }
 
-// P[m][n] = sum_k X[m][k] U[n][k] in double (operands of type T), M = T * B rows, N = d, K = in_dim.
-// 64 x 64 tiles, 16 of K per stage, 4 x 4 outputs per thread.
+// P[m][n] = sum_k X[m][k] U[n][k] in double (operands of type T), M = T * B rows, N = d, K = in_dim, every sum ascending
+// in k.  64 x 64 tiles, 16 of K per stage, a 32 x 16 tile per warp on the FP64 matrix instruction (which adds its four
+// products in ascending order, rounding each like an FMA): bound by the FP64 rate.
 template <typename T>
 __global__ void __launch_bounds__(256) proj_f64_kernel(const T* __restrict__ X, const T* __restrict__ U,
                                                        double* __restrict__ P, int64_t M, int N, int K) {
-  __shared__ __align__(16) double Xs[16][64 + 2];
-  __shared__ __align__(16) double Us[16][64 + 2];
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  constexpr int kPitch = 20;  // doubles per row of 16: the quads of a half-warp fall on distinct banks
+  __shared__ __align__(16) double Xs[64][kPitch];
+  __shared__ __align__(16) double Us[64][kPitch];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, lr = lane >> 2, lc = lane & 3;
   const int64_t m0 = (int64_t)blockIdx.y * 64;
-  const int n0 = blockIdx.x * 64;
-  double acc[4][4] = {};
+  const int n0 = blockIdx.x * 64, wm = (warp & 1) * 32, wn = (warp >> 1) * 16;
+  const int sr = threadIdx.x >> 2, sk = (threadIdx.x & 3) * 4;  // this thread stages 4 elements of one row of each operand
+  float xv[4], uv[4];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int k = k0 + sk + i;
+      xv[i] = (m0 + sr < M && k < K) ? to_f(X[(m0 + sr) * K + k]) : 0.0f;
+      uv[i] = (n0 + sr < N && k < K) ? to_f(U[(int64_t)(n0 + sr) * K + k]) : 0.0f;
+    }
+  };
+  double2 acc[4][2] = {};
+  fetch(0);
   for (int k0 = 0; k0 < K; k0 += 16) {
-    for (int i = threadIdx.x; i < 64 * 16; i += 256) {
-      const int r = i / 16, kk = i % 16, k = k0 + kk;
-      Xs[kk][r] = (m0 + r < M && k < K) ? (double)to_f(X[(m0 + r) * K + k]) : 0.0;
-      Us[kk][r] = (n0 + r < N && k < K) ? (double)to_f(U[(int64_t)(n0 + r) * K + k]) : 0.0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      Xs[sr][sk + i] = (double)xv[i];
+      Us[sr][sk + i] = (double)uv[i];
     }
     __syncthreads();
+    if (k0 + 16 < K) fetch(k0 + 16);
 #pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      double xa[4], ub[4];
+    for (int kk = 0; kk < 16; kk += 4) {
+      double a[4], b[2];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) xa[i] = Xs[kk][ty * 4 + i];
+      for (int i = 0; i < 4; ++i) a[i] = Xs[wm + 8 * i + lr][kk + lc];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) ub[j] = Us[kk][tx * 4 + j];
+      for (int j = 0; j < 2; ++j) b[j] = Us[wn + 8 * j + lr][kk + lc];
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(xa[i], ub[j], acc[i][j]);
+        for (int j = 0; j < 2; ++j) cell::dmma(acc[i][j], a[i], b[j]);
     }
     __syncthreads();
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const int64_t m = m0 + ty * 4 + i;
+    const int64_t m = m0 + wm + 8 * i + lr;
     if (m >= M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
-      if (n < N) P[m * N + n] = acc[i][j];
+    for (int j = 0; j < 2; ++j) {
+      const int n = n0 + wn + 8 * j + 2 * lc;  // (N is a multiple of 4)
+      if (n < N) *reinterpret_cast<double2*>(P + m * N + n) = acc[i][j];
     }
   }
 }
 
 template <typename T, int NW, bool BWD>
-bool launch_persistent(Launcher& lc, const PersistArgs& a) {
-  static PerDevice<int> state;  // 0 = not set up yet, 1 = usable on this device, -1 = clusters of 16 not schedulable here
+bool launch_persistent(Launcher& lc, const PersistArgs& a, bool ask) {
+  static PerDevice<int> state;  // 0 = not set up yet, clusters that run at a time, -1 = clusters of 16 not schedulable here
   int& st = state.here();
   auto kernel = rnn_persistent_kernel<T, NW, BWD>;
   constexpr int NT = NW * kKP / kCS * kKP, D = NW * kKP;
@@ -316,10 +330,11 @@ bool launch_persistent(Launcher& lc, const PersistArgs& a) {
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem) == cudaSuccess &&
         cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
         cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters >= 1)
-      st = 1;
+      st = clusters;
     cudaGetLastError();
   }
-  if (st != 1) return false;
+  if (ask) return st >= (a.B + kR - 1) / kR;  // whether all clusters would run at once
+  if (st < 1) return false;
   cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, a);
   if (e != cudaSuccess && lc.err == cudaSuccess) lc.err = e;
   lc.count();
@@ -328,11 +343,11 @@ bool launch_persistent(Launcher& lc, const PersistArgs& a) {
 }
 
 template <typename T, bool BWD>
-bool dispatch_persistent(Launcher& lc, const PersistArgs& a) {
+bool dispatch_persistent(Launcher& lc, const PersistArgs& a, bool ask = false) {
   switch (a.d) {
-    case 128: return launch_persistent<T, 128 / kKP, BWD>(lc, a);
-    case 256: return launch_persistent<T, 256 / kKP, BWD>(lc, a);
-    case 512: return launch_persistent<T, 512 / kKP, BWD>(lc, a);
+    case 128: return launch_persistent<T, 128 / kKP, BWD>(lc, a, ask);
+    case 256: return launch_persistent<T, 256 / kKP, BWD>(lc, a, ask);
+    case 512: return launch_persistent<T, 512 / kKP, BWD>(lc, a, ask);
     default: return false;  // other widths stay on the per-step kernels
   }
 }
@@ -344,26 +359,32 @@ size_t rnn_persistent_proj_bytes(int T, int64_t B, int d) {
   return (size_t)T * (size_t)B * (size_t)d * sizeof(double);
 }
 
+void rnn_project(Launcher& lc, int dtype, const void* X, const void* U, double* P, int64_t M, int d, int in_dim) {
+  dim3 grid((unsigned)((d + 63) / 64), (unsigned)((M + 63) / 64));
+  if (dtype == HBP_F32) proj_f64_kernel<float><<<grid, 256, 0, lc.stream>>>((const float*)X, (const float*)U, P, M, d, in_dim);
+  else proj_f64_kernel<bf16><<<grid, 256, 0, lc.stream>>>((const bf16*)X, (const bf16*)U, P, M, d, in_dim);
+  lc.count();
+  lc.check();
+}
+
+bool rnn_persistent_at_once(int dtype, bool backward, int B, int d) {
+  Launcher lc;
+  PersistArgs a = {};
+  a.B = B; a.d = d;
+  if (backward) return dtype == HBP_F32 ? dispatch_persistent<float, true>(lc, a, true) : dispatch_persistent<bf16, true>(lc, a, true);
+  return dtype == HBP_F32 ? dispatch_persistent<float, false>(lc, a, true) : dispatch_persistent<bf16, false>(lc, a, true);
+}
+
 bool rnn_forward_persistent(Launcher& lc, int dtype, const void* W, const void* U, const void* X, const void* gate,
                             const void* x0, double* P, void* x_all, void* deriv, int T, int B, int d, int in_dim, int* status) {
   if (!P || T <= 0 || B <= 0 || (d != 128 && d != 256 && d != 512)) return false;
   PersistArgs a = {};
   a.W = W; a.gate = gate; a.P = P; a.x0 = x0; a.states = x_all; a.deriv = deriv; a.delta = nullptr; a.status = status;
   a.T = T; a.B = B; a.d = d;
-  const int64_t M = (int64_t)T * B;
-  dim3 grid((unsigned)((d + 63) / 64), (unsigned)((M + 63) / 64));
   // (where clusters of 16 cannot be scheduled the dispatch returns false after the projection has been enqueued:
   // harmless, the caller then runs the per-step kernels)
-  if (dtype == HBP_F32) {
-    proj_f64_kernel<float><<<grid, 256, 0, lc.stream>>>((const float*)X, (const float*)U, P, M, d, in_dim);
-    lc.count();
-    lc.check();
-    return dispatch_persistent<float, false>(lc, a);
-  }
-  proj_f64_kernel<bf16><<<grid, 256, 0, lc.stream>>>((const bf16*)X, (const bf16*)U, P, M, d, in_dim);
-  lc.count();
-  lc.check();
-  return dispatch_persistent<bf16, false>(lc, a);
+  rnn_project(lc, dtype, X, U, P, (int64_t)T * B, d, in_dim);
+  return dtype == HBP_F32 ? dispatch_persistent<float, false>(lc, a) : dispatch_persistent<bf16, false>(lc, a);
 }
 
 bool rnn_backward_persistent(Launcher& lc, int dtype, const void* W, const void* gate, const void* deriv, const void* delta,
