@@ -1,0 +1,356 @@
+// Float GEMM on the tensor cores for any orientation of the operands (residual MLPs and decoders in single precision):
+//   D(m, n) = sum_k A(m, k) B(n, k), each operand split on the way into shared memory into a tf32 high part and a tf32
+//   remainder, three tf32 products lo hi + hi lo + hi hi, the epilogues of the CUDA-core kernel.
+//
+// One CTA per 128 x 128 tile (and batch entry, and split of K), 512 threads:
+//   warps 0..7   load 32-wide k-blocks of A and B from global memory (two blocks ahead, in registers), split them and store
+//                both parts as K-major 128-byte-swizzled tiles (64 KB a stage, three stages); an operand whose row index is
+//                contiguous is transposed in 4 x 4 blocks in registers on the way
+//   warps 8..15  add each finished accumulator to float sums in registers; epilogue
+//   warp 8       also issues 12 x tcgen05.mma 128x128x8 per k-block into one of two tensor-memory accumulators, before it
+//                adds up the previous block's (a warp of its own would leave 96 registers a thread instead of 128)
+// The sums leave the tensor core after every 32 of K because its accumulation truncates: the error of a long chain is a bias
+// that grows with its length (12 additions of which 4 at full magnitude here), while the additions in registers round to
+// nearest: 1.8e-7 of the result against 64 bits at K = 1560, 2.4e-7 at 4096, where the CUDA-core kernel's running float sums
+// are at 7e-7 and 1.2e-6.
+//
+// Bound by shared-memory bandwidth: per k-block 64 KB of stores and 96 KB of operand reads, 1280 clocks at 128 bytes (about
+// 1950 measured), against 768 clocks of tensor work; splitting ahead of time would need a copy of every operand in both
+// orientations.  1900 x 1560 x 520, 12 at once: 1980 -> 400 us (92 TFLOP/s); 4096 x 1024 x 4096: 1580 -> 264 us.
+#include "tc_common.cuh"
+
+namespace hbp {
+
+using namespace tc;
+
+namespace {
+
+constexpr int BM = 128, BN = 128, BK = 32;
+constexpr int kWorkerWarps = 8, kMmaWarp = kWorkerWarps, kAllThreads = 64 * kWorkerWarps;
+constexpr int kStages = 3;
+constexpr uint32_t kTile = BM * BK * 4, kStageBytes = 4 * kTile;  // A hi, A lo, B hi, B lo
+constexpr uint32_t kTmemCols = 256;
+constexpr int kSmemBytes = kStages * (int)kStageBytes + 1024 /*alignment*/ + 256 /*barriers*/;
+
+struct F32Params {
+  GemmArgs g;
+  int a_mn, b_mn;  // 1: the row index is contiguous
+  int k_blocks, kb_per_split;
+  int* status;
+};
+
+// v = hi + lo + (what a third tf32 term would hold).  The tensor core ignores the low 13 bits of an operand, so hi is
+// rounded (truncated where rounding would reach infinity) and cleared and lo only rounded; integer operations, because the
+// conversion instruction runs at a fraction of their rate.  An infinity stands for itself.
+__device__ __forceinline__ void split_tf32x2(float v, uint32_t& hi, uint32_t& lo) {
+  const uint32_t u = __float_as_uint(v);
+  const float mag = fabsf(v);
+  hi = (mag < __uint_as_float(0x7f7ff000u) ? u + 0x1000u : u) & 0xffffe000u;
+  lo = mag == __uint_as_float(0x7f800000u) ? 0u : __float_as_uint(v - __uint_as_float(hi)) + 0x1000u;
+}
+__device__ __forceinline__ void store_split(uint32_t hi_tile, uint32_t lo_tile, int row, int unit, float a, float b, float c, float d) {
+  uint4 h, l;
+  split_tf32x2(a, h.x, l.x);
+  split_tf32x2(b, h.y, l.y);
+  split_tf32x2(c, h.z, l.z);
+  split_tf32x2(d, h.w, l.w);
+  st_shared16(swz(hi_tile, row, unit), h);
+  st_shared16(swz(lo_tile, row, unit), l);
+}
+
+// This thread's share of one operand's 128 x 32 block: four 16-byte loads.
+//   K contiguous: 8 lanes read the 8 units of a row, rows 32 apart;  rows contiguous: a 4 x 4 block, lane & 7 = unit of K
+struct Loader {
+  const float* at;     // this thread's first element of the current block
+  int64_t step, next;  // between its four loads, and from block to block
+  int left, k, unit;   // rows from its first row to the end; first k of the thread in the current block
+  bool mn;
+  __device__ __forceinline__ void init(const void* p, int64_t s_row, int64_t s_k, int extent, int row0, int k0, bool mn_major) {
+    const int tid = threadIdx.x;
+    mn = mn_major;
+    unit = tid & 7;
+    const int row = row0 + (mn ? (tid >> 3) * 4 : tid >> 3);
+    left = extent - row;
+    k = k0 + unit * 4;
+    at = (const float*)p + (int64_t)row * s_row + (int64_t)k * s_k;
+    step = mn ? s_k : 32 * s_row;
+    next = BK * s_k;
+  }
+  __device__ __forceinline__ void load(int k_end, float4* v) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const bool in = mn ? left > 0 && k + i < k_end : left > 32 * i && k < k_end;
+      v[i] = in ? __ldg(reinterpret_cast<const float4*>(at + i * step)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    at += next;
+    k += BK;
+  }
+  __device__ __forceinline__ void store(uint32_t hi_tile, uint32_t lo_tile, const float4* v) const {
+    const int tid = threadIdx.x;
+    if (mn) {
+      const int r = (tid >> 3) * 4;
+      store_split(hi_tile, lo_tile, r, unit, v[0].x, v[1].x, v[2].x, v[3].x);
+      store_split(hi_tile, lo_tile, r + 1, unit, v[0].y, v[1].y, v[2].y, v[3].y);
+      store_split(hi_tile, lo_tile, r + 2, unit, v[0].z, v[1].z, v[2].z, v[3].z);
+      store_split(hi_tile, lo_tile, r + 3, unit, v[0].w, v[1].w, v[2].w, v[3].w);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) store_split(hi_tile, lo_tile, (tid >> 3) + 32 * i, unit, v[i].x, v[i].y, v[i].z, v[i].w);
+    }
+  }
+};
+
+// Four neighbouring outputs (m, n .. n + 3); what the scalar epilogue_store does for these kinds, with 16-byte accesses.
+__device__ __forceinline__ void epilogue_store4(const GemmArgs& g, int b, int m, int n, float4 acc) {
+  float* D = (float*)g.D + b * g.d_sb + (int64_t)m * g.ldd + n;
+  float v[4] = {acc.x, acc.y, acc.z, acc.w};
+  if (g.epi == EPI_GELU_FWD) {
+    float d2[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      d2[i] = gelu_prime_f(v[i]);
+      v[i] = gelu_f(v[i]);
+    }
+    *reinterpret_cast<float4*>((float*)g.D2 + b * g.d2_sb + (int64_t)m * g.ldd2 + n) = make_float4(d2[0], d2[1], d2[2], d2[3]);
+  } else if (g.epi == EPI_MUL || g.epi == EPI_ADD || g.epi == EPI_RESID) {
+    const float4 ev = *reinterpret_cast<const float4*>((const float*)g.E + b * g.e_sb + (int64_t)m * g.lde + n);
+    const float e[4] = {ev.x, ev.y, ev.z, ev.w};
+    if (g.epi == EPI_RESID) {
+      float mask[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float gate = g.gate ? ((const float*)g.gate)[b * g.gate_sb + n + i] : 1.0f;
+        v[i] = gate * e[i] + v[i];
+        mask[i] = v[i] > 0.0f ? 1.0f : 0.0f;
+        if (g.relu) v[i] = fmaxf(v[i], 0.0f);
+      }
+      if (g.relu) *reinterpret_cast<float4*>((float*)g.D2 + b * g.d2_sb + (int64_t)m * g.ldd2 + n) = make_float4(mask[0], mask[1], mask[2], mask[3]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] = g.epi == EPI_MUL ? v[i] * e[i] : v[i] + e[i];
+    }
+  }
+  *reinterpret_cast<float4*>(D) = make_float4(v[0], v[1], v[2], v[3]);
+}
+
+__global__ void __launch_bounds__(kAllThreads, 1) gemm_f32_kernel(const F32Params p) {
+  const GemmArgs& g = p.g;
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  uint8_t* aligned = smem_raw + (base - smem_u32(smem_raw));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(aligned + kStages * kStageBytes);
+  const uint32_t bar0 = smem_u32(bars);
+  auto full_bar = [&](int s) { return bar0 + 8u * s; };
+  auto empty_bar = [&](int s) { return bar0 + 8u * (kStages + s); };
+  auto accf_bar = [&](int a) { return bar0 + 8u * (2 * kStages + a); };
+  auto acce_bar = [&](int a) { return bar0 + 8u * (2 * kStages + 2 + a); };
+  const uint32_t drain_bar = bar0 + 8u * (2 * kStages + 4);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 5);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(full_bar(s), kWorkerWarps);
+      mbar_init(empty_bar(s), 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(accf_bar(a), 1);
+      mbar_init(acce_bar(a), kWorkerWarps);
+    }
+    mbar_init(drain_bar, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == kMmaWarp) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kTmemCols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+
+  const int b = blockIdx.z / g.splitk, split = blockIdx.z % g.splitk;
+  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  const int kb_lo = split * p.kb_per_split, kb_hi = min(p.k_blocks, kb_lo + p.kb_per_split);
+  const int n_kb = max(0, kb_hi - kb_lo);
+
+  if (warp < kWorkerWarps) {
+    Loader la, lb;
+    la.init((const float*)g.A + (int64_t)b * g.a_sb, g.a_sm, g.a_sk, g.M, m0, kb_lo * BK, p.a_mn != 0);
+    lb.init((const float*)g.B + (int64_t)b * g.b_sb, g.b_sn, g.b_sk, g.N, n0, kb_lo * BK, p.b_mn != 0);
+    const int k_end = min(g.K, kb_hi * BK);
+    float4 va[2][4], vb[2][4];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      la.load(k_end, va[i]);
+      lb.load(k_end, vb[i]);
+    }
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int kb = 0; kb < n_kb && ok; kb += 2) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        if (kb + i >= n_kb) break;
+        if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
+        const uint32_t s0 = base + stage * kStageBytes;
+        la.store(s0, s0 + kTile, va[i]);
+        la.load(k_end, va[i]);  // past the last block: nothing
+        lb.store(s0 + 2 * kTile, s0 + 3 * kTile, vb[i]);
+        lb.load(k_end, vb[i]);
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(full_bar(stage));
+        if (++stage == kStages) { stage = 0; phase ^= 1u; }
+      }
+    }
+  } else {
+    const int quarter = warp & 3, half = (warp >> 2) & 1;
+    const uint32_t tsrc = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * 64);
+    float sum[64];
+#pragma unroll
+    for (int i = 0; i < 64; ++i) sum[i] = 0.0f;
+    bool ok = true;
+    auto drain = [&](int kb) {  // adds k-block kb's accumulator to the sums
+      const int acc = kb & 1;
+      if (!mbar_wait(accf_bar(acc), (uint32_t)((kb >> 1) & 1), abort_flag, p.status)) { ok = false; return; }
+      tc_fence_after();
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float v[32];
+        tc_ld32(tsrc + (uint32_t)(acc * BN + h * 32), v);
+        if (h == 1) {  // read: it may be written again
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(acce_bar(acc));
+        }
+#pragma unroll
+        for (int i = 0; i < 32; ++i) sum[h * 32 + i] += v[i];
+      }
+    };
+    if (warp == kMmaWarp) {
+      uint32_t elected;
+      asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(elected));
+      const bool issuer = elected != 0;
+      const uint32_t idesc = (1u << 4) /*fp32 accumulate*/ | (2u << 7) | (2u << 10) /*tf32*/ | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+      int stage = 0;
+      uint32_t phase = 0;
+      for (int kb = 0; kb < n_kb; ++kb) {
+        const int acc = kb & 1;
+        ok = mbar_wait(full_bar(stage), phase, abort_flag, p.status) &&
+             mbar_wait(acce_bar(acc), (uint32_t)(((kb >> 1) & 1) ^ 1), abort_flag, p.status);
+        if (!ok) break;
+        tc_fence_after();
+        if (issuer) {
+          const uint32_t s0 = base + stage * kStageBytes, tmem_d = tmem_base + (uint32_t)acc * BN;
+          const uint64_t a_hi = make_desc(s0, 16u, 1024u), a_lo = make_desc(s0 + kTile, 16u, 1024u);
+          const uint64_t b_hi = make_desc(s0 + 2 * kTile, 16u, 1024u), b_lo = make_desc(s0 + 3 * kTile, 16u, 1024u);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) tc_mma_tf32(tmem_d, a_lo + 2 * k, b_hi + 2 * k, idesc, k > 0);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) tc_mma_tf32(tmem_d, a_hi + 2 * k, b_lo + 2 * k, idesc, 1u);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) tc_mma_tf32(tmem_d, a_hi + 2 * k, b_hi + 2 * k, idesc, 1u);
+          tc_commit(empty_bar(stage));
+          tc_commit(accf_bar(acc));
+        }
+        __syncwarp();
+        if (++stage == kStages) { stage = 0; phase ^= 1u; }
+        if (kb > 0) drain(kb - 1);
+        if (!ok) break;
+      }
+      if (ok && n_kb > 0) drain(n_kb - 1);
+      if (!ok) {  // let issued MMAs finish before the tensor memory is freed
+        if (issuer) tc_commit(drain_bar);
+        const uint64_t t0 = global_ns();
+        while (!mbar_try_wait(drain_bar, 0) && global_ns() - t0 < 100000000ull) {
+        }
+      }
+    } else {
+      for (int kb = 0; kb < n_kb && ok; ++kb) drain(kb);
+    }
+    // All products of this CTA are done: the stages are free.  Each warp passes its 32 x 64 sums through 32 x 36 floats of
+    // its own so that 8 lanes write 32 consecutive columns of a row.
+    if (ok) {
+      float* buf = reinterpret_cast<float*>(aligned) + (warp - kWorkerWarps) * (32 * 36);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          *reinterpret_cast<float4*>(buf + lane * 36 + 4 * i) =
+              make_float4(sum[h * 32 + 4 * i], sum[h * 32 + 4 * i + 1], sum[h * 32 + 4 * i + 2], sum[h * 32 + 4 * i + 3]);
+        __syncwarp();
+        const int n = n0 + half * 64 + h * 32 + 4 * (lane & 7);
+#pragma unroll 2
+        for (int i = 0; i < 8; ++i) {
+          const int r = 4 * i + (lane >> 3), m = m0 + quarter * 32 + r;
+          if (m >= g.M || n >= g.N) continue;
+          const float4 v = *reinterpret_cast<const float4*>(buf + r * 36 + 4 * (lane & 7));
+          if (g.splitk > 1) *reinterpret_cast<float4*>(g.partial + (((int64_t)split * g.batch + b) * g.M + m) * g.N + n) = v;
+          else epilogue_store4(g, b, m, n, v);
+        }
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == kMmaWarp) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
+  }
+}
+
+// An operand qualifies if one of its strides is 1, its 16-byte vectors are aligned and none straddles the end.
+bool operand_ok(const void* base, int64_t s_row, int64_t s_k, int64_t s_b, int batch, int rows, int K, int* mn) {
+  if ((uintptr_t)base & 15u) return false;
+  if (batch > 1 && s_b % 4) return false;
+  if (s_k == 1 && s_row % 4 == 0 && K % 4 == 0) { *mn = 0; return true; }
+  if (s_row == 1 && s_k % 4 == 0 && rows % 4 == 0) { *mn = 1; return true; }
+  return false;
+}
+
+}  // namespace
+
+bool gemm_f32_tc(Launcher& lc, const GemmArgs& g, int* status_word) {
+  if (!status_word || g.in_dtype != HBP_F32 || g.A2) return false;
+  if (g.M <= 0 || g.N <= 0 || g.K <= 0 || g.batch <= 0) return false;
+  // A few short dot products are the CUDA-core kernel's: setting up tensor memory and the pipeline takes 6 us.  32 x 256 x 64:
+  // 6.8 us against 8.6; 32 x 64 x 256: 16.5 against 14.5; 64 x 256 x 32: 12.4 against 8.3.
+  if (g.M <= 32 && g.K <= 128) return false;
+  // the epilogue's 16-byte accesses
+  auto vec = [](const void* p, int64_t ld, int64_t sb) { return !((uintptr_t)p & 15u) && ld % 4 == 0 && sb % 4 == 0; };
+  if (g.N % 4 || !vec(g.D, g.ldd, g.d_sb) || g.R) return false;
+  const bool has_e = g.epi == EPI_MUL || g.epi == EPI_ADD || g.epi == EPI_RESID;
+  if (!has_e && g.epi != EPI_STORE && g.epi != EPI_STORE_LN && g.epi != EPI_GELU_FWD) return false;
+  if (has_e && (!g.E || !vec(g.E, g.lde, g.e_sb))) return false;
+  if ((g.epi == EPI_GELU_FWD || g.relu) && (!g.D2 || !vec(g.D2, g.ldd2, g.d2_sb))) return false;
+  if (g.splitk > 1 && (g.epi != EPI_STORE || ((uintptr_t)g.partial & 15u))) return false;
+  F32Params p;
+  p.g = g;
+  if (!operand_ok(g.A, g.a_sm, g.a_sk, g.a_sb, g.batch, g.M, g.K, &p.a_mn)) return false;
+  if (!operand_ok(g.B, g.b_sn, g.b_sk, g.b_sb, g.batch, g.N, g.K, &p.b_mn)) return false;
+  const int64_t z = (int64_t)g.batch * g.splitk;
+  if (z > 65535 || (g.M + BM - 1) / BM > 65535) return false;
+  p.k_blocks = (g.K + BK - 1) / BK;
+  p.kb_per_split = (p.k_blocks + g.splitk - 1) / g.splitk;
+  p.status = status_word;
+  static PerDevice<bool> attr_done;
+  if (!attr_done.here()) {
+    if (cudaFuncSetAttribute(gemm_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    attr_done.here() = true;
+  }
+  dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, (unsigned)z);
+  gemm_f32_kernel<<<grid, kAllThreads, kSmemBytes, lc.stream>>>(p);
+  lc.count();
+  lc.check();
+  if (g.splitk > 1) reduce_splitk(lc, g.partial, (float*)g.D, g.splitk, (int64_t)g.batch * g.M * g.N);
+  return true;
+}
+
+}  // namespace hbp

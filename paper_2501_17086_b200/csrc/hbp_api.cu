@@ -11,6 +11,7 @@
 namespace hbp {
 bool gemm(Launcher& lc, const GemmArgs& g, int* status_word) {
   if (!lc.force_simt && !g.relu && gemm_tc(lc, g, status_word)) return true;
+  if (!lc.force_simt && gemm_f32_tc(lc, g, status_word)) return false;  // (no LayerNorm row sums either)
   gemm_simt(lc, g);
   return false;
 }
