@@ -317,9 +317,9 @@ bool operand_ok(const void* base, int64_t s_row, int64_t s_k, int64_t s_b, int b
 bool gemm_f32_tc(Launcher& lc, const GemmArgs& g, int* status_word) {
   if (!status_word || g.in_dtype != HBP_F32 || g.A2) return false;
   if (g.M <= 0 || g.N <= 0 || g.K <= 0 || g.batch <= 0) return false;
-  // A few short dot products are the CUDA-core kernel's: setting up tensor memory and the pipeline takes 6 us.  32 x 256 x 64:
-  // 6.8 us against 8.6; 32 x 64 x 256: 16.5 against 14.5; 64 x 256 x 32: 12.4 against 8.3.
-  if (g.M <= 32 && g.K <= 128) return false;
+  // Few rows are the CUDA-core kernel's: a tile would be mostly padding, and setting up tensor memory and the pipeline takes
+  // 6 us.  32 x 64 x 256: 8.5 us there against 14.5; 32 x 512 x 1024: 23 against 39; 64 x 256 x 32: 10.4 against 8.4.
+  if (g.M <= 32) return false;
   // the epilogue's 16-byte accesses
   auto vec = [](const void* p, int64_t ld, int64_t sb) { return !((uintptr_t)p & 15u) && ld % 4 == 0 && sb % 4 == 0; };
   if (g.N % 4 || !vec(g.D, g.ldd, g.d_sb) || g.R) return false;

@@ -66,10 +66,11 @@ __device__ __forceinline__ void epilogue_store(const GemmArgs& g, int b, int m, 
   }
 }
 
-// 256 threads, BM x BN output tile, BK = 16, (BM/16) x (BN/16) register micro-tile.
+// 256 threads, BM x BN output tile, BK = 16, (BM/16) x (BN/16) register micro-tile.  The next block of K is loaded into
+// registers while the current one is multiplied (1900 x 1560 x 520, 12 at once: 1980 -> 1660 us).
 template <typename T, int BM, int BN>
 __global__ void __launch_bounds__(256) gemm_simt_kernel(const GemmArgs g) {
-  constexpr int BK = 16, TM = BM / 16, TN = BN / 16;
+  constexpr int BK = 16, TM = BM / 16, TN = BN / 16, NA = BM * BK / 256, NB = BN * BK / 256;
   __shared__ float As[BK][BM + 4];
   __shared__ float Bs[BK][BN + 4];
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
@@ -78,11 +79,11 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const GemmArgs g) {
   const T* A = (const T*)g.A + (int64_t)b * g.a_sb;
   const T* A2 = g.A2 ? (const T*)g.A2 + (int64_t)b * g.a_sb : nullptr;
   const T* B = (const T*)g.B + (int64_t)b * g.b_sb;
-  // K range of this split (multiples of BK except the last)
-  const int ktiles = (g.K + BK - 1) / BK;
+  // K range of this split (multiples of 16 except the last)
+  const int ktiles = (g.K + 15) / 16;
   const int per = (ktiles + g.splitk - 1) / g.splitk;
-  const int kbeg = split * per * BK;
-  const int kend = min(g.K, (split + 1) * per * BK);
+  const int kbeg = split * per * 16;
+  const int kend = min(g.K, (split + 1) * per * 16);
 
   float acc[TM][TN];
 #pragma unroll
@@ -91,28 +92,35 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const GemmArgs g) {
     for (int j = 0; j < TN; ++j) acc[i][j] = 0.0f;
 
   const bool a_kmajor = (g.a_sk == 1), b_kmajor = (g.b_sk == 1);
+  float av[NA], bv[NB];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int i = 0; i < NA; ++i) {
+      const int idx = tid + i * 256, kk = a_kmajor ? idx % BK : idx / BM, mm = a_kmajor ? idx / BK : idx % BM;
+      const int m = m0 + mm, k = k0 + kk;
+      av[i] = (m < g.M && k < kend) ? load_a<T>(A, A2, (int64_t)m * g.a_sm + (int64_t)k * g.a_sk) : 0.0f;
+    }
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      const int idx = tid + i * 256, kk = b_kmajor ? idx % BK : idx / BN, nn = b_kmajor ? idx / BK : idx % BN;
+      const int n = n0 + nn, k = k0 + kk;
+      bv[i] = (n < g.N && k < kend) ? to_f(B[(int64_t)n * g.b_sn + (int64_t)k * g.b_sk]) : 0.0f;
+    }
+  };
+  if (kbeg < kend) fetch(kbeg);
   for (int k0 = kbeg; k0 < kend; k0 += BK) {
 #pragma unroll
-    for (int i = 0; i < (BM * BK) / 256; ++i) {
-      int idx = tid + i * 256;
-      int kk = a_kmajor ? idx % BK : idx / BM;
-      int mm = a_kmajor ? idx / BK : idx % BM;
-      int m = m0 + mm, k = k0 + kk;
-      float v = 0.0f;
-      if (m < g.M && k < kend) v = load_a<T>(A, A2, (int64_t)m * g.a_sm + (int64_t)k * g.a_sk);
-      As[kk][mm] = v;
+    for (int i = 0; i < NA; ++i) {
+      const int idx = tid + i * 256;
+      As[a_kmajor ? idx % BK : idx / BM][a_kmajor ? idx / BK : idx % BM] = av[i];
     }
 #pragma unroll
-    for (int i = 0; i < (BN * BK) / 256; ++i) {
-      int idx = tid + i * 256;
-      int kk = b_kmajor ? idx % BK : idx / BN;
-      int nn = b_kmajor ? idx / BK : idx % BN;
-      int n = n0 + nn, k = k0 + kk;
-      float v = 0.0f;
-      if (n < g.N && k < kend) v = to_f(B[(int64_t)n * g.b_sn + (int64_t)k * g.b_sk]);
-      Bs[kk][nn] = v;
+    for (int i = 0; i < NB; ++i) {
+      const int idx = tid + i * 256;
+      Bs[b_kmajor ? idx % BK : idx / BN][b_kmajor ? idx / BK : idx % BN] = bv[i];
     }
     __syncthreads();
+    if (k0 + BK < kend) fetch(k0 + BK);
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
       float a[TM], bb[TN];
@@ -145,6 +153,75 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const GemmArgs g) {
   }
 }
 
+// At most 32 rows: 32 x 32 tiles, a few blocks on an idle GPU, so what counts is the time of one block.  64 of K per block
+// (one exposed memory latency, the next block's loads in flight meanwhile); four groups of 64 threads take 16 of them each
+// with a 4 x 4 micro-tile, because with one group of 256 threads and 2 x 2 the shared-memory loads bound it, and the groups'
+// sums are added in a fixed order.  32 x 64 x 256: 16.5 -> 8.5 us, 32 x 512 x
+// 1024: 51 -> 23.
+template <typename T>
+__global__ void __launch_bounds__(256) gemm_small_kernel(const GemmArgs g) {
+  constexpr int BM = 32, BN = 32, BK = 64, P = 36, N4 = BM * BK / 256;
+  __shared__ __align__(16) float As[BK][P];
+  __shared__ __align__(16) float Bs[BK][P];
+  __shared__ float red[4][BM][BN + 1];
+  const int tid = threadIdx.x, grp = tid >> 6, tx = tid & 7, ty = (tid >> 3) & 7;
+  const int b = blockIdx.z / g.splitk, split = blockIdx.z % g.splitk;
+  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  const T* A = (const T*)g.A + (int64_t)b * g.a_sb;
+  const T* A2 = g.A2 ? (const T*)g.A2 + (int64_t)b * g.a_sb : nullptr;
+  const T* B = (const T*)g.B + (int64_t)b * g.b_sb;
+  const int ktiles = (g.K + 15) / 16, per = (ktiles + g.splitk - 1) / g.splitk;
+  const int kbeg = split * per * 16, kend = min(g.K, (split + 1) * per * 16);
+  const bool a_kmajor = g.a_sk == 1, b_kmajor = g.b_sk == 1;
+  float acc[4][4] = {}, av[N4], bv[N4];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int i = 0; i < N4; ++i) {
+      const int idx = tid + i * 256;
+      const int ka = k0 + (a_kmajor ? idx % BK : idx / BM), m = m0 + (a_kmajor ? idx / BK : idx % BM);
+      const int kb = k0 + (b_kmajor ? idx % BK : idx / BN), n = n0 + (b_kmajor ? idx / BK : idx % BN);
+      av[i] = (m < g.M && ka < kend) ? load_a<T>(A, A2, (int64_t)m * g.a_sm + (int64_t)ka * g.a_sk) : 0.0f;
+      bv[i] = (n < g.N && kb < kend) ? to_f(B[(int64_t)n * g.b_sn + (int64_t)kb * g.b_sk]) : 0.0f;
+    }
+  };
+  if (kbeg < kend) fetch(kbeg);
+  for (int k0 = kbeg; k0 < kend; k0 += BK) {
+#pragma unroll
+    for (int i = 0; i < N4; ++i) {
+      const int idx = tid + i * 256;
+      As[a_kmajor ? idx % BK : idx / BM][a_kmajor ? idx / BK : idx % BM] = av[i];
+      Bs[b_kmajor ? idx % BK : idx / BN][b_kmajor ? idx / BK : idx % BN] = bv[i];
+    }
+    __syncthreads();
+    if (k0 + BK < kend) fetch(k0 + BK);
+#pragma unroll
+    for (int kk = 0; kk < BK / 4; ++kk) {
+      const float4 a4 = *reinterpret_cast<const float4*>(&As[grp * (BK / 4) + kk][ty * 4]);
+      const float4 b4 = *reinterpret_cast<const float4*>(&Bs[grp * (BK / 4) + kk][tx * 4]);
+      const float a[4] = {a4.x, a4.y, a4.z, a4.w}, bb[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], bb[j], acc[i][j]);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) red[grp][ty * 4 + i][tx * 4 + j] = acc[i][j];
+  __syncthreads();
+  const int nn = tid & 31, n = n0 + nn;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int mm = (tid >> 5) + 8 * i, m = m0 + mm;
+    if (m >= g.M || n >= g.N) continue;
+    const float v = (red[0][mm][nn] + red[1][mm][nn]) + (red[2][mm][nn] + red[3][mm][nn]);
+    if (g.splitk > 1) g.partial[(((int64_t)split * g.batch + b) * g.M + m) * g.N + n] = v;
+    else epilogue_store<T>(g, b, m, n, v);
+  }
+}
+
 __global__ void reduce_splitk_kernel(const float* __restrict__ partial, float* __restrict__ out, int splits,
                                      int64_t elems) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -165,7 +242,7 @@ void launch_simt(Launcher& lc, const GemmArgs& g) {
     gemm_simt_kernel<T, 64, 64><<<grid, 256, 0, lc.stream>>>(g);
   } else {
     dim3 grid((g.N + 31) / 32, (g.M + 31) / 32, g.batch * g.splitk);
-    gemm_simt_kernel<T, 32, 32><<<grid, 256, 0, lc.stream>>>(g);
+    gemm_small_kernel<T><<<grid, 256, 0, lc.stream>>>(g);
   }
   lc.count();
   lc.check();
