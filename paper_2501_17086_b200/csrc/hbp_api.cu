@@ -331,8 +331,8 @@ struct Run {
   }
 
   // ---- MLP block: u = J^T g for layers [b0, b1) (b1 - b0 <= group), from states g[step+1] -------
-  // dA = G W2, dZ = dA * gelu'(Z) -> H1 (cached derivative);  dY = dZ W1 -> U[step].
-  void mlp_vjp(int b0, int b1, bool want_dy) {
+  // dA = G W2, dZ = dA * gelu'(Z) -> H1 from layer `slot` on (cached derivative);  dY = dZ W1 -> U[step].
+  void mlp_vjp(int b0, int b1, bool want_dy, int slot = 0) {
     const int nb = b1 - b0, ss = step_stride();
     GemmArgs a = base_args();
     a.M = (int)N; a.N = (int)h; a.K = (int)d; a.batch = nb;
@@ -340,12 +340,13 @@ struct Run {
     a.B = at(p->W2, (int64_t)b0 * d * h); a.b_sn = 1; a.b_sk = h; a.b_sb = d * h;
     a.epi = EPI_MUL;
     a.E = at(c->DACT, (int64_t)b0 * N * h); a.lde = h; a.e_sb = N * h;
-    a.D = c->H1; a.ldd = h; a.d_sb = N * h;
+    const char* dz = at(c->H1, (int64_t)slot * N * h);
+    a.D = const_cast<char*>(dz); a.ldd = h; a.d_sb = N * h;
     run_gemm(a);
     if (!want_dy) return;
     GemmArgs b = base_args();
     b.M = (int)N; b.N = (int)d; b.K = (int)h; b.batch = nb;
-    b.A = c->H1; b.a_sm = h; b.a_sk = 1; b.a_sb = N * h;
+    b.A = dz; b.a_sm = h; b.a_sk = 1; b.a_sb = N * h;
     b.B = at(p->W1, (int64_t)b0 * h * d); b.b_sn = 1; b.b_sk = d; b.b_sb = h * d;
     b.epi = EPI_STORE;
     b.D = at(c->U, (int64_t)mlp_step(b0) * state); b.ldd = d; b.d_sb = ss * state;
@@ -1163,19 +1164,27 @@ static hbp_status backward_common(hbp_ctx* ctx, const hbp_params* params, int32_
       }
       if (grads) r.lstm_wgrad(grads);
     } else {
+      // The chain of steps needs no parameter gradient: those of a whole group of layers (of all layers, for attention)
+      // follow in one batched product each, from the dZ (dQKV) the chain left behind.  One layer's weight gradient is 4 to
+      // 32 tiles for 148 SMs: a decoder of 6 layers, 512 wide, 2664 rows, 1590 -> 890 us.
+      int lo = 0, hi = 0;  // layers whose dZ is in H1, once the chain has come down to lo
       for (int l = steps - 1; l >= 0; --l) {
         const int b = tr ? l / 2 : l;
         const bool is_mlp = !tr || (l % 2 == 1);
         if (is_mlp) {
+          if (l == steps - 1 || b < lo) {
+            hi = b + 1;
+            lo = hi > ctx->group ? hi - ctx->group : 0;
+          }
           r.mask_gradients(b, b + 1);
-          r.mlp_vjp(b, b + 1, true);
-          if (grads) r.mlp_wgrad(b, b + 1, grads);
+          r.mlp_vjp(b, b + 1, true, b - lo);
+          if (grads && b == lo) r.mlp_wgrad(lo, hi, grads);
         } else {
           r.attn_vjp(b, b + 1, true);
-          if (grads) r.attn_wgrad(b, b + 1, grads);
         }
         r.scan_with_u(l, l + 1);
       }
+      if (grads && tr) r.attn_wgrad(0, ctx->layers, grads);
     }
     if (grads) r.gate_grads(grads);
   }
