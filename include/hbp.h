@@ -262,6 +262,14 @@ int64_t hbp_launch_count(const hbp_ctx* ctx);
  * device, so one process may hold contexts on several GPUs (each used with its device current). */
 int32_t hbp_context_modes(const hbp_ctx* ctx);
 
+/* Diagnostic, host only (no GPU is needed): how the one-launch recurrence of a cell is split - the forward pass of GRU and
+ * LSTM, exact backpropagation (backward != 0) of all three cells - on a device that runs at_once[cs] clusters of cs CTAs at
+ * a time (17 entries, cs = 0..16).  plan (8 entries) receives the units per CTA, the CTAs per cluster, the batch rows per
+ * cluster, the warps that share a tile's contraction (forward), the threads per CTA, the bytes of shared memory, the
+ * 16-byte words of packed weights, and one past the last of them that any thread reads; *pack_bytes what the workspace holds
+ * for them.  HBP_ERR_UNSUPPORTED: there is no such split, the cell runs one launch per step. */
+hbp_status hbp_recurrence_plan(const hbp_config* cfg, int32_t backward, const int32_t* at_once, int64_t* plan, size_t* pack_bytes);
+
 const char* hbp_status_string(hbp_status s);
 void hbp_destroy(hbp_ctx* ctx);
 

@@ -21,7 +21,7 @@ LOSS_FINAL, LOSS_EVERY_STEP = 0, 1
 
 EXPORTS = ["hbp_workspace_bytes", "hbp_create", "hbp_forward", "hbp_backward", "hbp_exact",
            "hbp_cumsumprod_scratch_bytes", "hbp_cumsumprod", "hbp_cumsumprod_status", "hbp_sync_status", "hbp_launch_count",
-           "hbp_context_modes", "hbp_selftest_wait_timeout",
+           "hbp_context_modes", "hbp_selftest_wait_timeout", "hbp_recurrence_plan",
            "hbp_profile_enable", "hbp_profile_read", "hbp_cumsumprod_static", "hbp_cumsumprod_static_max_bytes",
            "hbp_compare_scratch_bytes", "hbp_compare", "hbp_iterate", "hbp_add_carry", "hbp_param_grads",
            "hbp_status_string", "hbp_destroy"]
@@ -63,6 +63,7 @@ def _load():
     lib.hbp_cumsumprod.argtypes = [i32, i32, i32, i32, i64, i32, vp, vp, vp, vp, vp, sz, vp]
     lib.hbp_cumsumprod_status.argtypes = [i32, i32, i32, i32, i64, i32, vp, vp, vp, vp, vp, sz, vp, vp]
     lib.hbp_selftest_wait_timeout.argtypes = [vp, vp, sz, C.c_uint64, vp]
+    lib.hbp_recurrence_plan.argtypes = [C.POINTER(hbp_config), i32, C.POINTER(i32), C.POINTER(i64), C.POINTER(sz)]
     lib.hbp_context_modes.argtypes = [vp]
     lib.hbp_context_modes.restype = i32
     lib.hbp_cumsumprod_static.argtypes = [i32, i32, i32, i32, i64, i32, vp, vp, vp, vp, vp]
@@ -135,6 +136,18 @@ def workspace_bytes(cfg: hbp_config) -> int:
     n = C.c_size_t(0)
     _check(lib.hbp_workspace_bytes(C.byref(cfg), C.byref(n)), "hbp_workspace_bytes")
     return n.value
+
+
+def recurrence_plan(cfg: hbp_config, backward: bool, at_once) -> dict | None:
+    """The split of a cell's one-launch recurrence where ``at_once[cs]`` clusters of cs CTAs run at a time (17 entries),
+    or None where the cell runs one launch per step.  Needs no GPU."""
+    out, pack = (C.c_int64 * 8)(), C.c_size_t(0)
+    code = lib.hbp_recurrence_plan(C.byref(cfg), int(backward), (C.c_int32 * 17)(*at_once), out, C.byref(pack))
+    if code == 6:
+        return None
+    _check(code, "hbp_recurrence_plan")
+    names = ("units_per_cta", "cluster", "rows", "ksplit", "threads", "smem", "packed_words", "words_read")
+    return {**{n: int(v) for n, v in zip(names, out)}, "pack_bytes": pack.value}
 
 
 _GRAD_SHAPES = {

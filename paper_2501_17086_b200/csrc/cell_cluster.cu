@@ -118,6 +118,13 @@ __device__ __forceinline__ void tanh_pair(double v, double& t, double& s) {
   s = 4.0 * e * q * q;
 }
 
+// The warps that share a tile's contraction take its blocks in turn: warp ks takes blocks ks, ks + ks_n, ...  How many those
+// are (none for a warp beyond the last block: few inputs have one block of U for up to eight warps, and such a warp's base
+// lies past the packed blocks) ...
+__host__ __device__ constexpr int block_share(int blocks, int ks, int ks_n) { return ks < blocks ? (blocks - ks + ks_n - 1) / ks_n : 0; }
+// ... and which of them, out of n > 0 with `res` of them resident, ring slot s starts with (the last one again past the end).
+__host__ __device__ constexpr int ahead_block(int res, int s, int n) { return res + s < n ? res + s : n - 1; }
+
 // ------------------------------------------------------------------------------------------------ forward
 // The contraction index runs in blocks of 16 units; within a block lane c = l % 4 holds units 4c .. 4c + 3, one per
 // matrix instruction, so that a lane's share of W is one 16-byte load and its share of h two.  Outputs are finished one
@@ -157,7 +164,7 @@ __global__ void __launch_bounds__(max_threads(MT, EX), 1) cell_forward_kernel(co
 #pragma unroll
     for (int g = 0; g < G; ++g) b[g] = __ldg(M + (j * ks_n * G + g) * 32);
   };
-  const int jh = (kbh - ks + ks_n - 1) / ks_n, jx = ks < kbx ? (kbx - ks + ks_n - 1) / ks_n : 0;
+  const int jh = block_share(kbh, ks, ks_n), jx = block_share(kbx, ks, ks_n);
   const int res = min(p.res, jh), res_x = min(p.res_x, jx);
   const float4* my_w = wres + warp * p.res * G * 32 + lane;
   const float4* my_u = ures + warp * p.res_x * G * 32 + lane;
@@ -262,8 +269,10 @@ __global__ void __launch_bounds__(max_threads(MT, EX), 1) cell_forward_kernel(co
           }
       };
       float4 pre[kAhead][G];
+      if (jx > res_x) {
 #pragma unroll
-      for (int s = 0; s < kAhead; ++s) load_rows(gU, min(res_x + s, max(jx - 1, 0)), pre[s]);
+        for (int s = 0; s < kAhead; ++s) load_rows(gU, ahead_block(res_x, s, jx), pre[s]);
+      }
       if (p.stage_x) ok = bar_wait_cluster(xbar0 + 8 * cur, (uint32_t)((t >> 1) & 1), abort_flag) && ok;
       for (int j = 0; j < res_x; ++j) {
         float4 b[G];
@@ -285,7 +294,7 @@ __global__ void __launch_bounds__(max_threads(MT, EX), 1) cell_forward_kernel(co
     }
     float4 pre[kAhead][G];  // the first streamed blocks of W do not depend on the exchange either
 #pragma unroll
-    for (int s = 0; s < kAhead; ++s) load_rows(gW, min(res + s, jh - 1), pre[s]);
+    for (int s = 0; s < kAhead; ++s) load_rows(gW, ahead_block(res, s, jh), pre[s]);
     if (t > 0) ok = bar_wait_cluster(bar0 + 8 * cur, (uint32_t)(((t - 1) >> 1) & 1), abort_flag) && ok;
     if (ok) {
       const unsigned char* vb = cell_smem + cur * buf_bytes;
@@ -843,6 +852,30 @@ bool make_plan(int cell, bool bwd, int es, int64_t B, int u, int in, ActiveClust
   return best->uc != 0;
 }
 
+// One past the last 16-byte word of the packed weights (W, then U) that any lane reads under a plan, by the kernels' own
+// index arithmetic: the last warps of the last CTA reach furthest.
+int64_t packed_words_read(bool bwd, int gates, int in, const Plan& q) {
+  if (bwd) return packed_size(true, gates, q.cs * q.uc, in, q.uc).w;  // group < groups, block < kc by construction
+  const int kbh = (q.cs * q.uc + 15) / 16, kbx = (in + 15) / 16;
+  const int64_t tiles = (int64_t)q.cs * q.uc / 8, n_w = tiles * kbh * gates * 32;
+  int64_t end = 0;
+  for (int ks = 0; ks < q.ksplit; ++ks) {
+    const int jh = block_share(kbh, ks, q.ksplit), jx = block_share(kbx, ks, q.ksplit);
+    const int64_t w = ((tiles - 1) * kbh + ks) * gates * 32, x = n_w + ((tiles - 1) * kbx + ks) * gates * 32;
+    auto reach = [&](int64_t base, int j) {
+      const int64_t e = base + ((int64_t)j * q.ksplit * gates + gates) * 32;
+      if (e > end) end = e;
+    };
+    for (int j = 0; j < jh; ++j) reach(w, j);
+    for (int j = 0; j < jx; ++j) reach(x, j);
+    for (int s = 0; s < 4; ++s) {
+      reach(w, ahead_block(q.res, s, jh));
+      if (jx > q.res_x) reach(x, ahead_block(q.res_x, s, jx));
+    }
+  }
+  return end;
+}
+
 template <typename T, int CELL, bool BWD, int MT, int EX>
 auto cell_kernel() {
   if constexpr (BWD) return cell_backward_kernel<T, CELL, MT, EX>;
@@ -924,6 +957,17 @@ size_t cell_pack_bytes(int block, int u, int in_dim) {
     if (n > most) most = n;
   }
   return most;
+}
+
+bool cell_plan(int block, int dtype, bool backward, int64_t B, int u, int in_dim, const int32_t* at_once, int64_t* out) {
+  const int cell = block == HBP_BLOCK_GRU ? CELL_GRU : (block == HBP_BLOCK_LSTM ? CELL_LSTM : CELL_RNN);
+  const int gates = cell == CELL_RNN ? 1 : (cell == CELL_GRU ? 3 : 4), in = backward ? 0 : in_dim;
+  Plan q;
+  if (!make_plan(cell, backward, dtype == HBP_F32 ? 4 : 2, B, u, in, [&](int, int, int cs) { return (int)at_once[cs]; }, &q)) return false;
+  const Packed n = packed_size(backward, gates, u, in, q.uc);
+  const int64_t v[8] = {q.uc, q.cs, q.rows, q.ksplit, q.threads, (int64_t)q.smem, (int64_t)n.w + n.x, packed_words_read(backward, gates, in, q)};
+  for (int i = 0; i < 8; ++i) out[i] = v[i];
+  return true;
 }
 
 bool cell_forward_cluster(Launcher& lc, int dtype, int block, const void* W, const void* U, const void* X, const void* gate,

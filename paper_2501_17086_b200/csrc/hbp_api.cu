@@ -868,6 +868,18 @@ int64_t hbp_launch_count(const hbp_ctx* ctx) { return ctx ? ctx->launches : 0; }
 
 int32_t hbp_context_modes(const hbp_ctx* ctx) { return ctx ? (ctx->force_simt ? 1 : 0) | (ctx->gemm_pair ? 2 : 0) | (ctx->scan_operand ? 4 : 0) : 0; }
 
+hbp_status hbp_recurrence_plan(const hbp_config* cfg, int32_t backward, const int32_t* at_once, int64_t* plan, size_t* pack_bytes) {
+  if (!at_once || !plan || !pack_bytes) return HBP_ERR_INVALID_ARG;
+  const hbp_status st = check_config(cfg);
+  if (st != HBP_OK) return st;
+  const bool rnn = cfg->block == HBP_BLOCK_RNN_TANH;
+  if (!(rnn && backward) && cfg->block != HBP_BLOCK_GRU && cfg->block != HBP_BLOCK_LSTM) return HBP_ERR_UNSUPPORTED;
+  const int u = cfg->block == HBP_BLOCK_LSTM ? cfg->d / 2 : cfg->d;
+  *pack_bytes = cell_pack_bytes(cfg->block, u, cfg->in_dim);
+  if (!*pack_bytes || !cell_plan(cfg->block, cfg->dtype, backward != 0, cfg->tokens, u, cfg->in_dim, at_once, plan)) return HBP_ERR_UNSUPPORTED;
+  return HBP_OK;
+}
+
 hbp_status hbp_sync_status(hbp_ctx* ctx, void* cuda_stream) {
   if (!ctx) return HBP_ERR_INVALID_ARG;
   int word = 0;

@@ -1,0 +1,38 @@
+"""The splits of the one-launch recurrences, looked over on the host: what a plan makes the kernels read and hold stays within
+what is there for it."""
+import pytest
+
+from paper_2501_17086_b200.build import build_library
+
+# clusters of cs CTAs that a B200 runs at a time, cs = 0..16 (fewer than 148 / cs: a cluster stays within one GPC)
+AT_ONCE = [0, 148, 74, 45, 35, 28, 22, 15, 15, 15, 11, 7, 7, 7, 7, 7, 7]
+
+
+@pytest.fixture(scope="module")
+def B():
+    build_library()
+    from paper_2501_17086_b200 import binding
+    return binding
+
+
+def _config(B, block, dtype, u, rows, nin):
+    return B.make_config(block, dtype, 4, 2 * u if block == "lstm" else u, rows, hidden=u if block == "lstm" else 0, in_dim=nin,
+                         batch=rows, loss=B.LOSS_EVERY_STEP)
+
+
+@pytest.mark.parametrize("block", ["gru", "lstm", "rnn_tanh"])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_plans_stay_inside_the_packed_weights_and_shared_memory(B, block, dtype):
+    for u in (8, 16, 64, 72, 128, 200, 264, 512):
+        for rows in (1, 9, 32, 128, 200):
+            for nin in (8, 16, 24, 64, 212 if dtype == "f32" else 216):
+                for backward in (False, True):
+                    p = B.recurrence_plan(_config(B, block, dtype, u, rows, nin), backward, AT_ONCE)
+                    if block == "rnn_tanh" and not backward:
+                        assert p is None
+                        continue
+                    assert p is not None, (u, rows, nin, backward)
+                    assert p["words_read"] <= p["packed_words"], (u, rows, nin, backward, p)
+                    assert p["packed_words"] * 16 <= p["pack_bytes"]
+                    assert p["smem"] <= 227 * 1024 and p["threads"] <= 384 and p["cluster"] <= 16
+                    assert p["cluster"] * p["units_per_cta"] >= u and p["rows"] <= 24
