@@ -31,6 +31,9 @@ constexpr int kStages = 3;
 constexpr uint32_t kTile = BM * BK * 4, kStageBytes = 4 * kTile;  // A hi, A lo, B hi, B lo
 constexpr uint32_t kTmemCols = 256;
 constexpr int kSmemBytes = kStages * (int)kStageBytes + 1024 /*alignment*/ + 256 /*barriers*/;
+// what each adding warp uses of the stages once all products are done (refine_non_finite's two blocks, or the epilogue's one)
+constexpr int kRowPitch = 33, kColPitch = 68, kWarpFloats = BK * kRowPitch + BK * kColPitch;
+static_assert(kWorkerWarps * kWarpFloats * 4 <= kStages * (int)kStageBytes && 32 * 36 <= kWarpFloats, "stages");
 
 struct F32Params {
   GemmArgs g;
@@ -41,7 +44,8 @@ struct F32Params {
 
 // v = hi + lo + (what a third tf32 term would hold).  The tensor core ignores the low 13 bits of an operand, so hi is
 // rounded (truncated where rounding would reach infinity) and cleared and lo only rounded; integer operations, because the
-// conversion instruction runs at a fraction of their rate.  An infinity stands for itself.
+// conversion instruction runs at a fraction of their rate.  An infinity or a NaN leaves hi infinite or NaN, so that every sum
+// it enters is one of the two (which, refine_non_finite settles).
 __device__ __forceinline__ void split_tf32x2(float v, uint32_t& hi, uint32_t& lo) {
   const uint32_t u = __float_as_uint(v);
   const float mag = fabsf(v);
@@ -131,6 +135,51 @@ __device__ __forceinline__ void epilogue_store4(const GemmArgs& g, int b, int m,
     }
   }
   *reinterpret_cast<float4*>(D) = make_float4(v[0], v[1], v[2], v[3]);
+}
+
+// The sums of one warp's 32 x 64 outputs that are infinite or NaN, formed again as plain float sums in ascending order of k.
+// Three products of parts do not give what one product of the whole does there: an infinity times a remainder of zero, or of
+// the other sign, is NaN where infinity times the operand is infinity, a NaN may lose its payload and become an infinity, and a
+// part may overflow where the sum does not.  Whatever the operands, a finite sum has met neither.
+__device__ __forceinline__ void refine_non_finite(const GemmArgs& g, int b, int m0, int n0, int k_lo, int k_hi, float* smem, float (&sum)[64]) {
+  const int lane = threadIdx.x & 31;
+  float *As = smem, *Bs = smem + BK * kRowPitch;  // [k][row], [k][column]
+  const float* A = (const float*)g.A + (int64_t)b * g.a_sb;
+  const float* B = (const float*)g.B + (int64_t)b * g.b_sb;
+  // a [rows] x [BK] block, lanes along the index that is contiguous
+  auto stage = [&](float* to, int pitch, const float* from, int64_t s_row, int64_t s_k, int row0, int rows, int extent, int k0) {
+    for (int i = lane; i < rows * BK; i += 32) {
+      const int r = s_k == 1 ? i / BK : i % rows, kk = s_k == 1 ? i % BK : i / rows;
+      to[kk * pitch + r] = (row0 + r < extent && k0 + kk < k_hi) ? __ldg(from + (int64_t)(row0 + r) * s_row + (int64_t)(k0 + kk) * s_k) : 0.0f;
+    }
+  };
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    float acc[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) acc[i] = 0.0f;
+    for (int k0 = k_lo; k0 < k_hi; k0 += BK) {
+      __syncwarp();
+      stage(As, kRowPitch, A, g.a_sm, g.a_sk, m0, 32, g.M, k0);
+      stage(Bs, kColPitch, B, g.b_sn, g.b_sk, n0 + 32 * h, 32, g.N, k0);
+      __syncwarp();
+#pragma unroll 1
+      for (int kk = 0; kk < min(BK, k_hi - k0); ++kk) {
+        const float a = As[kk * kRowPitch + lane];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float4 v = *reinterpret_cast<const float4*>(Bs + kk * kColPitch + 4 * i);
+          acc[4 * i] = fmaf(a, v.x, acc[4 * i]);
+          acc[4 * i + 1] = fmaf(a, v.y, acc[4 * i + 1]);
+          acc[4 * i + 2] = fmaf(a, v.z, acc[4 * i + 2]);
+          acc[4 * i + 3] = fmaf(a, v.w, acc[4 * i + 3]);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 32; ++i)
+      if (!(fabsf(sum[32 * h + i]) < __uint_as_float(0x7f800000u))) sum[32 * h + i] = acc[i];
+  }
 }
 
 __global__ void __launch_bounds__(kAllThreads, 1) gemm_f32_kernel(const F32Params p) {
@@ -274,7 +323,12 @@ __global__ void __launch_bounds__(kAllThreads, 1) gemm_f32_kernel(const F32Param
     // All products of this CTA are done: the stages are free.  Each warp passes its 32 x 64 sums through 32 x 36 floats of
     // its own so that 8 lanes write 32 consecutive columns of a row.
     if (ok) {
-      float* buf = reinterpret_cast<float*>(aligned) + (warp - kWorkerWarps) * (32 * 36);
+      float* buf = reinterpret_cast<float*>(aligned) + (warp - kWorkerWarps) * kWarpFloats;
+      bool finite = true;
+#pragma unroll
+      for (int i = 0; i < 64; ++i) finite = finite && fabsf(sum[i]) < __uint_as_float(0x7f800000u);
+      if (__any_sync(0xffffffffu, !finite))
+        refine_non_finite(g, b, m0 + quarter * 32, n0 + half * 64, kb_lo * BK, min(g.K, kb_hi * BK), buf, sum);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         __syncwarp();

@@ -41,3 +41,36 @@ def test_non_finite_inputs_stay_non_finite():
         ctx.sync_status()
     assert torch.equal(finite[0][0], finite[1][0])
     assert torch.equal(finite[0][1].all(dim=1), finite[1][1].all(dim=1))
+
+
+def test_infinities_and_nans_have_the_value_a_plain_sum_gives():
+    """Weights of one sign per row, so that an infinite state element makes whole rows of the next state +inf or -inf (in three
+    products of parts an infinity meets remainders that are zero or of the other sign: NaN); 0.5 is exact in the tensor core's
+    type, the NaN's payload lies only in the bits it drops, and -3.4e38 is next to the largest float."""
+    w = Workload("t", "mlp", "f32", L=1, d=256, hidden=320, tokens=200, batch=1, seq=1, seed=8200)
+    inp = make_inputs(w, "cuda")
+    sign = torch.where(torch.arange(w.d, device="cuda") % 3 == 0, -1.0, 1.0)
+    inp["W1"].abs_()
+    inp["W1"][0, :160] = 0.5
+    inp["W2"].abs_().mul_(sign[None, :, None])
+    x0 = inp["x0"].abs_()
+    x0[3, 5], x0[40, 1], x0[150, 63] = float("inf"), float("inf"), -3.4e38
+    x0.view(torch.int32)[77, 0] = 0x7f800001
+    states = []
+    for simt in (False, True):
+        if simt:
+            os.environ["HBP_FORCE_SIMT"] = "1"
+        try:
+            ctx = harness.make_context(w)
+        finally:
+            os.environ.pop("HBP_FORCE_SIMT", None)
+        states.append(ctx.forward(harness.params_for(w, inp), x0)[1].clone())
+        ctx.sync_status()
+    got, want = states
+    assert torch.isinf(want[3]).all() and torch.isinf(want[40]).all() and torch.isnan(want[77]).all()
+    assert torch.equal(torch.isnan(got), torch.isnan(want))
+    assert torch.equal(torch.isinf(got), torch.isinf(want))
+    assert torch.equal(got[torch.isinf(want)], want[torch.isinf(want)])   # the signs
+    rest = torch.isfinite(want)
+    rest[150] = False
+    assert float((got[rest] - want[rest]).norm() / want[rest].norm()) < 1e-6
