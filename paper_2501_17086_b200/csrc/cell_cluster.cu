@@ -921,7 +921,10 @@ bool run_cell(Launcher& lc, CellArgs a) {
                   : q.mt == 1 ? cudaLaunchKernelEx(&cfg, cell_kernel<T, CELL, BWD, 1, 0>(), a)
                   : q.mt == 2 ? cudaLaunchKernelEx(&cfg, cell_kernel<T, CELL, BWD, 2, 0>(), a)
                               : cudaLaunchKernelEx(&cfg, cell_kernel<T, CELL, BWD, 3, 0>(), a);
-  if (e != cudaSuccess && lc.err == cudaSuccess) lc.err = e;
+  if (e != cudaSuccess) {  // clusters of this size cannot be placed here: the caller runs another form
+    cudaGetLastError();
+    return false;
+  }
   lc.count();
   lc.check();
   return true;

@@ -372,7 +372,10 @@ bool run_rnn(Launcher& lc, RnnArgs a) {
     e = q.mt == 1 ? launch(rnn_cluster_kernel<T, 1, 4, PARTS>) : (q.mt == 2 ? launch(rnn_cluster_kernel<T, 2, 4, PARTS>) : launch(rnn_cluster_kernel<T, 3, 4, PARTS>));
   else
     e = q.mt == 1 ? launch(rnn_cluster_kernel<T, 1, 8, PARTS>) : (q.mt == 2 ? launch(rnn_cluster_kernel<T, 2, 8, PARTS>) : launch(rnn_cluster_kernel<T, 3, 8, PARTS>));
-  if (e != cudaSuccess && lc.err == cudaSuccess) lc.err = e;
+  if (e != cudaSuccess) {  // clusters of this size cannot be placed here: the caller runs another form
+    cudaGetLastError();
+    return false;
+  }
   lc.count();
   lc.check();
   return true;

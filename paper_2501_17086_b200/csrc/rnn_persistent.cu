@@ -336,7 +336,10 @@ bool launch_persistent(Launcher& lc, const PersistArgs& a, bool ask) {
   if (ask) return st >= (a.B + kR - 1) / kR;  // whether all clusters would run at once
   if (st < 1) return false;
   cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, a);
-  if (e != cudaSuccess && lc.err == cudaSuccess) lc.err = e;
+  if (e != cudaSuccess) {  // clusters of this size cannot be placed here: the caller runs another form
+    cudaGetLastError();
+    return false;
+  }
   lc.count();
   lc.check();
   return true;
