@@ -262,6 +262,11 @@ int64_t hbp_launch_count(const hbp_ctx* ctx);
  * device, so one process may hold contexts on several GPUs (each used with its device current). */
 int32_t hbp_context_modes(const hbp_ctx* ctx);
 
+/* Diagnostic: the functions that the one-launch recurrences of GRU and LSTM form their gates from, in double, at v [n]
+ * (device): out [n][6] (device) receives e^-|v|, 1 / (1 + e^-|v|), sigmoid(v), 1 - sigmoid(v), tanh(v), 1 - tanh(v)^2.  n up
+ * to 2^32. */
+hbp_status hbp_selftest_gate_math(const double* v, double* out, int64_t n, void* cuda_stream);
+
 /* Diagnostic, host only (no GPU is needed): how the one-launch recurrence of a cell is split - the forward pass of GRU and
  * LSTM, exact backpropagation (backward != 0) of all three cells - on a device that runs at_once[cs] clusters of cs CTAs at
  * a time (17 entries, cs = 0..16).  plan (8 entries) receives the units per CTA, the CTAs per cluster, the batch rows per

@@ -21,7 +21,7 @@ LOSS_FINAL, LOSS_EVERY_STEP = 0, 1
 
 EXPORTS = ["hbp_workspace_bytes", "hbp_create", "hbp_forward", "hbp_backward", "hbp_exact",
            "hbp_cumsumprod_scratch_bytes", "hbp_cumsumprod", "hbp_cumsumprod_status", "hbp_sync_status", "hbp_launch_count",
-           "hbp_context_modes", "hbp_selftest_wait_timeout", "hbp_recurrence_plan",
+           "hbp_context_modes", "hbp_selftest_wait_timeout", "hbp_selftest_gate_math", "hbp_recurrence_plan",
            "hbp_profile_enable", "hbp_profile_read", "hbp_cumsumprod_static", "hbp_cumsumprod_static_max_bytes",
            "hbp_compare_scratch_bytes", "hbp_compare", "hbp_iterate", "hbp_add_carry", "hbp_param_grads",
            "hbp_status_string", "hbp_destroy"]
@@ -63,6 +63,7 @@ def _load():
     lib.hbp_cumsumprod.argtypes = [i32, i32, i32, i32, i64, i32, vp, vp, vp, vp, vp, sz, vp]
     lib.hbp_cumsumprod_status.argtypes = [i32, i32, i32, i32, i64, i32, vp, vp, vp, vp, vp, sz, vp, vp]
     lib.hbp_selftest_wait_timeout.argtypes = [vp, vp, sz, C.c_uint64, vp]
+    lib.hbp_selftest_gate_math.argtypes = [vp, vp, i64, vp]
     lib.hbp_recurrence_plan.argtypes = [C.POINTER(hbp_config), i32, C.POINTER(i32), C.POINTER(i64), C.POINTER(sz)]
     lib.hbp_context_modes.argtypes = [vp]
     lib.hbp_context_modes.restype = i32
@@ -136,6 +137,15 @@ def workspace_bytes(cfg: hbp_config) -> int:
     n = C.c_size_t(0)
     _check(lib.hbp_workspace_bytes(C.byref(cfg), C.byref(n)), "hbp_workspace_bytes")
     return n.value
+
+
+def gate_math(v):
+    """e^-|v|, 1 / (1 + e^-|v|), sigmoid(v), 1 - sigmoid(v), tanh(v), 1 - tanh(v)^2 of a float64 device tensor [n] as the
+    one-launch recurrences form them: [n, 6]."""
+    assert v.is_cuda and v.is_contiguous() and v.dtype == torch.float64
+    out = torch.empty((v.numel(), 6), dtype=torch.float64, device=v.device)
+    _check(lib.hbp_selftest_gate_math(_ptr(v), _ptr(out), v.numel(), _stream()), "hbp_selftest_gate_math")
+    return out
 
 
 def recurrence_plan(cfg: hbp_config, backward: bool, at_once) -> dict | None:

@@ -79,9 +79,10 @@ struct CellArgs {
   int stage_x;          // forward: the inputs of a step are copied to shared memory one step ahead
 };
 
-// e^x for x <= 0 (or NaN), 0 below -708 to within the smallest normal number: x = k ln 2 + r with |r| <= ln 2 / 2 and
-// the Taylor polynomial of degree 13 in r (remainder 4e-18), evaluated pairwise.  Without branches, so that the gates of
-// the two units a thread owns run interleaved: with exp() and the division operator a GRU's step spent 2870 clocks here.
+// e^x for x <= 0 (or NaN), below -708 the value there, 3.3e-308 (zero in float): x = k ln 2 + r with |r| <= ln 2 / 2 and
+// the Taylor polynomial of degree 13 in r (remainder 4e-18), evaluated pairwise: within one unit in the last place.  Without
+// branches, so that the gates of the two units a thread owns run interleaved: with exp() and the division operator a GRU's
+// step spent 2870 clocks here.
 __device__ __forceinline__ double exp_nonpos(double x) {
   x = x < -708.0 ? -708.0 : x;
   constexpr double kRound = 6755399441055744.0;  // 1.5 * 2^52: adding it leaves the nearest integer in the low word
@@ -95,10 +96,10 @@ __device__ __forceinline__ double exp_nonpos(double x) {
   const double a4 = fma(r, 1.0 / 362880.0, 1.0 / 40320.0), a5 = fma(r, 1.0 / 39916800.0, 1.0 / 3628800.0);
   const double a6 = fma(r, 1.0 / 6227020800.0, 1.0 / 479001600.0);
   const double b1 = fma(r2, a2, a1), b2 = fma(r2, a4, a3), b3 = fma(r2, a6, a5);
-  const double p = 1.0 + fma(r2, fma(r8, b3, fma(r4, b2, b1)), r);  // 1 last: below one unit in the last place
+  const double p = 1.0 + fma(r2, fma(r8, b3, fma(r4, b2, b1)), r);
   return p * __hiloint2double((1023 + k) << 20, 0);
 }
-// 1 / d for d in [1, 2] by Newton's iteration from the hardware's estimate
+// 1 / d for d in [1, 2], within one unit in the last place, by Newton's iteration from the hardware's estimate
 __device__ __forceinline__ double recip(double d) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
@@ -725,6 +726,17 @@ __global__ void __launch_bounds__(max_threads(MT, EX), 1) cell_backward_kernel(c
   tc::cluster_sync();
 }
 
+// the functions of the gates on their own: out[i] = {e^-|v|, 1 / (1 + e^-|v|), sigmoid(v), 1 - sigmoid(v), tanh(v), 1 - tanh(v)^2}
+__global__ void __launch_bounds__(256) gate_math_kernel(const double* __restrict__ v, double* __restrict__ out, int64_t n) {
+  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (i >= n) return;
+  double* o = out + 6 * i;
+  o[0] = exp_nonpos(-fabs(v[i]));
+  o[1] = recip(1.0 + o[0]);
+  sigmoid_pair(v[i], o[2], o[3]);
+  tanh_pair(v[i], o[4], o[5]);
+}
+
 // ------------------------------------------------------------------------------------------------ weights in blocks
 // forward: element (lane, i) of block (unit tile, k block, gate) is M[gate u + 8 tile + lane / 4][16 block + 4 (lane % 4) + i]
 template <typename T>
@@ -971,6 +983,12 @@ bool cell_plan(int block, int dtype, bool backward, int64_t B, int u, int in_dim
   const int64_t v[8] = {q.uc, q.cs, q.rows, q.ksplit, q.threads, (int64_t)q.smem, (int64_t)n.w + n.x, packed_words_read(backward, gates, in, q)};
   for (int i = 0; i < 8; ++i) out[i] = v[i];
   return true;
+}
+
+void cell_gate_math(Launcher& lc, const double* v, double* out, int64_t n) {
+  gate_math_kernel<<<(unsigned)((n + 255) / 256), 256, 0, lc.stream>>>(v, out, n);
+  lc.count();
+  lc.check();
 }
 
 bool cell_forward_cluster(Launcher& lc, int dtype, int block, const void* W, const void* U, const void* X, const void* gate,

@@ -868,6 +868,15 @@ int64_t hbp_launch_count(const hbp_ctx* ctx) { return ctx ? ctx->launches : 0; }
 
 int32_t hbp_context_modes(const hbp_ctx* ctx) { return ctx ? (ctx->force_simt ? 1 : 0) | (ctx->gemm_pair ? 2 : 0) | (ctx->scan_operand ? 4 : 0) : 0; }
 
+hbp_status hbp_selftest_gate_math(const double* v, double* out, int64_t n, void* cuda_stream) {
+  if (!v || !out) return HBP_ERR_INVALID_ARG;
+  if (n <= 0 || n > (int64_t)1 << 32) return HBP_ERR_SHAPE;
+  Launcher lc;
+  lc.stream = (cudaStream_t)cuda_stream;
+  cell_gate_math(lc, v, out, n);
+  return lc.err == cudaSuccess ? HBP_OK : HBP_ERR_CUDA;
+}
+
 hbp_status hbp_recurrence_plan(const hbp_config* cfg, int32_t backward, const int32_t* at_once, int64_t* plan, size_t* pack_bytes) {
   if (!at_once || !plan || !pack_bytes) return HBP_ERR_INVALID_ARG;
   const hbp_status st = check_config(cfg);
