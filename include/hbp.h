@@ -250,6 +250,16 @@ hbp_status hbp_profile_read(hbp_ctx* ctx, float* ms, int64_t* launches);
 /* Number of kernels this context has launched since creation (host counter). */
 int64_t hbp_launch_count(const hbp_ctx* ctx);
 
+/* How often since creation a call of this context has taken a form among several that would serve it: a recurrence as one
+ * launch (clusters of cell_cluster.cu; those of rnn_cluster.cu; clusters of 16 CTAs with four rows each, rnn_persistent.cu)
+ * or step by step (counted per step); a float product on the tensor cores with its operands split inside the kernel, or a
+ * product on the CUDA cores. */
+typedef enum {
+  HBP_FORM_CELL_CLUSTER = 0, HBP_FORM_RNN_CLUSTER = 1, HBP_FORM_RNN_FOUR_ROWS = 2, HBP_FORM_STEP = 3, HBP_FORM_GEMM_F32 = 4,
+  HBP_FORM_GEMM_SIMT = 5, HBP_FORM_COUNT = 6
+} hbp_form;
+int64_t hbp_form_count(const hbp_ctx* ctx, int32_t form);
+
 /* Kernel-selection modes of a context, fixed when it was created from the environment of that moment:
  * bit 0 = HBP_FORCE_SIMT=1 (every contraction on the CUDA-core kernels, a cross-check of the tensor-core ones),
  * bit 1 = the tensor-core GEMM pairs CTAs (tcgen05 cta_group::2, 256 x 256 tiles): the default; HBP_GEMM_PAIR=0

@@ -18,9 +18,10 @@ HBP_F32, HBP_BF16 = 0, 1
 BLOCKS = {"mlp": 0, "preln_mlp": 1, "rnn_tanh": 2, "preln_transformer": 3, "gru": 4, "lstm": 5, "relu_mlp": 6, "postln_mlp": 7}
 GATE_ONE, GATE_CHANNEL_SHARED, GATE_CHANNEL_PER_STEP = 0, 1, 2
 LOSS_FINAL, LOSS_EVERY_STEP = 0, 1
+FORMS = ("cell_cluster", "rnn_cluster", "rnn_four_rows", "step", "gemm_f32", "gemm_simt")
 
 EXPORTS = ["hbp_workspace_bytes", "hbp_create", "hbp_forward", "hbp_backward", "hbp_exact",
-           "hbp_cumsumprod_scratch_bytes", "hbp_cumsumprod", "hbp_cumsumprod_status", "hbp_sync_status", "hbp_launch_count",
+           "hbp_cumsumprod_scratch_bytes", "hbp_cumsumprod", "hbp_cumsumprod_status", "hbp_sync_status", "hbp_launch_count", "hbp_form_count",
            "hbp_context_modes", "hbp_selftest_wait_timeout", "hbp_selftest_gate_math", "hbp_recurrence_plan",
            "hbp_profile_enable", "hbp_profile_read", "hbp_cumsumprod_static", "hbp_cumsumprod_static_max_bytes",
            "hbp_compare_scratch_bytes", "hbp_compare", "hbp_iterate", "hbp_add_carry", "hbp_param_grads",
@@ -79,6 +80,8 @@ def _load():
     lib.hbp_profile_read.argtypes = [vp, C.POINTER(C.c_float), C.POINTER(i64)]
     lib.hbp_launch_count.argtypes = [vp]
     lib.hbp_launch_count.restype = i64
+    lib.hbp_form_count.argtypes = [vp, i32]
+    lib.hbp_form_count.restype = i64
     lib.hbp_status_string.argtypes = [C.c_int]
     lib.hbp_status_string.restype = C.c_char_p
     lib.hbp_destroy.argtypes = [vp]
@@ -86,7 +89,7 @@ def _load():
     for name in EXPORTS:
         if name in ("hbp_cumsumprod_static_max_bytes", "hbp_compare_scratch_bytes"):
             getattr(lib, name).restype = sz
-        elif name not in ("hbp_launch_count", "hbp_status_string", "hbp_destroy", "hbp_context_modes"):
+        elif name not in ("hbp_launch_count", "hbp_form_count", "hbp_status_string", "hbp_destroy", "hbp_context_modes"):
             getattr(lib, name).restype = C.c_int
     return lib
 
@@ -300,6 +303,11 @@ class Context:
     @property
     def launches(self) -> int:
         return int(lib.hbp_launch_count(self._h))
+
+    @property
+    def forms(self) -> dict:
+        """How often each form of a recurrence or product has been taken since creation (``FORMS``)."""
+        return {name: int(lib.hbp_form_count(self._h, i)) for i, name in enumerate(FORMS)}
 
 
 def cumsumprod_scratch_bytes(dtype, L, rows, d) -> int:

@@ -937,6 +937,7 @@ bool run_cell(Launcher& lc, CellArgs a) {
     cudaGetLastError();
     return false;
   }
+  lc.ran(HBP_FORM_CELL_CLUSTER);
   lc.count();
   lc.check();
   return true;

@@ -401,6 +401,7 @@ bool gemm_f32_tc(Launcher& lc, const GemmArgs& g, int* status_word) {
   }
   dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, (unsigned)z);
   gemm_f32_kernel<<<grid, kAllThreads, kSmemBytes, lc.stream>>>(p);
+  lc.ran(HBP_FORM_GEMM_F32);
   lc.count();
   lc.check();
   if (g.splitk > 1) reduce_splitk(lc, g.partial, (float*)g.D, g.splitk, (int64_t)g.batch * g.M * g.N);

@@ -244,6 +244,7 @@ void launch_simt(Launcher& lc, const GemmArgs& g) {
     dim3 grid((g.N + 31) / 32, (g.M + 31) / 32, g.batch * g.splitk);
     gemm_small_kernel<T><<<grid, 256, 0, lc.stream>>>(g);
   }
+  lc.ran(HBP_FORM_GEMM_SIMT);
   lc.count();
   lc.check();
 }

@@ -37,6 +37,7 @@ struct hbp_ctx {
   size_t ws_bytes = 0;
   bool forward_done = false;
   int64_t launches = 0;
+  int64_t forms[HBP_FORM_COUNT] = {};
   int es = 4;         // element size
   int steps = 0;      // residual steps seen by the scan
   int layers = 0;     // MLP layers (== steps for MLP kinds, decoder blocks for the Transformer)
@@ -264,6 +265,7 @@ struct Run {
   Run(hbp_ctx* ctx, const hbp_params* params, void* stream) : c(ctx), p(params) {
     lc.stream = (cudaStream_t)stream;
     lc.launches = &ctx->launches;
+    lc.forms = ctx->forms;
     lc.force_simt = ctx->force_simt;
     lc.gemm_pair = ctx->gemm_pair;
     N = ctx->cfg.tokens;
@@ -866,6 +868,8 @@ hbp_status hbp_profile_read(hbp_ctx* ctx, float* ms, int64_t* launches) {
 
 int64_t hbp_launch_count(const hbp_ctx* ctx) { return ctx ? ctx->launches : 0; }
 
+int64_t hbp_form_count(const hbp_ctx* ctx, int32_t form) { return ctx && form >= 0 && form < HBP_FORM_COUNT ? ctx->forms[form] : 0; }
+
 int32_t hbp_context_modes(const hbp_ctx* ctx) { return ctx ? (ctx->force_simt ? 1 : 0) | (ctx->gemm_pair ? 2 : 0) | (ctx->scan_operand ? 4 : 0) : 0; }
 
 hbp_status hbp_selftest_gate_math(const double* v, double* out, int64_t n, void* cuda_stream) {
@@ -949,6 +953,7 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
     for (int t = 0; t < T && !one_launch; ++t) {
       const double* sin = ctx->hres + (int64_t)(t & 1) * state;
       double* sout = ctx->hres + (int64_t)((t + 1) & 1) * state;
+      r.lc.ran(HBP_FORM_STEP);
       lstm_forward_step(r.lc, f.dtype, params->W, params->U, r.at(inputs, (int64_t)t * N * f.in_dim), sin, sout,
                         r.at(ctx->Fg, (int64_t)t * state), r.at(ctx->C5, (int64_t)t * N * 5 * u),
                         r.at(xa, (int64_t)(t + 1) * state), (int)N, (int)u, f.in_dim);
@@ -966,6 +971,7 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
     for (int t = 0; t < T && !one_launch; ++t) {
       const double* hin = ctx->hres + (int64_t)(t & 1) * state;
       double* hout = ctx->hres + (int64_t)((t + 1) & 1) * state;
+      r.lc.ran(HBP_FORM_STEP);
       gru_forward_step(r.lc, f.dtype, params->W, params->U, r.at(inputs, (int64_t)t * N * f.in_dim), hin, hout,
                        r.at(ctx->Zc, (int64_t)t * state), r.at(ctx->C4, (int64_t)t * 4 * state),
                        r.at(xa, (int64_t)(t + 1) * state), (int)N, (int)d, f.in_dim);
@@ -995,6 +1001,7 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
       for (int t = 0; t < T; ++t) {
         const double* hin = ctx->hres + (int64_t)(t & 1) * state;
         double* hout = ctx->hres + (int64_t)((t + 1) & 1) * state;
+        r.lc.ran(HBP_FORM_STEP);
         rnn_forward_step(r.lc, f.dtype, params->W, params->U, r.at(inputs, (int64_t)t * N * f.in_dim), r.gate_ptr(t), hin,
                          hout, r.at(ctx->C, (int64_t)t * state), r.at(xa, (int64_t)(t + 1) * state), (int)N, (int)d,
                          f.in_dim);
@@ -1150,6 +1157,7 @@ static hbp_status backward_common(hbp_ctx* ctx, const hbp_params* params, int32_
         for (int t = steps - 1; t >= 0; --t) {
           const double* gin = ctx->hres + (int64_t)((steps - 1 - t) & 1) * r.state;
           double* gout = ctx->hres + (int64_t)((steps - t) & 1) * r.state;
+          r.lc.ran(HBP_FORM_STEP);
           rnn_backward_step(r.lc, f.dtype, params->W, r.at(ctx->C, (int64_t)t * r.state),
                             f.loss == HBP_LOSS_EVERY_STEP ? r.at(r.delta, (int64_t)t * r.state) : nullptr, r.gate_ptr(t),
                             gin, gout, r.at(r.g, (int64_t)t * r.state), (int)r.N, (int)r.d);
@@ -1164,6 +1172,7 @@ static hbp_status backward_common(hbp_ctx* ctx, const hbp_params* params, int32_
       for (int t = steps - 1; t >= 0 && !one_launch; --t) {
         const double* gin = ctx->hres + (int64_t)((steps - 1 - t) & 1) * r.state;
         double* gout = ctx->hres + (int64_t)((steps - t) & 1) * r.state;
+        r.lc.ran(HBP_FORM_STEP);
         gru_backward_step(r.lc, f.dtype, params->W, r.at(ctx->Zc, (int64_t)t * r.state),
                           r.at(ctx->C4, (int64_t)t * 4 * r.state),
                           f.loss == HBP_LOSS_EVERY_STEP ? r.at(r.delta, (int64_t)t * r.state) : nullptr, gin, gout,
@@ -1178,6 +1187,7 @@ static hbp_status backward_common(hbp_ctx* ctx, const hbp_params* params, int32_
       for (int t = steps - 1; t >= 0 && !one_launch; --t) {
         const double* gin = ctx->hres + (int64_t)((steps - 1 - t) & 1) * r.state;
         double* gout = ctx->hres + (int64_t)((steps - t) & 1) * r.state;
+        r.lc.ran(HBP_FORM_STEP);
         lstm_backward_step(r.lc, f.dtype, params->W, r.at(ctx->Fg, (int64_t)t * r.state),
                            r.at(ctx->C5, (int64_t)t * r.N * 5 * (r.d / 2)),
                            f.loss == HBP_LOSS_EVERY_STEP ? r.at(r.delta, (int64_t)t * r.state) : nullptr, gin, gout,

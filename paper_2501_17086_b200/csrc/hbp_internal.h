@@ -77,15 +77,20 @@ struct PerDevice {
   T& here() { return v[current_device()]; }
 };
 
-// Counts launches and remembers the first CUDA error; carries the kernel-selection modes of the context it runs for.
+// Counts launches (all, and by form: hbp_form) and remembers the first CUDA error; carries the kernel-selection modes of the
+// context it runs for.
 struct Launcher {
   cudaStream_t stream = nullptr;
   int64_t* launches = nullptr;
+  int64_t* forms = nullptr;
   cudaError_t err = cudaSuccess;
   bool force_simt = false;  // keep every GEMM and attention product on the CUDA-core kernels (cross-checks)
   bool gemm_pair = true;    // tensor-core GEMM pairs CTAs (cta_group::2, 256 x 256 tiles) where there are two row blocks
   void count(int n = 1) {
     if (launches) *launches += n;
+  }
+  void ran(hbp_form form) {
+    if (forms) ++forms[form];
   }
   void check() {
     cudaError_t e = cudaGetLastError();

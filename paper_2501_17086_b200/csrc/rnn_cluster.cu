@@ -376,6 +376,7 @@ bool run_rnn(Launcher& lc, RnnArgs a) {
     cudaGetLastError();
     return false;
   }
+  lc.ran(HBP_FORM_RNN_CLUSTER);
   lc.count();
   lc.check();
   return true;

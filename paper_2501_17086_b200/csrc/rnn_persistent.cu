@@ -340,6 +340,7 @@ bool launch_persistent(Launcher& lc, const PersistArgs& a, bool ask) {
     cudaGetLastError();
     return false;
   }
+  lc.ran(HBP_FORM_RNN_FOUR_ROWS);
   lc.count();
   lc.check();
   return true;

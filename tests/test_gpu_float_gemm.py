@@ -21,7 +21,15 @@ pytestmark = pytest.mark.gpu
 def test_tile_edges_match_oracle(block, L, d, h, tokens):
     w = Workload("t", block, "f32", L=L, d=d, hidden=h, tokens=tokens, batch=1, seq=1, seed=8000 + d + tokens)
     inp = make_inputs(w, "cuda")
-    compare(w, run_gpu(w, inp, (1, L)), orun.run(w, inp, ks=(1, L), grads_for=("exact", L)), (1, L), ("exact", L))
+    gpu = run_gpu(w, inp, (1, L))
+    # forward: two products a layer; each pass: two per VJP over all layers (k of them, the exact pass one per layer) and, for the
+    # parameters, one VJP's first product again (not in the exact pass) and two batched weight gradients
+    forward = [(tokens, h, d), (tokens, d, h)] * L
+    vjp, weights = [(tokens, h, d), (tokens, d, h)], [(d, h, tokens), (h, d, tokens)]
+    products = forward + vjp * (1 + L) + ([vjp[0]] + weights) * 2 + vjp * L + weights
+    taken = sum(m > 32 for m, n, k in products)
+    assert gpu["ctx"].forms["gemm_f32"] == taken and gpu["ctx"].forms["gemm_simt"] == len(products) - taken
+    compare(w, gpu, orun.run(w, inp, ks=(1, L), grads_for=("exact", L)), (1, L), ("exact", L))
 
 
 def test_non_finite_inputs_stay_non_finite():
@@ -39,6 +47,7 @@ def test_non_finite_inputs_stay_non_finite():
             os.environ.pop("HBP_FORCE_SIMT", None)
         finite.append(torch.isfinite(ctx.forward(harness.params_for(w, inp), inp["x0"])))
         ctx.sync_status()
+        assert ctx.forms["gemm_simt" if simt else "gemm_f32"] == 2
     assert torch.equal(finite[0][0], finite[1][0])
     assert torch.equal(finite[0][1].all(dim=1), finite[1][1].all(dim=1))
 
@@ -66,6 +75,7 @@ def test_infinities_and_nans_have_the_value_a_plain_sum_gives():
             os.environ.pop("HBP_FORCE_SIMT", None)
         states.append(ctx.forward(harness.params_for(w, inp), x0)[1].clone())
         ctx.sync_status()
+        assert ctx.forms["gemm_simt" if simt else "gemm_f32"] == 2
     got, want = states
     assert torch.isinf(want[3]).all() and torch.isinf(want[40]).all() and torch.isnan(want[77]).all()
     assert torch.equal(torch.isnan(got), torch.isnan(want))

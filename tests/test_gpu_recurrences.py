@@ -19,11 +19,17 @@ def _workload(block, dtype, T, u, B, nin, loss="every_mse"):
                     batch=B, tokens=B, seed=7000 + T + u + B, loss=loss)
 
 
-def _forward(w, inp):
+def _forward(w, inp, form):
+    """The states, from a context whose forward pass has to take ``form`` (one launch, or one per step)."""
     ctx = harness.make_context(w)
     x = ctx.forward(harness.params_for(w, inp), inp["x0"], harness.rnn_inputs(w, inp))
     ctx.sync_status()
+    assert _recurrences(ctx) == {form: w.L if form == "step" else 1}
     return x
+
+
+def _recurrences(ctx):
+    return {n: c for n, c in ctx.forms.items() if c and n in ("cell_cluster", "rnn_cluster", "rnn_four_rows", "step")}
 
 
 @pytest.mark.parametrize("block,dtype,T,u,B,nin", [
@@ -37,11 +43,14 @@ def _forward(w, inp):
 def test_edges_of_the_splits_match_oracle(block, dtype, T, u, B, nin):
     w = _workload(block, dtype, T, u, B, nin)
     inp = make_inputs(w, "cuda")
-    compare(w, run_gpu(w, inp, (1,)), orun.run(w, inp, ks=(1,), grads_for=("exact", 1)), (1,), ("exact", 1))
+    gpu = run_gpu(w, inp, (1,))
+    # one forward and one exact pass, each one launch
+    assert _recurrences(gpu["ctx"]) == ({"rnn_cluster": 1, "cell_cluster": 1} if block == "rnn_tanh" else {"cell_cluster": 2})
+    compare(w, gpu, orun.run(w, inp, ks=(1,), grads_for=("exact", 1)), (1,), ("exact", 1))
 
 
 @pytest.mark.parametrize("dtype,T,u,B,nin", [
-    ("f32", 300, 512, 32, 256), ("f32", 100, 512, 190, 8), ("f32", 200, 256, 40, 64), ("f32", 120, 128, 61, 20), ("bf16", 60, 256, 33, 16),
+    ("f32", 300, 512, 32, 256), ("f32", 100, 512, 190, 8), ("f32", 200, 256, 40, 64), ("f32", 120, 128, 201, 20), ("bf16", 60, 256, 33, 16),
     ("f32", 200, 100, 50, 20), ("f32", 100, 508, 180, 256), ("f32", 50, 4, 5, 4), ("f32", 64, 436, 100, 36), ("bf16", 80, 264, 17, 40),
 ])
 def test_tanh_rnn_forms_agree_bit_for_bit(dtype, T, u, B, nin):
@@ -49,16 +58,16 @@ def test_tanh_rnn_forms_agree_bit_for_bit(dtype, T, u, B, nin):
     four at a time (128, 256 and 512 units), or against one launch per step."""
     w = _workload("rnn_tanh", dtype, T, u, B, nin)
     inp = make_inputs(w, "cuda")
-    x = _forward(w, inp)
+    x = _forward(w, inp, "rnn_cluster")
     if u in (128, 256, 512):
         for r in range(0, B, 4):
             n = min(4, B - r)
             part = dict(inp, X=inp["X"][:, r:r + n].contiguous(), x0=inp["x0"][r:r + n].contiguous())
-            assert torch.equal(_forward(_workload("rnn_tanh", dtype, T, u, n, nin), part), x[:, r:r + n])
+            assert torch.equal(_forward(_workload("rnn_tanh", dtype, T, u, n, nin), part, "rnn_four_rows"), x[:, r:r + n])
     else:
         os.environ["HBP_FORCE_SIMT"] = "1"
         try:
-            assert torch.equal(_forward(w, inp), x)
+            assert torch.equal(_forward(w, inp, "step"), x)
         finally:
             del os.environ["HBP_FORCE_SIMT"]
 
@@ -70,5 +79,5 @@ def test_unaligned_weights_take_the_per_step_form(block):
     inp = make_inputs(w, "cuda")
     moved = torch.empty(inp["W"].numel() + 1, device="cuda")[1:].view_as(inp["W"])
     moved.copy_(inp["W"])
-    x, y = _forward(w, inp), _forward(w, dict(inp, W=moved))
+    x, y = _forward(w, inp, "cell_cluster"), _forward(w, dict(inp, W=moved), "step")
     assert float((x - y).norm() / x.norm()) < 1e-6

@@ -57,6 +57,7 @@ for block, u in (("gru", 64), ("lstm", 40), ("rnn_tanh", 128), ("rnn_tanh", 100)
         ctx.sync_status()
         if not steps:
             assert forward_refused > 0 and refused.value - before > forward_refused, (block, u, refused.value)
+        assert ctx.forms["step"] == 2 * T and not any(ctx.forms[f] for f in ("cell_cluster", "rnn_cluster", "rnn_four_rows")), ctx.forms
         outs.append((x, g))
     # the same per-step kernels on both sides (every cluster refused, theirs too): the same bits
     assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1]), (block, u)
