@@ -267,6 +267,8 @@ int64_t hbp_form_count(const hbp_ctx* ctx, int32_t form);
  * bit 2 = on the float tanh RNN the reverse scan between two all-step VJPs (Eq. 9 followed by Eq. 8) also writes
  * the next VJP's left operand g_{t+1} * tanh'(z_t), split for the tensor cores, instead of the intermediate
  * iterate: the default; HBP_SCAN_OPERAND=0 keeps the separate pass (same bits in every result, a cross-check).
+ * HBP_LAYER_GROUP=n (no bit) caps the layers whose hidden-size scratch is held at once at n, where the stack's size asks for no
+ * smaller group already: a small stack then takes the group by group path of the largest ones.
  * The modes belong to the context: contexts created
  * under other settings, before or after, keep their own.  One-time kernel set-up is likewise remembered per
  * device, so one process may hold contexts on several GPUs (each used with its device current). */

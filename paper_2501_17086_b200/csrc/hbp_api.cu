@@ -27,8 +27,8 @@ struct ProfSeg {
 
 struct hbp_ctx {
   hbp_config cfg;
-  // kernel-selection modes, read from the environment (HBP_FORCE_SIMT=1, HBP_GEMM_PAIR=0, HBP_SCAN_OPERAND=0) when
-  // THIS context is created and kept with it: another context created later under other settings does not change them
+  // kernel-selection modes, read from the environment (HBP_FORCE_SIMT=1, HBP_GEMM_PAIR=0, HBP_SCAN_OPERAND=0,
+  // HBP_LAYER_GROUP=n: `group` below) when THIS context is created and kept with it: another context created later under other settings does not change them
   bool force_simt = false, gemm_pair = false, scan_operand = true;
   bool profiling = false;
   std::vector<ProfSeg> segs;       // recorded, not yet read
@@ -820,6 +820,9 @@ hbp_status hbp_create(const hbp_config* cfg, void* workspace, size_t workspace_b
   c->gemm_pair = !(pm && pm[0] == '0');  // pairs by default
   const char* so = std::getenv("HBP_SCAN_OPERAND");
   c->scan_operand = !(so && so[0] == '0');  // the scan writes the next VJP's operand by default (float tanh RNN)
+  const char* lg = std::getenv("HBP_LAYER_GROUP");
+  const int cap = lg ? std::atoi(lg) : 0;
+  if (cap > 0 && cap < c->group) c->group = cap;  // (the scratch is carved for the larger group)
   if (cudaMemset(c->status, 0, 256) != cudaSuccess) {
     delete c;
     return HBP_ERR_CUDA;

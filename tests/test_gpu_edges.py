@@ -318,6 +318,27 @@ def test_scan_that_writes_the_next_vjp_operand_changes_no_bit(monkeypatch, T, d,
             assert torch.equal(got[0][1][n], got[1][1][n]), n
 
 
+@pytest.mark.parametrize("group", [2, 3])
+@pytest.mark.parametrize("block,dtype", [("preln_mlp", "f32"), ("preln_mlp", "bf16"), ("postln_mlp", "f32"), ("relu_mlp", "f32"),
+                                         ("preln_transformer", "bf16")])
+def test_layer_groups_match_the_oracle(block, dtype, group, monkeypatch):
+    """Stacks whose hidden-size scratch does not hold all layers work through groups of them, the last one shorter: five
+    layers in groups of two and of three (HBP_LAYER_GROUP), in the exact pass and in the truncated one."""
+    from oracle import run as orun
+    from paper_2501_17086_b200.workloads import Workload, make_inputs
+    from test_gpu_parity import compare, run_gpu
+    tr = block == "preln_transformer"
+    w = Workload("t", block, dtype, L=5, d=128, hidden=256, n_heads=2 if tr else 0, head_dim=64 if tr else 0, seq=40 if tr else 1,
+                 batch=3 if tr else 1, tokens=120, seed=8300, init="small" if block == "postln_mlp" else "")
+    inp = make_inputs(w, "cuda")
+    whole = run_gpu(w, inp, (2,))
+    monkeypatch.setenv("HBP_LAYER_GROUP", str(group))
+    gpu = run_gpu(w, inp, (2,))
+    assert gpu["ctx"].launches > whole["ctx"].launches   # more and smaller products
+    compare(w, gpu, orun.run(w, inp, ks=(2,), grads_for=("exact", 2)), (2,), ("exact", 2))
+    assert torch.equal(gpu["exact"], whole["exact"]) and torch.equal(gpu["hbp"][2], whole["hbp"][2])
+
+
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 def test_compare_matches_the_definition(dtype):
     from paper_2501_17086_b200 import binding as B
