@@ -76,6 +76,7 @@ struct CellArgs {
   int uc;               // units per CTA
   int ksplit;           // forward: warps that share one 8-unit tile's contraction
   int res, res_x;       // blocks of W (U) per warp that stay in shared memory
+  int kc;               // backward: blocks of 16 of a CTA's own contraction, padding included
   int stage_x;          // forward: the inputs of a step are copied to shared memory one step ahead
 };
 
@@ -479,7 +480,7 @@ __global__ void __launch_bounds__(max_threads(MT, EX), 1) cell_backward_kernel(c
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, lr = lane >> 2, lc = lane & 3;
   const int row0 = (int)cluster_index() * R;
   const int half = uc / 2, items = R * half;
-  const int kl = G * uc, kc = (kl + 15) / 16;             // own contraction length and its blocks of 16
+  const int kc = p.kc;                                    // blocks of 16 of the own contraction (G uc long)
   const int groups = (cs * uc + 31) / 32;
   const int my_groups = groups > warp ? (groups - warp + kWarps - 1) / kWarps : 0;
   const int rb = p.res, nb = kc - rb;                     // blocks of each group that are resident; streamed
@@ -764,23 +765,22 @@ __global__ void __launch_bounds__(256) pack_backward_kernel(const T* __restrict_
 struct Packed {
   int w, x;  // float4 values of W (and U)
 };
-Packed packed_size(bool bwd, int gates, int u, int in, int uc) {
+Packed packed_size(bool bwd, int gates, int u, int in, int uc, int kc) {  // (kc: backward only)
   const int cs = (u + uc - 1) / uc;
-  if (bwd) return {cs * ((cs * uc + 31) / 32) * ((gates * uc + 15) / 16) * 128, 0};
+  if (bwd) return {cs * ((cs * uc + 31) / 32) * kc * 128, 0};
   return {cs * (uc / 8) * ((cs * uc + 15) / 16) * gates * 32, cs * (uc / 8) * ((in + 15) / 16) * gates * 32};
 }
 
 struct Plan {
-  int uc = 0, cs = 0, mt = 0, ex = 0, rows = 0, ksplit = 1, threads = 0, res = 0, res_x = 0, stage_x = 0;
+  int uc = 0, cs = 0, mt = 0, ex = 0, rows = 0, ksplit = 1, threads = 0, res = 0, res_x = 0, stage_x = 0, kc = 0;
   size_t smem = 0;
 };
 
+constexpr size_t v_block_bytes(int mt, int ex) { return mt * 1024 + ex * 128; }  // a block of 16 of the backward contraction's v
+
 size_t smem_without_weights(int cell, bool bwd, int uc, int cs, int mt, int ex, int rows, int ksplit, size_t x_bytes) {
   const int gates = cell == CELL_RNN ? 1 : (cell == CELL_GRU ? 3 : 4), acc = cell == CELL_RNN ? 1 : 4;
-  if (bwd) {
-    const size_t kc = (gates * uc + 15) / 16;
-    return (size_t)2 * cs * rows * (uc / 2) * 16 + kc * 4 * mt * 32 * 8 + ex * kc * 16 * 8 + 64;
-  }
+  if (bwd) return (size_t)2 * cs * rows * (uc / 2) * 16 + (gates * uc + 15) / 16 * v_block_bytes(mt, ex) + 64;
   const size_t outs = (size_t)(8 * mt + ex) * uc, kbh = (cs * uc + 15) / 16;
   return 2 * kbh * (mt * 1024 + ex * 128) + (2 * x_bytes + 15) / 16 * 16 + (ksplit * acc + (cell == CELL_LSTM)) * outs * 8 + 64;
 }
@@ -841,13 +841,17 @@ bool make_plan(int cell, bool bwd, int es, int64_t B, int u, int in, ActiveClust
         // what is left of the shared memory holds blocks of W, then of U
         size_t left = (size_t)kSmemLimit - base;
         if (bwd) {
-          // as many blocks of every column group as fit, the streamed rest a multiple of the blocks in flight
+          // as many blocks of every column group as fit, the streamed rest a multiple of the blocks in flight: with blocks
+          // of zeros behind it where not even the remainder fits
           const int ahead = mt == 1 ? kAheadBackward<1> : kAheadBackward<2>;
           const size_t block = (size_t)groups * 2048;
           q.res = (int)(left / block < (size_t)kc ? left / block : (size_t)kc);
           q.res = kc - (kc - q.res + ahead - 1) / ahead * ahead;
-          if (q.res < 0) continue;
-          q.smem = base + q.res * block;
+          const int padding = q.res < 0 ? -q.res : 0;
+          if (padding * v_block_bytes(mt, ex) > left) continue;
+          q.res += padding;
+          q.kc = kc + padding;
+          q.smem = base + padding * v_block_bytes(mt, ex) + q.res * block;
         } else {
           const size_t block = (size_t)warps * gates * 512;
           const int jh = (kbh + q.ksplit - 1) / q.ksplit, jx = (kbx + q.ksplit - 1) / q.ksplit;
@@ -867,7 +871,7 @@ bool make_plan(int cell, bool bwd, int es, int64_t B, int u, int in, ActiveClust
 // One past the last 16-byte word of the packed weights (W, then U) that any lane reads under a plan, by the kernels' own
 // index arithmetic: the last warps of the last CTA reach furthest.
 int64_t packed_words_read(bool bwd, int gates, int in, const Plan& q) {
-  if (bwd) return packed_size(true, gates, q.cs * q.uc, in, q.uc).w;  // group < groups, block < kc by construction
+  if (bwd) return packed_size(true, gates, q.cs * q.uc, in, q.uc, q.kc).w;  // group < groups, block < kc by construction
   const int kbh = (q.cs * q.uc + 15) / 16, kbx = (in + 15) / 16;
   const int64_t tiles = (int64_t)q.cs * q.uc / 8, n_w = tiles * kbh * gates * 32;
   int64_t end = 0;
@@ -913,11 +917,11 @@ bool run_cell(Launcher& lc, CellArgs a) {
   };
   Plan q;
   if (!make_plan(CELL, BWD, (int)sizeof(T), a.B, a.u, a.in, active, &q)) return false;
-  const Packed n = packed_size(BWD, Cell<CELL>::kGates, a.u, a.in, q.uc);
+  const Packed n = packed_size(BWD, Cell<CELL>::kGates, a.u, a.in, q.uc, q.kc);
   a.Up = a.Wp + n.w;
   if (BWD) {
-    const int kc = (Cell<CELL>::kGates * q.uc + 15) / 16, groups = (q.cs * q.uc + 31) / 32;
-    pack_backward_kernel<T><<<(n.w + 255) / 256, 256, 0, lc.stream>>>((const T*)a.W, a.Wp, a.u, Cell<CELL>::kGates, q.uc, kc, groups, n.w);
+    const int groups = (q.cs * q.uc + 31) / 32;
+    pack_backward_kernel<T><<<(n.w + 255) / 256, 256, 0, lc.stream>>>((const T*)a.W, a.Wp, a.u, Cell<CELL>::kGates, q.uc, q.kc, groups, n.w);
     lc.count();
   } else {
     pack_forward_kernel<T><<<(n.w + 255) / 256, 256, 0, lc.stream>>>((const T*)a.W, a.Wp, a.u, a.u, Cell<CELL>::kGates, (q.cs * q.uc + 15) / 16, n.w);
@@ -925,7 +929,7 @@ bool run_cell(Launcher& lc, CellArgs a) {
     lc.count(2);
   }
   lc.check();
-  a.rows = q.rows; a.uc = q.uc; a.ksplit = q.ksplit; a.res = q.res; a.res_x = q.res_x; a.stage_x = q.stage_x;
+  a.rows = q.rows; a.uc = q.uc; a.ksplit = q.ksplit; a.res = q.res; a.res_x = q.res_x; a.stage_x = q.stage_x; a.kc = q.kc;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr;
   launch_config(cfg, attr, (a.B + q.rows - 1) / q.rows, q.cs, q.threads, q.smem, lc.stream);
@@ -968,7 +972,8 @@ size_t cell_pack_bytes(int block, int u, int in_dim) {
   size_t most = 0;
   for (int uc = 8; uc <= 96; uc += 8) {
     if ((u + uc - 1) / uc > kMaxCluster) continue;
-    const Packed f = packed_size(false, gates, u, in_dim, uc), b = packed_size(true, gates, u, in_dim, uc);
+    const int kc = (gates * uc + 15) / 16 + 3;  // with the most padding a plan adds (fewer blocks than are in flight)
+    const Packed f = packed_size(false, gates, u, in_dim, uc, 0), b = packed_size(true, gates, u, in_dim, uc, kc);
     const size_t n = (size_t)(f.w + f.x > b.w ? f.w + f.x : b.w) * sizeof(float4);
     if (n > most) most = n;
   }
@@ -980,7 +985,7 @@ bool cell_plan(int block, int dtype, bool backward, int64_t B, int u, int in_dim
   const int gates = cell == CELL_RNN ? 1 : (cell == CELL_GRU ? 3 : 4), in = backward ? 0 : in_dim;
   Plan q;
   if (!make_plan(cell, backward, dtype == HBP_F32 ? 4 : 2, B, u, in, [&](int, int, int cs) { return (int)at_once[cs]; }, &q)) return false;
-  const Packed n = packed_size(backward, gates, u, in, q.uc);
+  const Packed n = packed_size(backward, gates, u, in, q.uc, q.kc);
   const int64_t v[8] = {q.uc, q.cs, q.rows, q.ksplit, q.threads, (int64_t)q.smem, (int64_t)n.w + n.x, packed_words_read(backward, gates, in, q)};
   for (int i = 0; i < 8; ++i) out[i] = v[i];
   return true;

@@ -39,6 +39,8 @@ def _recurrences(ctx):
     ("lstm", "f32", 3, 372, 150, 100), ("lstm", "bf16", 4, 40, 26, 8),
     ("rnn_tanh", "f32", 1, 4, 1, 4), ("rnn_tanh", "f32", 6, 68, 50, 12), ("rnn_tanh", "f32", 4, 508, 180, 256),
     ("rnn_tanh", "f32", 4, 512, 190, 8), ("rnn_tanh", "bf16", 5, 264, 17, 40),
+    # more units: 72 to 96 per CTA, all weights streamed, blocks of padding in the backward contraction
+    ("gru", "f32", 2, 1100, 10, 20), ("gru", "f32", 2, 1536, 9, 16), ("lstm", "f32", 2, 1300, 60, 8), ("lstm", "f32", 2, 1536, 8, 4),
 ])
 def test_edges_of_the_splits_match_oracle(block, dtype, T, u, B, nin):
     w = _workload(block, dtype, T, u, B, nin)
@@ -81,3 +83,11 @@ def test_unaligned_weights_take_the_per_step_form(block):
     moved.copy_(inp["W"])
     x, y = _forward(w, inp, "cell_cluster"), _forward(w, dict(inp, W=moved), "step")
     assert float((x - y).norm() / x.norm()) < 1e-6
+
+
+def test_exact_pass_of_wide_tanh_rnns_is_one_launch():
+    w = _workload("rnn_tanh", "f32", 2, 1536, 40, 8)
+    inp = make_inputs(w, "cuda")
+    gpu = run_gpu(w, inp, (1,))
+    assert gpu["ctx"].forms["cell_cluster"] == 1   # (the forward pass of that width is step by step)
+    compare(w, gpu, orun.run(w, inp, ks=(1,), grads_for=("exact", 1)), (1,), ("exact", 1))

@@ -32,7 +32,26 @@ def test_plans_stay_inside_the_packed_weights_and_shared_memory(B, block, dtype)
                         assert p is None
                         continue
                     assert p is not None, (u, rows, nin, backward)
-                    assert p["words_read"] <= p["packed_words"], (u, rows, nin, backward, p)
-                    assert p["packed_words"] * 16 <= p["pack_bytes"]
-                    assert p["smem"] <= 227 * 1024 and p["threads"] <= 384 and p["cluster"] <= 16
-                    assert p["cluster"] * p["units_per_cta"] >= u and p["rows"] <= 24
+                    _check(p, u, (u, rows, nin, backward))
+
+
+@pytest.mark.parametrize("block", ["gru", "lstm", "rnn_tanh"])
+def test_every_width_up_to_1536_has_a_split(B, block):
+    """Both directions; beyond 1536 units (96 per CTA, 16 CTAs) neither."""
+    for u in range(520, 1537, 8):
+        for rows in (1, 8, 32, 64, 100, 128, 300, 1000):
+            for backward in (False, True):
+                if block == "rnn_tanh" and not backward:
+                    continue
+                p = B.recurrence_plan(_config(B, block, "f32", u, rows, 64), backward, AT_ONCE)
+                assert p is not None, (u, rows, backward)
+                _check(p, u, (u, rows, backward))
+    for backward in (False, True):
+        assert B.recurrence_plan(_config(B, block, "f32", 1544, 32, 64), backward, AT_ONCE) is None
+
+
+def _check(p, u, what):
+    assert p["words_read"] <= p["packed_words"], (what, p)
+    assert p["packed_words"] * 16 <= p["pack_bytes"], (what, p)
+    assert p["smem"] <= 227 * 1024 and p["threads"] <= 384 and p["cluster"] <= 16, (what, p)
+    assert p["cluster"] * p["units_per_cta"] >= u and p["rows"] <= 24, (what, p)
