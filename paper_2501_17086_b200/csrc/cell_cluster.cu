@@ -714,6 +714,8 @@ __global__ void __launch_bounds__(max_threads(MT, EX), 1) cell_backward_kernel(c
           } else {
             store2(out, g[it].x, g[it].y);
           }
+        } else {  // padding stays zero: an infinity times its zero weights would be a NaN that the next step multiplies on
+          g[it] = gc[it] = make_double2(0.0, 0.0);
         }
       }
     }

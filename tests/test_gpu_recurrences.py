@@ -91,3 +91,23 @@ def test_exact_pass_of_wide_tanh_rnns_is_one_launch():
     gpu = run_gpu(w, inp, (1,))
     assert gpu["ctx"].forms["cell_cluster"] == 1   # (the forward pass of that width is step by step)
     compare(w, gpu, orun.run(w, inp, ks=(1,), grads_for=("exact", 1)), (1,), ("exact", 1))
+
+
+@pytest.mark.parametrize("u", [12, 100])
+def test_an_infinite_gradient_stays_infinite_beside_padding_units(u):
+    """Exact backpropagation of a tanh RNN with weights >= 0 (tanh' > 0): an infinite gradient of one unit makes all gradients of
+    its row infinite from the step before on, and no NaN, also where the last 8-unit tile has padding."""
+    w = _workload("rnn_tanh", "f32", 6, u, 9, 8)
+    inp = make_inputs(w, "cuda")
+    inp["W"].abs_().mul_(0.1)
+    params, xin = harness.params_for(w, inp), harness.rnn_inputs(w, inp)
+    ctx = harness.make_context(w)
+    x = ctx.forward(params, inp["x0"], xin)
+    delta = torch.ones_like(x)
+    delta[-1, 4, 2] = float("inf")
+    g = ctx.exact(params, delta, x, xin)
+    ctx.sync_status()
+    assert ctx.forms["cell_cluster"] == 1 and ctx.forms["step"] == 0
+    assert torch.isposinf(g[:-1, 4]).all()
+    others = [r for r in range(9) if r != 4]
+    assert torch.isfinite(g[:, others]).all()
