@@ -172,12 +172,8 @@ __global__ void __launch_bounds__(max_threads(MT, EX), 1) cell_forward_kernel(co
   const float4* my_u = ures + warp * p.res_x * G * 32 + lane;
 
   auto fetch_x = [&](int t) {  // one thread: the rows of a step are one contiguous block
-    const uint32_t bar = xbar0 + 8 * (t & 1), bytes = (uint32_t)live_rows * in * (uint32_t)sizeof(T);
-    tc::mbar_expect_tx(bar, bytes);
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     tc::smem_u32(xs) + (t & 1) * x_bytes),
-                 "l"((const T*)p.X + ((int64_t)t * p.B + row0) * in), "r"(bytes), "r"(bar)
-                 : "memory");
+    fetch_rows(tc::smem_u32(xs) + (t & 1) * x_bytes, (const T*)p.X + ((int64_t)t * p.B + row0) * in,
+               (uint32_t)live_rows * in * (uint32_t)sizeof(T), xbar0 + 8 * (t & 1));
   };
   if (tid == 0) {
     for (int i = 0; i < 4; ++i) tc::mbar_init(bar0 + 8 * i, 1);
@@ -453,12 +449,7 @@ __global__ void __launch_bounds__(max_threads(MT, EX), 1) cell_forward_kernel(co
         if (rounds > 4) finish(Const<4>{}, Const<2>{});
     }
   }
-  if (!ok) {
-    if (tid == 0 && p.status) atomicExch(p.status, (int)HBP_ERR_TIMEOUT);
-    const uint64_t t0 = tc::global_ns();  // copies of our own and stores of peers that may still be in flight
-    while (tc::global_ns() - t0 < 2000000ull) {
-    }
-  }
+  if (!ok) after_timeout(p.status);
   tc::cluster_sync();
 }
 
@@ -720,12 +711,7 @@ __global__ void __launch_bounds__(max_threads(MT, EX), 1) cell_backward_kernel(c
       }
     }
   }
-  if (__syncthreads_or(!ok)) {
-    if (tid == 0 && p.status) atomicExch(p.status, (int)HBP_ERR_TIMEOUT);
-    const uint64_t t0 = tc::global_ns();
-    while (tc::global_ns() - t0 < 2000000ull) {
-    }
-  }
+  if (__syncthreads_or(!ok)) after_timeout(p.status);
   tc::cluster_sync();
 }
 
@@ -781,7 +767,7 @@ struct Plan {
 constexpr size_t v_block_bytes(int mt, int ex) { return mt * 1024 + ex * 128; }  // a block of 16 of the backward contraction's v
 
 size_t smem_without_weights(int cell, bool bwd, int uc, int cs, int mt, int ex, int rows, int ksplit, size_t x_bytes) {
-  const int gates = cell == CELL_RNN ? 1 : (cell == CELL_GRU ? 3 : 4), acc = cell == CELL_RNN ? 1 : 4;
+  const int gates = cell == CELL_RNN ? 1 : (cell == CELL_GRU ? 3 : 4), acc = 4;  // (the tanh cell: backward only)
   if (bwd) return (size_t)2 * cs * rows * (uc / 2) * 16 + (gates * uc + 15) / 16 * v_block_bytes(mt, ex) + 64;
   const size_t outs = (size_t)(8 * mt + ex) * uc, kbh = (cs * uc + 15) / 16;
   return 2 * kbh * (mt * 1024 + ex * 128) + (2 * x_bytes + 15) / 16 * 16 + (ksplit * acc + (cell == CELL_LSTM)) * outs * 8 + 64;
@@ -828,7 +814,7 @@ bool make_plan(int cell, bool bwd, int es, int64_t B, int u, int in, ActiveClust
         q.stage_x = !bwd && smem_without_weights(cell, bwd, uc, cs, mt, ex, q.rows, q.ksplit, x_bytes) <= (size_t)kSmemLimit;
         const size_t base = smem_without_weights(cell, bwd, uc, cs, mt, ex, q.rows, q.ksplit, q.stage_x ? x_bytes : 0);
         if (base > (size_t)kSmemLimit) continue;
-        const double exchange = cs > 1 ? 500.0 + q.rows * cs * uc * 8 / 17.0 : 0.0;
+        const double exchange = exchange_clocks(cs, q.rows, uc);
         double cost;
         if (bwd) {
           cost = (double)kc * 16 * tile_clocks * ((groups + 3) / 4) + exchange;
@@ -895,27 +881,22 @@ int64_t packed_words_read(bool bwd, int gates, int in, const Plan& q) {
 }
 
 template <typename T, int CELL, bool BWD, int MT, int EX>
-auto cell_kernel() {
+constexpr auto cell_kernel() {
   if constexpr (BWD) return cell_backward_kernel<T, CELL, MT, EX>;
   else return cell_forward_kernel<T, CELL, MT, EX>;
 }
-
 template <typename T, int CELL, bool BWD, int MT, int EX>
-int active_clusters(int cs) {
-  struct Known { int n[kMaxCluster + 1]; };  // 1 + the answer, 0 = not asked yet
-  static PerDevice<Known> known;
-  int& k = known.here().n[cs];
-  if (k == 0) k = 1 + max_active_clusters(cell_kernel<T, CELL, BWD, MT, EX>(), cs, max_threads(MT, EX));
-  return k - 1;
+int active_cells(int cs) {
+  return active_clusters<cell_kernel<T, CELL, BWD, MT, EX>()>(cs, max_threads(MT, EX));
 }
 
 template <typename T, int CELL, bool BWD>
 bool run_cell(Launcher& lc, CellArgs a) {
   auto active = [](int mt, int ex, int cs) {
-    return ex        ? active_clusters<T, CELL, BWD, 1, 1>(cs)
-           : mt == 1 ? active_clusters<T, CELL, BWD, 1, 0>(cs)
-           : mt == 2 ? active_clusters<T, CELL, BWD, 2, 0>(cs)
-                     : active_clusters<T, CELL, BWD, 3, 0>(cs);
+    return ex        ? active_cells<T, CELL, BWD, 1, 1>(cs)
+           : mt == 1 ? active_cells<T, CELL, BWD, 1, 0>(cs)
+           : mt == 2 ? active_cells<T, CELL, BWD, 2, 0>(cs)
+                     : active_cells<T, CELL, BWD, 3, 0>(cs);
   };
   Plan q;
   if (!make_plan(CELL, BWD, (int)sizeof(T), a.B, a.u, a.in, active, &q)) return false;
@@ -999,11 +980,11 @@ void cell_gate_math(Launcher& lc, const double* v, double* out, int64_t n) {
   lc.check();
 }
 
-bool cell_forward_cluster(Launcher& lc, int dtype, int block, const void* W, const void* U, const void* X, const void* gate,
-                          const void* x0, void* x_all, void* keep, void* coef, int T, int B, int u, int in_dim, void* pack, int* status) {
+bool cell_forward_cluster(Launcher& lc, int dtype, int block, const void* W, const void* U, const void* X, const void* x0,
+                          void* x_all, void* keep, void* coef, int T, int B, int u, int in_dim, void* pack, int* status) {
   CellArgs a = {};
   a.Wp = (float4*)pack;
-  a.W = W; a.U = U; a.X = X; a.gate = gate; a.x0 = x0; a.states = x_all; a.keep = keep; a.coef = coef; a.status = status;
+  a.W = W; a.U = U; a.X = X; a.x0 = x0; a.states = x_all; a.keep = keep; a.coef = coef; a.status = status;
   a.T = T; a.B = B; a.u = u; a.in = in_dim;
   return dispatch_cell<false>(lc, dtype, block, a);
 }

@@ -71,6 +71,25 @@ __device__ __forceinline__ void store2(bf16* p, double a, double b) {
 __device__ __forceinline__ float lane4(const float4& v, int i) { return i == 0 ? v.x : (i == 1 ? v.y : (i == 2 ? v.z : v.w)); }
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
+// One thread: `bytes` contiguous bytes (a multiple of 16, both ends aligned to 16) from global to shared memory, counted by
+// the mbarrier.
+__device__ __forceinline__ void fetch_rows(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  tc::mbar_expect_tx(bar, bytes);
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+// The whole CTA, once a wait has given up: records it and lets copies of its own and stores of peers that may still be in
+// flight arrive.
+__device__ __forceinline__ void after_timeout(int* status) {
+  if (threadIdx.x == 0 && status) atomicExch(status, (int)HBP_ERR_TIMEOUT);
+  const uint64_t t0 = tc::global_ns();
+  while (tc::global_ns() - t0 < 2000000ull) {
+  }
+}
+
+// Estimated clocks of a step's exchange: 500 of latency and 17 bytes per clock received, both measured.
+inline double exchange_clocks(int cs, int rows, int uc) { return cs > 1 ? 500.0 + rows * cs * uc * 8 / 17.0 : 0.0; }
+
 inline void launch_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& attr, int64_t clusters, int cs, int threads, size_t smem, cudaStream_t stream) {
   cfg = cudaLaunchConfig_t{};
   cfg.gridDim = dim3((unsigned)(clusters * cs));
@@ -99,6 +118,16 @@ int max_active_clusters(K kernel, int cs, int threads) {
     n = 0;
   cudaGetLastError();
   return n;
+}
+
+// The same, asked once per device, kernel and cluster size.
+template <auto Kernel>
+int active_clusters(int cs, int threads) {
+  struct Known { int n[kMaxCluster + 1]; };  // 1 + the answer, 0 = not asked yet
+  static PerDevice<Known> known;
+  int& k = known.here().n[cs];
+  if (k == 0) k = 1 + max_active_clusters(Kernel, cs, threads);
+  return k - 1;
 }
 
 }  // namespace cell

@@ -950,7 +950,7 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
     const int T = f.L;
     const int64_t u = d / 2;
     // all T steps in one launch where that form applies, else one launch per step (likewise below)
-    const bool one_launch = !ctx->force_simt && cell_forward_cluster(r.lc, f.dtype, f.block, params->W, params->U, inputs, nullptr, x0, xa,
+    const bool one_launch = !ctx->force_simt && cell_forward_cluster(r.lc, f.dtype, f.block, params->W, params->U, inputs, x0, xa,
                                                                      ctx->Fg, ctx->C5, T, (int)N, (int)u, f.in_dim, ctx->pack, ctx->status);
     if (!one_launch) convert_to_f64(r.lc, f.dtype, x0, ctx->hres, state);
     for (int t = 0; t < T && !one_launch; ++t) {
@@ -968,7 +968,7 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
     }
   } else if (f.block == HBP_BLOCK_GRU) {
     const int T = f.L;
-    const bool one_launch = !ctx->force_simt && cell_forward_cluster(r.lc, f.dtype, f.block, params->W, params->U, inputs, nullptr, x0, xa,
+    const bool one_launch = !ctx->force_simt && cell_forward_cluster(r.lc, f.dtype, f.block, params->W, params->U, inputs, x0, xa,
                                                                      ctx->Zc, ctx->C4, T, (int)N, (int)d, f.in_dim, ctx->pack, ctx->status);
     if (!one_launch) convert_to_f64(r.lc, f.dtype, x0, ctx->hres, state);
     for (int t = 0; t < T && !one_launch; ++t) {

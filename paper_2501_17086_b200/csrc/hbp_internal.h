@@ -234,8 +234,8 @@ size_t cell_pack_bytes(int block, int u, int in_dim);
 bool cell_plan(int block, int dtype, bool backward, int64_t B, int u, int in_dim, const int32_t* at_once, int64_t* out);
 // The gates' functions on their own, as hbp_selftest_gate_math gives them.
 void cell_gate_math(Launcher& lc, const double* v, double* out, int64_t n);
-bool cell_forward_cluster(Launcher& lc, int dtype, int block, const void* W, const void* U, const void* X, const void* gate,
-                          const void* x0, void* x_all, void* keep, void* coef, int T, int B, int u, int in_dim, void* pack, int* status);
+bool cell_forward_cluster(Launcher& lc, int dtype, int block, const void* W, const void* U, const void* X, const void* x0,
+                          void* x_all, void* keep, void* coef, int T, int B, int u, int in_dim, void* pack, int* status);
 bool cell_backward_cluster(Launcher& lc, int dtype, int block, const void* W, const void* gate, const void* keep, const void* coef,
                            const void* delta, void* g_all, int T, int B, int u, void* pack, int* status);
 

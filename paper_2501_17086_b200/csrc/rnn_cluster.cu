@@ -94,12 +94,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rnn_cluster_kernel(const RnnAr
   const float4* my_w = wres + warp * p.res * (NCW / 4) * 32 + lane;
 
   auto fetch_x = [&](int t) {  // one thread: the rows of a step are one contiguous block
-    const uint32_t bar = xbar0 + 8 * (t & 1), bytes = (uint32_t)live_rows * in * (uint32_t)sizeof(T);
-    tc::mbar_expect_tx(bar, bytes);
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     tc::smem_u32(xs) + (t & 1) * x_bytes),
-                 "l"((const T*)p.X + ((int64_t)t * p.B + row0) * in), "r"(bytes), "r"(bar)
-                 : "memory");
+    fetch_rows(tc::smem_u32(xs) + (t & 1) * x_bytes, (const T*)p.X + ((int64_t)t * p.B + row0) * in,
+               (uint32_t)live_rows * in * (uint32_t)sizeof(T), xbar0 + 8 * (t & 1));
   };
   if (tid == 0) {
     for (int i = 0; i < 4; ++i) tc::mbar_init(bar0 + 8 * i, 1);
@@ -270,12 +266,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) rnn_cluster_kernel(const RnnAr
       }
     }
   }
-  if (!ok) {
-    if (tid == 0 && p.status) atomicExch(p.status, (int)HBP_ERR_TIMEOUT);
-    const uint64_t t0 = tc::global_ns();  // copies of our own and stores of peers that may still be in flight
-    while (tc::global_ns() - t0 < 2000000ull) {
-    }
-  }
+  if (!ok) after_timeout(p.status);
   tc::cluster_sync();
 }
 
@@ -302,8 +293,8 @@ struct RnnPlan {
   size_t smem = 0;
 };
 
-// As make_plan in cell_cluster.cu: matrix instructions at 16 clocks each on a warp's quarter of the SM, the exchange at
-// 500 clocks and 17 bytes per clock, 1200 clocks for the rest of a step, times the waves of clusters.
+// As make_plan in cell_cluster.cu: matrix instructions at 16 clocks each on a warp's quarter of the SM, the exchange, 1200
+// clocks for the rest of a step, times the waves of clusters.
 template <typename ActiveClusters>
 bool make_rnn_plan(bool parts, int es, int B, int u, int in, ActiveClusters active, RnnPlan* best) {
   const int nc = parts ? 16 : 8, n_k = parts ? u : u + in, steps = chain_steps(parts, n_k);
@@ -328,7 +319,7 @@ bool make_rnn_plan(bool parts, int es, int B, int u, int in, ActiveClusters acti
         if (base > (size_t)kSmemLimit) continue;
         const int waves = ((B + q.rows - 1) / q.rows + at_once - 1) / at_once;
         const double cost = waves * (16.0 * steps * ncw * mt * ((warps + 3) / 4) + 1200.0 + 150.0 * mt +
-                                     (cs > 1 ? 500.0 + q.rows * cs * uc * 8 / 17.0 : 0.0));
+                                     exchange_clocks(cs, q.rows, uc));
         if (best->uc && cost >= best_cost) continue;
         const size_t block = (size_t)warps * (ncw / 4) * 512, left = (size_t)kSmemLimit - base;
         q.res = (int)(left / block < (size_t)steps ? left / block : (size_t)steps);
@@ -342,19 +333,15 @@ bool make_rnn_plan(bool parts, int es, int B, int u, int in, ActiveClusters acti
 }
 
 template <typename T, int MT, int NCW, bool PARTS>
-int active_clusters(int cs) {
-  struct Known { int n[kMaxCluster + 1]; };  // 1 + the answer, 0 = not asked yet
-  static PerDevice<Known> known;
-  int& k = known.here().n[cs];
-  if (k == 0) k = 1 + max_active_clusters(rnn_cluster_kernel<T, MT, NCW, PARTS>, cs, kMaxThreads);
-  return k - 1;
+int active_rnns(int cs) {
+  return active_clusters<rnn_cluster_kernel<T, MT, NCW, PARTS>>(cs, kMaxThreads);
 }
 
 template <typename T, bool PARTS>
 bool run_rnn(Launcher& lc, RnnArgs a) {
   auto active = [](int mt, int ncw, int cs) {
-    if (ncw == 4) return mt == 1 ? active_clusters<T, 1, 4, PARTS>(cs) : (mt == 2 ? active_clusters<T, 2, 4, PARTS>(cs) : active_clusters<T, 3, 4, PARTS>(cs));
-    return mt == 1 ? active_clusters<T, 1, 8, PARTS>(cs) : (mt == 2 ? active_clusters<T, 2, 8, PARTS>(cs) : active_clusters<T, 3, 8, PARTS>(cs));
+    if (ncw == 4) return mt == 1 ? active_rnns<T, 1, 4, PARTS>(cs) : (mt == 2 ? active_rnns<T, 2, 4, PARTS>(cs) : active_rnns<T, 3, 4, PARTS>(cs));
+    return mt == 1 ? active_rnns<T, 1, 8, PARTS>(cs) : (mt == 2 ? active_rnns<T, 2, 8, PARTS>(cs) : active_rnns<T, 3, 8, PARTS>(cs));
   };
   RnnPlan q;
   if (!make_rnn_plan(PARTS, (int)sizeof(T), a.B, a.u, a.in, active, &q)) return false;
