@@ -773,6 +773,16 @@ size_t smem_without_weights(int cell, bool bwd, int uc, int cs, int mt, int ex, 
   return 2 * kbh * (mt * 1024 + ex * 128) + (2 * x_bytes + 15) / 16 * 16 + (ksplit * acc + (cell == CELL_LSTM)) * outs * 8 + 64;
 }
 
+// Clocks of a step of the per-step forward kernels (gru.cu, lstm.cu) at 1.92 GHz, fitted to 400 measurements at 8 to 1536 units and
+// 1 to 2304 rows (standard deviation 6 %): 32 x 32 tiles, the contraction split over two CTAs where that still leaves at most
+// two per SM, the CTAs of an SM sharing its FP64 units.
+double per_step_clocks(int gates, int64_t B, int u, int in) {
+  const int64_t cols = (u + 31) / 32, tiles = cols * ((B + 31) / 32);
+  const int split = tiles <= 148 && cols >= 8 ? 2 : 1;
+  const int64_t per_sm = (tiles * split + 147) / 148;
+  return 17000.0 + 6800.0 * (per_sm - 1) + gates * (u + in) * 2.0 / split * (per_sm == 1 ? 20.6 : 17.7 * per_sm);
+}
+
 // The split with the smallest estimated time of a step, in clocks per SM: matrix instructions at 16 clocks each on a
 // warp's quarter of the SM (at least 60 between two that add to the same sums), the exchange (500 clocks of latency and
 // 17 bytes per clock received, both measured; the input projection overlaps it in the forward pass) and the elementwise
@@ -784,6 +794,7 @@ template <typename ActiveClusters>
 bool make_plan(int cell, bool bwd, int es, int64_t B, int u, int in, ActiveClusters active, Plan* best) {
   const int gates = cell == CELL_RNN ? 1 : (cell == CELL_GRU ? 3 : 4);
   double best_cost = 0.0;
+  int best_waves = 0;
   best->uc = 0;
   for (int uc = 8; uc <= 96; uc += 8) {
     const int cs = (u + uc - 1) / uc, ntu = uc / 8;
@@ -850,8 +861,19 @@ bool make_plan(int cell, bool bwd, int es, int64_t B, int u, int in, ActiveClust
         }
         *best = q;
         best_cost = cost;
+        best_waves = waves;
       }
     }
+  }
+  // The estimate ranks splits; against another kernel it is short of 4100 clocks and 3.3 per unit a wave, 6100 more with a ninth
+  // row and 3600 per further tile of rows (the same measurements, 6 %; weights streamed from L2 add nothing).  One launch per
+  // step is the faster forward pass where the last wave of 7 clusters is nearly empty and the per-step tiles just fill the
+  // chip: 1056 to 1184 units with 57 to 64 or 113 to 128 rows (GRU, 1152 units: 70 us a step against 56 with 64 rows, 101 against
+  // 90 with 128), LSTM, 512 units, 288 rows (67 against 62).  Elsewhere one launch is up to 6 times as fast, and exact
+  // backpropagation 1.3 to 10 times at all sizes.
+  if (!bwd && best->uc) {
+    const double one = 1.04 * best_cost + best_waves * (4100.0 + 3.3 * u + 6100.0 * best->ex + 3600.0 * (best->mt - 1));
+    if (per_step_clocks(gates, B, u, in) < 0.95 * one) best->uc = 0;
   }
   return best->uc != 0;
 }

@@ -226,8 +226,9 @@ bool rnn_forward_cluster(Launcher& lc, int dtype, const void* W, const void* U, 
 // all T steps: clusters of up to 16 CTAs own 8 to 24 batch rows, contractions on the FP64 matrix instruction.  u = units
 // (LSTM states are 2u wide); keep = the GRU's z or the LSTM's [f | 0]; coef = tanh', C4 or C5; delta may be null.
 // pack: scratch of cell_pack_bytes bytes for the weights in the kernels' order (0 = more units than this form takes).
-// false when nothing was done for the recurrence (more than 1536 units, unaligned pointers, clusters that cannot be scheduled
-// or whose launch is refused; the packing may have been enqueued): the caller then runs the per-step kernels.
+// false when nothing was done for the recurrence (more than 1536 units, a forward pass that is faster step by step, unaligned
+// pointers, clusters that cannot be scheduled or whose launch is refused; the packing may have been enqueued): the caller then
+// runs the per-step kernels.
 size_t cell_pack_bytes(int block, int u, int in_dim);
 // The split of a recurrence that these would choose where at_once[cs] clusters of cs CTAs run at a time (cs <= 16), as
 // hbp_recurrence_plan gives it; false = none.
