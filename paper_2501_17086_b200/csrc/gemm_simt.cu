@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const GemmArgs g) {
   }
 }
 
-// At most 32 rows: 32 x 32 tiles, a few blocks on an idle GPU, so what counts is the time of one block.  64 of K per block
+// At most 32 rows and a long contraction: 32 x 32 tiles, a few blocks on an idle GPU, so what counts is the time of one block.  64 of K per block
 // (one exposed memory latency, the next block's loads in flight meanwhile); four groups of 64 threads take 16 of them each
 // with a 4 x 4 micro-tile, because with one group of 256 threads and 2 x 2 the shared-memory loads bound it, and the groups'
 // sums are added in a fixed order.  32 x 64 x 256: 16.5 -> 8.5 us, 32 x 512 x
@@ -241,8 +241,12 @@ void launch_simt(Launcher& lc, const GemmArgs& g) {
     dim3 grid((g.N + 63) / 64, (g.M + 63) / 64, g.batch * g.splitk);
     gemm_simt_kernel<T, 64, 64><<<grid, 256, 0, lc.stream>>>(g);
   } else {
+    // At most 32 rows.  Up to 128 of K the plain kernel is never the slower one (a block of the small one takes 64 of K at a time
+    // and 1 to 2 us however short the contraction): 32 x 2048 x 32, 64 at once, 31 us against 82; 32 x 1024 x 64, 16 at once, 10.7
+    // against 14.7; a few tiles the same (7.9).  From 192 on the small one is: a few tiles 8 against 10.5, many 1.1 to 2.5 times.
     dim3 grid((g.N + 31) / 32, (g.M + 31) / 32, g.batch * g.splitk);
-    gemm_small_kernel<T><<<grid, 256, 0, lc.stream>>>(g);
+    if (g.K <= 128 * g.splitk) gemm_simt_kernel<T, 32, 32><<<grid, 256, 0, lc.stream>>>(g);
+    else gemm_small_kernel<T><<<grid, 256, 0, lc.stream>>>(g);
   }
   lc.ran(HBP_FORM_GEMM_SIMT);
   lc.count();
