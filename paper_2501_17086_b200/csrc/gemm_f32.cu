@@ -1,22 +1,29 @@
 // Float GEMM on the tensor cores for any orientation of the operands (residual MLPs and decoders in single precision):
-//   D(m, n) = sum_k A(m, k) B(n, k), each operand split on the way into shared memory into a tf32 high part and a tf32
-//   remainder, three tf32 products lo hi + hi lo + hi hi, the epilogues of the CUDA-core kernel.
+//   D(m, n) = sum_k A(m, k) B(n, k), each operand split on the way into shared memory into three bf16 parts that add up to it
+//   exactly, six bf16 products of parts (all but the three below 2^-26 of the whole), the epilogues of the CUDA-core kernel.
 //
 // One CTA per 128 x 128 tile (and batch entry, and split of K), 512 threads:
 //   warps 0..7   load 32-wide k-blocks of A and B from global memory (two blocks ahead, in registers), split them and store
-//                both parts as K-major 128-byte-swizzled tiles (64 KB a stage, three stages); an operand whose row index is
+//                the parts as K-major 128-byte-swizzled rows (48 KB a stage, four stages); an operand whose row index is
 //                contiguous is transposed in 4 x 4 blocks in registers on the way
 //   warps 8..15  add each finished accumulator to float sums in registers; epilogue
-//   warp 8       also issues 12 x tcgen05.mma 128x128x8 per k-block into one of two tensor-memory accumulators, before it
+//   warp 8       also issues 12 x tcgen05.mma 128x128x16 per k-block into one of two tensor-memory accumulators, before it
 //                adds up the previous block's (a warp of its own would leave 96 registers a thread instead of 128)
 // The sums leave the tensor core after every 32 of K because its accumulation truncates: the error of a long chain is a bias
-// that grows with its length (12 additions of which 4 at full magnitude here), while the additions in registers round to
-// nearest: 1.8e-7 of the result against 64 bits at K = 1560, 2.4e-7 at 4096, where the CUDA-core kernel's running float sums
-// are at 7e-7 and 1.2e-6.
+// that grows with its length, while the additions in registers round to nearest.  What is left of the bias is taken out there
+// (kOneUp).  Error against 64 bits, normal operands (2-norm): the CUDA-core kernel's running float sums; here; two tf32 parts
+// and three products, which hold 22 bits and are biased:
+//   K =   32  1.0e-7  0.7e-7  1.3e-7        K =  520  4.1e-7  1.05e-7  1.5e-7
+//   K =  128  2.0e-7  0.8e-7  1.35e-7       K = 4096  1.1e-6  2.2e-7  2.4e-7
+// and less for positive operands.  Weight gradients of float MLP stacks of 2 and 8 layers, 64 to 520 wide, 32 to 4000 rows: 0.18
+// to 1.0 times the error on the CUDA cores.  Contractions of at most one block stay there: a float sum of a few terms rounds
+// less than a block truncates (K = 4: 3.9e-8 against 4.6e-8).
 //
-// Bound by shared-memory bandwidth: per k-block 64 KB of stores and 96 KB of operand reads, 1280 clocks at 128 bytes (about
-// 1950 measured), against 768 clocks of tensor work; splitting ahead of time would need a copy of every operand in both
-// orientations.  1900 x 1560 x 520, 12 at once: 1980 -> 400 us (92 TFLOP/s); 4096 x 1024 x 4096: 1580 -> 264 us.
+// The six bf16 products cost the tensor time of three tf32 ones (768 clocks of a k-block), the parts take 48 KB of stores
+// instead of 64.  1900 x 1560 x 520, 12 at once: CUDA cores 1800 us, tf32 363, here 350 (106 TFLOP/s); rows contiguous 1700, 473,
+// 467; 4096 x 1024 x 4096: 1390, 282, 254.  Bound by the loading warps, no one thing in them: of the 350 (467) us 50 (162) go
+// without the global loads, 40 (19) without the split's arithmetic, 14 (38) without two of the three stores, 16 (29) without ten
+// of the twelve MMAs.
 #include "tc_common.cuh"
 
 namespace hbp {
@@ -26,12 +33,18 @@ using namespace tc;
 namespace {
 
 constexpr int BM = 128, BN = 128, BK = 32;
+constexpr int kShortK = BK;  // contractions up to here are the CUDA-core kernel's
 constexpr int kWorkerWarps = 8, kMmaWarp = kWorkerWarps, kAllThreads = 64 * kWorkerWarps;
-constexpr int kStages = 3;
-constexpr uint32_t kTile = BM * BK * 4, kStageBytes = 4 * kTile;  // A hi, A lo, B hi, B lo
+constexpr int kStages = 4;
+// 128 rows of 128 bytes: the high and middle parts of 32 elements of A; of B; the low parts of A and of B
+constexpr uint32_t kTile = BM * 128, kStageBytes = 3 * kTile;
 constexpr uint32_t kTmemCols = 256;
+// The tensor core truncates: a block's sums are 4.5e-8 of themselves (normal operands) to 5.1e-8 (of one sign) too small on average,
+// which adds up over the products of a stack where the float sums' roundings do not (weight gradients of 8 layers: 2.7 times the
+// error).  Three of eight blocks of a row, others in the next row, count 2^-23 = 1.19e-7 more.
+constexpr float kOneUp = 1.00000011920928955f;
 constexpr int kSmemBytes = kStages * (int)kStageBytes + 1024 /*alignment*/ + 256 /*barriers*/;
-// what each adding warp uses of the stages once all products are done (refine_non_finite's two blocks, or the epilogue's one)
+// what each adding warp uses of the stages once all products are done (refine's two blocks, or the epilogue's one)
 constexpr int kRowPitch = 33, kColPitch = 68, kWarpFloats = BK * kRowPitch + BK * kColPitch;
 static_assert(kWorkerWarps * kWarpFloats * 4 <= kStages * (int)kStageBytes && 32 * 36 <= kWarpFloats, "stages");
 
@@ -42,38 +55,51 @@ struct F32Params {
   int* status;
 };
 
-// v = hi + lo + (what a third tf32 term would hold).  The tensor core ignores the low 13 bits of an operand, so hi is
-// rounded (truncated where rounding would reach infinity) and cleared and lo only rounded; integer operations, because the
-// conversion instruction runs at a fraction of their rate.  An infinity or a NaN leaves hi infinite or NaN, so that every sum
-// it enters is one of the two (which, refine_non_finite settles).
-__device__ __forceinline__ void split_tf32x2(float v, uint32_t& hi, uint32_t& lo) {
-  const uint32_t u = __float_as_uint(v);
-  const float mag = fabsf(v);
-  hi = (mag < __uint_as_float(0x7f7ff000u) ? u + 0x1000u : u) & 0xffffe000u;
-  lo = mag == __uint_as_float(0x7f800000u) ? 0u : __float_as_uint(v - __uint_as_float(hi)) + 0x1000u;
+// a and b, each as three bf16 parts that add up to it exactly (24 bits; below 2^-109 the low part runs into the denormals and
+// loses bits), packed in pairs.  An infinity or a NaN leaves a part NaN, so that every sum it enters is not finite, which refine
+// settles.
+__device__ __forceinline__ void split_bf16x3(float a, float b, uint32_t& h, uint32_t& m, uint32_t& l) {
+  auto pack = [](float x, float y) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(x, y);
+    return *reinterpret_cast<const uint32_t*>(&v);
+  };
+  h = pack(a, b);
+  const float ra = a - __uint_as_float(h << 16), rb = b - __uint_as_float(h & 0xffff0000u);
+  m = pack(ra, rb);
+  l = pack(ra - __uint_as_float(m << 16), rb - __uint_as_float(m & 0xffff0000u));
 }
-__device__ __forceinline__ void store_split(uint32_t hi_tile, uint32_t lo_tile, int row, int unit, float a, float b, float c, float d) {
-  uint4 h, l;
-  split_tf32x2(a, h.x, l.x);
-  split_tf32x2(b, h.y, l.y);
-  split_tf32x2(c, h.z, l.z);
-  split_tf32x2(d, h.w, l.w);
-  st_shared16(swz(hi_tile, row, unit), h);
-  st_shared16(swz(lo_tile, row, unit), l);
+__device__ __forceinline__ void st_shared8(uint32_t addr, uint32_t a, uint32_t b) {
+  asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
+}
+// Four neighbours in k (unit of 4 out of 8) of a row: high and middle parts to the operand's tile, low parts to its half
+// (0 = A, 4 = B, in 16-byte units) of the common one.
+__device__ __forceinline__ void store_split(uint32_t tile, uint32_t low_tile, int low_half, int row, int unit, float a, float b, float c, float d) {
+  uint32_t h0, m0, l0, h1, m1, l1;
+  split_bf16x3(a, b, h0, m0, l0);
+  split_bf16x3(c, d, h1, m1, l1);
+  const uint32_t at = (uint32_t)(unit & 1) * 8u;
+  st_shared8(swz(tile, row, unit >> 1) + at, h0, h1);
+  st_shared8(swz(tile, row, 4 + (unit >> 1)) + at, m0, m1);
+  st_shared8(swz(low_tile, row, low_half + (unit >> 1)) + at, l0, l1);
 }
 
 // This thread's share of one operand's 128 x 32 block: four 16-byte loads.
-//   K contiguous: 8 lanes read the 8 units of a row, rows 32 apart;  rows contiguous: a 4 x 4 block, lane & 7 = unit of K
+//   K contiguous: 8 lanes read the 8 units of a row, rows 32 apart;  rows contiguous: a 4 x 4 block, lane & 7 = unit of K.
+// Either way the two rows that a half-warp stores to are 4 apart (modulo 8), and the swizzle puts them on distinct banks.
 struct Loader {
   const float* at;     // this thread's first element of the current block
   int64_t step, next;  // between its four loads, and from block to block
   int left, k, unit;   // rows from its first row to the end; first k of the thread in the current block
   bool mn;
+  __device__ __forceinline__ int k_row() const {  // of 32, for K contiguous
+    const int g = threadIdx.x >> 3;
+    return (g & ~7) | ((g & 1) << 2) | ((g >> 1) & 3);
+  }
   __device__ __forceinline__ void init(const void* p, int64_t s_row, int64_t s_k, int extent, int row0, int k0, bool mn_major) {
     const int tid = threadIdx.x;
     mn = mn_major;
     unit = tid & 7;
-    const int row = row0 + (mn ? (tid >> 3) * 4 : tid >> 3);
+    const int row = row0 + (mn ? (tid >> 3) * 4 : k_row());
     left = extent - row;
     k = k0 + unit * 4;
     at = (const float*)p + (int64_t)row * s_row + (int64_t)k * s_k;
@@ -89,17 +115,16 @@ struct Loader {
     at += next;
     k += BK;
   }
-  __device__ __forceinline__ void store(uint32_t hi_tile, uint32_t lo_tile, const float4* v) const {
-    const int tid = threadIdx.x;
+  __device__ __forceinline__ void store(uint32_t tile, uint32_t low_tile, int low_half, const float4* v) const {
     if (mn) {
-      const int r = (tid >> 3) * 4;
-      store_split(hi_tile, lo_tile, r, unit, v[0].x, v[1].x, v[2].x, v[3].x);
-      store_split(hi_tile, lo_tile, r + 1, unit, v[0].y, v[1].y, v[2].y, v[3].y);
-      store_split(hi_tile, lo_tile, r + 2, unit, v[0].z, v[1].z, v[2].z, v[3].z);
-      store_split(hi_tile, lo_tile, r + 3, unit, v[0].w, v[1].w, v[2].w, v[3].w);
+      const int r = (threadIdx.x >> 3) * 4;
+      store_split(tile, low_tile, low_half, r, unit, v[0].x, v[1].x, v[2].x, v[3].x);
+      store_split(tile, low_tile, low_half, r + 1, unit, v[0].y, v[1].y, v[2].y, v[3].y);
+      store_split(tile, low_tile, low_half, r + 2, unit, v[0].z, v[1].z, v[2].z, v[3].z);
+      store_split(tile, low_tile, low_half, r + 3, unit, v[0].w, v[1].w, v[2].w, v[3].w);
     } else {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) store_split(hi_tile, lo_tile, (tid >> 3) + 32 * i, unit, v[i].x, v[i].y, v[i].z, v[i].w);
+      for (int i = 0; i < 4; ++i) store_split(tile, low_tile, low_half, k_row() + 32 * i, unit, v[i].x, v[i].y, v[i].z, v[i].w);
     }
   }
 };
@@ -137,11 +162,13 @@ __device__ __forceinline__ void epilogue_store4(const GemmArgs& g, int b, int m,
   *reinterpret_cast<float4*>(D) = make_float4(v[0], v[1], v[2], v[3]);
 }
 
-// The sums of one warp's 32 x 64 outputs that are infinite or NaN, formed again as plain float sums in ascending order of k.
-// Three products of parts do not give what one product of the whole does there: an infinity times a remainder of zero, or of
-// the other sign, is NaN where infinity times the operand is infinity, a NaN may lose its payload and become an infinity, and a
-// part may overflow where the sum does not.  Whatever the operands, a finite sum has met neither.
-__device__ __forceinline__ void refine_non_finite(const GemmArgs& g, int b, int m0, int n0, int k_lo, int k_hi, float* smem, float (&sum)[64]) {
+// Sums that the parts may not give as the operands would: infinite or NaN ones.
+__device__ __forceinline__ bool in_doubt(float sum) { return !(fabsf(sum) < __uint_as_float(0x7f800000u)); }
+// The sums in doubt of one warp's 32 x 64 outputs, formed again as plain float sums in ascending order of k.  Products of parts
+// do not give what one product of the whole does where an operand is not finite: an infinity times a part of zero, or of the
+// other sign, is NaN where infinity times the operand is infinity, a NaN may lose its payload and become an infinity, and a
+// part may overflow where the sum does not.  Whatever the operands, a finite sum has met none of that.
+__device__ __forceinline__ void refine(const GemmArgs& g, int b, int m0, int n0, int k_lo, int k_hi, float* smem, float (&sum)[64]) {
   const int lane = threadIdx.x & 31;
   float *As = smem, *Bs = smem + BK * kRowPitch;  // [k][row], [k][column]
   const float* A = (const float*)g.A + (int64_t)b * g.a_sb;
@@ -178,7 +205,7 @@ __device__ __forceinline__ void refine_non_finite(const GemmArgs& g, int b, int 
     }
 #pragma unroll
     for (int i = 0; i < 32; ++i)
-      if (!(fabsf(sum[32 * h + i]) < __uint_as_float(0x7f800000u))) sum[32 * h + i] = acc[i];
+      if (in_doubt(sum[32 * h + i])) sum[32 * h + i] = acc[i];
   }
 }
 
@@ -245,9 +272,9 @@ __global__ void __launch_bounds__(kAllThreads, 1) gemm_f32_kernel(const F32Param
         if (kb + i >= n_kb) break;
         if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
         const uint32_t s0 = base + stage * kStageBytes;
-        la.store(s0, s0 + kTile, va[i]);
+        la.store(s0, s0 + 2 * kTile, 0, va[i]);
         la.load(k_end, va[i]);  // past the last block: nothing
-        lb.store(s0 + 2 * kTile, s0 + 3 * kTile, vb[i]);
+        lb.store(s0 + kTile, s0 + 2 * kTile, 4, vb[i]);
         lb.load(k_end, vb[i]);
         fence_async_smem();
         __syncwarp();
@@ -264,6 +291,7 @@ __global__ void __launch_bounds__(kAllThreads, 1) gemm_f32_kernel(const F32Param
     bool ok = true;
     auto drain = [&](int kb) {  // adds k-block kb's accumulator to the sums
       const int acc = kb & 1;
+      const float unbias = ((3 * kb + lane) & 7) < 3 ? kOneUp : 1.0f;
       if (!mbar_wait(accf_bar(acc), (uint32_t)((kb >> 1) & 1), abort_flag, p.status)) { ok = false; return; }
       tc_fence_after();
 #pragma unroll
@@ -276,14 +304,14 @@ __global__ void __launch_bounds__(kAllThreads, 1) gemm_f32_kernel(const F32Param
           if (lane == 0) mbar_arrive(acce_bar(acc));
         }
 #pragma unroll
-        for (int i = 0; i < 32; ++i) sum[h * 32 + i] += v[i];
+        for (int i = 0; i < 32; ++i) sum[h * 32 + i] = fmaf(v[i], unbias, sum[h * 32 + i]);
       }
     };
     if (warp == kMmaWarp) {
       uint32_t elected;
       asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(elected));
       const bool issuer = elected != 0;
-      const uint32_t idesc = (1u << 4) /*fp32 accumulate*/ | (2u << 7) | (2u << 10) /*tf32*/ | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+      const uint32_t idesc = (1u << 4) /*fp32 accumulate*/ | (1u << 7) | (1u << 10) /*bf16*/ | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
       int stage = 0;
       uint32_t phase = 0;
       for (int kb = 0; kb < n_kb; ++kb) {
@@ -294,14 +322,13 @@ __global__ void __launch_bounds__(kAllThreads, 1) gemm_f32_kernel(const F32Param
         tc_fence_after();
         if (issuer) {
           const uint32_t s0 = base + stage * kStageBytes, tmem_d = tmem_base + (uint32_t)acc * BN;
-          const uint64_t a_hi = make_desc(s0, 16u, 1024u), a_lo = make_desc(s0 + kTile, 16u, 1024u);
-          const uint64_t b_hi = make_desc(s0 + 2 * kTile, 16u, 1024u), b_lo = make_desc(s0 + 3 * kTile, 16u, 1024u);
+          const uint64_t a_h = make_desc(s0, 16u, 1024u), b_h = make_desc(s0 + kTile, 16u, 1024u);
+          const uint64_t a_l = make_desc(s0 + 2 * kTile, 16u, 1024u), a_m = a_h + 4, b_m = b_h + 4, b_l = a_l + 4;
+          const uint64_t as[6] = {a_l, a_h, a_m, a_m, a_h, a_h}, bs[6] = {b_h, b_l, b_m, b_h, b_m, b_h};  // the small terms first
 #pragma unroll
-          for (int k = 0; k < 4; ++k) tc_mma_tf32(tmem_d, a_lo + 2 * k, b_hi + 2 * k, idesc, k > 0);
+          for (int q = 0; q < 6; ++q)
 #pragma unroll
-          for (int k = 0; k < 4; ++k) tc_mma_tf32(tmem_d, a_hi + 2 * k, b_lo + 2 * k, idesc, 1u);
-#pragma unroll
-          for (int k = 0; k < 4; ++k) tc_mma_tf32(tmem_d, a_hi + 2 * k, b_hi + 2 * k, idesc, 1u);
+            for (int k = 0; k < 2; ++k) tc_mma(tmem_d, as[q] + 2 * k, bs[q] + 2 * k, idesc, q + k > 0);
           tc_commit(empty_bar(stage));
           tc_commit(accf_bar(acc));
         }
@@ -324,11 +351,11 @@ __global__ void __launch_bounds__(kAllThreads, 1) gemm_f32_kernel(const F32Param
     // its own so that 8 lanes write 32 consecutive columns of a row.
     if (ok) {
       float* buf = reinterpret_cast<float*>(aligned) + (warp - kWorkerWarps) * kWarpFloats;
-      bool finite = true;
+      bool doubt = false;
 #pragma unroll
-      for (int i = 0; i < 64; ++i) finite = finite && fabsf(sum[i]) < __uint_as_float(0x7f800000u);
-      if (__any_sync(0xffffffffu, !finite))
-        refine_non_finite(g, b, m0 + quarter * 32, n0 + half * 64, kb_lo * BK, min(g.K, kb_hi * BK), buf, sum);
+      for (int i = 0; i < 64; ++i) doubt = doubt || in_doubt(sum[i]);
+      if (__any_sync(0xffffffffu, doubt))
+        refine(g, b, m0 + quarter * 32, n0 + half * 64, kb_lo * BK, min(g.K, kb_hi * BK), buf, sum);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         __syncwarp();
@@ -372,8 +399,10 @@ bool gemm_f32_tc(Launcher& lc, const GemmArgs& g, int* status_word) {
   if (!status_word || g.in_dtype != HBP_F32 || g.A2) return false;
   if (g.M <= 0 || g.N <= 0 || g.K <= 0 || g.batch <= 0) return false;
   // Few rows are the CUDA-core kernel's: a tile would be mostly padding, and setting up tensor memory and the pipeline takes
-  // 6 us.  32 x 64 x 256: 8.5 us there against 14.5; 32 x 512 x 1024: 23 against 39; 64 x 256 x 32: 10.4 against 8.4.
-  if (g.M <= 32) return false;
+  // 6 us.  32 x 64 x 256: 9 us there against 14.5; 32 x 512 x 1024: 23 against 39.  (Many such products at once, 500 tiles or more,
+  // would take half the time here, 32 x 1024 x 4096, 16 at once, 160 us against 290: the rule does not look at that.)  So are
+  // short contractions, whose float sums have few roundings (above); 64 x 256 x 32, 8 at once: 10.4 us there against 8.7.
+  if (g.M <= 32 || g.K <= kShortK) return false;
   // the epilogue's 16-byte accesses
   auto vec = [](const void* p, int64_t ld, int64_t sb) { return !((uintptr_t)p & 15u) && ld % 4 == 0 && sb % 4 == 0; };
   if (g.N % 4 || !vec(g.D, g.ldd, g.d_sb) || g.R) return false;

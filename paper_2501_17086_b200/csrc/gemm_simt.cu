@@ -1,6 +1,6 @@
 // CUDA-core (FFMA) GEMM with arbitrary operand strides, fp32 accumulation and fused epilogues.
-// Serves the float configurations (where 1e-5 accuracy rules out reduced-precision tensor-core
-// inputs) and every bf16 problem whose shape the tcgen05 kernel does not take.
+// Serves the float products that the split-operand tensor-core kernel declines (few rows, short contractions, unaligned
+// operands) and every bf16 problem whose shape the tcgen05 kernel does not take.
 #include "hbp_internal.h"
 
 namespace hbp {

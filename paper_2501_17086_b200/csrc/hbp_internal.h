@@ -103,8 +103,8 @@ void gemm_simt(Launcher& lc, const GemmArgs& g);
 // tcgen05 / TMEM / TMA GEMM for bf16 operands; returns false if the problem does not meet its
 // alignment rules, in which case nothing was launched (gemm_tc.cu).
 bool gemm_tc(Launcher& lc, const GemmArgs& g, int* status_word);
-// Three tf32 products on the tensor cores for plain float operands of any orientation (gemm_f32.cu); false if the problem
-// does not meet its alignment rules or is too small to gain, in which case nothing was launched.
+// Six bf16 products of three parts each on the tensor cores for plain float operands of any orientation (gemm_f32.cu); false if
+// the problem does not meet its alignment rules or is too small to gain, in which case nothing was launched.
 bool gemm_f32_tc(Launcher& lc, const GemmArgs& g, int* status_word);
 // Picks gemm_tc when it applies, else gemm_simt (EPI_STORE_LN then degrades to EPI_STORE); returns
 // whether the tensor-core kernel ran.
