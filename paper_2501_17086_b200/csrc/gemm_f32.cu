@@ -16,8 +16,8 @@
 //   K =   32  1.0e-7  0.7e-7  1.3e-7        K =  520  4.1e-7  1.05e-7  1.5e-7
 //   K =  128  2.0e-7  0.8e-7  1.35e-7       K = 4096  1.1e-6  2.2e-7  2.4e-7
 // and less for positive operands.  Weight gradients of float MLP stacks of 2 and 8 layers, 64 to 520 wide, 32 to 4000 rows: 0.18
-// to 1.0 times the error on the CUDA cores.  Contractions of at most one block stay there: a float sum of a few terms rounds
-// less than a block truncates (K = 4: 3.9e-8 against 4.6e-8).
+// to 1.0 times the error on the CUDA cores.  Contractions up to 16 stay there: a float sum of a few terms rounds no more than a
+// block truncates (K = 4: 3.9e-8, 16: 7.3e-8, 20: 8.2e-8, 32: 1.03e-7 against 6.8e-8 for any K up to 32).
 //
 // The six bf16 products cost the tensor time of three tf32 ones (768 clocks of a k-block), the parts take 48 KB of stores
 // instead of 64.  1900 x 1560 x 520, 12 at once: CUDA cores 1800 us, tf32 363, here 350 (106 TFLOP/s); rows contiguous 1700, 473,
@@ -33,7 +33,7 @@ using namespace tc;
 namespace {
 
 constexpr int BM = 128, BN = 128, BK = 32;
-constexpr int kShortK = BK;  // contractions up to here are the CUDA-core kernel's
+constexpr int kShortK = 16;  // contractions up to here are the CUDA-core kernel's
 constexpr int kWorkerWarps = 8, kMmaWarp = kWorkerWarps, kAllThreads = 64 * kWorkerWarps;
 constexpr int kStages = 4;
 // 128 rows of 128 bytes: the high and middle parts of 32 elements of A; of B; the low parts of A and of B
@@ -405,7 +405,7 @@ bool gemm_f32_tc(Launcher& lc, const GemmArgs& g, int* status_word) {
   // Few rows are the CUDA-core kernel's: a tile would be mostly padding, and setting up tensor memory and the pipeline takes
   // 6 us.  32 x 64 x 256: 9 us there against 14.5; 32 x 512 x 1024: 23 against 39.  (Many such products at once, 500 tiles or more,
   // would take half the time here, 32 x 1024 x 4096, 16 at once, 160 us against 290: the rule does not look at that.)  So are
-  // short contractions, whose float sums have few roundings (above); 64 x 256 x 32, 8 at once: 10.4 us there against 8.7.
+  // short contractions, whose float sums have few roundings (above).
   if (g.M <= 32 || g.K <= kShortK) return false;
   // the epilogue's 16-byte accesses
   auto vec = [](const void* p, int64_t ld, int64_t sb) { return !((uintptr_t)p & 15u) && ld % 4 == 0 && sb % 4 == 0; };

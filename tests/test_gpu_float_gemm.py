@@ -27,7 +27,7 @@ def test_tile_edges_match_oracle(block, L, d, h, tokens):
     forward = [(tokens, h, d), (tokens, d, h)] * L
     vjp, weights = [(tokens, h, d), (tokens, d, h)], [(d, h, tokens), (h, d, tokens)]
     products = forward + vjp * (1 + L) + ([vjp[0]] + weights) * 2 + vjp * L + weights
-    taken = sum(m > 32 and k > 32 for m, n, k in products)
+    taken = sum(m > 32 and k > 16 for m, n, k in products)
     assert gpu["ctx"].forms["gemm_f32"] == taken and gpu["ctx"].forms["gemm_simt"] == len(products) - taken
     compare(w, gpu, orun.run(w, inp, ks=(1, L), grads_for=("exact", L)), (1, L), ("exact", L))
 
