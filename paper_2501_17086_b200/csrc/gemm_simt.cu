@@ -241,11 +241,12 @@ void launch_simt(Launcher& lc, const GemmArgs& g) {
     dim3 grid((g.N + 63) / 64, (g.M + 63) / 64, g.batch * g.splitk);
     gemm_simt_kernel<T, 64, 64><<<grid, 256, 0, lc.stream>>>(g);
   } else {
-    // At most 32 rows.  Up to 128 of K the plain kernel is never the slower one (a block of the small one takes 64 of K at a time
-    // and 1 to 2 us however short the contraction): 32 x 2048 x 32, 64 at once, 31 us against 82; 32 x 1024 x 64, 16 at once, 10.7
-    // against 14.7; a few tiles the same (7.9).  From 192 on the small one is: a few tiles 8 against 10.5, many 1.1 to 2.5 times.
+    // At most 32 rows.  Few tiles, or a long contraction, are the small kernel's; but a block of it takes 64 of K at a time and 1
+    // to 2 us however short the contraction, which counts where an SM gets several: 32 x 1024 x 64, 16 at once (512 tiles), 14.7
+    // us against 10.7 for the plain kernel; 32 x 2048 x 32, 64 at once, 82 against 31.  Up to 128 tiles the two are the same at 64
+    // of K (7.9 us with the launch); from 192 of K on the small one is never slower (a few tiles 8 against 10.5).
     dim3 grid((g.N + 31) / 32, (g.M + 31) / 32, g.batch * g.splitk);
-    if (g.K <= 128 * g.splitk) gemm_simt_kernel<T, 32, 32><<<grid, 256, 0, lc.stream>>>(g);
+    if (g.K <= 128 * g.splitk && (int64_t)grid.x * grid.y * grid.z > 148) gemm_simt_kernel<T, 32, 32><<<grid, 256, 0, lc.stream>>>(g);
     else gemm_small_kernel<T><<<grid, 256, 0, lc.stream>>>(g);
   }
   lc.ran(HBP_FORM_GEMM_SIMT);
