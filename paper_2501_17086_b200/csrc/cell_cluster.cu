@@ -1,4 +1,4 @@
-// The recurrences of the gated cells as ONE launch over all T steps, any number of units:
+// The recurrences of the gated cells as ONE launch over all T steps, up to 1536 units (16 CTAs of 96):
 //     forward     (GRU, LSTM) next state, stored state and the coefficients of the backward pass, from h_0 and all inputs
 //     exact BPTT  (tanh RNN, GRU, LSTM) g_t from g_{t+1}, delta_t and the stored coefficients (Section 2.2)
 // both carried in double, contractions on the FP64 matrix instruction (mma.m8n8k4.f64).
@@ -24,7 +24,7 @@
 // streaming ran at 12 bytes per clock and SM and cost more than the products.
 //
 // Measured against one launch per step (128 rows, 512 units, 212 inputs, us per step): GRU forward 35.2 -> 17.5, exact
-// 43.1 -> 11.8; LSTM forward 44.8 -> 21.1, exact 65.6 -> 15.3.  128 rows, 64 units, 4 inputs: GRU 12.4 -> 2.0 and 8.6 -> 1.8.
+// 43.1 -> 11.8; LSTM forward 44.8 -> 21.1, exact 65.6 -> 14.8.  128 rows, 64 units, 4 inputs: GRU 12.4 -> 2.0 and 8.6 -> 1.8.
 // What is left of a 512-unit GRU's forward step: 18 of 34 thousand clocks are h's products, 10 the input projection, the
 // rest the exchange and the gates.
 //

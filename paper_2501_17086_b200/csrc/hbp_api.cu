@@ -987,8 +987,10 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
   } else if (f.block == HBP_BLOCK_RNN_TANH) {
     const int T = f.L;
     // All T steps in one launch where that form applies, else one launch per step.  Of the two one-launch forms the one
-    // with 4 rows per cluster has the shorter step (512 units, 8 rows, 16 inputs: 2.4 us against 2.7) as long as its clusters run at once;
-    // with more rows they queue (32 rows, 256 inputs: 5.5 us against 3.2).
+    // with 4 rows per cluster has the shorter step as long as its clusters run at once (28 rows at 256 and 512 units, 80
+    // at 128); then they queue.  Time of the other form over its time, 1 to 28 (80) rows, 16 and 256 inputs: 512 units
+    // 0.99-1.07, 256 1.06-1.15, 128 1.03-1.19; with 4 to 16 rows more than run at once 0.63-0.72.  Exact backpropagation (there
+    // the other form is cell_cluster.cu's): 1.05-1.20, 1.20-1.59, 1.37-1.55; beyond 0.69 at 512 units, 0.90 at 256.
     const bool one_form = !ctx->force_simt && f.gate != HBP_GATE_CHANNEL_PER_STEP;
     auto four_rows = [&]() {
       return ctx->Pd && rnn_forward_persistent(r.lc, f.dtype, params->W, params->U, inputs, r.gate_ptr(0), x0, ctx->Pd, xa, ctx->C, T,
