@@ -56,8 +56,8 @@ struct F32Params {
 };
 
 // a and b, each as three bf16 parts that add up to it exactly (24 bits; below 2^-109 the low part runs into the denormals and
-// loses bits, below 2^-133 the high part vanishes), packed in pairs.  An infinity or a NaN leaves a part NaN, so that every sum
-// it enters is not finite.  refine settles both.
+// loses bits), packed in pairs.  An infinity or a NaN leaves a part NaN, so that every sum it enters is not finite, which refine
+// settles.
 __device__ __forceinline__ void split_bf16x3(float a, float b, uint32_t& h, uint32_t& m, uint32_t& l) {
   auto pack = [](float x, float y) {
     const __nv_bfloat162 v = __floats2bfloat162_rn(x, y);
@@ -162,12 +162,8 @@ __device__ __forceinline__ void epilogue_store4(const GemmArgs& g, int b, int m,
   *reinterpret_cast<float4*>(D) = make_float4(v[0], v[1], v[2], v[3]);
 }
 
-// Sums that the parts may not give as the operands would: infinite or NaN ones, and those below 2^-96, whose operands may have
-// parts in the denormals (operands of 1e-35: error 2.7e-6, of 1e-37: 2.7e-4).  A sum of exactly zero stands.
-__device__ __forceinline__ bool in_doubt(float sum) {
-  const float mag = fabsf(sum);
-  return !(mag < __uint_as_float(0x7f800000u)) || (mag < __uint_as_float(0x0f800000u) && mag > 0.0f);
-}
+// Sums that the parts may not give as the operands would: infinite or NaN ones.
+__device__ __forceinline__ bool in_doubt(float sum) { return !(fabsf(sum) < __uint_as_float(0x7f800000u)); }
 // The sums in doubt of one warp's 32 x 64 outputs, formed again as plain float sums in ascending order of k.  Products of parts
 // do not give what one product of the whole does where an operand is not finite: an infinity times a part of zero, or of the
 // other sign, is NaN where infinity times the operand is infinity, a NaN may lose its payload and become an infinity, and a
