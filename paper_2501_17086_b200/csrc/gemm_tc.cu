@@ -4,11 +4,11 @@
 //   D(m, n) = sum_k A(m, k) B(n, k), fp32 accumulate, batched (one launch covers all layers of a group).
 //
 // Persistent kernel, one CTA per SM, 320 threads:
-//   warp 0      TMA producer (one lane): fills a 4-stage ring of {A 128x64, B 256x64} bf16 tiles
-//   warp 1      MMA issuer (one lane): 4 x tcgen05.mma 128x256x16 per stage; owns the TMEM allocation
+//   warp 0      TMA producer (one lane): fills a ring of {A 128x64, B 128x64 (pairs) or 256x64} bf16 tiles
+//   warp 1      MMA issuer (one lane): 4 x tcgen05.mma of 16 of K per stage; owns the TMEM allocation
 //   warps 2..9  epilogue: two warps per 32-lane TMEM quarter, 128 accumulator columns each; each warp
-//               stages 32-row chunks through a private 4 KB swizzled buffer, so every global access of
-//               the epilogue is a TMA tile copy (the cached gelu' in, the result out)
+//               stages 32-row chunks through private 4 KB swizzled buffers, so every global access of
+//               the epilogue is a TMA tile copy (the cached gelu' in, the result out or added to what is there)
 // The 512 TMEM columns hold two 128x256 fp32 accumulators, so the epilogue of tile i overlaps the main
 // loop of tile i+1.  Either operand may be K-major (contraction index contiguous in memory) or MN-major
 // (row/column index contiguous); both are supported natively through the matrix descriptors, so neither
@@ -29,19 +29,22 @@ constexpr int BM = 128, BN = 256, BK = 64;
 constexpr int A_BYTES = BM * BK * 2;
 // Single CTA: a 128 x 256 tile, stages of {A 128 x 64, B 256 x 64} (B 64 or 128 rows for a product at most that wide).
 // CTA pair (two CTAs of a cluster on one 256 x 256 tile, tcgen05 cta_group::2): each CTA stages its own 128 rows of A
-// and its own 128 of the 256 columns of B, so a stage is 32 KB instead of 48 KB for the same flops per SM, and six
-// stages fit.
+// and its own 128 of the 256 columns of B, so a stage is 32 KB instead of 48 KB for the same flops per SM: five stages
+// and two staging buffers per epilogue warp fit (six stages and one buffer: the same main loop, 16384 x 8192 x 2048 x 4
+// 1115 -> 1174 TFLOP/s, but an epilogue that waits for each of its copies).  Single CTAs keep the deeper ring.
+constexpr int PAIR_STAGE_BYTES = A_BYTES + 128 * BK * 2;
 template <bool kPair>
 struct Mode {
   static constexpr int kBRows = kPair ? 128 : 256;
   static constexpr int kTileM = kPair ? 256 : 128;
+  static constexpr int kEpiBufs = kPair ? 2 : 1;  // staging buffers per epilogue warp
+  static constexpr int kRingBytes = kPair ? 5 * PAIR_STAGE_BYTES : 4 * (A_BYTES + 256 * BK * 2);
 };
-constexpr int PAIR_STAGES = 6, PAIR_STAGE_BYTES = A_BYTES + 128 * BK * 2;
-constexpr int RING_BYTES = 4 * (A_BYTES + 256 * BK * 2);  // = 6 stages of the pair mode
 constexpr int EPI_WARPS = 8, THREADS = 64 + 32 * EPI_WARPS;
 constexpr uint32_t TMEM_COLS = 512;
-constexpr int EPI_BUF_BYTES = 4096;  // 32 rows x 128 bytes per epilogue warp
-constexpr int SMEM_BYTES = RING_BYTES + EPI_WARPS * EPI_BUF_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
+constexpr int EPI_BUF_BYTES = 4096;  // 32 rows x 128 bytes
+constexpr int SMEM_BYTES = Mode<true>::kRingBytes + 2 * EPI_WARPS * EPI_BUF_BYTES + 1024 /*alignment slack*/ + 512 /*barriers*/;
+static_assert(Mode<false>::kRingBytes + EPI_WARPS * EPI_BUF_BYTES == Mode<true>::kRingBytes + 2 * EPI_WARPS * EPI_BUF_BYTES, "one size");
 
 struct TcParams {
   int M, N, K, batch;
@@ -65,23 +68,54 @@ struct TcParams {
 };
 
 // ------------------------------------------------------------------------------------------- epilogue math
-// Phi(z) and the normal density for bf16 outputs: erf by Abramowitz & Stegun 7.1.26 (|error| < 1.5e-7),
+// Two floats in one 64-bit register: one instruction does both (the forward GELU is bound by how many it issues).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float x, float y) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& x, float& y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v)); }
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 both(float c) { return pack2(c, c); }
+
+// z[0], z[1] -> gelu(z) in place, gelu'(z) in dz, for bf16 outputs: erf by Abramowitz & Stegun 7.1.26 (|error| < 1.5e-7),
 // sharing exp(-z^2/2) between erf and the density; the tail is formed without cancellation.
-__device__ __forceinline__ void normal_cdf_pdf(float z, float& cdf, float& pdf) {
-  const float ax = fabsf(z) * 0.70710678118654752440f;
-  float t;  // 1 / (1 + p |z| / sqrt 2) by the hardware reciprocal (relative error 2^-23: far below the formula's own)
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(0.3275911f, ax, 1.0f)));
-  const float e = __expf(-0.5f * z * z);
-  float poly = fmaf(t, 1.061405429f, -1.453152027f);
-  poly = fmaf(t, poly, 1.421413741f);
-  poly = fmaf(t, poly, -0.284496736f);
-  poly = fmaf(t, poly, 0.254829592f);
-  const float half_tail = 0.5f * poly * t * e;  // 0.5 * erfc(|z| / sqrt 2)
-  cdf = z < 0.0f ? half_tail : 1.0f - half_tail;
-  pdf = e * 0.39894228040143267794f;
+__device__ __forceinline__ void gelu_pair(float* z, float* dz) {
+  const f32x2 z2 = pack2(z[0], z[1]);
+  float t0, t1, e0, e1;
+  // 1 / (1 + p |z| / sqrt 2) by the hardware reciprocal (relative error 2^-23: far below the formula's own)
+  unpack2(fma2(both(0.3275911f * 0.70710678118654752440f), pack2(fabsf(z[0]), fabsf(z[1])), both(1.0f)), t0, t1);
+  asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(t0));
+  asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(t1));
+  unpack2(mul2(mul2(z2, z2), both(-0.5f * 1.44269504088896340736f)), e0, e1);  // exp(-z^2/2) = 2^(-z^2 log2(e) / 2)
+  asm("ex2.approx.ftz.f32 %0, %0;" : "+f"(e0));
+  asm("ex2.approx.ftz.f32 %0, %0;" : "+f"(e1));
+  const f32x2 t = pack2(t0, t1), e = pack2(e0, e1);
+  f32x2 poly = fma2(t, both(0.5f * 1.061405429f), both(0.5f * -1.453152027f));
+  poly = fma2(t, poly, both(0.5f * 1.421413741f));
+  poly = fma2(t, poly, both(0.5f * -0.284496736f));
+  poly = fma2(t, poly, both(0.5f * 0.254829592f));
+  const f32x2 tail = mul2(mul2(poly, t), e);  // 0.5 erfc(|z| / sqrt 2)
+  float lo0, lo1, hi0, hi1;
+  unpack2(tail, lo0, lo1);
+  unpack2(fma2(tail, both(-1.0f), both(1.0f)), hi0, hi1);
+  const f32x2 cdf = pack2(z[0] < 0.0f ? lo0 : hi0, z[1] < 0.0f ? lo1 : hi1);
+  unpack2(fma2(z2, mul2(e, both(0.39894228040143267794f)), cdf), dz[0], dz[1]);
+  unpack2(mul2(z2, cdf), z[0], z[1]);
 }
 
-// Residual update of the forward pass, written straight from registers (not on the hot path):
+// Residual update of the forward pass with a gate or without a float copy of the stream (EPI_ACCUM is the other one), written
+// straight from registers:
 // one thread owns `row` and the 32 accumulator columns starting at col0.
 __device__ __forceinline__ void residual_chunk(const TcParams& p, int b, int row, int col0, float* v) {
   if (row >= p.M) return;
@@ -127,7 +161,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   // same 192 KB ring is 4, 6 or 8 stages deep: the bytes in flight, not the stage count, hide the load latency
   constexpr int MAX_STAGES = 8;
   const int STAGE_BYTES = kPair ? PAIR_STAGE_BYTES : A_BYTES + p.n_mma * 128;
-  const int STAGES = kPair ? PAIR_STAGES : RING_BYTES / STAGE_BYTES;
+  constexpr int RING_BYTES = Mode<kPair>::kRingBytes, EPI_BUFS = Mode<kPair>::kEpiBufs;
+  const int STAGES = RING_BYTES / STAGE_BYTES;
   constexpr int B_ROWS = Mode<kPair>::kBRows, TILE_M = Mode<kPair>::kTileM;
   // pair mode: rank of this CTA in its pair; the even CTA (leader) owns the pipeline's full barriers and
   // issues the MMAs, its peer's tile loads signal the leader's barriers
@@ -139,18 +174,18 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   // the swizzled tiles need 1024-byte alignment
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* aligned = smem_raw + (base - smem_u32(smem_raw));
-  const uint32_t epi_base = base + RING_BYTES;  // EPI_WARPS x 4 KB, each 1024-byte aligned
-  uint64_t* bars = reinterpret_cast<uint64_t*>(aligned + RING_BYTES + EPI_WARPS * EPI_BUF_BYTES);
+  const uint32_t epi_base = base + RING_BYTES;  // EPI_WARPS x EPI_BUFS x 4 KB, each 1024-byte aligned
+  uint64_t* bars = reinterpret_cast<uint64_t*>(aligned + RING_BYTES + EPI_WARPS * EPI_BUFS * EPI_BUF_BYTES);
   // with S = MAX_STAGES: bars[0..S) full, [S..2S) empty, [2S..2S+2) accumulator full, [2S+2..2S+4) accumulator empty,
-  // [2S+4] drain, [2S+5 .. 2S+5+EPI_WARPS) one per epilogue warp for its staged operand loads
+  // [2S+4] drain, [2S+5 .. 2S+5+2*EPI_WARPS) one per staging buffer for its operand loads
   const uint32_t bar0 = smem_u32(bars);
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
   auto empty_bar = [&](int s) { return bar0 + 8u * (MAX_STAGES + s); };
   auto accf_bar = [&](int a) { return bar0 + 8u * (2 * MAX_STAGES + a); };
   auto acce_bar = [&](int a) { return bar0 + 8u * (2 * MAX_STAGES + 2 + a); };
   const uint32_t drain_bar = bar0 + 8u * (2 * MAX_STAGES + 4);
-  auto epi_bar = [&](int w) { return bar0 + 8u * (2 * MAX_STAGES + 5 + w); };
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * MAX_STAGES + 5 + EPI_WARPS);
+  auto epi_bar = [&](int w, int i) { return bar0 + 8u * (2 * MAX_STAGES + 5 + 2 * w + i); };
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * MAX_STAGES + 5 + 2 * EPI_WARPS);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -164,7 +199,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       mbar_init(acce_bar(a), kPair ? 2 * EPI_WARPS : EPI_WARPS);  // pair: both CTAs' epilogue warps arrive at the leader
     }
     mbar_init(drain_bar, 1);
-    for (int w = 0; w < EPI_WARPS; ++w) mbar_init(epi_bar(w), 1);
+    for (int w = 0; w < EPI_WARPS; ++w)
+      for (int i = 0; i < 2; ++i) mbar_init(epi_bar(w, i), 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -333,12 +369,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   } else {
     // ------------------------------------------------------------------ epilogue
     const int quarter = warp & 3, half = (warp - 2) >> 2, ew = warp - 2;
-    const uint32_t buf = epi_base + ew * EPI_BUF_BYTES;
-    const uint32_t ebar = epi_bar(ew);
-    uint32_t e_phase = 0;
-    bool e_pending = false;  // lane 0: a staged operand load is in flight
+    const uint32_t buf0 = epi_base + ew * EPI_BUFS * EPI_BUF_BYTES;
+    uint32_t e_phase = 0;    // bit i: parity of the next load into buffer i
+    uint32_t e_pending = 0;  // lane 0, bit i: a load into buffer i is in flight
     int acc = 0;
     uint32_t acc_phase = 0;
+    uint32_t next_buf = 0;
     const bool staged = p.epi != EPI_RESID;
     const bool has_e = p.epi == EPI_MUL || p.epi == EPI_STORE_LN || p.epi == EPI_ADD;
     const int cw = p.d_f32 ? 32 : 64;      // accumulator columns per staged chunk (128 bytes of output per row)
@@ -356,10 +392,17 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       const int b = tile / tiles_per_batch, r = tile % tiles_per_batch;
       const int m0 = (r / p.n_tiles) * TILE_M + (int)rank * BM, n0 = (r % p.n_tiles) * BN;  // this CTA's 128 rows
       const int row0 = m0 + quarter * 32, colw = n0 + half * 128;
-      if (has_e && lane == 0 && nchunks > 0) {  // the buffer is free here: fetch the first chunk of E while the MMAs still run
-        mbar_expect_tx(ebar, EPI_BUF_BYTES);
-        tma_load_3d(buf, &tmE, ebar, colw, row0, b);
-        e_pending = true;
+      // chunk c of E goes through buffer c % EPI_BUFS, where the result replaces it
+      auto load_e = [&](int c) {
+        const uint32_t i = c % EPI_BUFS;
+        mbar_expect_tx(epi_bar(ew, i), EPI_BUF_BYTES);
+        tma_load_3d(buf0 + i * EPI_BUF_BYTES, &tmE, epi_bar(ew, i), colw + c * cw, row0, b);
+        e_pending |= 1u << i;
+      };
+      if (has_e && lane == 0 && nchunks > 0) {  // the first chunks, while the MMAs still run
+        tma_store_wait_read();
+        load_e(0);
+        if (EPI_BUFS > 1 && nchunks > 1) load_e(1);
       }
       if (!mbar_wait(accf_bar(acc), acc_phase, abort_flag, p.status, p.wait_limit_ns)) break;
       tc_fence_after();
@@ -384,18 +427,27 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll 1
         for (int c = 0; c < nchunks; ++c) {
           float v[64];
-          tc_ld32(tsrc + c * cw, v);
-          if (!p.d_f32) tc_ld32(tsrc + c * cw + 32, v + 32);
+          tc_ld32_async(tsrc + c * cw, v);
+          if (!p.d_f32) tc_ld32_async(tsrc + c * cw + 32, v + 32);
+          tc_ld_wait();
           if (c == nchunks - 1) {  // last read of this accumulator: hand it back to the MMA warp
             tc_fence_before();
             __syncwarp();
             if (lane == 0) release_acc(acc);
           }
           const int col = colw + c * cw;
+          // the buffer this chunk goes through; without E the oldest one, once its last copy out has read it
+          const uint32_t bi = has_e ? (uint32_t)(c % EPI_BUFS) : next_buf;
+          uint32_t buf = buf0 + bi * EPI_BUF_BYTES;
+          auto take_buffer = [&]() {
+            if (lane == 0) tma_store_wait_read<EPI_BUFS - 1>();
+            __syncwarp();
+            next_buf = (next_buf + 1) % EPI_BUFS;
+          };
           if (has_e) {
-            if (!mbar_wait(ebar, e_phase, abort_flag, p.status, p.wait_limit_ns)) { ok = false; break; }
-            e_phase ^= 1u;
-            e_pending = false;
+            if (!mbar_wait(epi_bar(ew, bi), (e_phase >> bi) & 1u, abort_flag, p.status, p.wait_limit_ns)) { ok = false; break; }
+            e_phase ^= 1u << bi;
+            e_pending &= ~(1u << bi);
             if (p.epi == EPI_ADD) {  // float tile: 32 columns
 #pragma unroll
               for (int u = 0; u < 8; ++u) {
@@ -429,6 +481,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             s1 = s2 = 0.0f;
           }
           if (p.d_f32) {
+            if (!has_e) take_buffer();
 #pragma unroll
             for (int u = 0; u < 8; ++u)
               st_shared16(swz(buf, lane, u), make_uint4(__float_as_uint(v[4 * u]), __float_as_uint(v[4 * u + 1]),
@@ -436,36 +489,30 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           } else if (p.epi == EPI_GELU_FWD) {
             float dv[64];
 #pragma unroll
-            for (int i = 0; i < 64; ++i) {
-              float cdf, pdf;
-              normal_cdf_pdf(v[i], cdf, pdf);
-              dv[i] = fmaf(v[i], pdf, cdf);
-              v[i] *= cdf;
-            }
+            for (int i = 0; i < 64; i += 2) gelu_pair(v + i, dv + i);
+            take_buffer();
 #pragma unroll
             for (int u = 0; u < 8; ++u) st_shared16(swz(buf, lane, u), pack8(dv + 8 * u));
             fence_async_smem();
             __syncwarp();
-            if (lane == 0) {
-              tma_store_3d(&tmD2, buf, col, row0, b);
-              tma_store_wait_read();
-            }
-            __syncwarp();
+            if (lane == 0) tma_store_3d(&tmD2, buf, col, row0, b);
+            buf = buf0 + next_buf * EPI_BUF_BYTES;
+            take_buffer();
 #pragma unroll
             for (int u = 0; u < 8; ++u) st_shared16(swz(buf, lane, u), pack8(v + 8 * u));
           } else {
+            if (!has_e) take_buffer();
 #pragma unroll
             for (int u = 0; u < 8; ++u) st_shared16(swz(buf, lane, u), pack8(v + 8 * u));
           }
           fence_async_smem();
           __syncwarp();
           if (lane == 0) {
-            tma_store_3d(&tmD, buf, col, row0, b);
-            tma_store_wait_read();  // the buffer may be overwritten once the copy has read it
-            if (has_e && c + 1 < nchunks) {
-              mbar_expect_tx(ebar, EPI_BUF_BYTES);
-              tma_load_3d(buf, &tmE, ebar, col + cw, row0, b);
-              e_pending = true;
+            if (p.epi == EPI_ACCUM) tma_add_3d(&tmD, buf, col, row0, b);
+            else tma_store_3d(&tmD, buf, col, row0, b);
+            if (has_e && c + EPI_BUFS < nchunks) {
+              tma_store_wait_read();  // the buffer may be overwritten once the copy has read it
+              load_e(c + EPI_BUFS);
             }
           }
           __syncwarp();
@@ -476,11 +523,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
     if (lane == 0) {
       tma_store_wait_all();
-      if (e_pending) {  // only after an abort: do not leave with a copy into our buffer in flight
-        uint64_t t0 = global_ns();
-        while (!mbar_try_wait(ebar, e_phase) && global_ns() - t0 < 100000000ull) {
+      for (int i = 0; i < EPI_BUFS; ++i)
+        if ((e_pending >> i) & 1u) {  // only after an abort: do not leave with a copy into our buffer in flight
+          uint64_t t0 = global_ns();
+          while (!mbar_try_wait(epi_bar(ew, i), (e_phase >> i) & 1u) && global_ns() - t0 < 100000000ull) {
+          }
         }
-      }
     }
   }
 
@@ -583,12 +631,13 @@ bool gemm_tc(Launcher& lc, const GemmArgs& g, int* status_word) {
   const int vec = f32 ? 4 : 8;  // elements per 16 bytes
   if (g.N % vec || g.K % vec) return false;
   if (g.epi != EPI_STORE && g.epi != EPI_GELU_FWD && g.epi != EPI_MUL && g.epi != EPI_RESID && g.epi != EPI_STORE_LN &&
-      g.epi != EPI_ADD)
+      g.epi != EPI_ADD && g.epi != EPI_ACCUM)
     return false;
   if (g.epi == EPI_ADD && (!g.E || !(g.d_f32 || g.in_dtype == HBP_F32) || g.splitk > 1)) return false;  // float outputs only
   if (g.epi == EPI_STORE_LN && (!g.stats || !g.E)) return false;
   const bool out_f32 = g.d_f32 || f32;
-  if (out_f32 && g.epi != EPI_STORE && g.epi != EPI_ADD) return false;
+  if (out_f32 && g.epi != EPI_STORE && g.epi != EPI_ADD && g.epi != EPI_ACCUM) return false;
+  if (g.epi == EPI_ACCUM && (!g.d_f32 || f32 || g.splitk > 1)) return false;
   if (g.splitk > 1 && (g.epi != EPI_STORE || !out_f32 || !g.partial || g.ldd != g.N || (g.batch > 1 && g.d_sb != (int64_t)g.M * g.N)))
     return false;
   const void* A0 = f32 ? (const void*)g.A_hi : g.A;

@@ -1028,19 +1028,29 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
         if (e != cudaSuccess && r.lc.err == cudaSuccess) r.lc.err = e;
       }
     }
-    // residual update x_{l+1} = a * x_l + F through the float master copy when there is one
-    auto resid_epilogue = [&](GemmArgs& a, int step) {
+    // Residual update x_{l+1} = a * x_l + F through the float master copy when there is one.  Where the next thing done with
+    // the state is its LayerNorm, whose kernel reads the master row by row, that kernel writes the state in dtype too (ln_of),
+    // and the product only adds itself to the master.  (gates of one; the tensor-core kernel's conditions)
+    const bool ln_writes = ctx->xres && (ctx->preln || f.block == HBP_BLOCK_POSTLN_MLP);
+    auto resid_gemm = [&](GemmArgs& a, int step) {
+      if (ln_writes && !ctx->force_simt && f.gate == HBP_GATE_ONE) {
+        a.epi = EPI_ACCUM; a.d_f32 = true;
+        a.D = ctx->xres; a.ldd = d;
+        if (gemm_tc(r.lc, a, ctx->status)) return;
+        a.d_f32 = false;
+      }
       a.epi = EPI_RESID;
       a.gate = r.gate_ptr(step);
       if (ctx->xres) a.R = ctx->xres;
       else { a.E = r.at(xa, (int64_t)step * state); a.lde = d; }
       a.D = r.at(xa, (int64_t)(step + 1) * state); a.ldd = d;
       if (ctx->MASK) { a.relu = true; a.D2 = r.at(ctx->MASK, (int64_t)step * state); a.ldd2 = d; }
+      r.run_gemm(a);
     };
     auto ln_of = [&](int step) {
-      const void* src = ctx->xres ? (const void*)ctx->xres : (const void*)r.at(xa, (int64_t)step * state);
-      layernorm_fwd(r.lc, f.dtype, src, ctx->xres != nullptr, r.at(ctx->Y, (int64_t)step * state),
-                    ctx->rstd + (int64_t)step * N, N, (int)d, f.ln_eps);
+      const float* src = ctx->xres ? ctx->xres : (const float*)r.at(xa, (int64_t)step * state);
+      layernorm_fwd(r.lc, f.dtype, src, r.at(ctx->Y, (int64_t)step * state), ctx->rstd + (int64_t)step * N, N, (int)d, f.ln_eps,
+                    nullptr, ctx->xres && step > 0 ? r.at(xa, (int64_t)step * state) : nullptr);
     };
     for (int b = 0; b < f.L; ++b) {
       if (tr) {
@@ -1063,8 +1073,7 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
         o.M = (int)N; o.N = (int)d; o.K = (int)d;
         o.A = r.at(ctx->O, (int64_t)b * state); o.a_sm = d; o.a_sk = 1;
         o.B = r.at(params->Wo, (int64_t)b * d * d); o.b_sn = d; o.b_sk = 1;
-        resid_epilogue(o, step);
-        r.run_gemm(o);
+        resid_gemm(o, step);
       }
       const int step = r.mlp_step(b);
       if (ctx->preln) ln_of(step);
@@ -1080,14 +1089,14 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
       c2.M = (int)N; c2.N = (int)d; c2.K = (int)h;
       c2.A = r.at(ctx->ACT, (int64_t)b * N * h); c2.a_sm = h; c2.a_sk = 1;
       c2.B = r.at(params->W2, (int64_t)b * d * h); c2.b_sn = h; c2.b_sk = 1;
-      resid_epilogue(c2, step);
-      r.run_gemm(c2);
+      resid_gemm(c2, step);
       if (f.block == HBP_BLOCK_POSTLN_MLP) {  // x_{l+1} = LN(x_l + Block(x_l)), normalised in place; 1/sigma is the gate
-        const void* src = ctx->xres ? (const void*)ctx->xres : (const void*)r.at(xa, (int64_t)(step + 1) * state);
-        layernorm_fwd(r.lc, f.dtype, src, ctx->xres != nullptr, r.at(xa, (int64_t)(step + 1) * state),
-                      ctx->rstd + (int64_t)step * N, N, (int)d, f.ln_eps, ctx->xres);
+        const float* src = ctx->xres ? ctx->xres : (const float*)r.at(xa, (int64_t)(step + 1) * state);
+        layernorm_fwd(r.lc, f.dtype, src, r.at(xa, (int64_t)(step + 1) * state), ctx->rstd + (int64_t)step * N, N, (int)d,
+                      f.ln_eps, ctx->xres);
       }
     }
+    if (ctx->xres && ctx->preln) convert_from_f32(r.lc, ctx->xres, (bf16*)r.at(xa, (int64_t)ctx->steps * state), state);
   }
   ctx->forward_done = true;
   return r.result();

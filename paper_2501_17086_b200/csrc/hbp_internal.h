@@ -21,6 +21,7 @@ enum Epilogue {
   EPI_AFFINE = 4,    // D = (E ? E[m,n] : 0) + gate[n] * E2[m,n] + acc
   EPI_STORE_LN = 6,  // D = acc, plus per-row partial sums (sum acc, sum acc * E[m,n]) per 64 columns -> stats
   EPI_ADD = 7,       // D = acc + E[m,n]   (u_t + delta_t: the scan then reads one tensor less)
+  EPI_ACCUM = 8,     // D += acc, D float (bf16 operands on the tensor cores only: gemm_tc; gemm() does not take it)
   EPI_RNN_FWD = 5,   // c = tanh(acc + E[m,n]);  D2 = 1 - c^2;  D = gate[n] * E2[m,n] + c
 };
 
@@ -169,10 +170,11 @@ void copy_state(Launcher& lc, int dtype, void* dst, const void* src, int64_t ele
 void mul_elementwise(Launcher& lc, int dtype, void* dst, const void* a, const void* b, int64_t elems);
 // states[s][e] += carry[e] for s in [0, count)
 void add_to_states(Launcher& lc, int dtype, void* states, const void* carry, int count, int64_t elems);
-// LayerNorm forward of one state: x (float master or dtype) -> xhat (dtype), rstd (float).
-// (master, if given, receives the normalised values in float as well)
-void layernorm_fwd(Launcher& lc, int dtype, const void* x, bool x_is_f32, void* xhat, float* rstd, int64_t rows,
-                   int d, float eps, float* master = nullptr);
+// LayerNorm forward of one state in float: xhat (dtype), rstd (float); where given, master receives the normalised values in
+// float as well, and state the rows themselves in dtype.
+void layernorm_fwd(Launcher& lc, int dtype, const float* x, void* xhat, float* rstd, int64_t rows, int d, float eps,
+                   float* master = nullptr, void* state = nullptr);
+void convert_from_f32(Launcher& lc, const float* src, bf16* dst, int64_t elems);  // elems a multiple of 4
 // t = rstd (g - mean g - xo mean(g xo)) and c = t - rstd g per row (post-LN layers; xo = the layer's output state)
 void postln_prepass(Launcher& lc, int dtype, const void* g, const void* xo, const float* rstd, void* t_out, void* c_out,
                     int64_t rows, int d);

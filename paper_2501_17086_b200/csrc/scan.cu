@@ -449,54 +449,68 @@ __global__ void to_f32_kernel(const T* __restrict__ src, float* __restrict__ dst
   if (i < n) dst[i] = to_f(src[i]);
 }
 
-// xhat = (x - mean) * rstd over the last axis, biased variance; one block per row, two passes in registers.
-template <typename T, typename X>
-__global__ void __launch_bounds__(1024) layernorm_fwd_kernel(const X* __restrict__ x, T* __restrict__ xhat,
-                                                             float* __restrict__ rstd, int d, float eps,
-                                                             float* __restrict__ master) {
-  constexpr int V = Vec<T>::N;
-  __shared__ float red[2][32];
-  const int64_t row = blockIdx.x;
-  const bool active = (int)threadIdx.x * V < d;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = (blockDim.x + 31) >> 5;
-  float val[V];
+// xhat = (x - mean) * rstd over the last axis, biased variance, two passes in registers.  `wpr` warps (1, 2 or 4) of a block
+// of four hold a row, NV float4 per lane, so that a row's loads are all in flight at once and a row of up to 2048 needs no
+// block barrier.  Bound: bytes.  8192 x 1024 float -> bf16, with the state written too (67 MB): 17.6 -> 9.4 us (one block per
+// row before, without the state).  master receives the normalised values in float (post-LN layers: the float copy of the
+// residual stream continues from them), state the row itself in T (the float copy is the only one kept during the pass).
+__device__ __forceinline__ void store4(float* p, const float4& v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ __forceinline__ void store4(bf16* p, const float4& v) {
+  const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+  *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+}
+__global__ void from_f32_kernel(const float* __restrict__ src, bf16* __restrict__ dst, int64_t nvec) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < nvec) store4(dst + 4 * i, *reinterpret_cast<const float4*>(src + 4 * i));
+}
+
+constexpr int kLnWarps = 4;
+template <typename T, int NV>
+__global__ void __launch_bounds__(kLnWarps * 32) layernorm_fwd_kernel(const float* __restrict__ x, T* __restrict__ xhat,
+                                                                      float* __restrict__ rstd, int64_t rows, int d, float eps,
+                                                                      float* __restrict__ master, T* __restrict__ state, int wpr) {
+  __shared__ float red[2][kLnWarps];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t row = (int64_t)blockIdx.x * (kLnWarps / wpr) + warp / wpr;
+  const int first = (warp % wpr) * 32 + lane, nvec = row < rows ? d / 4 : 0;
+  const float* xr = x + row * d;
+  float4 v[NV];
 #pragma unroll
-  for (int i = 0; i < V; ++i) val[i] = active ? to_f(x[row * d + threadIdx.x * V + i]) : 0.0f;
-  float s1 = 0.0f;
-#pragma unroll
-  for (int i = 0; i < V; ++i) s1 += val[i];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-  if (lane == 0) red[0][warp] = s1;
-  __syncthreads();
-  float t = 0.0f;
-  for (int w = 0; w < nwarps; ++w) t += red[0][w];
-  const float mu = t / (float)d;
-  float s2 = 0.0f;
-#pragma unroll
-  for (int i = 0; i < V; ++i) {
-    const float c = active ? val[i] - mu : 0.0f;
-    s2 = fmaf(c, c, s2);
+  for (int i = 0; i < NV; ++i) {
+    const int c = first + i * wpr * 32;
+    v[i] = c < nvec ? *reinterpret_cast<const float4*>(xr + 4 * c) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   }
+  auto row_sum = [&](float s, int k) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-  if (lane == 0) red[1][warp] = s2;
-  __syncthreads();
-  t = 0.0f;
-  for (int w = 0; w < nwarps; ++w) t += red[1][w];
-  const float r = rsqrtf(t / (float)d + eps);
-  if (threadIdx.x == 0) rstd[row] = r;
-  if (active) {
-    float o[V];
-#pragma unroll
-    for (int i = 0; i < V; ++i) o[i] = (val[i] - mu) * r;
-    Vec<T> out;
-    out.set(o);
-    stv<T>(xhat + row * d + threadIdx.x * V, out);
-    if (master) {  // the float copy of the residual stream continues from the normalised values (post-LN layers)
-#pragma unroll
-      for (int i = 0; i < V; ++i) master[row * d + threadIdx.x * V + i] = o[i];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (wpr > 1) {
+      if (lane == 0) red[k][warp] = s;
+      __syncthreads();
+      s = 0.0f;
+      for (int w = 0; w < wpr; ++w) s += red[k][warp / wpr * wpr + w];
     }
+    return s;
+  };
+  float s1 = 0.0f, s2 = 0.0f;
+#pragma unroll
+  for (int i = 0; i < NV; ++i) s1 += (v[i].x + v[i].y) + (v[i].z + v[i].w);
+  const float mu = row_sum(s1, 0) / (float)d;
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    if (first + i * wpr * 32 >= nvec) continue;
+    const float a = v[i].x - mu, b = v[i].y - mu, c = v[i].z - mu, e = v[i].w - mu;
+    s2 += fmaf(a, a, b * b) + fmaf(c, c, e * e);
+  }
+  const float r = rsqrtf(row_sum(s2, 1) / (float)d + eps);
+  if (first == 0 && row < rows) rstd[row] = r;
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const int c = first + i * wpr * 32;
+    if (c >= nvec) continue;
+    const float4 o = make_float4((v[i].x - mu) * r, (v[i].y - mu) * r, (v[i].z - mu) * r, (v[i].w - mu) * r);
+    store4(xhat + row * d + 4 * c, o);
+    if (master) store4(master + row * d + 4 * c, o);
+    if (state) store4(state + row * d + 4 * c, v[i]);
   }
 }
 
@@ -765,16 +779,27 @@ void convert_to_f32(Launcher& lc, int dtype, const void* src, float* dst, int64_
   lc.check();
 }
 
-void layernorm_fwd(Launcher& lc, int dtype, const void* x, bool x_is_f32, void* xhat, float* rstd, int64_t rows,
-                   int d, float eps, float* master) {
-  const int V = dtype == HBP_F32 ? 4 : 8;
-  const int threads = row_block_threads(d, V);
-  if (dtype == HBP_F32)
-    layernorm_fwd_kernel<float, float><<<(unsigned)rows, threads, 0, lc.stream>>>((const float*)x, (float*)xhat, rstd, d, eps, master);
-  else if (x_is_f32)
-    layernorm_fwd_kernel<bf16, float><<<(unsigned)rows, threads, 0, lc.stream>>>((const float*)x, (bf16*)xhat, rstd, d, eps, master);
-  else
-    layernorm_fwd_kernel<bf16, bf16><<<(unsigned)rows, threads, 0, lc.stream>>>((const bf16*)x, (bf16*)xhat, rstd, d, eps, master);
+template <typename T>
+static void layernorm_launch(Launcher& lc, const float* x, T* xhat, float* rstd, int64_t rows, int d, float eps, float* master,
+                             T* state) {
+  const int nvec = d / 4, wpr = nvec <= 512 ? 1 : (nvec <= 1024 ? 2 : 4);  // at most 16 float4 per lane (d <= 8192)
+  const int per_lane = (nvec + 32 * wpr - 1) / (32 * wpr);
+  const int64_t per_block = kLnWarps / wpr;
+  const unsigned grid = (unsigned)((rows + per_block - 1) / per_block);
+  auto kernel = per_lane <= 4 ? layernorm_fwd_kernel<T, 4> : (per_lane <= 8 ? layernorm_fwd_kernel<T, 8> : layernorm_fwd_kernel<T, 16>);
+  kernel<<<grid, kLnWarps * 32, 0, lc.stream>>>(x, xhat, rstd, rows, d, eps, master, state, wpr);
+  lc.count();
+  lc.check();
+}
+
+void layernorm_fwd(Launcher& lc, int dtype, const float* x, void* xhat, float* rstd, int64_t rows, int d, float eps,
+                   float* master, void* state) {
+  if (dtype == HBP_F32) layernorm_launch<float>(lc, x, (float*)xhat, rstd, rows, d, eps, master, (float*)state);
+  else layernorm_launch<bf16>(lc, x, (bf16*)xhat, rstd, rows, d, eps, master, (bf16*)state);
+}
+
+void convert_from_f32(Launcher& lc, const float* src, bf16* dst, int64_t elems) {
+  from_f32_kernel<<<(unsigned)((elems / 4 + 255) / 256), 256, 0, lc.stream>>>(src, dst, elems / 4);
   lc.count();
   lc.check();
 }
