@@ -33,6 +33,18 @@ struct RingAcc<float> {
   typedef double type;  // thousands of dependent steps at 1e-5: the running value is carried in double
 };
 
+// Conversions and the step itself in the order they are written down: the interleaving of three chains is the point.
+__device__ __forceinline__ void widen(float x, double& y) { asm volatile("cvt.f64.f32 %0, %1;" : "=d"(y) : "f"(x)); }
+__device__ __forceinline__ void widen(float x, float& y) { y = x; }
+__device__ __forceinline__ void narrow(double x, float& y) { asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(y) : "d"(x)); }
+__device__ __forceinline__ void narrow(float x, float& y) { y = x; }
+__device__ __forceinline__ double step(double a, double g, double u) {
+  double r;
+  asm volatile("fma.rn.f64 %0, %1, %2, %3;" : "=d"(r) : "d"(a), "d"(g), "d"(u));
+  return r;
+}
+__device__ __forceinline__ float step(float a, float g, float u) { return a * g + u; }
+
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int c0, int c1) {
   asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(dst),
                "l"(tm), "r"(bar), "r"(c0), "r"(c1)
@@ -89,7 +101,8 @@ __global__ void __launch_bounds__((kConsumerWarps * (kOp ? 2 : 1) + 1) * 32) sca
   const int kRows = rows_ps;                       // steps per ring stage
   const int kStageBytes = rows_ps * kRowBytes;  // per stream
   extern __shared__ __align__(128) unsigned char ring_raw[];
-  unsigned char* ring = reinterpret_cast<unsigned char*>(((uintptr_t)ring_raw + 127) & ~(uintptr_t)127);
+  // (pointer arithmetic on the array itself: through an integer the compiler loses that this is shared memory)
+  unsigned char* ring = ring_raw + ((0u - smem_u32(ring_raw)) & 127u);
   uint64_t* bars = reinterpret_cast<uint64_t*>(ring + (size_t)nstages * STREAMS * kStageBytes);
   constexpr int kBarsPerStage = 2 + (kOp ? kConsumerWarps : 0);
   int* abort_flag = reinterpret_cast<int*>(bars + kBarsPerStage * nstages);
@@ -137,6 +150,8 @@ __global__ void __launch_bounds__((kConsumerWarps * (kOp ? 2 : 1) + 1) * 32) sca
         if (kOp) tma_load_2d(dst + OP_STREAM * kStageBytes, &m.mc, full_bar(slot), x0, y - 1);  // rows below 0: zero fill
       };
       int issued = 0, taken = 0;
+      // with a few stages to spare a slot is refilled one stage late, so that this lane does not wait for the box it has just sent
+      const bool late = nstages >= 4;
       for (; issued < niter && issued < nstages; ++issued) load_stage(issued);
       for (int k = 0; k < niter; ++k) {
         const int slot = k % nstages;
@@ -144,6 +159,7 @@ __global__ void __launch_bounds__((kConsumerWarps * (kOp ? 2 : 1) + 1) * 32) sca
         taken = k + 1;
         const int l_base = s.l_hi - (k + 1) * kRows;
         if (l_base >= l_box) {
+          fence_async_smem();  // the warps' results, seen through the barrier, are read by the async proxy
           const uint32_t src = smem_u32(ring + (size_t)slot * STREAMS * kStageBytes);
           if (kOp) {
             tma_store_2d(&m.oh, src, x0, l_base - 1);
@@ -152,9 +168,11 @@ __global__ void __launch_bounds__((kConsumerWarps * (kOp ? 2 : 1) + 1) * 32) sca
             tma_store_2d(&m.og, src, x0, l_base);
           }
           asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-          tma_store_wait_read();  // the slot may be overwritten once the box has been read out of it
+          // a slot may be overwritten once the box has been read out of it
+          if (late) tma_store_wait_read<1>();
+          else tma_store_wait_read();
         }
-        if (issued < niter) load_stage(issued++);
+        if (issued < niter && issued < (late ? k : k + 1) + nstages) load_stage(issued++);
       }
       // nothing of this block may still be in flight when it ends: loads that no one took (only after an abort) ...
       for (int k = taken; k < issued; ++k) {
@@ -218,7 +236,6 @@ __global__ void __launch_bounds__((kConsumerWarps * (kOp ? 2 : 1) + 1) * 32) sca
           }
         }
       }
-      fence_async_smem();  // the box is read by the async proxy
       __syncwarp();
       if (lane == 0) mbar_arrive(done_bar(slot));
     }
@@ -241,69 +258,129 @@ __global__ void __launch_bounds__((kConsumerWarps * (kOp ? 2 : 1) + 1) * 32) sca
 #pragma unroll
     for (int e = 0; e < EPT; ++e) a0[e] = to_f(((const T*)s.a)[(e0 + e) % s.d]);
   }
-  T* gp = g + (int64_t)(s.l_hi - 1) * state + e0;  // where the next step's value goes
-  // kSub rows of one stage, later steps first.  direct = the threads store g themselves (a stage that reaches below
-  // the first step, where they also stop there; or g wanted beside the operand)
-  auto sub_block = [&](unsigned char* stg, int l_top, auto direct_t, auto check_t) {
-    constexpr bool kDirect = decltype(direct_t)::value, kCheck = decltype(check_t)::value;
-    float uu[kSubRows][EPT], aa[kSubRows][EPT];
+  // A warp is alone on its scheduler, so nothing hides its latencies but its own instructions: while the kSubRows current
+  // steps are worked on, the next ones are read from shared memory and converted (8.8 clocks of issue per conversion, 18 of
+  // latency; 8.2 of latency for the multiply-add).  2048 steps x 11100 channels of two float streams on 87 SMs: 65 -> 52 clocks
+  // a step, 68 -> 54 us, 5.05 TB/s; with no work done between the copies in and out 52 us.  Shorter stages cost more: 16 rows
+  // instead of 32, 78 us.  uu, aa: the current steps, ready to use.
+  constexpr int RAW = NS + (kElemGate ? 1 : 0);
+  A uu[kSubRows][EPT], aa[kSubRows][EPT];
 #pragma unroll
-    for (int r = 0; r < kSubRows; ++r) {
+  for (int r = 0; r < kSubRows; ++r)
 #pragma unroll
-      for (int e = 0; e < EPT; ++e) {
-        uu[r][e] = 0.0f;
-        aa[r][e] = a0[e];
-      }
-      if (NS >= 1) unpack_word<T>(*reinterpret_cast<const uint32_t*>(stg + r * kRowBytes), uu[r]);
-      if (NS >= 2) {
-        float t[EPT];
-        unpack_word<T>(*reinterpret_cast<const uint32_t*>(stg + kStageBytes + r * kRowBytes), t);
-#pragma unroll
-        for (int e = 0; e < EPT; ++e) uu[r][e] += t[e];
-      }
-      if (kElemGate) unpack_word<T>(*reinterpret_cast<const uint32_t*>(stg + NS * kStageBytes + r * kRowBytes), aa[r]);
+    for (int e = 0; e < EPT; ++e) {
+      uu[r][e] = (A)0;
+      aa[r][e] = (A)a0[e];
     }
+  auto read = [&](const unsigned char* stg, uint32_t (*w)[kSubRows]) {
 #pragma unroll
-    for (int r = kSubRows - 1; r >= 0; --r) {
-      if (kCheck && l_top - (kSubRows - 1 - r) < s.l_lo) break;
+    for (int i = 0; i < RAW; ++i)
 #pragma unroll
-      for (int e = 0; e < EPT; ++e) carry[e] = (A)aa[r][e] * carry[e] + (A)uu[r][e];
-      uint32_t out;  // g_l as it is stored: one float, or two bf16
-      if (EPT == 1) {
-        out = __float_as_uint((float)carry[0]);
-      } else {
-        const __nv_bfloat162 b2 = __floats2bfloat162_rn((float)carry[0], (float)carry[EPT - 1]);
-        out = *reinterpret_cast<const uint32_t*>(&b2);
+      for (int r = 0; r < kSubRows; ++r) w[i][r] = *reinterpret_cast<const uint32_t*>(stg + i * kStageBytes + r * kRowBytes);
+  };
+  auto prepare = [&](uint32_t (*w)[kSubRows], int r) {
+    float f[EPT], t[EPT];
+    if (NS >= 1) {
+      unpack_word<T>(w[0][r], f);
+      if (NS >= 2) {
+        unpack_word<T>(w[NS - 1][r], t);
+#pragma unroll
+        for (int e = 0; e < EPT; ++e) f[e] += t[e];
       }
-      if (kDirect && live) *reinterpret_cast<uint32_t*>(gp) = out;
-      gp -= state;
-      // left in the first stream's place: for the box that goes out, or for the operand warps
-      if (!kDirect || kOp) *reinterpret_cast<uint32_t*>(stg + r * kRowBytes) = out;
+#pragma unroll
+      for (int e = 0; e < EPT; ++e) widen(f[e], uu[r][e]);
+    }
+    if (kElemGate) {
+      unpack_word<T>(w[RAW - 1][r], f);
+#pragma unroll
+      for (int e = 0; e < EPT; ++e) widen(f[e], aa[r][e]);
     }
   };
-  for (int k = 0; k < niter; ++k) {
-    const int slot = k % nstages;
-    if (!mbar_wait(full_bar(slot), (uint32_t)((k / nstages) & 1), abort_flag, status)) break;
-    unsigned char* stg = ring + (size_t)slot * STREAMS * kStageBytes + word * 4;
-    const int l_base = s.l_hi - (k + 1) * kRows;
-    if (l_base < s.l_lo) {
-#pragma unroll 1
-      for (int sb = kRows / kSubRows - 1; sb >= 0; --sb) {
-        if (store_g) sub_block(stg + sb * kSubRows * kRowBytes, l_base + sb * kSubRows + kSubRows - 1, std::true_type(), std::true_type());
-        else sub_block(stg + sb * kSubRows * kRowBytes, l_base + sb * kSubRows + kSubRows - 1, std::false_type(), std::true_type());
+  auto stage_of = [&](int k) { return ring + (size_t)(k % nstages) * STREAMS * kStageBytes + word * 4; };
+  const int sub_bytes = kSubRows * kRowBytes, top = (kRows / kSubRows - 1) * sub_bytes;  // the last rows of a stage come first
+  // kSub rows of one stage, later steps first; next = where the following ones are.  direct = the threads store g themselves
+  // (a stage that reaches below the first step, where they also stop there; or g wanted beside the operand)
+  auto sub_block = [&](unsigned char* stg, const unsigned char* next, int l_top, auto direct_t, auto check_t) {
+    constexpr bool kDirect = decltype(direct_t)::value, kCheck = decltype(check_t)::value;
+    uint32_t w[RAW][kSubRows];
+    read(next, w);
+    A was[EPT];
+    auto put = [&](int r) {
+      float o[EPT];
+#pragma unroll
+      for (int e = 0; e < EPT; ++e) narrow(was[e], o[e]);
+      uint32_t out;  // g_l as it is stored: one float, or two bf16
+      if (EPT == 1) {
+        out = __float_as_uint(o[0]);
+      } else {
+        const __nv_bfloat162 b2 = __floats2bfloat162_rn(o[0], o[EPT - 1]);
+        out = *reinterpret_cast<const uint32_t*>(&b2);
       }
-    } else if (kOp ? store_g : l_base < l_box) {
-#pragma unroll 1
-      for (int sb = kRows / kSubRows - 1; sb >= 0; --sb)
-        sub_block(stg + sb * kSubRows * kRowBytes, l_base + sb * kSubRows + kSubRows - 1, std::true_type(), std::false_type());
-    } else {
-#pragma unroll 1
-      for (int sb = kRows / kSubRows - 1; sb >= 0; --sb)
-        sub_block(stg + sb * kSubRows * kRowBytes, l_base + sb * kSubRows + kSubRows - 1, std::false_type(), std::false_type());
+      if (kDirect && live) *reinterpret_cast<uint32_t*>(g + (int64_t)(l_top - (kSubRows - 1 - r)) * state + e0) = out;
+      // left in the first stream's place: for the box that goes out, or for the operand warps
+      if (!kDirect || kOp) *reinterpret_cast<uint32_t*>(stg + r * kRowBytes) = out;
+    };
+#pragma unroll
+    for (int r = kSubRows - 1; r >= 0; --r) {
+      if (kCheck && l_top - (kSubRows - 1 - r) < s.l_lo) {
+        if (r < kSubRows - 1) put(r + 1);
+        return;
+      }
+      A is[EPT];
+#pragma unroll
+      for (int e = 0; e < EPT; ++e) is[e] = step(aa[r][e], carry[e], uu[r][e]);
+      prepare(w, r);
+      if (r < kSubRows - 1) put(r + 1);
+#pragma unroll
+      for (int e = 0; e < EPT; ++e) was[e] = carry[e] = is[e];
     }
-    if (!kOp) fence_async_smem();  // the box is read by the async proxy
+    put(0);
+  };
+  bool ready = mbar_wait(full_bar(0), 0, abort_flag, status);
+  if (ready) {
+    uint32_t w[RAW][kSubRows];
+    read(stage_of(0) + top, w);
+#pragma unroll
+    for (int r = 0; r < kSubRows; ++r) prepare(w, r);
+  }
+  for (int k = 0; k < niter && ready; ++k) {
+    const int slot = k % nstages;
+    unsigned char* sub = stage_of(k) + top;
+    const int l_base = s.l_hi - (k + 1) * kRows;
+    const bool last = k + 1 == niter;
+    const uint32_t next_full = full_bar((k + 1) % nstages), next_parity = (uint32_t)(((k + 1) / nstages) & 1);
+    bool early = false;
+    // the first rows of the next stage if they are there already; this stage is not held up for them
+    auto next_stage = [&]() -> const unsigned char* {
+      early = !last && mbar_test_wait(next_full, next_parity);
+      return early ? stage_of(k + 1) + top : stage_of(k);
+    };
+    auto stage = [&](auto direct_t, auto check_t) {
+#pragma unroll 1
+      for (int l_top = l_base + kRows - 1; l_top > l_base + kSubRows; l_top -= kSubRows, sub -= sub_bytes)
+        sub_block(sub, sub - sub_bytes, l_top, direct_t, check_t);
+      const unsigned char* next = next_stage();
+      sub_block(sub, next, l_base + kSubRows - 1, direct_t, check_t);
+    };
+    if (l_base < s.l_lo) {
+      if (store_g) stage(std::true_type(), std::true_type());
+      else stage(std::false_type(), std::true_type());
+    } else if (kOp ? store_g : l_base < l_box) {
+      stage(std::true_type(), std::false_type());
+    } else {
+      stage(std::false_type(), std::false_type());
+    }
     __syncwarp();
     if (lane == 0) mbar_arrive(kOp ? chain_bar(slot, warp) : done_bar(slot));
+    if (!last && !early) {
+      ready = mbar_wait(next_full, next_parity, abort_flag, status);
+      if (ready) {
+        uint32_t w[RAW][kSubRows];
+        read(stage_of(k + 1) + top, w);
+#pragma unroll
+        for (int r = 0; r < kSubRows; ++r) prepare(w, r);
+      }
+    }
   }
 }
 
