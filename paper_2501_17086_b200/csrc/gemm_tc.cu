@@ -31,20 +31,21 @@ constexpr int A_BYTES = BM * BK * 2;
 // CTA pair (two CTAs of a cluster on one 256 x 256 tile, tcgen05 cta_group::2): each CTA stages its own 128 rows of A
 // and its own 128 of the 256 columns of B, so a stage is 32 KB instead of 48 KB for the same flops per SM: five stages
 // and two staging buffers per epilogue warp fit (six stages and one buffer: the same main loop, 16384 x 8192 x 2048 x 4
-// 1115 -> 1174 TFLOP/s, but an epilogue that waits for each of its copies).  Single CTAs keep the deeper ring.
+// 1115 -> 1174 TFLOP/s, but an epilogue that waits for each of its copies).  Single CTAs and float operands, whose main loop
+// moves three times the bytes per flop and whose epilogue only stores, keep the deeper ring.
 constexpr int PAIR_STAGE_BYTES = A_BYTES + 128 * BK * 2;
-template <bool kPair>
+template <bool kPair, bool kTf32>
 struct Mode {
   static constexpr int kBRows = kPair ? 128 : 256;
   static constexpr int kTileM = kPair ? 256 : 128;
-  static constexpr int kEpiBufs = kPair ? 2 : 1;  // staging buffers per epilogue warp
-  static constexpr int kRingBytes = kPair ? 5 * PAIR_STAGE_BYTES : 4 * (A_BYTES + 256 * BK * 2);
+  static constexpr int kEpiBufs = kPair && !kTf32 ? 2 : 1;  // staging buffers per epilogue warp
+  static constexpr int kRingBytes = (kEpiBufs == 2 ? 5 : 6) * PAIR_STAGE_BYTES;  // single CTAs: 4, 6 or 8 stages
 };
 constexpr int EPI_WARPS = 8, THREADS = 64 + 32 * EPI_WARPS;
 constexpr uint32_t TMEM_COLS = 512;
 constexpr int EPI_BUF_BYTES = 4096;  // 32 rows x 128 bytes
-constexpr int SMEM_BYTES = Mode<true>::kRingBytes + 2 * EPI_WARPS * EPI_BUF_BYTES + 1024 /*alignment slack*/ + 512 /*barriers*/;
-static_assert(Mode<false>::kRingBytes + EPI_WARPS * EPI_BUF_BYTES == Mode<true>::kRingBytes + 2 * EPI_WARPS * EPI_BUF_BYTES, "one size");
+constexpr int SMEM_BYTES = Mode<true, false>::kRingBytes + 2 * EPI_WARPS * EPI_BUF_BYTES + 1024 /*alignment slack*/ + 512 /*barriers*/;
+static_assert(Mode<false, false>::kRingBytes + EPI_WARPS * EPI_BUF_BYTES == Mode<true, false>::kRingBytes + 2 * EPI_WARPS * EPI_BUF_BYTES, "one size");
 
 struct TcParams {
   int M, N, K, batch;
@@ -161,9 +162,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   // same 192 KB ring is 4, 6 or 8 stages deep: the bytes in flight, not the stage count, hide the load latency
   constexpr int MAX_STAGES = 8;
   const int STAGE_BYTES = kPair ? PAIR_STAGE_BYTES : A_BYTES + p.n_mma * 128;
-  constexpr int RING_BYTES = Mode<kPair>::kRingBytes, EPI_BUFS = Mode<kPair>::kEpiBufs;
+  constexpr int RING_BYTES = Mode<kPair, kTf32>::kRingBytes, EPI_BUFS = Mode<kPair, kTf32>::kEpiBufs;
   const int STAGES = RING_BYTES / STAGE_BYTES;
-  constexpr int B_ROWS = Mode<kPair>::kBRows, TILE_M = Mode<kPair>::kTileM;
+  constexpr int B_ROWS = Mode<kPair, kTf32>::kBRows, TILE_M = Mode<kPair, kTf32>::kTileM;
   // pair mode: rank of this CTA in its pair; the even CTA (leader) owns the pipeline's full barriers and
   // issues the MMAs, its peer's tile loads signal the leader's barriers
   const uint32_t rank = kPair ? cluster_ctarank() : 0u;
@@ -672,7 +673,7 @@ bool gemm_tc(Launcher& lc, const GemmArgs& g, int* status_word) {
   const bool narrow = g.N <= 128 && g.epi != EPI_STORE_LN;
   const bool pair = lc.gemm_pair && sms >= 2 && g.M > BM && !narrow;
   const int n_mma = !narrow ? BN : (g.N <= 64 ? 64 : 128);
-  const int b_rows = pair ? Mode<true>::kBRows : n_mma;
+  const int b_rows = pair ? Mode<true, false>::kBRows : n_mma;
   CUtensorMap tmA, tmB;
   if (!make_map(&tmA, A0, g.M, g.K, g.batch, a_sm, a_sk, g.a_sb, a_mn, BM, f32)) return false;
   if (!make_map(&tmB, B0, g.N, g.K, g.batch, b_sn, b_sk, g.b_sb, b_mn, b_rows, f32)) return false;
