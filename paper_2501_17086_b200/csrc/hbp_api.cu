@@ -6,6 +6,7 @@
 #include <new>
 #include <vector>
 
+#include "float_parts.cuh"
 #include "hbp_internal.h"
 
 namespace hbp {
@@ -59,6 +60,11 @@ struct hbp_ctx {
   float *Whi = nullptr, *Wlo = nullptr;
   char* U = nullptr;       // [steps][N][d] block VJP outputs (dY before the LayerNorm finish)
   char* H1 = nullptr;      // [group][N][h] dZ
+  // Float residual MLP stacks: the operands of every product as three bf16 planes (gemm_parts.cu).  OPp = what W1 is applied to
+  // [L][N][d], ACTp, DZp in the memory of ACT and H1, Gp = what the blocks are differentiated against [group][N][d]
+  bool parts = false;      // fixed by the configuration; use_parts: and by the context's modes
+  bool use_parts = false;
+  Planes OPp, ACTp, Gp, DZp, W1p, W2p;
   float2* lnpart = nullptr;  // [steps][N][slots] partial row sums of dY and dY * xhat from the GEMM epilogue
   float4* lnstat = nullptr;  // [steps][N] {rstd, mean dY, mean dY * xhat, 0}
   int ln_slots = 0;
@@ -129,6 +135,15 @@ hbp_status check_config(const hbp_config* c) {
     if (c->head_dim != 32 && c->head_dim != 64 && c->head_dim != 128) return HBP_ERR_UNSUPPORTED;
   }
   return HBP_OK;
+}
+
+// Whether a float residual MLP stack keeps its operands in parts.  Training step and exact pass, time without over time with:
+// 8 layers 64 wide (256 hidden), 64 rows 1.20 and 1.21; 64 (128) x 4096 rows 1.98 and 2.31; 132 (260) x 1000 1.33 and 1.44;
+// 1024 (4096) x 40 rows 2.0 and 2.2, x 2000 rows 2.1.  Below 64 wide the tiles are mostly padding (36 (64) x 40 rows 0.91 and
+// 0.94), and up to 32 rows the CUDA cores are faster (gemm_f32.cu).
+bool keeps_parts(const hbp_config& f) {
+  return f.dtype == HBP_F32 && (f.block == HBP_BLOCK_MLP || f.block == HBP_BLOCK_PRELN_MLP || f.block == HBP_BLOCK_RELU_MLP || f.block == HBP_BLOCK_POSTLN_MLP) &&
+         f.tokens > 32 && f.d >= 64 && f.hidden >= 64;
 }
 
 // Lays the workspace out; with base == nullptr only the total size is computed.
@@ -226,14 +241,30 @@ size_t carve(hbp_ctx* c, char* base) {
       c->CB = take(steps * N * d * es);
       c->rstd = (float*)take(steps * N * 4);
     }
-    c->ACT = take((size_t)c->layers * N * h * es);
-    c->DACT = take((size_t)c->layers * N * h * es);
+    auto take_planes = [&](Planes& P, size_t entries, size_t rows, size_t cols) {
+      P.ld = (int64_t)((cols + 63) / 64 * 64); P.sb = (int64_t)rows * P.ld; P.plane = (int64_t)entries * P.sb;
+      P.p = (bf16*)take(3 * (size_t)P.plane * 2);
+    };
+    c->parts = keeps_parts(f);
+    const size_t layers = (size_t)c->layers;
+    if (c->parts) {
+      take_planes(c->OPp, layers, N, d);
+      take_planes(c->W1p, layers, h, d);
+      take_planes(c->W2p, layers, d, h);
+      take_planes(c->ACTp, layers, N, h);
+    }
+    c->ACT = c->parts ? (char*)c->ACTp.p : take(layers * N * h * es);
+    c->DACT = take(layers * N * h * es);
     const size_t per_layer = N * h * es;
     size_t grp = ((size_t)6 << 30) / per_layer;
     if (grp < 1) grp = 1;
     if (grp > (size_t)c->layers) grp = (size_t)c->layers;
     c->group = (int)grp;
-    c->H1 = take(grp * per_layer);
+    if (c->parts) {
+      take_planes(c->Gp, grp, N, d);
+      take_planes(c->DZp, grp, N, h);
+    }
+    c->H1 = c->parts ? (char*)c->DZp.p : take(grp * per_layer);
   }
   if (f.block == HBP_BLOCK_PRELN_TRANSFORMER) {
     const size_t Lb = (size_t)f.L;
@@ -314,6 +345,45 @@ struct Run {
     b.stats_sb = (int64_t)ss * N * c->ln_slots;
   }
 
+  // ---- operands in parts (use_parts) ---------------------------------------------------------------
+  bool weights_in_parts = false;  // once per call: the caller's weights may be others in the next
+  void split_weights() {
+    if (weights_in_parts) return;
+    weights_in_parts = true;
+    split_parts(lc, (const float*)p->W1, c->W1p, c->layers * h, (int)d);
+    split_parts(lc, (const float*)p->W2, c->W2p, c->layers * d, (int)h);
+  }
+  PartsGemm parts_args(int64_t m, int64_t n, int64_t k, int batch, const Planes& A, bool a_mn, const Planes& B, bool b_mn) const {
+    PartsGemm a;
+    a.M = (int)m; a.N = (int)n; a.K = (int)k; a.batch = batch;
+    a.A = A; a.a_mn = a_mn; a.B = B; a.b_mn = b_mn;
+    return a;
+  }
+  void mlp_vjp_parts(int b0, int b1, bool want_dy, int slot) {
+    const int nb = b1 - b0;
+    split_weights();
+    split_parts(lc, (const float*)upstream(b0), c->Gp.at(slot), (int64_t)nb * N, (int)d);
+    PartsGemm a = parts_args(N, h, d, nb, c->Gp.at(slot), false, c->W2p.at(b0), true);
+    a.epi = EPI_MUL;
+    a.E = (const float*)c->DACT + (int64_t)b0 * N * h; a.lde = h; a.e_sb = N * h;
+    a.Dp = c->DZp.at(slot);
+    gemm_parts(lc, a, c->status);
+    if (!want_dy) return;
+    PartsGemm b = parts_args(N, d, h, nb, c->DZp.at(slot), false, c->W1p.at(b0), true);
+    b.D = (float*)c->U + (int64_t)b0 * state; b.ldd = d; b.d_sb = state;
+    gemm_parts(lc, b, c->status);
+  }
+  void mlp_wgrad_parts(int b0, int b1, const hbp_grads* gr) {
+    const int nb = b1 - b0;
+    PartsGemm a = parts_args(d, h, N, nb, c->Gp, true, c->ACTp.at(b0), true);
+    a.D = gr->dW2 + (int64_t)b0 * d * h; a.ldd = h; a.d_sb = d * h;
+    gemm_parts(lc, a, c->status);
+    if (!c->preln) split_parts(lc, (const float*)x_all + (int64_t)b0 * state, c->OPp.at(b0), (int64_t)nb * N, (int)d);
+    PartsGemm b = parts_args(h, d, N, nb, c->DZp, true, c->OPp.at(b0), true);
+    b.D = gr->dW1 + (int64_t)b0 * h * d; b.ldd = d; b.d_sb = h * d;
+    gemm_parts(lc, b, c->status);
+  }
+
   // What the MLP block of layer b0 is differentiated against: g_{l+1}, or mask_l * g_{l+1} for ReLU(x + Block(x))
   // (mask_gradients fills GM first).
   const char* upstream(int b0) const {
@@ -335,6 +405,7 @@ struct Run {
   // ---- MLP block: u = J^T g for layers [b0, b1) (b1 - b0 <= group), from states g[step+1] -------
   // dA = G W2, dZ = dA * gelu'(Z) -> H1 from layer `slot` on (cached derivative);  dY = dZ W1 -> U[step].
   void mlp_vjp(int b0, int b1, bool want_dy, int slot = 0) {
+    if (c->use_parts) return mlp_vjp_parts(b0, b1, want_dy, slot);
     const int nb = b1 - b0, ss = step_stride();
     GemmArgs a = base_args();
     a.M = (int)N; a.N = (int)h; a.K = (int)d; a.batch = nb;
@@ -358,6 +429,7 @@ struct Run {
   }
   // dW2 = G^T gelu(Z), dW1 = dZ^T y for layers [b0, b1); needs dZ in H1 from mlp_vjp.
   void mlp_wgrad(int b0, int b1, const hbp_grads* gr) {
+    if (c->use_parts) return mlp_wgrad_parts(b0, b1, gr);
     const int nb = b1 - b0, ss = step_stride();
     GemmArgs a = base_args();
     a.M = (int)d; a.N = (int)h; a.K = (int)N; a.batch = nb;
@@ -816,6 +888,7 @@ hbp_status hbp_create(const hbp_config* cfg, void* workspace, size_t workspace_b
   c->ws_bytes = workspace_bytes;
   const char* env = std::getenv("HBP_FORCE_SIMT");
   c->force_simt = env && env[0] == '1';
+  c->use_parts = c->parts && !c->force_simt;
   const char* pm = std::getenv("HBP_GEMM_PAIR");
   c->gemm_pair = !(pm && pm[0] == '0');  // pairs by default
   const char* so = std::getenv("HBP_SCAN_OPERAND");
@@ -1050,8 +1123,25 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
     auto ln_of = [&](int step) {
       const float* src = ctx->xres ? ctx->xres : (const float*)r.at(xa, (int64_t)step * state);
       layernorm_fwd(r.lc, f.dtype, src, r.at(ctx->Y, (int64_t)step * state), ctx->rstd + (int64_t)step * N, N, (int)d, f.ln_eps,
-                    nullptr, ctx->xres && step > 0 ? r.at(xa, (int64_t)step * state) : nullptr);
+                    nullptr, ctx->xres && step > 0 ? r.at(xa, (int64_t)step * state) : nullptr,
+                    ctx->use_parts ? ctx->OPp.at(step) : Planes());
     };
+    auto mlp_parts = [&](int b) {
+      if (!ctx->preln) split_parts(r.lc, (const float*)xa + (int64_t)b * state, ctx->OPp.at(b), N, (int)d);
+      PartsGemm a = r.parts_args(N, h, d, 1, ctx->OPp.at(b), false, ctx->W1p.at(b), false);
+      a.epi = EPI_GELU_FWD;
+      a.Dp = ctx->ACTp.at(b);
+      a.D2 = (float*)ctx->DACT + (int64_t)b * N * h; a.ldd2 = h;
+      gemm_parts(r.lc, a, ctx->status);
+      PartsGemm o = r.parts_args(N, d, h, 1, ctx->ACTp.at(b), false, ctx->W2p.at(b), false);
+      o.epi = EPI_RESID;
+      o.E = (const float*)xa + (int64_t)b * state; o.lde = d;
+      o.gate = (const float*)r.gate_ptr(b);
+      o.D = (float*)xa + (int64_t)(b + 1) * state; o.ldd = d;
+      if (ctx->MASK) { o.relu = true; o.D2 = (float*)ctx->MASK + (int64_t)b * state; o.ldd2 = d; }
+      gemm_parts(r.lc, o, ctx->status);
+    };
+    if (ctx->use_parts) r.split_weights();
     for (int b = 0; b < f.L; ++b) {
       if (tr) {
         const int step = 2 * b;
@@ -1077,23 +1167,27 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
       }
       const int step = r.mlp_step(b);
       if (ctx->preln) ln_of(step);
-      GemmArgs a = r.base_args();
-      a.M = (int)N; a.N = (int)h; a.K = (int)d;
-      a.A = r.mlp_operand(b); a.a_sm = d; a.a_sk = 1;
-      a.B = r.at(params->W1, (int64_t)b * h * d); a.b_sn = d; a.b_sk = 1;
-      a.epi = EPI_GELU_FWD;
-      a.D = r.at(ctx->ACT, (int64_t)b * N * h); a.ldd = h;
-      a.D2 = r.at(ctx->DACT, (int64_t)b * N * h); a.ldd2 = h;
-      r.run_gemm(a);
-      GemmArgs c2 = r.base_args();
-      c2.M = (int)N; c2.N = (int)d; c2.K = (int)h;
-      c2.A = r.at(ctx->ACT, (int64_t)b * N * h); c2.a_sm = h; c2.a_sk = 1;
-      c2.B = r.at(params->W2, (int64_t)b * d * h); c2.b_sn = h; c2.b_sk = 1;
-      resid_gemm(c2, step);
+      if (ctx->use_parts) {
+        mlp_parts(b);
+      } else {
+        GemmArgs a = r.base_args();
+        a.M = (int)N; a.N = (int)h; a.K = (int)d;
+        a.A = r.mlp_operand(b); a.a_sm = d; a.a_sk = 1;
+        a.B = r.at(params->W1, (int64_t)b * h * d); a.b_sn = d; a.b_sk = 1;
+        a.epi = EPI_GELU_FWD;
+        a.D = r.at(ctx->ACT, (int64_t)b * N * h); a.ldd = h;
+        a.D2 = r.at(ctx->DACT, (int64_t)b * N * h); a.ldd2 = h;
+        r.run_gemm(a);
+        GemmArgs c2 = r.base_args();
+        c2.M = (int)N; c2.N = (int)d; c2.K = (int)h;
+        c2.A = r.at(ctx->ACT, (int64_t)b * N * h); c2.a_sm = h; c2.a_sk = 1;
+        c2.B = r.at(params->W2, (int64_t)b * d * h); c2.b_sn = h; c2.b_sk = 1;
+        resid_gemm(c2, step);
+      }
       if (f.block == HBP_BLOCK_POSTLN_MLP) {  // x_{l+1} = LN(x_l + Block(x_l)), normalised in place; 1/sigma is the gate
         const float* src = ctx->xres ? ctx->xres : (const float*)r.at(xa, (int64_t)(step + 1) * state);
         layernorm_fwd(r.lc, f.dtype, src, r.at(xa, (int64_t)(step + 1) * state), ctx->rstd + (int64_t)step * N, N, (int)d,
-                      f.ln_eps, ctx->xres);
+                      f.ln_eps, ctx->xres, nullptr, Planes());
       }
     }
     if (ctx->xres && ctx->preln) convert_from_f32(r.lc, ctx->xres, (bf16*)r.at(xa, (int64_t)ctx->steps * state), state);

@@ -171,9 +171,10 @@ void mul_elementwise(Launcher& lc, int dtype, void* dst, const void* a, const vo
 // states[s][e] += carry[e] for s in [0, count)
 void add_to_states(Launcher& lc, int dtype, void* states, const void* carry, int count, int64_t elems);
 // LayerNorm forward of one state in float: xhat (dtype), rstd (float); where given, master receives the normalised values in
-// float as well, and state the rows themselves in dtype.
+// float as well, state the rows themselves in dtype, and parts (float data) the output as bf16 planes (float_parts.cuh).
+struct Planes;
 void layernorm_fwd(Launcher& lc, int dtype, const float* x, void* xhat, float* rstd, int64_t rows, int d, float eps,
-                   float* master = nullptr, void* state = nullptr);
+                   float* master, void* state, const Planes& parts);
 void convert_from_f32(Launcher& lc, const float* src, bf16* dst, int64_t elems);  // elems a multiple of 4
 // t = rstd (g - mean g - xo mean(g xo)) and c = t - rstd g per row (post-LN layers; xo = the layer's output state)
 void postln_prepass(Launcher& lc, int dtype, const void* g, const void* xo, const float* rstd, void* t_out, void* c_out,

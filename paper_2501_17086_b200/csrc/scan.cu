@@ -1,6 +1,7 @@
 // Reverse diagonal scan over depth or time (Eq. 9 / Eq. 12 with diagonal K) and the row-wise
 // elementwise kernels around it.  All access is 128-bit and coalesced along the channel axis; the
 // running value is kept in float and rounded only when stored.
+#include "float_parts.cuh"
 #include "hbp_internal.h"
 
 namespace hbp {
@@ -453,7 +454,8 @@ __global__ void to_f32_kernel(const T* __restrict__ src, float* __restrict__ dst
 // of four hold a row, NV float4 per lane, so that a row's loads are all in flight at once and a row of up to 2048 needs no
 // block barrier.  Bound: bytes.  8192 x 1024 float -> bf16, with the state written too (67 MB): 17.6 -> 9.4 us (one block per
 // row before, without the state).  master receives the normalised values in float (post-LN layers: the float copy of the
-// residual stream continues from them), state the row itself in T (the float copy is the only one kept during the pass).
+// residual stream continues from them), state the row itself in T (the float copy is the only one kept during the pass), parts
+// (float data) the output again as the next product reads it.
 __device__ __forceinline__ void store4(float* p, const float4& v) { *reinterpret_cast<float4*>(p) = v; }
 __device__ __forceinline__ void store4(bf16* p, const float4& v) {
   const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
@@ -468,7 +470,7 @@ constexpr int kLnWarps = 4;
 template <typename T, int NV>
 __global__ void __launch_bounds__(kLnWarps * 32) layernorm_fwd_kernel(const float* __restrict__ x, T* __restrict__ xhat,
                                                                       float* __restrict__ rstd, int64_t rows, int d, float eps,
-                                                                      float* __restrict__ master, T* __restrict__ state, int wpr) {
+                                                                      float* __restrict__ master, T* __restrict__ state, Planes parts, int wpr) {
   __shared__ float red[2][kLnWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t row = (int64_t)blockIdx.x * (kLnWarps / wpr) + warp / wpr;
@@ -511,6 +513,7 @@ __global__ void __launch_bounds__(kLnWarps * 32) layernorm_fwd_kernel(const floa
     store4(xhat + row * d + 4 * c, o);
     if (master) store4(master + row * d + 4 * c, o);
     if (state) store4(state + row * d + 4 * c, v[i]);
+    if (sizeof(T) == 4 && parts.p) store_parts4(parts.p + row * parts.ld + 4 * c, parts.plane, o);
   }
 }
 
@@ -781,21 +784,21 @@ void convert_to_f32(Launcher& lc, int dtype, const void* src, float* dst, int64_
 
 template <typename T>
 static void layernorm_launch(Launcher& lc, const float* x, T* xhat, float* rstd, int64_t rows, int d, float eps, float* master,
-                             T* state) {
+                             T* state, const Planes& parts) {
   const int nvec = d / 4, wpr = nvec <= 512 ? 1 : (nvec <= 1024 ? 2 : 4);  // at most 16 float4 per lane (d <= 8192)
   const int per_lane = (nvec + 32 * wpr - 1) / (32 * wpr);
   const int64_t per_block = kLnWarps / wpr;
   const unsigned grid = (unsigned)((rows + per_block - 1) / per_block);
   auto kernel = per_lane <= 4 ? layernorm_fwd_kernel<T, 4> : (per_lane <= 8 ? layernorm_fwd_kernel<T, 8> : layernorm_fwd_kernel<T, 16>);
-  kernel<<<grid, kLnWarps * 32, 0, lc.stream>>>(x, xhat, rstd, rows, d, eps, master, state, wpr);
+  kernel<<<grid, kLnWarps * 32, 0, lc.stream>>>(x, xhat, rstd, rows, d, eps, master, state, parts, wpr);
   lc.count();
   lc.check();
 }
 
 void layernorm_fwd(Launcher& lc, int dtype, const float* x, void* xhat, float* rstd, int64_t rows, int d, float eps,
-                   float* master, void* state) {
-  if (dtype == HBP_F32) layernorm_launch<float>(lc, x, (float*)xhat, rstd, rows, d, eps, master, (float*)state);
-  else layernorm_launch<bf16>(lc, x, (bf16*)xhat, rstd, rows, d, eps, master, (bf16*)state);
+                   float* master, void* state, const Planes& parts) {
+  if (dtype == HBP_F32) layernorm_launch<float>(lc, x, (float*)xhat, rstd, rows, d, eps, master, (float*)state, parts);
+  else layernorm_launch<bf16>(lc, x, (bf16*)xhat, rstd, rows, d, eps, master, (bf16*)state, parts);
 }
 
 void convert_from_f32(Launcher& lc, const float* src, bf16* dst, int64_t elems) {

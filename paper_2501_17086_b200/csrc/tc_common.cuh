@@ -82,8 +82,11 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
+// Arrives at a barrier of another CTA of the cluster after reads of tensor memory (completed, and fenced by
+// tcgen05.fence::before_thread_sync): no write of this thread has to be seen there, and a release at cluster scope, which
+// waits for all of its earlier accesses, takes 1000 to 1800 clocks while tile copies are in flight.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 // tile load of a pair: the destination is this CTA's shared memory, the barrier may be the peer's (a
 // shared::cluster address).  Each CTA fetches its own half; nothing is broadcast across the pair.
@@ -92,6 +95,13 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
   asm volatile(
       "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
       ::"r"(dst), "l"(tm), "r"(bar_cluster), "r"(c0), "r"(c1), "r"(c2)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap* tm, uint32_t bar_cluster, int c0, int c1,
+                                                 int c2, int c3) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
+      ::"r"(dst), "l"(tm), "r"(bar_cluster), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
       : "memory");
 }
 // arrives on the barrier at the same offset in both CTAs of the pair once the MMAs issued so far have completed:
@@ -192,6 +202,11 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lead_byte
   d |= (uint64_t)1 << 46;  // descriptor version of this architecture
   d |= (uint64_t)2 << 61;  // 128-byte swizzle
   return d;
+}
+
+// The same for K-major rows of 64 bytes (32 elements of K) and the 64-byte swizzle: 8-row groups 512 bytes apart.
+__device__ __forceinline__ uint64_t make_desc64(uint32_t saddr) {
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | (uint64_t)1 << 16 | (uint64_t)(512u >> 4) << 32 | (uint64_t)1 << 46 | (uint64_t)4 << 61;
 }
 
 __device__ __forceinline__ void unpack8(const uint4& raw, float* f) {
