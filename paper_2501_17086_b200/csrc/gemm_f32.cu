@@ -246,6 +246,8 @@ __global__ void __launch_bounds__(kAllThreads, 1) gemm_f32_kernel(const F32Param
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  chain_next();
+  chain_wait();
 
   const int b = blockIdx.z / g.splitk, split = blockIdx.z % g.splitk;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
@@ -429,10 +431,8 @@ bool gemm_f32_tc(Launcher& lc, const GemmArgs& g, int* status_word) {
     attr_done.here() = true;
   }
   dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, (unsigned)z);
-  gemm_f32_kernel<<<grid, kAllThreads, kSmemBytes, lc.stream>>>(p);
+  launch_chained(lc, gemm_f32_kernel, grid, kAllThreads, kSmemBytes, 1, p);
   lc.ran(HBP_FORM_GEMM_F32);
-  lc.count();
-  lc.check();
   if (g.splitk > 1) reduce_splitk(lc, g.partial, (float*)g.D, g.splitk, (int64_t)g.batch * g.M * g.N);
   return true;
 }

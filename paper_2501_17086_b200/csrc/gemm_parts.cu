@@ -124,6 +124,8 @@ gemm_parts_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   cluster_sync();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  chain_next();
+  chain_wait();
   const int tiles_per_batch = p.m_tiles * p.n_tiles, half_n = p.n_tile / 2;
 
   if (warp < 4) {
@@ -420,6 +422,8 @@ gemm_parts_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 // src [rows][4 per_row] -> planes, four floats per thread (one load where src is 16-byte aligned)
 template <bool kAligned>
 __global__ void split_parts_kernel(const float* __restrict__ src, Planes dst, int64_t n, int per_row) {
+  chain_next();
+  chain_wait();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int64_t row = i / per_row;
@@ -454,10 +458,7 @@ bool map_floats(CUtensorMap* tm, const float* base, int M, int N, int batch, int
 void split_parts(Launcher& lc, const float* src, const Planes& dst, int64_t rows, int cols) {
   const int64_t n = rows * (cols / 4);
   const unsigned grid = (unsigned)((n + 255) / 256);
-  if ((uintptr_t)src & 15u) split_parts_kernel<false><<<grid, 256, 0, lc.stream>>>(src, dst, n, cols / 4);
-  else split_parts_kernel<true><<<grid, 256, 0, lc.stream>>>(src, dst, n, cols / 4);
-  lc.count();
-  lc.check();
+  launch_chained(lc, (uintptr_t)src & 15u ? split_parts_kernel<false> : split_parts_kernel<true>, dim3(grid), 256, 0, 1, src, dst, n, cols / 4);
 }
 
 void gemm_parts(Launcher& lc, const PartsGemm& g, int* status_word) {
@@ -511,23 +512,9 @@ void gemm_parts(Launcher& lc, const PartsGemm& g, int* status_word) {
     }
     attr_done.here() = true;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(2 * (p.num_tiles < pairs ? p.num_tiles : pairs));
-  cfg.blockDim = dim3(THREADS);
-  cfg.dynamicSmemBytes = SMEM_BYTES;
-  cfg.stream = lc.stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_parts_kernel, tmA, tmB, tmD, tmD2, tmE, tmP, p);
-  if (e != cudaSuccess && lc.err == cudaSuccess) lc.err = e;
+  launch_chained(lc, gemm_parts_kernel, dim3(2 * (p.num_tiles < pairs ? p.num_tiles : pairs)), THREADS, SMEM_BYTES, 2, tmA, tmB, tmD, tmD2,
+                 tmE, tmP, p);
   lc.ran(HBP_FORM_GEMM_F32);
-  lc.count();
-  lc.check();
 }
 
 }  // namespace hbp

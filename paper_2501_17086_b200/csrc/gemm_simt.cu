@@ -224,6 +224,8 @@ __global__ void __launch_bounds__(256) gemm_small_kernel(const GemmArgs g) {
 
 __global__ void reduce_splitk_kernel(const float* __restrict__ partial, float* __restrict__ out, int splits,
                                      int64_t elems) {
+  chain_next();
+  chain_wait();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= elems) return;
   double s = 0.0;
@@ -257,9 +259,7 @@ void launch_simt(Launcher& lc, const GemmArgs& g) {
 }  // namespace
 
 void reduce_splitk(Launcher& lc, const float* partial, float* out, int splits, int64_t elems) {
-  reduce_splitk_kernel<<<(unsigned)((elems + 255) / 256), 256, 0, lc.stream>>>(partial, out, splits, elems);
-  lc.count();
-  lc.check();
+  launch_chained(lc, reduce_splitk_kernel, dim3((unsigned)((elems + 255) / 256)), 256, 0, 1, partial, out, splits, elems);
 }
 
 void gemm_simt(Launcher& lc, const GemmArgs& g) {

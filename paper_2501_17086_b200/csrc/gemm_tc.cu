@@ -224,6 +224,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   if (kPair) cluster_sync();  // the peer's barriers and tensor memory exist before anything signals them
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  chain_next();
+  chain_wait();
   const int tiles_per_batch = p.m_tiles * p.n_tiles;
   // per element size: elements per 128-byte row (= K elements per stage), bytes of one MN-major block
   const int row_elems = kTf32 ? 32 : 64;
@@ -742,28 +744,13 @@ bool gemm_tc(Launcher& lc, const GemmArgs& g, int* status_word) {
   p.stall = g.test_stall;
   if (pair) {
     const int pairs = p.num_tiles < sms / 2 ? p.num_tiles : sms / 2;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * pairs);
-    cfg.blockDim = dim3(THREADS);
-    cfg.dynamicSmemBytes = SMEM_BYTES;
-    cfg.stream = lc.stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaError_t e = f32 ? cudaLaunchKernelEx(&cfg, gemm_tc_kernel<true, true>, tmA, tmB, tmA1, tmB1, tmA2, tmB2, tmD, tmD2, tmE, p)
-                        : cudaLaunchKernelEx(&cfg, gemm_tc_kernel<true, false>, tmA, tmB, tmA1, tmB1, tmA2, tmB2, tmD, tmD2, tmE, p);
-    if (e != cudaSuccess && lc.err == cudaSuccess) lc.err = e;
+    launch_chained(lc, f32 ? gemm_tc_kernel<true, true> : gemm_tc_kernel<true, false>, dim3(2 * pairs), THREADS, SMEM_BYTES, 2, tmA, tmB,
+                   tmA1, tmB1, tmA2, tmB2, tmD, tmD2, tmE, p);
   } else {
     const int grid = p.num_tiles < sms ? p.num_tiles : sms;
-    if (f32) gemm_tc_kernel<false, true><<<grid, THREADS, SMEM_BYTES, lc.stream>>>(tmA, tmB, tmA1, tmB1, tmA2, tmB2, tmD, tmD2, tmE, p);
-    else gemm_tc_kernel<false, false><<<grid, THREADS, SMEM_BYTES, lc.stream>>>(tmA, tmB, tmA1, tmB1, tmA2, tmB2, tmD, tmD2, tmE, p);
+    launch_chained(lc, f32 ? gemm_tc_kernel<false, true> : gemm_tc_kernel<false, false>, dim3(grid), THREADS, SMEM_BYTES, 1, tmA, tmB, tmA1,
+                   tmB1, tmA2, tmB2, tmD, tmD2, tmE, p);
   }
-  lc.count();
-  lc.check();
   if (splits > 1) reduce_splitk(lc, g.partial, (float*)g.D, splits, (int64_t)g.batch * g.M * g.N);
   return true;
 }

@@ -171,6 +171,8 @@ __global__ void __launch_bounds__(256) scan_depth_kernel(const ScanArgs s) {
 // produced dy, so no reduction is needed here.  u holds dy, the VJP is rstd * (dy - m1 - xhat * m2).
 template <typename T, bool kShift>
 __global__ void __launch_bounds__(256) scan_depth_lnstat_kernel(const ScanArgs s) {
+  chain_next();
+  chain_wait();
   constexpr int V = Vec<T>::N;
   const int64_t state_elems = s.rows * s.d;
   const int64_t nvec = state_elems / V;
@@ -227,6 +229,8 @@ __global__ void __launch_bounds__(256) scan_depth_lnstat_kernel(const ScanArgs s
 
 __global__ void ln_stats_finish_kernel(const float2* __restrict__ stats, int slots, const float* __restrict__ rstd,
                                        float4* __restrict__ lnstat, int64_t count, float inv_d) {
+  chain_next();
+  chain_wait();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   float s1 = 0.0f, s2 = 0.0f;
@@ -242,6 +246,8 @@ __global__ void ln_stats_finish_kernel(const float2* __restrict__ stats, int slo
 // u holds dY = dL/d(LN(x)); the step's VJP is rstd * (dy - mean(dy) - xhat * mean(dy * xhat)).
 template <typename T>
 __global__ void __launch_bounds__(1024) scan_depth_ln_kernel(const ScanArgs s) {
+  chain_next();
+  chain_wait();
   constexpr int V = Vec<T>::N;
   __shared__ float red[2][32][2];
   const int64_t row = blockIdx.x;
@@ -446,6 +452,8 @@ __global__ void add_to_states_kernel(T* __restrict__ states, const T* __restrict
 
 template <typename T>
 __global__ void to_f32_kernel(const T* __restrict__ src, float* __restrict__ dst, int64_t n) {
+  chain_next();
+  chain_wait();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) dst[i] = to_f(src[i]);
 }
@@ -462,6 +470,8 @@ __device__ __forceinline__ void store4(bf16* p, const float4& v) {
   *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
 }
 __global__ void from_f32_kernel(const float* __restrict__ src, bf16* __restrict__ dst, int64_t nvec) {
+  chain_next();
+  chain_wait();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < nvec) store4(dst + 4 * i, *reinterpret_cast<const float4*>(src + 4 * i));
 }
@@ -471,6 +481,8 @@ template <typename T, int NV>
 __global__ void __launch_bounds__(kLnWarps * 32) layernorm_fwd_kernel(const float* __restrict__ x, T* __restrict__ xhat,
                                                                       float* __restrict__ rstd, int64_t rows, int d, float eps,
                                                                       float* __restrict__ master, T* __restrict__ state, Planes parts, int wpr) {
+  chain_next();
+  chain_wait();
   __shared__ float red[2][kLnWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t row = (int64_t)blockIdx.x * (kLnWarps / wpr) + warp / wpr;
@@ -667,22 +679,18 @@ void scan_reverse(Launcher& lc, const ScanArgs& s) {
     const unsigned grid = (unsigned)((nvec + 255) / 256);
     const bool shift = s.gamma != 0.0f;
     if (s.dtype == HBP_F32) {
-      if (shift) scan_depth_lnstat_kernel<float, true><<<grid, 256, 0, lc.stream>>>(s);
-      else scan_depth_lnstat_kernel<float, false><<<grid, 256, 0, lc.stream>>>(s);
+      if (shift) launch_chained(lc, scan_depth_lnstat_kernel<float, true>, dim3(grid), 256, 0, 1, s);
+      else launch_chained(lc, scan_depth_lnstat_kernel<float, false>, dim3(grid), 256, 0, 1, s);
     } else {
-      if (shift) scan_depth_lnstat_kernel<bf16, true><<<grid, 256, 0, lc.stream>>>(s);
-      else scan_depth_lnstat_kernel<bf16, false><<<grid, 256, 0, lc.stream>>>(s);
+      if (shift) launch_chained(lc, scan_depth_lnstat_kernel<bf16, true>, dim3(grid), 256, 0, 1, s);
+      else launch_chained(lc, scan_depth_lnstat_kernel<bf16, false>, dim3(grid), 256, 0, 1, s);
     }
-    lc.count();
-    lc.check();
     return;
   }
   if (s.xhat) {
     const int threads = row_block_threads(s.d, V);
-    if (s.dtype == HBP_F32) scan_depth_ln_kernel<float><<<(unsigned)s.rows, threads, 0, lc.stream>>>(s);
-    else scan_depth_ln_kernel<bf16><<<(unsigned)s.rows, threads, 0, lc.stream>>>(s);
-    lc.count();
-    lc.check();
+    if (s.dtype == HBP_F32) launch_chained(lc, scan_depth_ln_kernel<float>, dim3((unsigned)s.rows), threads, 0, 1, s);
+    else launch_chained(lc, scan_depth_ln_kernel<bf16>, dim3((unsigned)s.rows), threads, 0, 1, s);
     return;
   }
   const int steps = s.l_hi - s.l_lo;
@@ -727,10 +735,7 @@ void scan_reverse(Launcher& lc, const ScanArgs& s) {
 
 void ln_stats_finish(Launcher& lc, const float2* stats, int slots, const float* rstd, float4* lnstat, int64_t count,
                      int d) {
-  ln_stats_finish_kernel<<<(unsigned)((count + 255) / 256), 256, 0, lc.stream>>>(stats, slots, rstd, lnstat, count,
-                                                                                1.0f / (float)d);
-  lc.count();
-  lc.check();
+  launch_chained(lc, ln_stats_finish_kernel, dim3((unsigned)((count + 255) / 256)), 256, 0, 1, stats, slots, rstd, lnstat, count, 1.0f / (float)d);
 }
 
 void copy_state(Launcher& lc, int dtype, void* dst, const void* src, int64_t elems) {
@@ -776,10 +781,8 @@ void add_to_states(Launcher& lc, int dtype, void* states, const void* carry, int
 
 void convert_to_f32(Launcher& lc, int dtype, const void* src, float* dst, int64_t elems) {
   const unsigned grid = (unsigned)((elems + 255) / 256);
-  if (dtype == HBP_F32) to_f32_kernel<float><<<grid, 256, 0, lc.stream>>>((const float*)src, dst, elems);
-  else to_f32_kernel<bf16><<<grid, 256, 0, lc.stream>>>((const bf16*)src, dst, elems);
-  lc.count();
-  lc.check();
+  if (dtype == HBP_F32) launch_chained(lc, to_f32_kernel<float>, dim3(grid), 256, 0, 1, (const float*)src, dst, elems);
+  else launch_chained(lc, to_f32_kernel<bf16>, dim3(grid), 256, 0, 1, (const bf16*)src, dst, elems);
 }
 
 template <typename T>
@@ -790,9 +793,7 @@ static void layernorm_launch(Launcher& lc, const float* x, T* xhat, float* rstd,
   const int64_t per_block = kLnWarps / wpr;
   const unsigned grid = (unsigned)((rows + per_block - 1) / per_block);
   auto kernel = per_lane <= 4 ? layernorm_fwd_kernel<T, 4> : (per_lane <= 8 ? layernorm_fwd_kernel<T, 8> : layernorm_fwd_kernel<T, 16>);
-  kernel<<<grid, kLnWarps * 32, 0, lc.stream>>>(x, xhat, rstd, rows, d, eps, master, state, parts, wpr);
-  lc.count();
-  lc.check();
+  launch_chained(lc, kernel, dim3(grid), kLnWarps * 32, 0, 1, x, xhat, rstd, rows, d, eps, master, state, parts, wpr);
 }
 
 void layernorm_fwd(Launcher& lc, int dtype, const float* x, void* xhat, float* rstd, int64_t rows, int d, float eps,
@@ -802,9 +803,7 @@ void layernorm_fwd(Launcher& lc, int dtype, const float* x, void* xhat, float* r
 }
 
 void convert_from_f32(Launcher& lc, const float* src, bf16* dst, int64_t elems) {
-  from_f32_kernel<<<(unsigned)((elems / 4 + 255) / 256), 256, 0, lc.stream>>>(src, dst, elems / 4);
-  lc.count();
-  lc.check();
+  launch_chained(lc, from_f32_kernel, dim3((unsigned)((elems / 4 + 255) / 256)), 256, 0, 1, src, dst, elems / 4);
 }
 
 void split_tf32(Launcher& lc, const float* a, const float* b, float* hi, float* lo, int64_t elems) {
