@@ -12,6 +12,7 @@
 // [c_r | c_z | c_n] instead of the first three.  Like the tanh RNN, the recurrence itself and exact
 // backpropagation through time are carried in double beside the stored values.
 #include "cluster_split.cuh"
+#include "split_transposed.cuh"
 
 namespace hbp {
 
@@ -232,33 +233,12 @@ __global__ void gru_split_kernel(const float* __restrict__ g, const float* __res
   lo[i] = make_float4(l[0], l[1], l[2], l[3]);
 }
 
-// tf32 split of g * C4 written transposed, [4d][rows] (the weight-gradient GEMMs contract over rows)
-__global__ void __launch_bounds__(256) gru_split_transposed_kernel(const float* __restrict__ g,
-                                                                   const float* __restrict__ c4, float* __restrict__ hiT,
-                                                                   float* __restrict__ loT, int64_t rows, int d) {
-  __shared__ float th[32][33], tl[32][33];
-  const int64_t r0 = (int64_t)blockIdx.x * 32;
-  const int c0 = blockIdx.y * 32;  // column of C4 in [0, 4d)
-  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
-  for (int i = ty; i < 32; i += 8) {
-    const int64_t r = r0 + i;
-    const int c = c0 + tx;
-    float v = 0.0f;
-    if (r < rows && c < 4 * d) v = g[r * d + c % d] * c4[r * 4 * d + c];
-    const float h = round_tf32(v);
-    th[i][tx] = h;
-    tl[i][tx] = round_tf32(v - h);
-  }
-  __syncthreads();
-  for (int i = ty; i < 32; i += 8) {
-    const int c = c0 + i;
-    const int64_t r = r0 + tx;
-    if (c < 4 * d && r < rows) {
-      hiT[(int64_t)c * rows + r] = th[tx][i];
-      loT[(int64_t)c * rows + r] = tl[tx][i];
-    }
-  }
-}
+// g * c4 in [rows][4d]
+struct GruOperand {
+  const float *g, *c4;
+  int d;
+  __device__ __forceinline__ float4 operator()(int64_t r, int c) const { return mul4(load4(g + r * d + c % d), load4(c4 + r * 4 * d + c)); }
+};
 
 }  // namespace
 
@@ -341,10 +321,7 @@ void gru_split(Launcher& lc, const float* g, const float* c4, float* hi, float* 
 }
 
 void gru_split_transposed(Launcher& lc, const float* g, const float* c4, float* hiT, float* loT, int64_t rows, int d) {
-  dim3 grid((unsigned)((rows + 31) / 32), (unsigned)((4 * d + 31) / 32));
-  gru_split_transposed_kernel<<<grid, 256, 0, lc.stream>>>(g, c4, hiT, loT, rows, d);
-  lc.count();
-  lc.check();
+  launch_split_transposed(lc, GruOperand{g, c4, d}, hiT, loT, rows, 4 * d);
 }
 
 }  // namespace hbp

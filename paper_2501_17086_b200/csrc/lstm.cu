@@ -8,6 +8,7 @@
 // parameter gradients contract the same four-block operand with h and with x_t.  As for the other recurrent cells,
 // the recurrence itself and exact backpropagation through time are carried in double beside the stored values.
 #include "cluster_split.cuh"
+#include "split_transposed.cuh"
 
 namespace hbp {
 
@@ -139,7 +140,6 @@ __global__ void __launch_bounds__(256) lstm_step_kernel(const T* __restrict__ W,
 }
 
 __device__ __forceinline__ double as_d(double v) { return v; }
-__device__ __forceinline__ double as_d(float v) { return (double)v; }
 
 // element (row, column k of the [4u] operand) from the upstream gradient [g_c | g_h] and the coefficients
 // (C = the type to compute in: double for exact backpropagation, float for GEMM operands)
@@ -277,33 +277,19 @@ __global__ void __launch_bounds__(256) lstm_split_kernel(const float* __restrict
   if (uo) write_uc<float>(g_row, c5 + row * 5 * u, fg + row * 2 * u, delta ? delta + row * 2 * u : nullptr, uo + row * 2 * u, u, n);
 }
 
-// the same operand written transposed, [4u][rows] (the weight-gradient GEMMs contract over rows)
-__global__ void __launch_bounds__(256) lstm_split_transposed_kernel(const float* __restrict__ g, const float* __restrict__ c5,
-                                                                    float* __restrict__ hiT, float* __restrict__ loT,
-                                                                    int64_t rows, int u) {
-  __shared__ float th[32][33], tl[32][33];
-  const int64_t r0 = (int64_t)blockIdx.x * 32;
-  const int c0 = blockIdx.y * 32;
-  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
-  for (int i = ty; i < 32; i += 8) {
-    const int64_t r = r0 + i;
-    const int c = c0 + tx;
-    float v = 0.0f;
-    if (r < rows && c < 4 * u) v = operand_value<float, float, float>(g + r * 2 * u, c5 + r * 5 * u, u, c);
-    const float h = round_tf32(v);
-    th[i][tx] = h;
-    tl[i][tx] = round_tf32(v - h);
+// four neighbouring columns of the [4u] operand (operand_value)
+struct LstmOperand {
+  const float *g, *c5;
+  int u;
+  __device__ __forceinline__ float4 operator()(int64_t r, int c) const {
+    const float *gr = g + r * 2 * u, *cr = c5 + r * 5 * u;
+    const int q = c / u, n = c - q * u;
+    const float4 gh = load4(gr + u + n);
+    if (q == 3) return mul4(gh, load4(cr + 3 * u + n));
+    const float4 gc = load4(gr + n), ch = load4(cr + 4 * u + n);
+    return mul4(make_float4(gc.x + gh.x * ch.x, gc.y + gh.y * ch.y, gc.z + gh.z * ch.z, gc.w + gh.w * ch.w), load4(cr + q * u + n));
   }
-  __syncthreads();
-  for (int i = ty; i < 32; i += 8) {
-    const int c = c0 + i;
-    const int64_t r = r0 + tx;
-    if (c < 4 * u && r < rows) {
-      hiT[(int64_t)c * rows + r] = th[tx][i];
-      loT[(int64_t)c * rows + r] = tl[tx][i];
-    }
-  }
-}
+};
 
 }  // namespace
 
@@ -391,10 +377,7 @@ void lstm_split(Launcher& lc, const float* g, const float* c5, const float* fg, 
 }
 
 void lstm_split_transposed(Launcher& lc, const float* g, const float* c5, float* hiT, float* loT, int64_t rows, int u) {
-  dim3 grid((unsigned)((rows + 31) / 32), (unsigned)((4 * u + 31) / 32));
-  lstm_split_transposed_kernel<<<grid, 256, 0, lc.stream>>>(g, c5, hiT, loT, rows, u);
-  lc.count();
-  lc.check();
+  launch_split_transposed(lc, LstmOperand{g, c5, u}, hiT, loT, rows, 4 * u);
 }
 
 }  // namespace hbp

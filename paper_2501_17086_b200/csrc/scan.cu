@@ -3,6 +3,7 @@
 // running value is kept in float and rounded only when stored.
 #include "float_parts.cuh"
 #include "hbp_internal.h"
+#include "split_transposed.cuh"
 
 namespace hbp {
 
@@ -626,35 +627,25 @@ __global__ void split_tf32_kernel(const float4* __restrict__ a, const float4* __
   hi[i] = h;
   lo[i] = l;
 }
-__global__ void __launch_bounds__(256) split_tf32_transposed_kernel(const float* __restrict__ a, const float* __restrict__ b,
-                                                                    float* __restrict__ hiT, float* __restrict__ loT,
-                                                                    int64_t rows, int cols, int64_t ld) {
-  __shared__ float th[32][33], tl[32][33];
-  const int64_t r0 = (int64_t)blockIdx.x * 32;
-  const int c0 = blockIdx.y * 32;
-  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;  // ty in 0..7
-  for (int i = ty; i < 32; i += 8) {
-    const int64_t r = r0 + i;
-    const int c = c0 + tx;
-    float v = 0.0f;
-    if (r < rows && c < cols) {
-      v = a[r * ld + c];
-      if (b) v *= b[r * ld + c];
-    }
-    const float h = round_tf32(v);
-    th[i][tx] = h;
-    tl[i][tx] = round_tf32(v - h);
+
+// a, or a * b, with ld elements between rows
+struct ProductValue {
+  const float *a, *b;
+  int64_t ld;
+  __device__ __forceinline__ float4 operator()(int64_t r, int c) const {
+    const float4 v = load4(a + r * ld + c);
+    return b ? mul4(v, load4(b + r * ld + c)) : v;
   }
-  __syncthreads();
-  for (int i = ty; i < 32; i += 8) {
-    const int c = c0 + i;
-    const int64_t r = r0 + tx;
-    if (c < cols && r < rows) {
-      hiT[(int64_t)c * rows + r] = th[tx][i];
-      loT[(int64_t)c * rows + r] = tl[tx][i];
-    }
+};
+// the same where a is not 16-byte aligned (a caller's inputs or weights)
+struct UnalignedValue {
+  const float* a;
+  int64_t ld;
+  __device__ __forceinline__ float4 operator()(int64_t r, int c) const {
+    const float* p = a + r * ld + c;
+    return make_float4(p[0], p[1], p[2], p[3]);
   }
-}
+};
 
 inline int row_block_threads(int d, int V) {
   int t = (d / V + 31) / 32 * 32;
@@ -816,10 +807,9 @@ void split_tf32(Launcher& lc, const float* a, const float* b, float* hi, float* 
 
 void split_tf32_transposed(Launcher& lc, const float* a, const float* b, float* hiT, float* loT, int64_t rows, int cols,
                            int64_t ld) {
-  dim3 grid((unsigned)((rows + 31) / 32), (unsigned)((cols + 31) / 32));
-  split_tf32_transposed_kernel<<<grid, 256, 0, lc.stream>>>(a, b, hiT, loT, rows, cols, ld > 0 ? ld : cols);
-  lc.count();
-  lc.check();
+  if (ld <= 0) ld = cols;
+  if ((uintptr_t)a & 15u) launch_split_transposed(lc, UnalignedValue{a, ld}, hiT, loT, rows, cols);  // (never with b)
+  else launch_split_transposed(lc, ProductValue{a, b, ld}, hiT, loT, rows, cols);
 }
 
 void gate_grad(Launcher& lc, int dtype, const void* g, const void* x, int64_t rows_total, int d, float* da,
