@@ -1,4 +1,5 @@
-// Float GEMM on the tensor cores for any orientation of the operands (residual MLPs and decoders in single precision):
+// Float GEMM on the tensor cores for any orientation of the operands (decoders in single precision, MLP stacks up to 63 wide; wider
+// ones keep their operands in parts: gemm_parts.cu):
 //   D(m, n) = sum_k A(m, k) B(n, k), each operand split on the way into shared memory into three bf16 parts that add up to it
 //   exactly, six bf16 products of parts (all but the three below 2^-26 of the whole), the epilogues of the CUDA-core kernel.
 //
