@@ -58,30 +58,30 @@ def config_of(w, k, touched_bytes=None):
 # profiles/.  An entry is used only while the kernel's sources still hash to the value recorded with the capture and
 # the workload has the captured shapes; otherwise the bench line carries "traffic": null.
 TRAFFIC = {
-    # gemm_tc_kernel, VJP pair (dA + dY): c5_small (4 layers x 16384 tokens): 2050.448 + 1063.307 and 2531.918 + 292.011 MB;
-    # c2_small (8 layers x 8192 tokens): 738.928 + 506.633 and 809.241 + 133.026 MB
+    # gemm_tc_kernel, VJP pair (dA + dY): c5_small (4 layers x 16384 tokens): 2063.204 + 1055.452 and 2749.347 + 279.092 MB;
+    # c2_small (8 layers x 8192 tokens): 738.612 + 504.159 and 790.034 + 129.739 MB
     "gemm_vjp": [
-        {"sources": ("gemm_tc.cu", "tc_common.cuh"), "sha256": "a0699ad7953dac89", "shape": ("preln_mlp", "bf16", 2048, 8192),
-         "bytes_per_token_layer": (2050.448e6 + 1063.307e6 + 2531.918e6 + 292.011e6) / (4 * 16384),
+        {"sources": ("gemm_tc.cu", "tc_common.cuh"), "sha256": "d3caab9167812b48", "shape": ("preln_mlp", "bf16", 2048, 8192),
+         "bytes_per_token_layer": (2063.204e6 + 1055.452e6 + 2749.347e6 + 279.092e6) / (4 * 16384),
          "profile": "profiles/gemm_tc_kernel_c5_small.md"},
-        {"sources": ("gemm_tc.cu", "tc_common.cuh"), "sha256": "a0699ad7953dac89", "shape": ("preln_mlp", "bf16", 1024, 4096),
-         "bytes_per_token_layer": (738.928e6 + 506.633e6 + 809.241e6 + 133.026e6) / (8 * 8192),
+        {"sources": ("gemm_tc.cu", "tc_common.cuh"), "sha256": "d3caab9167812b48", "shape": ("preln_mlp", "bf16", 1024, 4096),
+         "bytes_per_token_layer": (738.612e6 + 504.159e6 + 790.034e6 + 129.739e6) / (8 * 8192),
          "profile": "profiles/gemm_tc_kernel_c2_small.md"}],
-    # scan_depth_lnstat_kernel: c5_small 605.152 MB read + 213.872 MB written for 4 steps x 16384 x 2048 elements; c2_small
-    # 286.336 + 80.986 MB for 8 x 8192 x 1024 (the writes still in L2 when such a small launch ends are not in the counter)
+    # scan_depth_lnstat_kernel: c5_small 605.051 MB read + 213.533 MB written for 4 steps x 16384 x 2048 elements; c2_small
+    # 286.285 + 80.494 MB for 8 x 8192 x 1024 (the writes still in L2 when such a small launch ends are not in the counter)
     "scan_lnstat": [
-        {"sources": ("scan.cu",), "sha256": "981b284763a28eb7", "shape": ("preln_mlp", "bf16", 2048, 8192),
-         "bytes_per_state_element_step": (605.152e6 + 213.872e6) / (4 * 16384 * 2048),
+        {"sources": ("scan.cu",), "sha256": "0f92d71cff018e9f", "shape": ("preln_mlp", "bf16", 2048, 8192),
+         "bytes_per_state_element_step": (605.051e6 + 213.533e6) / (4 * 16384 * 2048),
          "profile": "profiles/scan_depth_lnstat_kernel_c5_small.md"},
-        {"sources": ("scan.cu",), "sha256": "981b284763a28eb7", "shape": ("preln_mlp", "bf16", 1024, 4096),
-         "bytes_per_state_element_step": (286.336e6 + 80.986e6) / (8 * 8192 * 1024),
+        {"sources": ("scan.cu",), "sha256": "0f92d71cff018e9f", "shape": ("preln_mlp", "bf16", 1024, 4096),
+         "bytes_per_state_element_step": (286.285e6 + 80.494e6) / (8 * 8192 * 1024),
          "profile": "profiles/scan_depth_lnstat_kernel_c2_small.md"}],
     # scan_ring_kernel on c3 (dram__bytes.sum.per_second x gpu__time_duration of the capture): the scan that writes the
-    # next VJP's split operand 6.166 TB/s x 165.2 us, the plain one 4.769 TB/s x 101.6 us
+    # next VJP's split operand 6.111 TB/s x 167.2 us, the plain one 5.752 TB/s x 83.6 us
     "scan_ring": [
-        {"sources": ("scan_ring.cu", "tc_common.cuh"), "sha256": "636a8f78eb8620ef", "shape": ("rnn_tanh", "f32", 512, 0),
-         "bytes_per_state_element_step": 4.769e12 * 101.6e-6 / (4096 * 32 * 512),
-         "bytes_per_state_element_step_operand": 6.166e12 * 165.2e-6 / (4096 * 32 * 512),
+        {"sources": ("scan_ring.cu", "tc_common.cuh"), "sha256": "895d1a866a4af682", "shape": ("rnn_tanh", "f32", 512, 0),
+         "bytes_per_state_element_step": 5.752e12 * 83.6e-6 / (4096 * 32 * 512),
+         "bytes_per_state_element_step_operand": 6.111e12 * 167.2e-6 / (4096 * 32 * 512),
          "profile": "profiles/scan_ring_kernel_c3.md"}],
 }
 
