@@ -70,7 +70,8 @@ struct PartsGemm {
   const float* gate = nullptr;
   bool relu = false;
 };
-void gemm_parts(Launcher& lc, const PartsGemm& g, int* status_word);
+// false: not launched (the device refuses launches in clusters, or no tensor map could be made); nothing has run then.
+bool gemm_parts(Launcher& lc, const PartsGemm& g, int* status_word);
 // src [rows][cols] (cols contiguous and a multiple of 4, any alignment) -> dst rows of the first batch entry on
 void split_parts(Launcher& lc, const float* src, const Planes& dst, int64_t rows, int cols);
 

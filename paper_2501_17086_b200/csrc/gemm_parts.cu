@@ -461,10 +461,7 @@ void split_parts(Launcher& lc, const float* src, const Planes& dst, int64_t rows
   launch_chained(lc, (uintptr_t)src & 15u ? split_parts_kernel<false> : split_parts_kernel<true>, dim3(grid), 256, 0, 1, src, dst, n, cols / 4);
 }
 
-void gemm_parts(Launcher& lc, const PartsGemm& g, int* status_word) {
-  auto fail = [&]() {
-    if (lc.err == cudaSuccess) lc.err = cudaErrorInvalidValue;
-  };
+bool gemm_parts(Launcher& lc, const PartsGemm& g, int* status_word) {
   Params p;
   p.g = g;
   p.status = status_word;
@@ -503,18 +500,20 @@ void gemm_parts(Launcher& lc, const PartsGemm& g, int* status_word) {
   else if (!p.direct) ok = ok && map_floats(&tmD, g.D, g.M, g.N, g.batch, g.ldd, g.d_sb);
   if (g.D2) ok = ok && map_floats(&tmD2, g.D2, g.M, g.N, g.batch, g.ldd2, g.d2_sb);
   if (g.E) ok = ok && map_floats(&tmE, g.E, g.M, g.N, g.batch, g.lde, g.e_sb);
-  if (!ok) return fail();
+  if (!ok) return false;
   static PerDevice<bool> attr_done;
   if (!attr_done.here()) {
     if (cudaFuncSetAttribute(gemm_parts_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) != cudaSuccess) {
       cudaGetLastError();
-      return fail();
+      return false;
     }
     attr_done.here() = true;
   }
-  launch_chained(lc, gemm_parts_kernel, dim3(2 * (p.num_tiles < pairs ? p.num_tiles : pairs)), THREADS, SMEM_BYTES, 2, tmA, tmB, tmD, tmD2,
-                 tmE, tmP, p);
+  if (try_launch_chained(lc, gemm_parts_kernel, dim3(2 * (p.num_tiles < pairs ? p.num_tiles : pairs)), THREADS, SMEM_BYTES, 2, tmA, tmB, tmD,
+                         tmD2, tmE, tmP, p) != cudaSuccess)
+    return false;
   lc.ran(HBP_FORM_GEMM_F32);
+  return true;
 }
 
 }  // namespace hbp

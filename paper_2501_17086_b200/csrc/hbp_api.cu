@@ -62,8 +62,8 @@ struct hbp_ctx {
   char* H1 = nullptr;      // [group][N][h] dZ
   // Float residual MLP stacks: the operands of every product as three bf16 planes (gemm_parts.cu).  OPp = what W1 is applied to
   // [L][N][d], ACTp, DZp in the memory of ACT and H1, Gp = what the blocks are differentiated against [group][N][d]
-  bool parts = false;      // fixed by the configuration; use_parts: and by the context's modes
-  bool use_parts = false;
+  bool parts = false;      // fixed by the configuration; use_parts: and by the context's modes (no CUDA cores, CTA pairs), and given
+  bool use_parts = false;  // up by a forward pass whose first such product the device refuses
   Planes OPp, ACTp, Gp, DZp, W1p, W2p;
   float2* lnpart = nullptr;  // [steps][N][slots] partial row sums of dY and dY * xhat from the GEMM epilogue
   float4* lnstat = nullptr;  // [steps][N] {rstd, mean dY, mean dY * xhat, 0}
@@ -359,6 +359,9 @@ struct Run {
     a.A = A; a.a_mn = a_mn; a.B = B; a.b_mn = b_mn;
     return a;
   }
+  void product(const PartsGemm& a) {  // (the forward pass has found that these can be launched)
+    if (!gemm_parts(lc, a, c->status) && lc.err == cudaSuccess) lc.err = cudaErrorLaunchFailure;
+  }
   void mlp_vjp_parts(int b0, int b1, bool want_dy, int slot) {
     const int nb = b1 - b0;
     split_weights();
@@ -367,21 +370,21 @@ struct Run {
     a.epi = EPI_MUL;
     a.E = (const float*)c->DACT + (int64_t)b0 * N * h; a.lde = h; a.e_sb = N * h;
     a.Dp = c->DZp.at(slot);
-    gemm_parts(lc, a, c->status);
+    product(a);
     if (!want_dy) return;
     PartsGemm b = parts_args(N, d, h, nb, c->DZp.at(slot), false, c->W1p.at(b0), true);
     b.D = (float*)c->U + (int64_t)b0 * state; b.ldd = d; b.d_sb = state;
-    gemm_parts(lc, b, c->status);
+    product(b);
   }
   void mlp_wgrad_parts(int b0, int b1, const hbp_grads* gr) {
     const int nb = b1 - b0;
     PartsGemm a = parts_args(d, h, N, nb, c->Gp, true, c->ACTp.at(b0), true);
     a.D = gr->dW2 + (int64_t)b0 * d * h; a.ldd = h; a.d_sb = d * h;
-    gemm_parts(lc, a, c->status);
+    product(a);
     if (!c->preln) split_parts(lc, (const float*)x_all + (int64_t)b0 * state, c->OPp.at(b0), (int64_t)nb * N, (int)d);
     PartsGemm b = parts_args(h, d, N, nb, c->DZp, true, c->OPp.at(b0), true);
     b.D = gr->dW1 + (int64_t)b0 * h * d; b.ldd = d; b.d_sb = h * d;
-    gemm_parts(lc, b, c->status);
+    product(b);
   }
 
   // What the MLP block of layer b0 is differentiated against: g_{l+1}, or mask_l * g_{l+1} for ReLU(x + Block(x))
@@ -888,9 +891,9 @@ hbp_status hbp_create(const hbp_config* cfg, void* workspace, size_t workspace_b
   c->ws_bytes = workspace_bytes;
   const char* env = std::getenv("HBP_FORCE_SIMT");
   c->force_simt = env && env[0] == '1';
-  c->use_parts = c->parts && !c->force_simt;
   const char* pm = std::getenv("HBP_GEMM_PAIR");
   c->gemm_pair = !(pm && pm[0] == '0');  // pairs by default
+  c->use_parts = c->parts && !c->force_simt && c->gemm_pair;
   const char* so = std::getenv("HBP_SCAN_OPERAND");
   c->scan_operand = !(so && so[0] == '0');  // the scan writes the next VJP's operand by default (float tanh RNN)
   const char* lg = std::getenv("HBP_LAYER_GROUP");
@@ -1132,14 +1135,14 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
       a.epi = EPI_GELU_FWD;
       a.Dp = ctx->ACTp.at(b);
       a.D2 = (float*)ctx->DACT + (int64_t)b * N * h; a.ldd2 = h;
-      gemm_parts(r.lc, a, ctx->status);
+      if (!gemm_parts(r.lc, a, ctx->status)) return false;
       PartsGemm o = r.parts_args(N, d, h, 1, ctx->ACTp.at(b), false, ctx->W2p.at(b), false);
       o.epi = EPI_RESID;
       o.E = (const float*)xa + (int64_t)b * state; o.lde = d;
       o.gate = (const float*)r.gate_ptr(b);
       o.D = (float*)xa + (int64_t)(b + 1) * state; o.ldd = d;
       if (ctx->MASK) { o.relu = true; o.D2 = (float*)ctx->MASK + (int64_t)b * state; o.ldd2 = d; }
-      gemm_parts(r.lc, o, ctx->status);
+      return gemm_parts(r.lc, o, ctx->status);
     };
     if (ctx->use_parts) r.split_weights();
     for (int b = 0; b < f.L; ++b) {
@@ -1168,7 +1171,11 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
       const int step = r.mlp_step(b);
       if (ctx->preln) ln_of(step);
       if (ctx->use_parts) {
-        mlp_parts(b);
+        if (!mlp_parts(b)) {  // the device refuses these launches: this context's products split their operands themselves
+          ctx->use_parts = false;
+          b = -1;  // (and its caches are filled from the first layer on; x_0 is as it was)
+          continue;
+        }
       } else {
         GemmArgs a = r.base_args();
         a.M = (int)N; a.N = (int)h; a.K = (int)d;

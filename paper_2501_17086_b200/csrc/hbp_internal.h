@@ -105,7 +105,7 @@ struct Launcher {
 // 742 us; float stack of 12 layers 520 wide 2746 -> 2668.  Not for the CUDA-core kernels: launched like this 34 of them of 4 to 8 us
 // each (8 layers 64 wide, 32 rows) are bound by the launching thread, 246 -> 315 us.
 template <typename... P, typename... A>
-void launch_chained(Launcher& lc, void (*kernel)(P...), dim3 grid, int threads, size_t smem, int cluster, A&&... args) {
+cudaError_t try_launch_chained(Launcher& lc, void (*kernel)(P...), dim3 grid, int threads, size_t smem, int cluster, A&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(threads);
@@ -121,8 +121,14 @@ void launch_chained(Launcher& lc, void (*kernel)(P...), dim3 grid, int threads, 
   cfg.attrs = attr;
   cfg.numAttrs = cluster > 1 ? 2 : 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+  if (e == cudaSuccess) lc.count();
+  else cudaGetLastError();
+  return e;
+}
+template <typename... P, typename... A>
+void launch_chained(Launcher& lc, void (*kernel)(P...), dim3 grid, int threads, size_t smem, int cluster, A&&... args) {
+  const cudaError_t e = try_launch_chained(lc, kernel, grid, threads, smem, cluster, args...);
   if (e != cudaSuccess && lc.err == cudaSuccess) lc.err = e;
-  lc.count();
   lc.check();
 }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

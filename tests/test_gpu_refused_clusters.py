@@ -1,5 +1,5 @@
-"""The one-launch recurrences where the device refuses their cluster launches: a stand-in for the runtime's launch call,
-loaded ahead of it in a process of its own, answers "out of resources" to every launch in clusters."""
+"""The one-launch recurrences and the float MLP stacks where the device refuses their cluster launches: a stand-in for the
+runtime's launch call, loaded ahead of it in a process of its own, answers "out of resources" to every launch in clusters."""
 import os
 import subprocess
 import sys
@@ -65,13 +65,57 @@ print("REFUSED", refused.value)
 """
 
 
-def test_refused_cluster_launches_fall_back_to_one_launch_per_step(tmp_path):
+STACKS = r"""
+import ctypes, os
+import torch
+from paper_2501_17086_b200 import harness
+from paper_2501_17086_b200.workloads import Workload, make_inputs
+
+refused = ctypes.c_int.in_dll(ctypes.CDLL(os.environ["LD_PRELOAD"]), "refused_launches")
+for block in ("mlp", "preln_mlp", "relu_mlp", "postln_mlp"):
+    w = Workload("t", block, "f32", L=3, d=132, hidden=260, tokens=300, batch=1, seq=1, seed=9050, init="small" if block == "postln_mlp" else "")
+    inp = make_inputs(w, "cuda")
+    params = harness.params_for(w, inp)
+    outs = []
+    for single in (False, True):
+        if single:
+            os.environ["HBP_GEMM_PAIR"] = "0"
+        ctx = harness.make_context(w)
+        os.environ.pop("HBP_GEMM_PAIR", None)
+        before = refused.value
+        x = ctx.forward(params, inp["x0"])
+        delta = harness.loss_delta(w, x, inp)
+        got = [x]
+        for exact in (False, True):
+            grads = ctx.new_grads()
+            got.append(ctx.exact(params, delta, x, grads=grads) if exact else ctx.backward(params, 2, delta, x, grads=grads))
+            got += [grads[n] for n in sorted(grads)]
+        ctx.forward(params, inp["x0"], x_all=x)
+        ctx.sync_status()
+        # paired CTAs: the first product is refused, and none is asked for again; single CTAs by request: none is asked for
+        assert refused.value - before == (0 if single else 1), (block, single, refused.value - before)
+        outs.append(got)
+    assert all(torch.equal(a, b) for a, b in zip(*outs)), block
+print("REFUSED", refused.value)
+"""
+
+
+def _run_refused(tmp_path, child):
     src, lib = tmp_path / "refuse.c", tmp_path / "librefuse.so"
     src.write_text(REFUSE)
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     subprocess.check_call(["gcc", "-shared", "-fPIC", "-I" + os.path.join(cuda, "include"), str(src), "-o", str(lib), "-ldl"])
     env = dict(os.environ, LD_PRELOAD=str(lib), PYTHONPATH=ROOT)
-    env.pop("HBP_FORCE_SIMT", None)
-    out = subprocess.run([sys.executable, "-c", CHILD], env=env, cwd=ROOT, capture_output=True, text=True, timeout=300)
+    for name in ("HBP_FORCE_SIMT", "HBP_GEMM_PAIR"):
+        env.pop(name, None)
+    out = subprocess.run([sys.executable, "-c", child], env=env, cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert out.returncode == 0, out.stdout[-2000:] + out.stderr[-4000:]
     assert "REFUSED" in out.stdout
+
+
+def test_refused_cluster_launches_fall_back_to_one_launch_per_step(tmp_path):
+    _run_refused(tmp_path, CHILD)
+
+
+def test_float_stacks_need_no_clusters(tmp_path):
+    _run_refused(tmp_path, STACKS)
