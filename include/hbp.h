@@ -136,12 +136,17 @@ typedef struct {
 } hbp_grads;
 
 /* Bytes of caller-provided device workspace a context for `cfg` needs (activation caches of the
- * last forward, per-iteration scratch, a status word).  HBP_ERR_SHAPE / _DTYPE / _UNSUPPORTED on a
- * bad config. */
+ * last forward, per-iteration scratch, a status word), under the kernel-selection modes of the moment (see
+ * hbp_context_modes).  HBP_ERR_SHAPE / _DTYPE / _UNSUPPORTED on a bad config.
+ * Float MLP stacks of more than 32 rows, 64 wide or more, keep the operands of their products split for the tensor cores, in
+ * a workspace of at most three times the size without (or 64 MiB more) and at most 90 GiB.  They take less too, down to the
+ * size without, which is the one under HBP_GEMM_PAIR=0: the weights of fewer layers are then held split at a time, or the
+ * products split their operands themselves (the results are the same). */
 hbp_status hbp_workspace_bytes(const hbp_config* cfg, size_t* bytes);
 
 /* Makes a context over `workspace` (device, 256-byte aligned, >= hbp_workspace_bytes).  The
- * workspace is borrowed until hbp_destroy.  *out is host memory owned by the library. */
+ * workspace is borrowed until hbp_destroy.  *out is host memory owned by the library.  HBP_ERR_WORKSPACE if the workspace
+ * is smaller than any form of the products needs (float MLP stacks: see hbp_workspace_bytes) or misaligned. */
 hbp_status hbp_create(const hbp_config* cfg, void* workspace, size_t workspace_bytes, hbp_ctx** out);
 
 /* Section 3, h_i = f_i(h_{i-1}): runs the steps from x0 [N][d] and stores every state in

@@ -32,7 +32,7 @@ __device__ __forceinline__ void split_parts2(float a, float b, uint32_t& h, uint
 }
 
 // A matrix [batch][rows][cols] held as three such planes, columns contiguous: part q of element (b, r, c) at
-// p[q * plane + b * sb + r * ld + c].  ld is a multiple of 64 (128 bytes), what lies beyond cols is never read.
+// p[q * plane + b * sb + r * ld + c].  ld is a multiple of 16 (32 bytes), what lies beyond cols is never read.
 struct Planes {
   bf16* p = nullptr;
   int64_t ld = 0, sb = 0, plane = 0;
@@ -72,6 +72,8 @@ struct PartsGemm {
 };
 // false: not launched (the device refuses launches in clusters, or no tensor map could be made); nothing has run then.
 bool gemm_parts(Launcher& lc, const PartsGemm& g, int* status_word);
+// Whether `batch` products with M x N outputs have tiles for half of the CTA pairs.
+bool parts_fill(int M, int N, int batch);
 // src [rows][cols] (cols contiguous and a multiple of 4, any alignment) -> dst rows of the first batch entry on
 void split_parts(Launcher& lc, const float* src, const Planes& dst, int64_t rows, int cols);
 

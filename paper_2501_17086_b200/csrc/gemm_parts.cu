@@ -461,6 +461,10 @@ void split_parts(Launcher& lc, const float* src, const Planes& dst, int64_t rows
   launch_chained(lc, (uintptr_t)src & 15u ? split_parts_kernel<false> : split_parts_kernel<true>, dim3(grid), 256, 0, 1, src, dst, n, cols / 4);
 }
 
+bool parts_fill(int M, int N, int batch) {
+  return (int64_t)((M + TILE_M - 1) / TILE_M) * ((N + kMaxTileN - 1) / kMaxTileN) * batch >= sm_count() / 4;
+}
+
 bool gemm_parts(Launcher& lc, const PartsGemm& g, int* status_word) {
   Params p;
   p.g = g;
@@ -512,7 +516,6 @@ bool gemm_parts(Launcher& lc, const PartsGemm& g, int* status_word) {
   if (try_launch_chained(lc, gemm_parts_kernel, dim3(2 * (p.num_tiles < pairs ? p.num_tiles : pairs)), THREADS, SMEM_BYTES, 2, tmA, tmB, tmD,
                          tmD2, tmE, tmP, p) != cudaSuccess)
     return false;
-  lc.ran(HBP_FORM_GEMM_F32);
   return true;
 }
 

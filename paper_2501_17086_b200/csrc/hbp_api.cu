@@ -1,6 +1,7 @@
 // C ABI of libhbp: configuration checks, workspace carve-up and the kernel sequences of
 // hbp_forward / hbp_backward / hbp_exact.  No device memory is allocated here; every buffer is either
 // the caller's or a slice of the caller's workspace.
+#include <cstdint>
 #include <cstdlib>
 #include <cstring>
 #include <new>
@@ -61,9 +62,10 @@ struct hbp_ctx {
   char* U = nullptr;       // [steps][N][d] block VJP outputs (dY before the LayerNorm finish)
   char* H1 = nullptr;      // [group][N][h] dZ
   // Float residual MLP stacks: the operands of every product as three bf16 planes (gemm_parts.cu).  OPp = what W1 is applied to
-  // [L][N][d], ACTp, DZp in the memory of ACT and H1, Gp = what the blocks are differentiated against [group][N][d]
-  bool parts = false;      // fixed by the configuration; use_parts: and by the context's modes (no CUDA cores, CTA pairs), and given
-  bool use_parts = false;  // up by a forward pass whose first such product the device refuses
+  // [L][N][d], ACTp, DZp in the memory of ACT and H1, Gp = what the blocks are differentiated against [group][N][d], W1p, W2p = the
+  // weights of weight_layers layers at a time (0: no planes)
+  int weight_layers = 0;
+  bool use_parts = false;  // weight_layers > 0, until a forward pass whose first such product the device refuses
   Planes OPp, ACTp, Gp, DZp, W1p, W2p;
   float2* lnpart = nullptr;  // [steps][N][slots] partial row sums of dY and dY * xhat from the GEMM epilogue
   float4* lnstat = nullptr;  // [steps][N] {rstd, mean dY, mean dY * xhat, 0}
@@ -146,8 +148,9 @@ bool keeps_parts(const hbp_config& f) {
          f.tokens > 32 && f.d >= 64 && f.hidden >= 64;
 }
 
-// Lays the workspace out; with base == nullptr only the total size is computed.
-size_t carve(hbp_ctx* c, char* base) {
+// Lays the workspace out, with planes for the weights of weight_layers layers (0: none at all); with base == nullptr only the
+// total size is computed.
+size_t carve(hbp_ctx* c, char* base, int weight_layers) {
   const hbp_config& f = c->cfg;
   size_t off = 0;
   auto take = [&](size_t bytes) -> char* {
@@ -161,6 +164,8 @@ size_t carve(hbp_ctx* c, char* base) {
   c->preln = f.block == HBP_BLOCK_PRELN_MLP || f.block == HBP_BLOCK_PRELN_TRANSFORMER;
   c->steps = f.block == HBP_BLOCK_PRELN_TRANSFORMER ? 2 * f.L : f.L;
   c->layers = f.L;
+  c->weight_layers = weight_layers;
+  const bool parts = weight_layers > 0;
   const size_t steps = (size_t)c->steps;
   c->status = (int*)take(256);
   c->U = take(steps * N * d * es);
@@ -242,29 +247,28 @@ size_t carve(hbp_ctx* c, char* base) {
       c->rstd = (float*)take(steps * N * 4);
     }
     auto take_planes = [&](Planes& P, size_t entries, size_t rows, size_t cols) {
-      P.ld = (int64_t)((cols + 63) / 64 * 64); P.sb = (int64_t)rows * P.ld; P.plane = (int64_t)entries * P.sb;
+      P.ld = (int64_t)((cols + 15) / 16 * 16); P.sb = (int64_t)rows * P.ld; P.plane = (int64_t)entries * P.sb;
       P.p = (bf16*)take(3 * (size_t)P.plane * 2);
     };
-    c->parts = keeps_parts(f);
     const size_t layers = (size_t)c->layers;
-    if (c->parts) {
+    if (parts) {
       take_planes(c->OPp, layers, N, d);
-      take_planes(c->W1p, layers, h, d);
-      take_planes(c->W2p, layers, d, h);
+      take_planes(c->W1p, weight_layers, h, d);
+      take_planes(c->W2p, weight_layers, d, h);
       take_planes(c->ACTp, layers, N, h);
     }
-    c->ACT = c->parts ? (char*)c->ACTp.p : take(layers * N * h * es);
+    c->ACT = parts ? (char*)c->ACTp.p : take(layers * N * h * es);
     c->DACT = take(layers * N * h * es);
     const size_t per_layer = N * h * es;
     size_t grp = ((size_t)6 << 30) / per_layer;
     if (grp < 1) grp = 1;
     if (grp > (size_t)c->layers) grp = (size_t)c->layers;
     c->group = (int)grp;
-    if (c->parts) {
+    if (parts) {
       take_planes(c->Gp, grp, N, d);
       take_planes(c->DZp, grp, N, h);
     }
-    c->H1 = c->parts ? (char*)c->DZp.p : take(grp * per_layer);
+    c->H1 = parts ? (char*)c->DZp.p : take(grp * per_layer);
   }
   if (f.block == HBP_BLOCK_PRELN_TRANSFORMER) {
     const size_t Lb = (size_t)f.L;
@@ -282,6 +286,45 @@ size_t carve(hbp_ctx* c, char* base) {
   }
   c->partial = (float*)take(c->partial_floats * 4);
   return off;
+}
+
+// The kernel-selection modes, from the environment.
+void read_modes(hbp_ctx* c) {
+  const char* env = std::getenv("HBP_FORCE_SIMT");
+  c->force_simt = env && env[0] == '1';
+  const char* pm = std::getenv("HBP_GEMM_PAIR");
+  c->gemm_pair = !(pm && pm[0] == '0');  // pairs by default
+  const char* so = std::getenv("HBP_SCAN_OPERAND");
+  c->scan_operand = !(so && so[0] == '0');  // the scan writes the next VJP's operand by default (float tanh RNN)
+}
+
+// The layers whose weights are held in parts at once, in a workspace of at most `limit` bytes; 0: no operand in parts.  The planes
+// of the weights are scratch that the other kernels do without, and they do not shrink with the rows (16 layers 1024 (4096),
+// 33 rows: 29 MB without, 850 with those of all layers), so with planes the workspace is at most three times what it is without,
+// or 64 MiB larger, and no more than half of the device's memory, so that a stack that fills it still fits.  (From some 2000
+// rows on all planes of such a stack take 0.5 to 0.9 of what the rest does.)  Weights of the layers that do not fit are split
+// again where they are needed, in runs of one length.  Forward, backward(4) with gradients and exact pass of 16 layers 1024 (4096)
+// in us, split inside / runs / all planes: 400 rows 3010, 7900, 5100 / 1400, 4560, 2180 / 1380, 3890, 2560; 128 rows
+// 3070, 2550, 4400 / 1280, 2190, 1620 / 1290, 1830, 1720.
+int weight_layers_in(hbp_ctx* c, size_t limit) {
+  if (!keeps_parts(c->cfg) || c->force_simt || !c->gemm_pair) return 0;
+  const size_t without = carve(c, nullptr, 0), small = (size_t)64 << 20, half = (size_t)90 << 30;
+  size_t most = without + (2 * without > small ? 2 * without : small);
+  if (most > half) most = half;
+  if (limit > most) limit = most;
+  int fits = 0;
+  for (int lo = 1, hi = c->cfg.L; lo <= hi;) {
+    const int mid = lo + (hi - lo) / 2;
+    if (carve(c, nullptr, mid) <= limit) {
+      fits = mid;
+      lo = mid + 1;
+    } else {
+      hi = mid - 1;
+    }
+  }
+  if (fits == 0) return 0;
+  const int runs = (c->cfg.L + fits - 1) / fits;
+  return (c->cfg.L + runs - 1) / runs;
 }
 
 struct Run {
@@ -346,45 +389,54 @@ struct Run {
   }
 
   // ---- operands in parts (use_parts) ---------------------------------------------------------------
-  bool weights_in_parts = false;  // once per call: the caller's weights may be others in the next
-  void split_weights() {
-    if (weights_in_parts) return;
-    weights_in_parts = true;
-    split_parts(lc, (const float*)p->W1, c->W1p, c->layers * h, (int)d);
-    split_parts(lc, (const float*)p->W2, c->W2p, c->layers * d, (int)h);
+  // The layers whose weights the planes hold, split by this call (the caller's may be others in the next).
+  struct Held { int lo = 0, hi = 0; } held1, held2;
+  Planes weights(Held& held, const Planes& P, const void* W, int64_t rows, int64_t cols, int b) {
+    if (b < held.lo || b >= held.hi) {
+      held.lo = b - b % c->weight_layers;
+      held.hi = held.lo + c->weight_layers < c->layers ? held.lo + c->weight_layers : c->layers;
+      split_parts(lc, (const float*)W + held.lo * rows * cols, P, (held.hi - held.lo) * rows, (int)cols);
+    }
+    return P.at(b - held.lo);
   }
+  Planes weights1(int b) { return weights(held1, c->W1p, p->W1, h, d, b); }
+  Planes weights2(int b) { return weights(held2, c->W2p, p->W2, d, h, b); }
   PartsGemm parts_args(int64_t m, int64_t n, int64_t k, int batch, const Planes& A, bool a_mn, const Planes& B, bool b_mn) const {
     PartsGemm a;
     a.M = (int)m; a.N = (int)n; a.K = (int)k; a.batch = batch;
     a.A = A; a.a_mn = a_mn; a.B = B; a.b_mn = b_mn;
     return a;
   }
-  void product(const PartsGemm& a) {  // (the forward pass has found that these can be launched)
+  void launch_product(const PartsGemm& a) {  // (the forward pass has found that these can be launched)
     if (!gemm_parts(lc, a, c->status) && lc.err == cudaSuccess) lc.err = cudaErrorLaunchFailure;
   }
   void mlp_vjp_parts(int b0, int b1, bool want_dy, int slot) {
-    const int nb = b1 - b0;
-    split_weights();
-    split_parts(lc, (const float*)upstream(b0), c->Gp.at(slot), (int64_t)nb * N, (int)d);
-    PartsGemm a = parts_args(N, h, d, nb, c->Gp.at(slot), false, c->W2p.at(b0), true);
-    a.epi = EPI_MUL;
-    a.E = (const float*)c->DACT + (int64_t)b0 * N * h; a.lde = h; a.e_sb = N * h;
-    a.Dp = c->DZp.at(slot);
-    product(a);
-    if (!want_dy) return;
-    PartsGemm b = parts_args(N, d, h, nb, c->DZp.at(slot), false, c->W1p.at(b0), true);
-    b.D = (float*)c->U + (int64_t)b0 * state; b.ldd = d; b.d_sb = state;
-    product(b);
+    split_parts(lc, (const float*)upstream(b0), c->Gp.at(slot), (int64_t)(b1 - b0) * N, (int)d);
+    for (int l = b0, end; l < b1; l = end) {  // runs of layers whose weights are held together
+      const Planes W2 = weights2(l), G = c->Gp.at(slot + l - b0), DZ = c->DZp.at(slot + l - b0);
+      end = held2.hi < b1 ? held2.hi : b1;
+      PartsGemm a = parts_args(N, h, d, end - l, G, false, W2, true);
+      a.epi = EPI_MUL;
+      a.E = (const float*)c->DACT + (int64_t)l * N * h; a.lde = h; a.e_sb = N * h;
+      a.Dp = DZ;
+      launch_product(a);
+      if (!want_dy) continue;
+      PartsGemm b = parts_args(N, d, h, end - l, DZ, false, weights1(l), true);
+      b.D = (float*)c->U + (int64_t)l * state; b.ldd = d; b.d_sb = state;
+      launch_product(b);
+    }
+    for (int i = 0; i < 1 + want_dy; ++i) lc.ran(HBP_FORM_GEMM_F32);  // products, not launches
   }
   void mlp_wgrad_parts(int b0, int b1, const hbp_grads* gr) {
     const int nb = b1 - b0;
     PartsGemm a = parts_args(d, h, N, nb, c->Gp, true, c->ACTp.at(b0), true);
     a.D = gr->dW2 + (int64_t)b0 * d * h; a.ldd = h; a.d_sb = d * h;
-    product(a);
+    launch_product(a);
     if (!c->preln) split_parts(lc, (const float*)x_all + (int64_t)b0 * state, c->OPp.at(b0), (int64_t)nb * N, (int)d);
     PartsGemm b = parts_args(h, d, N, nb, c->DZp, true, c->OPp.at(b0), true);
     b.D = gr->dW1 + (int64_t)b0 * h * d; b.ldd = d; b.d_sb = h * d;
-    product(b);
+    launch_product(b);
+    for (int i = 0; i < 2; ++i) lc.ran(HBP_FORM_GEMM_F32);
   }
 
   // What the MLP block of layer b0 is differentiated against: g_{l+1}, or mask_l * g_{l+1} for ReLU(x + Block(x))
@@ -408,7 +460,12 @@ struct Run {
   // ---- MLP block: u = J^T g for layers [b0, b1) (b1 - b0 <= group), from states g[step+1] -------
   // dA = G W2, dZ = dA * gelu'(Z) -> H1 from layer `slot` on (cached derivative);  dY = dZ W1 -> U[step].
   void mlp_vjp(int b0, int b1, bool want_dy, int slot = 0) {
-    if (c->use_parts) return mlp_vjp_parts(b0, b1, want_dy, slot);
+    // One launch over all layers with the operands split inside, rather than a launch and a split pass for each run of layers
+    // whose weights fit the planes, where such a run is too small for the chip (the parameter pass reads dZ as planes).  backward(1)
+    // of 16 layers 1024 (4096), inside / in runs of n tiles: 128 rows, n = 6, 428 / 1269 us; 250, 12, 764 / 1304; 500, 60, 1468 / 912;
+    // 8 layers 512 (1024) x 300, 24, 123 / 155
+    const bool runs = c->weight_layers >= b1 - b0 || parts_fill((int)N, (int)d, c->weight_layers);
+    if (c->use_parts && (runs || !want_dy)) return mlp_vjp_parts(b0, b1, want_dy, slot);
     const int nb = b1 - b0, ss = step_stride();
     GemmArgs a = base_args();
     a.M = (int)N; a.N = (int)h; a.K = (int)d; a.batch = nb;
@@ -869,7 +926,8 @@ hbp_status hbp_workspace_bytes(const hbp_config* cfg, size_t* bytes) {
   if (st != HBP_OK) return st;
   hbp_ctx tmp;
   tmp.cfg = *cfg;
-  *bytes = carve(&tmp, nullptr);
+  read_modes(&tmp);
+  *bytes = carve(&tmp, nullptr, weight_layers_in(&tmp, SIZE_MAX));
   return HBP_OK;
 }
 
@@ -882,20 +940,15 @@ hbp_status hbp_create(const hbp_config* cfg, void* workspace, size_t workspace_b
   hbp_ctx* c = new (std::nothrow) hbp_ctx;
   if (!c) return HBP_ERR_INVALID_ARG;
   c->cfg = *cfg;
-  const size_t need = carve(c, (char*)workspace);
+  read_modes(c);
+  const size_t need = carve(c, (char*)workspace, weight_layers_in(c, workspace_bytes));
   if (workspace_bytes < need) {
     delete c;
     return HBP_ERR_WORKSPACE;
   }
   c->ws = (char*)workspace;
   c->ws_bytes = workspace_bytes;
-  const char* env = std::getenv("HBP_FORCE_SIMT");
-  c->force_simt = env && env[0] == '1';
-  const char* pm = std::getenv("HBP_GEMM_PAIR");
-  c->gemm_pair = !(pm && pm[0] == '0');  // pairs by default
-  c->use_parts = c->parts && !c->force_simt && c->gemm_pair;
-  const char* so = std::getenv("HBP_SCAN_OPERAND");
-  c->scan_operand = !(so && so[0] == '0');  // the scan writes the next VJP's operand by default (float tanh RNN)
+  c->use_parts = c->weight_layers > 0;
   const char* lg = std::getenv("HBP_LAYER_GROUP");
   const int cap = lg ? std::atoi(lg) : 0;
   if (cap > 0 && cap < c->group) c->group = cap;  // (the scratch is carved for the larger group)
@@ -1131,20 +1184,22 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
     };
     auto mlp_parts = [&](int b) {
       if (!ctx->preln) split_parts(r.lc, (const float*)xa + (int64_t)b * state, ctx->OPp.at(b), N, (int)d);
-      PartsGemm a = r.parts_args(N, h, d, 1, ctx->OPp.at(b), false, ctx->W1p.at(b), false);
+      PartsGemm a = r.parts_args(N, h, d, 1, ctx->OPp.at(b), false, r.weights1(b), false);
       a.epi = EPI_GELU_FWD;
       a.Dp = ctx->ACTp.at(b);
       a.D2 = (float*)ctx->DACT + (int64_t)b * N * h; a.ldd2 = h;
       if (!gemm_parts(r.lc, a, ctx->status)) return false;
-      PartsGemm o = r.parts_args(N, d, h, 1, ctx->ACTp.at(b), false, ctx->W2p.at(b), false);
+      r.lc.ran(HBP_FORM_GEMM_F32);
+      PartsGemm o = r.parts_args(N, d, h, 1, ctx->ACTp.at(b), false, r.weights2(b), false);
       o.epi = EPI_RESID;
       o.E = (const float*)xa + (int64_t)b * state; o.lde = d;
       o.gate = (const float*)r.gate_ptr(b);
       o.D = (float*)xa + (int64_t)(b + 1) * state; o.ldd = d;
       if (ctx->MASK) { o.relu = true; o.D2 = (float*)ctx->MASK + (int64_t)b * state; o.ldd2 = d; }
-      return gemm_parts(r.lc, o, ctx->status);
+      if (!gemm_parts(r.lc, o, ctx->status)) return false;
+      r.lc.ran(HBP_FORM_GEMM_F32);
+      return true;
     };
-    if (ctx->use_parts) r.split_weights();
     for (int b = 0; b < f.L; ++b) {
       if (tr) {
         const int step = 2 * b;
