@@ -246,8 +246,9 @@ size_t carve(hbp_ctx* c, char* base, int weight_layers) {
       c->CB = take(steps * N * d * es);
       c->rstd = (float*)take(steps * N * 4);
     }
+    auto plane_cols = [](size_t cols) { return (cols + 15) / 16 * 16; };
     auto take_planes = [&](Planes& P, size_t entries, size_t rows, size_t cols) {
-      P.ld = (int64_t)((cols + 15) / 16 * 16); P.sb = (int64_t)rows * P.ld; P.plane = (int64_t)entries * P.sb;
+      P.ld = (int64_t)plane_cols(cols); P.sb = (int64_t)rows * P.ld; P.plane = (int64_t)entries * P.sb;
       P.p = (bf16*)take(3 * (size_t)P.plane * 2);
     };
     const size_t layers = (size_t)c->layers;
@@ -259,7 +260,7 @@ size_t carve(hbp_ctx* c, char* base, int weight_layers) {
     }
     c->ACT = parts ? (char*)c->ACTp.p : take(layers * N * h * es);
     c->DACT = take(layers * N * h * es);
-    const size_t per_layer = N * h * es;
+    const size_t per_layer = parts ? 3 * 2 * N * (plane_cols(d) + plane_cols(h)) : N * h * es;  // Gp and DZp, or H1
     size_t grp = ((size_t)6 << 30) / per_layer;
     if (grp < 1) grp = 1;
     if (grp > (size_t)c->layers) grp = (size_t)c->layers;

@@ -39,6 +39,14 @@ def test_split_operands_are_bounded(monkeypatch, block, L, d, h, tokens):
         assert most > without
 
 
+@pytest.mark.parametrize("d,h,tokens", [(1024, 4096, 8192), (1024, 1024, 32768), (2048, 8192, 4096)])
+def test_scratch_of_a_layer_group_stays_within_6_gib(monkeypatch, d, h, tokens):
+    for forms in range(2):  # with planes, without
+        a, b = (_sizes(monkeypatch, "preln_mlp", L, d, h, tokens)[forms] for L in (64, 65))
+        scratch = a - 64 * (b - a)  # what does not grow with the layers: the group, and partial sums of d channels
+        assert 4 << 30 < scratch <= (6 << 30) + 256 * d * 4 + (1 << 16)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("group", ["", "2"])
 @pytest.mark.parametrize("block", BLOCKS)
