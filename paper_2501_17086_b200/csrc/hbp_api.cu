@@ -411,6 +411,12 @@ struct Run {
   void launch_product(const PartsGemm& a) {  // (the forward pass has found that these can be launched)
     if (!gemm_parts(lc, a, c->status) && lc.err == cudaSuccess) lc.err = cudaErrorLaunchFailure;
   }
+  void count_products(int n) {  // products, not launches
+    for (int i = 0; i < n; ++i) {
+      lc.ran(HBP_FORM_GEMM_F32);
+      lc.ran(HBP_FORM_GEMM_PARTS);
+    }
+  }
   void mlp_vjp_parts(int b0, int b1, bool want_dy, int slot) {
     split_parts(lc, (const float*)upstream(b0), c->Gp.at(slot), (int64_t)(b1 - b0) * N, (int)d);
     for (int l = b0, end; l < b1; l = end) {  // runs of layers whose weights are held together
@@ -426,7 +432,7 @@ struct Run {
       b.D = (float*)c->U + (int64_t)l * state; b.ldd = d; b.d_sb = state;
       launch_product(b);
     }
-    for (int i = 0; i < 1 + want_dy; ++i) lc.ran(HBP_FORM_GEMM_F32);  // products, not launches
+    count_products(want_dy ? 2 : 1);
   }
   void mlp_wgrad_parts(int b0, int b1, const hbp_grads* gr) {
     const int nb = b1 - b0;
@@ -437,7 +443,7 @@ struct Run {
     PartsGemm b = parts_args(h, d, N, nb, c->DZp, true, c->OPp.at(b0), true);
     b.D = gr->dW1 + (int64_t)b0 * h * d; b.ldd = d; b.d_sb = h * d;
     launch_product(b);
-    for (int i = 0; i < 2; ++i) lc.ran(HBP_FORM_GEMM_F32);
+    count_products(2);
   }
 
   // What the MLP block of layer b0 is differentiated against: g_{l+1}, or mask_l * g_{l+1} for ReLU(x + Block(x))
@@ -1190,7 +1196,7 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
       a.Dp = ctx->ACTp.at(b);
       a.D2 = (float*)ctx->DACT + (int64_t)b * N * h; a.ldd2 = h;
       if (!gemm_parts(r.lc, a, ctx->status)) return false;
-      r.lc.ran(HBP_FORM_GEMM_F32);
+      r.count_products(1);
       PartsGemm o = r.parts_args(N, d, h, 1, ctx->ACTp.at(b), false, r.weights2(b), false);
       o.epi = EPI_RESID;
       o.E = (const float*)xa + (int64_t)b * state; o.lde = d;
@@ -1198,7 +1204,7 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
       o.D = (float*)xa + (int64_t)(b + 1) * state; o.ldd = d;
       if (ctx->MASK) { o.relu = true; o.D2 = (float*)ctx->MASK + (int64_t)b * state; o.ldd2 = d; }
       if (!gemm_parts(r.lc, o, ctx->status)) return false;
-      r.lc.ran(HBP_FORM_GEMM_F32);
+      r.count_products(1);
       return true;
     };
     for (int b = 0; b < f.L; ++b) {

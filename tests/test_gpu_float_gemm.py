@@ -1,6 +1,6 @@
-"""The float tensor-core GEMM (operands split into three bf16 parts inside the kernel) at the edges of its tiles: rows, columns
-and contraction lengths around 32 and 128, every orientation of the operands and every epilogue of the float MLP and decoder
-kinds, against the oracle."""
+"""The float tensor-core GEMMs at the edges of their tiles: rows, columns and contraction lengths around 32 and 128, every
+orientation of the operands and every epilogue of the float MLP and decoder kinds, against the oracle.  Each test runs on the kernel
+that splits its operands into three bf16 parts itself, and on the one that reads them already split where a stack keeps them so."""
 import os
 
 import pytest
@@ -14,9 +14,29 @@ from test_gpu_parity import compare, rel_l2, run_gpu, to_np
 pytestmark = pytest.mark.gpu
 
 
+@pytest.fixture(params=["split_inside", "planes"], autouse=True)
+def operands(request, monkeypatch):
+    """HBP_GEMM_PAIR=0 contexts split inside the kernel.  Every context that a test made has to have taken the products meant."""
+    made, make = [], harness.make_context
+
+    def make_context(w):
+        made.append((w, make(w), os.environ.get("HBP_FORCE_SIMT") == "1"))
+        return made[-1][1]
+
+    monkeypatch.setattr(harness, "make_context", make_context)
+    if request.param == "split_inside":
+        monkeypatch.setenv("HBP_GEMM_PAIR", "0")
+    yield request.param
+    for w, ctx, simt in made:
+        kept = request.param == "planes" and not simt and w.tokens > 32 and w.d >= 64 and w.hidden >= 64
+        assert ctx.forms["gemm_parts"] == (ctx.forms["gemm_f32"] if kept else 0)
+        assert not simt or ctx.forms["gemm_f32"] == 0
+
+
 @pytest.mark.parametrize("block,L,d,h,tokens", [
     ("mlp", 2, 4, 8, 33), ("mlp", 2, 128, 256, 127), ("mlp", 3, 132, 260, 129), ("preln_mlp", 2, 36, 388, 257),
     ("preln_mlp", 2, 260, 124, 1000), ("relu_mlp", 2, 100, 132, 70), ("postln_mlp", 2, 132, 300, 161), ("mlp", 1, 1028, 1032, 40),
+    ("relu_mlp", 2, 388, 36, 257), ("postln_mlp", 2, 60, 520, 130),
 ])
 def test_tile_edges_match_oracle(block, L, d, h, tokens):
     w = Workload("t", block, "f32", L=L, d=d, hidden=h, tokens=tokens, batch=1, seq=1, seed=8000 + d + tokens)

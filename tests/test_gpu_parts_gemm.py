@@ -25,7 +25,9 @@ def _workload(block, L, d, h, tokens, seed):
 def test_tile_edges_match_oracle(block, L, d, h, tokens):
     w = _workload(block, L, d, h, tokens, 9000 + d + tokens)
     inp = make_inputs(w, "cuda")
-    compare(w, run_gpu(w, inp, (1, 2)), orun.run(w, inp, ks=(1, 2), grads_for=("exact", 2)), (1, 2), ("exact", 2))
+    gpu = run_gpu(w, inp, (1, 2))
+    assert gpu["ctx"].forms["gemm_parts"] == gpu["ctx"].forms["gemm_f32"] > 0
+    compare(w, gpu, orun.run(w, inp, ks=(1, 2), grads_for=("exact", 2)), (1, 2), ("exact", 2))
 
 
 def _shifted(t):
