@@ -1167,12 +1167,14 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
     // Residual update x_{l+1} = a * x_l + F through the float master copy when there is one.  Where the next thing done with
     // the state is its LayerNorm, whose kernel reads the master row by row, that kernel writes the state in dtype too (ln_of),
     // and the product only adds itself to the master.  (gates of one; the tensor-core kernel's conditions)
+    bool state_due = false;  // the last product left the state in the float master only
     const bool ln_writes = ctx->xres && (ctx->preln || f.block == HBP_BLOCK_POSTLN_MLP);
     auto resid_gemm = [&](GemmArgs& a, int step) {
       if (ln_writes && !ctx->force_simt && f.gate == HBP_GATE_ONE) {
         a.epi = EPI_ACCUM; a.d_f32 = true;
         a.D = ctx->xres; a.ldd = d;
-        if (gemm_tc(r.lc, a, ctx->status)) return;
+        state_due = gemm_tc(r.lc, a, ctx->status);
+        if (state_due) return;
         a.d_f32 = false;
       }
       a.epi = EPI_RESID;
@@ -1186,8 +1188,8 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
     auto ln_of = [&](int step) {
       const float* src = ctx->xres ? ctx->xres : (const float*)r.at(xa, (int64_t)step * state);
       layernorm_fwd(r.lc, f.dtype, src, r.at(ctx->Y, (int64_t)step * state), ctx->rstd + (int64_t)step * N, N, (int)d, f.ln_eps,
-                    nullptr, ctx->xres && step > 0 ? r.at(xa, (int64_t)step * state) : nullptr,
-                    ctx->use_parts ? ctx->OPp.at(step) : Planes());
+                    nullptr, state_due ? r.at(xa, (int64_t)step * state) : nullptr, ctx->use_parts ? ctx->OPp.at(step) : Planes());
+      state_due = false;
     };
     auto mlp_parts = [&](int b) {
       if (!ctx->preln) split_parts(r.lc, (const float*)xa + (int64_t)b * state, ctx->OPp.at(b), N, (int)d);
@@ -1257,9 +1259,10 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
         const float* src = ctx->xres ? ctx->xres : (const float*)r.at(xa, (int64_t)(step + 1) * state);
         layernorm_fwd(r.lc, f.dtype, src, r.at(xa, (int64_t)(step + 1) * state), ctx->rstd + (int64_t)step * N, N, (int)d,
                       f.ln_eps, ctx->xres, nullptr, Planes());
+        state_due = false;
       }
     }
-    if (ctx->xres && ctx->preln) convert_from_f32(r.lc, ctx->xres, (bf16*)r.at(xa, (int64_t)ctx->steps * state), state);
+    if (state_due) convert_from_f32(r.lc, ctx->xres, (bf16*)r.at(xa, (int64_t)ctx->steps * state), state);
   }
   ctx->forward_done = true;
   return r.result();

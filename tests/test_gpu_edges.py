@@ -423,3 +423,26 @@ def test_backward_replays_from_a_cuda_graph(name, k):
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(g_all, want2)
+
+
+@pytest.mark.parametrize("block", ["preln_mlp", "preln_transformer"])
+def test_a_gated_bf16_stack_stores_each_state_once(block):
+    """Its residual products store the state themselves; only products that add to the float stream (no gate) leave the last state
+    to one more launch."""
+    from paper_2501_17086_b200 import binding as B
+    heads = dict(n_heads=2, head_dim=64, seq=100, batch=3) if block == "preln_transformer" else {}
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(77)
+    shapes = {"W1": (2, 256, 128), "W2": (2, 128, 256), **({n: (2, 128, 128) for n in ("Wq", "Wk", "Wv", "Wo")} if heads else {})}
+    params = {n: (0.1 * torch.randn(s, generator=gen, device="cuda")).bfloat16() for n, s in shapes.items()}
+    x0 = torch.randn((300, 128), generator=gen, device="cuda").bfloat16()
+    launches, last = [], []
+    for gate in (B.GATE_ONE, B.GATE_CHANNEL_SHARED):
+        ctx = B.Context(B.make_config(block, "bf16", 2, 128, 300, hidden=256, gate=gate, **heads))
+        params["a"] = torch.ones((128,), device="cuda", dtype=torch.bfloat16) if gate else None
+        last.append(ctx.forward(params, x0)[-1].float())
+        ctx.sync_status()
+        launches.append(ctx.launches)
+    assert launches[1] == launches[0] - 1
+    # gates of one: the same sums (float additions of the same two values, one rounding to bf16)
+    assert torch.equal(last[0], last[1])
