@@ -70,7 +70,8 @@ struct PartsGemm {
   const float* gate = nullptr;
   bool relu = false;
 };
-// false: not launched (the device refuses launches in clusters, or no tensor map could be made); nothing has run then.
+// false: not launched (the device refuses launches in clusters, no tensor map could be made, or D is not 16-byte aligned in
+// another epilogue than EPI_STORE); nothing has run then.
 bool gemm_parts(Launcher& lc, const PartsGemm& g, int* status_word);
 // Whether `batch` products with M x N outputs have tiles for half of the CTA pairs.
 bool parts_fill(int M, int N, int batch);

@@ -493,6 +493,7 @@ bool gemm_parts(Launcher& lc, const PartsGemm& g, int* status_word) {
   p.stages = (int)(kRingBytes / (kABytes + p.b_bytes));
   if (p.stages > kMaxStages) p.stages = kMaxStages;
   p.direct = g.D && ((uintptr_t)g.D & 15u) != 0;
+  if (p.direct && g.epi != EPI_STORE) return false;  // (element by element neither E nor the mask is taken along)
   CUtensorMap tmA, tmB, tmD, tmD2, tmE, tmP;
   bool ok = g.a_mn ? map_planes(&tmA, g.A, g.M, g.K, g.batch, 64, BK, CU_TENSOR_MAP_SWIZZLE_128B)
                    : map_planes(&tmA, g.A, g.K, g.M, g.batch, BK, BM, CU_TENSOR_MAP_SWIZZLE_64B);
