@@ -598,16 +598,14 @@ bool operand_ok(const void* base, int64_t s_mn, int64_t s_k, int64_t s_b, int ba
 
 namespace tc {
 EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  static bool tried = false;
-  if (!tried) {
-    tried = true;
+  static const EncodeTiledFn fn = []() -> EncodeTiledFn {  // (one thread looks it up, others wait for it)
     void* ptr = nullptr;
     cudaDriverEntryPointQueryResult q;
     if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &q) == cudaSuccess &&
         q == cudaDriverEntryPointSuccess)
-      fn = (EncodeTiledFn)ptr;
-  }
+      return (EncodeTiledFn)ptr;
+    return nullptr;
+  }();
   return fn;
 }
 
