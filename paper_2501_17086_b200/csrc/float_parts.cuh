@@ -13,7 +13,8 @@ __device__ __forceinline__ void split_rest2(uint32_t h, float ra, float rb, uint
   l = pack_bf16(ra - __uint_as_float(m << 16), rb - __uint_as_float(m & 0xffff0000u));
 }
 // a and b, each as three bf16 parts that add up to it exactly (24 bits; below 2^-109 the low part runs into the denormals and
-// loses bits), packed in pairs.  For magnitudes (as bits) below kPlainParts, whose high part rounds to a finite value.
+// loses bits), packed in pairs.  For magnitudes (as bits) below kPlainParts, whose high part rounds to a finite value (from there on
+// a part is infinite or NaN).
 constexpr uint32_t kPlainParts = 0x7f7f8000u;
 __device__ __forceinline__ void split_plain2(float a, float b, uint32_t& h, uint32_t& m, uint32_t& l) {
   h = pack_bf16(a, b);
@@ -30,6 +31,11 @@ __device__ __forceinline__ void split_parts2(float a, float b, uint32_t& h, uint
   if (ub >= kPlainParts && ub < inf) h = (h & 0x0000ffffu) | (__float_as_uint(b) & 0xffff0000u);
   split_rest2(h, ua < inf ? a - __uint_as_float(h << 16) : 0.0f, ub < inf ? b - __uint_as_float(h & 0xffff0000u) : 0.0f, m, l);
 }
+
+// The tensor core truncates: the sums of 32 of K are 4.5e-8 of themselves (normal operands) to 5.1e-8 (of one sign) too small on
+// average, which adds up over the products of a stack where the float sums' roundings do not (weight gradients of 8 layers: 2.7 times
+// the error).  Three of eight blocks of a row, others in the next row, count 2^-23 = 1.19e-7 more.
+constexpr float kOneUp = 1.00000011920928955f;
 
 // A matrix [batch][rows][cols] held as three such planes, columns contiguous: part q of element (b, r, c) at
 // p[q * plane + b * sb + r * ld + c].  ld is a multiple of 16 (32 bytes), what lies beyond cols is never read.

@@ -1,5 +1,5 @@
 // Float GEMM on the tensor cores for any orientation of the operands (decoders in single precision, MLP stacks up to 63 wide; wider
-// ones keep their operands in parts: gemm_parts.cu):
+// ones keep their operands in parts, gemm_parts.cu, where their workspace and the device allow it):
 //   D(m, n) = sum_k A(m, k) B(n, k), each operand split on the way into shared memory into three bf16 parts that add up to it
 //   exactly, six bf16 products of parts (all but the three below 2^-26 of the whole), the epilogues of the CUDA-core kernel.
 //
@@ -16,8 +16,8 @@
 // and three products, which hold 22 bits and are biased:
 //   K =   32  1.0e-7  0.7e-7  1.3e-7        K =  520  4.1e-7  1.05e-7  1.5e-7
 //   K =  128  2.0e-7  0.8e-7  1.35e-7       K = 4096  1.1e-6  2.2e-7  2.4e-7
-// and less for positive operands.  Weight gradients of float MLP stacks of 2 and 8 layers, 64 to 520 wide, 32 to 4000 rows: 0.18
-// to 1.0 times the error on the CUDA cores.  Contractions up to 16 stay there: a float sum of a few terms rounds no more than a
+// and less for positive operands.  Weight gradients of float MLP stacks of 2 and 8 layers, 64 to 520 wide, 32 to 4000 rows (here under
+// HBP_GEMM_PAIR=0; in parts they have the same bits): 0.18 to 1.0 times the error on the CUDA cores.  Contractions up to 16 stay there: a float sum of a few terms rounds no more than a
 // block truncates (K = 4: 3.9e-8, 16: 7.3e-8, 20: 8.2e-8, 32: 1.03e-7 against 6.8e-8 for any K up to 32).
 //
 // The six bf16 products cost the tensor time of three tf32 ones (768 clocks of a k-block), the parts take 48 KB of stores
@@ -25,6 +25,7 @@
 // 467; 4096 x 1024 x 4096: 1390, 282, 254.  Bound by the loading warps, no one thing in them: of the 350 (467) us 50 (162) go
 // without the global loads, 40 (19) without the split's arithmetic, 14 (38) without two of the three stores, 16 (29) without ten
 // of the twelve MMAs.
+#include "float_parts.cuh"
 #include "tc_common.cuh"
 
 namespace hbp {
@@ -40,10 +41,6 @@ constexpr int kStages = 4;
 // 128 rows of 128 bytes: the high and middle parts of 32 elements of A; of B; the low parts of A and of B
 constexpr uint32_t kTile = BM * 128, kStageBytes = 3 * kTile;
 constexpr uint32_t kTmemCols = 256;
-// The tensor core truncates: a block's sums are 4.5e-8 of themselves (normal operands) to 5.1e-8 (of one sign) too small on average,
-// which adds up over the products of a stack where the float sums' roundings do not (weight gradients of 8 layers: 2.7 times the
-// error).  Three of eight blocks of a row, others in the next row, count 2^-23 = 1.19e-7 more.
-constexpr float kOneUp = 1.00000011920928955f;
 constexpr int kSmemBytes = kStages * (int)kStageBytes + 1024 /*alignment*/ + 256 /*barriers*/;
 // what each adding warp uses of the stages once all products are done (refine's two blocks, or the epilogue's one)
 constexpr int kRowPitch = 33, kColPitch = 68, kWarpFloats = BK * kRowPitch + BK * kColPitch;
@@ -56,28 +53,16 @@ struct F32Params {
   int* status;
 };
 
-// a and b, each as three bf16 parts that add up to it exactly (24 bits; below 2^-109 the low part runs into the denormals and
-// loses bits), packed in pairs.  An infinity or a NaN leaves a part NaN, so that every sum it enters is not finite, which refine
-// settles.
-__device__ __forceinline__ void split_bf16x3(float a, float b, uint32_t& h, uint32_t& m, uint32_t& l) {
-  auto pack = [](float x, float y) {
-    const __nv_bfloat162 v = __floats2bfloat162_rn(x, y);
-    return *reinterpret_cast<const uint32_t*>(&v);
-  };
-  h = pack(a, b);
-  const float ra = a - __uint_as_float(h << 16), rb = b - __uint_as_float(h & 0xffff0000u);
-  m = pack(ra, rb);
-  l = pack(ra - __uint_as_float(m << 16), rb - __uint_as_float(m & 0xffff0000u));
-}
 __device__ __forceinline__ void st_shared8(uint32_t addr, uint32_t a, uint32_t b) {
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
 }
 // Four neighbours in k (unit of 4 out of 8) of a row: high and middle parts to the operand's tile, low parts to its half
-// (0 = A, 4 = B, in 16-byte units) of the common one.
+// (0 = A, 4 = B, in 16-byte units) of the common one.  An infinity, a NaN or a value whose high part rounds to one leaves a part NaN,
+// so that every sum it enters is not finite, which refine settles.
 __device__ __forceinline__ void store_split(uint32_t tile, uint32_t low_tile, int low_half, int row, int unit, float a, float b, float c, float d) {
   uint32_t h0, m0, l0, h1, m1, l1;
-  split_bf16x3(a, b, h0, m0, l0);
-  split_bf16x3(c, d, h1, m1, l1);
+  split_plain2(a, b, h0, m0, l0);
+  split_plain2(c, d, h1, m1, l1);
   const uint32_t at = (uint32_t)(unit & 1) * 8u;
   st_shared8(swz(tile, row, unit >> 1) + at, h0, h1);
   st_shared8(swz(tile, row, 4 + (unit >> 1)) + at, m0, m1);

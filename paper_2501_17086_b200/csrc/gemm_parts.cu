@@ -42,7 +42,6 @@ constexpr int kRegsFew = 56, kRegsMany = 224;
 constexpr uint32_t kFloatBuf = 4096, kPartBuf = 3 * 32 * 64, kEpiBytes = kFloatBuf + kPartBuf;
 constexpr uint32_t TMEM_COLS = 512;
 constexpr int SMEM_BYTES = (int)kRingBytes + EPI_WARPS * (int)kEpiBytes + 1024 /*alignment*/ + 512 /*barriers*/;
-constexpr float kOneUp = 1.00000011920928955f;  // see gemm_f32.cu
 
 struct Params {
   PartsGemm g;
@@ -443,15 +442,6 @@ bool map_planes(CUtensorMap* tm, const Planes& P, int cols, int rows, int batch,
   return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, P.p, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
-bool map_floats(CUtensorMap* tm, const float* base, int M, int N, int batch, int64_t ld, int64_t sb) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn) return false;
-  const cuuint64_t dims[3] = {(cuuint64_t)N, (cuuint64_t)M, (cuuint64_t)batch};
-  const cuuint64_t strides[2] = {(cuuint64_t)ld * 4, (cuuint64_t)(batch > 1 ? sb : ld * M) * 4};
-  const cuuint32_t box[3] = {32, 32, 1}, estr[3] = {1, 1, 1};
-  return fn(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
 
 }  // namespace
 
@@ -473,7 +463,9 @@ bool gemm_parts(Launcher& lc, const PartsGemm& g, int* status_word) {
   p.m_tiles = (g.M + TILE_M - 1) / TILE_M;
   // The width of a tile: the one whose waves over the SM pairs take the least time.  A block of 32 of K is 12 instructions of
   // n_tile / 2 clocks (narrow ones 40: A is read from shared memory either way) and a tile ends with an epilogue that only the
-  // next tile's first blocks run under.
+  // next tile's first blocks run under: 1500 clocks, and 12 a column, 60 where the GELU is formed (from the kernel's times).  Of 7
+  // stacks, 64 (256) x 300 to 1024 (2048) x 4000, in each of their products the width chosen so is the fastest of the six or
+  // within 4 % of it; a wrong one costs up to 1.9 times (1900 x 520 x 1560, 12 at once: 192 columns 502 us of VJP, 32 863).
   const int pairs = sm_count() / 2;
   int64_t best = 0;
   for (int n = 32; n <= kMaxTileN; n += 32) {
@@ -502,9 +494,9 @@ bool gemm_parts(Launcher& lc, const PartsGemm& g, int* status_word) {
   tmD = tmD2 = tmE = tmP = tmA;  // placeholders when unused
   const bool to_parts = g.epi == EPI_GELU_FWD || g.epi == EPI_MUL;
   if (to_parts) ok = ok && map_planes(&tmP, g.Dp, g.N, g.M, g.batch, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
-  else if (!p.direct) ok = ok && map_floats(&tmD, g.D, g.M, g.N, g.batch, g.ldd, g.d_sb);
-  if (g.D2) ok = ok && map_floats(&tmD2, g.D2, g.M, g.N, g.batch, g.ldd2, g.d2_sb);
-  if (g.E) ok = ok && map_floats(&tmE, g.E, g.M, g.N, g.batch, g.lde, g.e_sb);
+  else if (!p.direct) ok = ok && make_map_epi(&tmD, g.D, true, g.M, g.N, g.batch, g.ldd, g.d_sb);
+  if (g.D2) ok = ok && make_map_epi(&tmD2, g.D2, true, g.M, g.N, g.batch, g.ldd2, g.d2_sb);
+  if (g.E) ok = ok && make_map_epi(&tmE, g.E, true, g.M, g.N, g.batch, g.lde, g.e_sb);
   if (!ok) return false;
   static PerDevice<bool> attr_done;
   if (!attr_done.here()) {

@@ -569,20 +569,6 @@ bool make_map(CUtensorMap* tm, const void* base, int extent_mn, int K, int batch
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Tensor map of an epilogue operand [batch][M][N] (leading dimension ld, batch stride sb, in elements):
-// boxes of 32 rows x 128 bytes, the chunk one epilogue warp stages.
-bool make_map_epi(CUtensorMap* tm, const void* base, bool f32, int M, int N, int batch, int64_t ld, int64_t sb) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn) return false;
-  const cuuint64_t es = f32 ? 4 : 2;
-  cuuint64_t dims[3] = {(cuuint64_t)N, (cuuint64_t)M, (cuuint64_t)batch};
-  cuuint64_t strides[2] = {(cuuint64_t)ld * es, batch > 1 ? (cuuint64_t)sb * es : (cuuint64_t)ld * es * (cuuint64_t)M};
-  cuuint32_t box[3] = {f32 ? 32u : 64u, 32u, 1u}, estr[3] = {1, 1, 1};
-  return fn(tm, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims,
-            strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 // An operand qualifies if one of its two strides is 1 and the others keep every row 16-byte aligned.
@@ -597,6 +583,18 @@ bool operand_ok(const void* base, int64_t s_mn, int64_t s_k, int64_t s_b, int ba
 }  // namespace
 
 namespace tc {
+bool make_map_epi(CUtensorMap* tm, const void* base, bool f32, int M, int N, int batch, int64_t ld, int64_t sb) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  const cuuint64_t es = f32 ? 4 : 2;
+  cuuint64_t dims[3] = {(cuuint64_t)N, (cuuint64_t)M, (cuuint64_t)batch};
+  cuuint64_t strides[2] = {(cuuint64_t)ld * es, batch > 1 ? (cuuint64_t)sb * es : (cuuint64_t)ld * es * (cuuint64_t)M};
+  cuuint32_t box[3] = {f32 ? 32u : 64u, 32u, 1u}, estr[3] = {1, 1, 1};
+  return fn(tm, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims,
+            strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 EncodeTiledFn encode_fn() {
   static const EncodeTiledFn fn = []() -> EncodeTiledFn {  // (one thread looks it up, others wait for it)
     void* ptr = nullptr;
@@ -666,7 +664,8 @@ bool gemm_tc(Launcher& lc, const GemmArgs& g, int* status_word) {
   if (g.epi == EPI_RESID && !g.R && !g.E) return false;
 
   // CTA pairs wherever there are at least two 128-row blocks (unless the context asks for single CTAs): a stage is
-  // 32 KB instead of 48 KB for the same flops per SM, so the ring is six stages deep and draws a third less from L2
+  // 32 KB instead of 48 KB for the same flops per SM: five stages beside two staging buffers per epilogue warp (float operands
+  // six and one) where single CTAs have four, and a third less is drawn from L2
   const int sms = sm_count();
   // A product at most 128 columns wide runs on single CTAs with MMAs of 64 or 128 columns, so that most of the tile is
   // not padding (64-wide recurrent states).  The LayerNorm row sums keep the full tile: their slots are per 64 columns.

@@ -139,10 +139,11 @@ hbp_status check_config(const hbp_config* c) {
   return HBP_OK;
 }
 
-// Whether a float residual MLP stack keeps its operands in parts.  Training step and exact pass, time without over time with:
-// 8 layers 64 wide (256 hidden), 64 rows 1.20 and 1.21; 64 (128) x 4096 rows 1.98 and 2.31; 132 (260) x 1000 1.33 and 1.44;
-// 1024 (4096) x 40 rows 2.0 and 2.2, x 2000 rows 2.1.  Below 64 wide the tiles are mostly padding (36 (64) x 40 rows 0.91 and
-// 0.94), and up to 32 rows the CUDA cores are faster (gemm_f32.cu).
+// Whether a float residual MLP stack keeps its operands in parts (if the workspace allows it: weight_layers_in).  Forward and
+// backward(4) with gradients, and the exact pass alone, time without over time with: 8 layers 64 wide (256 hidden), 64 rows 1.38 and
+// 1.48; 16 layers 68 (136) x 4096 rows 1.72 and 1.68; 8 layers 132 (260) x 1000 1.50 and 1.53; 16 layers 1024 (4096) x 40 rows 1.60
+// and 2.85, x 2000 1.89 and 2.06.  Below 64 wide the tiles are mostly padding (36 (64) x 40 rows 0.91 and 0.94), and up to 32 rows
+// the CUDA cores are faster (gemm_f32.cu).
 bool keeps_parts(const hbp_config& f) {
   return f.dtype == HBP_F32 && (f.block == HBP_BLOCK_MLP || f.block == HBP_BLOCK_PRELN_MLP || f.block == HBP_BLOCK_RELU_MLP || f.block == HBP_BLOCK_POSTLN_MLP) &&
          f.tokens > 32 && f.d >= 64 && f.hidden >= 64;

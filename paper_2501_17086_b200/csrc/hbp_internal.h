@@ -46,7 +46,7 @@ struct GemmArgs {
   const void* gate = nullptr;  // [N] per batch entry (stride gate_sb), nullptr = ones
   int64_t gate_sb = 0;
   float* R = nullptr;  // fp32 master copy of the residual stream [M][N], leading dim N
-  bool relu = false;   // EPI_RESID on the CUDA-core kernel only: v = max(v, 0) and D2[m,n] = (v > 0) as 0/1 (the mask that gates this step)
+  bool relu = false;   // EPI_RESID of float products: v = max(v, 0) and D2[m,n] = (v > 0) as 0/1 (the mask that gates this step)
   float2* stats = nullptr;  // EPI_STORE_LN: [batch][M][stats_slots] partial sums; batch stride stats_sb (in float2)
   int64_t stats_sb = 0;
   // float operands for the tensor cores: each of A (after the A2 product) and B split into a tf32-exact

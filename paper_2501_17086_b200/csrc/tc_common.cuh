@@ -84,7 +84,9 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank) {
 }
 // Arrives at a barrier of another CTA of the cluster after reads of tensor memory (completed, and fenced by
 // tcgen05.fence::before_thread_sync): no write of this thread has to be seen there, and a release at cluster scope, which
-// waits for all of its earlier accesses, takes 1000 to 1800 clocks while tile copies are in flight.
+// waits for all of its earlier accesses, takes 1000 to 1800 clocks while tile copies are in flight: with it a training step of 12 float layers
+// 520 (1560) x 1900 rows takes 3558 us instead of 2647, the exact pass of a 6-layer decoder 512 wide 776 instead of 743, a training
+// step of 64 bf16 layers 1024 (4096) x 8192 rows 40.2 ms instead of 39.4.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
@@ -258,6 +260,9 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link against libcuda); nullptr if absent.
 EncodeTiledFn encode_fn();
+// Tensor map of an epilogue operand [batch][M][N] (leading dimension ld, batch stride sb, in elements): boxes of 32 rows x 128
+// bytes, the chunk one epilogue warp stages.
+bool make_map_epi(CUtensorMap* tm, const void* base, bool f32, int M, int N, int batch, int64_t ld, int64_t sb);
 int sm_count();
 
 }  // namespace tc
