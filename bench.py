@@ -58,14 +58,14 @@ def config_of(w, k, touched_bytes=None):
 # profiles/.  An entry is used only while the kernel's sources still hash to the value recorded with the capture and
 # the workload has the captured shapes; otherwise the bench line carries "traffic": null.
 TRAFFIC = {
-    # gemm_tc_kernel, VJP pair (dA + dY): c5_small (4 layers x 16384 tokens): 2063.204 + 1055.452 and 2749.347 + 279.092 MB;
-    # c2_small (8 layers x 8192 tokens): 738.612 + 504.159 and 790.034 + 129.739 MB
+    # gemm_tc_kernel, VJP pair (dA + dY): c5_small (4 layers x 16384 tokens): 2036.314 + 1054.398 and 3038.729 + 279.232 MB;
+    # c2_small (8 layers x 8192 tokens): 738.478 + 504.902 and 790.265 + 129.146 MB
     "gemm_vjp": [
-        {"sources": ("gemm_tc.cu", "tc_common.cuh"), "sha256": "d3caab9167812b48", "shape": ("preln_mlp", "bf16", 2048, 8192),
-         "bytes_per_token_layer": (2063.204e6 + 1055.452e6 + 2749.347e6 + 279.092e6) / (4 * 16384),
+        {"sources": ("gemm_tc.cu", "tc_common.cuh"), "sha256": "5ddffe2221713528", "shape": ("preln_mlp", "bf16", 2048, 8192),
+         "bytes_per_token_layer": (2036.314e6 + 1054.398e6 + 3038.729e6 + 279.232e6) / (4 * 16384),
          "profile": "profiles/gemm_tc_kernel_c5_small.md"},
-        {"sources": ("gemm_tc.cu", "tc_common.cuh"), "sha256": "d3caab9167812b48", "shape": ("preln_mlp", "bf16", 1024, 4096),
-         "bytes_per_token_layer": (738.612e6 + 504.159e6 + 790.034e6 + 129.739e6) / (8 * 8192),
+        {"sources": ("gemm_tc.cu", "tc_common.cuh"), "sha256": "5ddffe2221713528", "shape": ("preln_mlp", "bf16", 1024, 4096),
+         "bytes_per_token_layer": (738.478e6 + 504.902e6 + 790.265e6 + 129.146e6) / (8 * 8192),
          "profile": "profiles/gemm_tc_kernel_c2_small.md"}],
     # scan_depth_lnstat_kernel: c5_small 605.051 MB read + 213.533 MB written for 4 steps x 16384 x 2048 elements; c2_small
     # 286.285 + 80.494 MB for 8 x 8192 x 1024 (the writes still in L2 when such a small launch ends are not in the counter)
@@ -77,11 +77,11 @@ TRAFFIC = {
          "bytes_per_state_element_step": (286.285e6 + 80.494e6) / (8 * 8192 * 1024),
          "profile": "profiles/scan_depth_lnstat_kernel_c2_small.md"}],
     # scan_ring_kernel on c3 (dram__bytes.sum.per_second x gpu__time_duration of the capture): the scan that writes the
-    # next VJP's split operand 6.111 TB/s x 167.2 us, the plain one 5.752 TB/s x 83.6 us
+    # next VJP's split operand 6.046 TB/s x 169.0 us, the plain one 5.680 TB/s x 84.7 us
     "scan_ring": [
-        {"sources": ("scan_ring.cu", "tc_common.cuh"), "sha256": "895d1a866a4af682", "shape": ("rnn_tanh", "f32", 512, 0),
-         "bytes_per_state_element_step": 5.752e12 * 83.6e-6 / (4096 * 32 * 512),
-         "bytes_per_state_element_step_operand": 6.111e12 * 167.2e-6 / (4096 * 32 * 512),
+        {"sources": ("scan_ring.cu", "tc_common.cuh"), "sha256": "926e6b3b23b4c4d9", "shape": ("rnn_tanh", "f32", 512, 0),
+         "bytes_per_state_element_step": 5.680e12 * 84.7e-6 / (4096 * 32 * 512),
+         "bytes_per_state_element_step_operand": 6.046e12 * 169.0e-6 / (4096 * 32 * 512),
          "profile": "profiles/scan_ring_kernel_c3.md"}],
 }
 
