@@ -38,7 +38,7 @@ __device__ __forceinline__ void split_parts2(float a, float b, uint32_t& h, uint
 constexpr float kOneUp = 1.00000011920928955f;
 
 // A matrix [batch][rows][cols] held as three such planes, columns contiguous: part q of element (b, r, c) at
-// p[q * plane + b * sb + r * ld + c].  ld is a multiple of 16 (32 bytes), what lies beyond cols is never read.
+// p[q * plane + b * sb + r * ld + c].  ld is a multiple of 16 (32 bytes) or 64, what lies beyond cols is never read.
 struct Planes {
   bf16* p = nullptr;
   int64_t ld = 0, sb = 0, plane = 0;

@@ -247,7 +247,13 @@ size_t carve(hbp_ctx* c, char* base, int weight_layers) {
       c->CB = take(steps * N * d * es);
       c->rstd = (float*)take(steps * N * 4);
     }
-    auto plane_cols = [](size_t cols) { return (cols + 15) / 16 * 16; };
+    // Rows of a plane start at 128 bytes (a pass over 112 to 1400 columns takes 1 to 6 % less so: 3 layers 356 (1196) x 127 rows 229 us
+    // instead of 242, 5 layers 424 (932) x 1219 488 instead of 503) unless that adds more than a quarter of the memory, where it
+    // gains nothing (96 (220) x 79 rows 301 instead of 294).
+    auto plane_cols = [](size_t cols) {
+      const size_t line = (cols + 63) / 64 * 64;
+      return 4 * line <= 5 * cols ? line : (cols + 15) / 16 * 16;
+    };
     auto take_planes = [&](Planes& P, size_t entries, size_t rows, size_t cols) {
       P.ld = (int64_t)plane_cols(cols); P.sb = (int64_t)rows * P.ld; P.plane = (int64_t)entries * P.sb;
       P.p = (bf16*)take(3 * (size_t)P.plane * 2);
