@@ -477,8 +477,8 @@ struct Run {
     // One launch over all layers with the operands split inside, rather than a launch and a split pass for each run of layers
     // whose weights fit the planes, where such a run is too small for the chip (the parameter pass reads dZ as planes).  backward(1)
     // of 16 layers 1024 (4096), inside / in runs of n tiles: 128 rows, n = 6, 428 / 1269 us; 250, 12, 764 / 1304; 500, 60, 1468 / 912;
-    // 8 layers 512 (1024) x 300, 24, 123 / 155
-    const bool runs = c->weight_layers >= b1 - b0 || parts_fill((int)N, (int)d, c->weight_layers);
+    // 8 layers 512 (1024) x 300, 24, 123 / 155.  (Weights that are not 16-byte aligned can only be split into planes.)
+    const bool runs = c->weight_layers >= b1 - b0 || parts_fill((int)N, (int)d, c->weight_layers) || (((uintptr_t)p->W1 | (uintptr_t)p->W2) & 15u);
     if (c->use_parts && (runs || !want_dy)) return mlp_vjp_parts(b0, b1, want_dy, slot);
     const int nb = b1 - b0, ss = step_stride();
     GemmArgs a = base_args();

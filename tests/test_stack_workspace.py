@@ -62,7 +62,11 @@ def test_stacks_run_with_less(monkeypatch, block, group):
     params = harness.params_for(w, inp)
     one_layer = 6 * (w.hidden * 144 + w.d * 320)  # both weights in three planes of two bytes, 132 columns rounded up to 16, 260 to 64
 
-    def run(nbytes, pair=True):
+    def shifted(t):  # the same values four bytes past a 16-byte boundary
+        out = torch.empty(t.numel() + 4, device="cuda")[1:1 + t.numel()].view(t.shape)
+        return out.copy_(t)
+
+    def run(nbytes, pair=True, params=params):
         with monkeypatch.context() as m:
             m.setattr(B, "workspace_bytes", lambda cfg: nbytes)
             if not pair:
@@ -83,6 +87,8 @@ def test_stacks_run_with_less(monkeypatch, block, group):
         some, more, n = run(most - (w.L - layers) * one_layer)
         assert more > launches and 0 < n <= products  # (batched VJPs of so few layers may split inside)
         assert all(torch.equal(a, b) for a, b in zip(some, all_layers))
+    some, _, n = run(most - (w.L - 1) * one_layer, params={k: shifted(t) for k, t in params.items()})
+    assert n == products and all(torch.equal(a, b) for a, b in zip(some, all_layers))
     # the operands split inside the kernel: the same arithmetic
     (inside, *n0), (least, *n1) = run(without, pair=False), run(without)
     assert n0 == n1 and n0[0] < launches and n0[1] == 0
