@@ -366,30 +366,28 @@ def measure(env, wname, k, steps, warmup, headline, detail):
             roofline["traffic"] = t["bytes_per_token_layer"] * w.tokens * w.L * kk * steps / max(1, vjp_launches)
             roofline["traffic_source"] = t["profile"] + " (scaled by tokens x layers per launch)"
     else:
-        # float data: the contraction runs on the tensor cores as three tf32 products per algorithmic product
-        # (split operands), so the hardware does 3x the algorithmic flops; tf32 peak = measured bf16 peak x the
-        # nominal tf32/bf16 ratio (1.1 / 2.25).  The operand split is inside the measured phase.
+        # float data: the contraction runs on the tensor cores as six bf16 products of parts per algorithmic product, so the hardware
+        # does 6x the algorithmic flops.  Splitting the operands is inside the measured phase.  These launches are short and run
+        # at the full clock (no power cap in the clock record), so the burst figure is the peak they are held to; the fraction of
+        # the sustained one is given beside it.
         alg = (vjp_flops * kk * steps / (vjp_ms * 1e-3) / 1e12) if vjp_ms else None
-        # These launches are short and run at the full clock (no power cap in the clock record), so the burst figure
-        # is the peak they are held to; the fraction of the sustained one is given beside it.
-        tf32_peak = peaks.get("bf16_tflops", 1590.0) * 1.1 / 2.25
-        tf32_sustained = bf16_peak * 1.1 / 2.25
-        scan_writes_operand = w.block == "rnn_tanh" and os.environ.get("HBP_SCAN_OPERAND", "1") != "0"
-        split_note = "the operand split is written by the preceding scan" if scan_writes_operand else "incl. the operand split"
-        roofline = {"bound": "tensor", "kernel": f"gemm_tc_kernel, tf32 x3 (VJP phase, {split_note})",
-                    "achieved": 3 * alg if alg else None, "peak": tf32_peak, "unit": "TFLOP/s (tf32, 3 per algorithmic flop)",
-                    "frac": (3 * alg / tf32_peak) if alg else None, "algorithmic_tflops": alg,
-                    "algorithmic_frac": (alg / tf32_peak) if alg else None,
+        peak = peaks.get("bf16_tflops", 1590.0)
+        kernel = "gemm_cell_kernel" if w.block in ("rnn_tanh", "gru", "lstm") else "gemm_parts_kernel"
+        roofline = {"bound": "tensor", "kernel": f"{kernel}, bf16 x 6 (VJP phase, incl. the operand split)",
+                    "achieved": 6 * alg if alg else None, "peak": peak, "unit": "TFLOP/s (bf16, 6 per algorithmic flop)",
+                    "frac": (6 * alg / peak) if alg else None, "algorithmic_tflops": alg,
+                    "algorithmic_frac": (alg / peak) if alg else None,
                     "fp32_alu_peak_tflops": 148 * 128 * 2 * 1.965e9 / 1e12,
-                    "frac_of_sustained": (3 * alg / tf32_sustained) if alg else None,
-                    "peak_source": "of measured burst bf16 x nominal tf32/bf16 ratio" if peaks else "of fallback", "traffic": None}
+                    "frac_of_sustained": (6 * alg / bf16_peak) if alg else None,
+                    "peak_source": "of measured (burst bf16 GEMM)" if peaks else "of fallback", "traffic": None}
     # scan: read u (+ xhat when the LayerNorm finish is fused, + the per-element gate of a GRU), write g
     tensors = 2 + (1 if w.block in ("preln_mlp", "preln_transformer", "gru", "lstm") else 0)  # per-step delta is added by the VJP GEMM epilogue
     if w.block == "postln_mlp":  # u, the non-block part c, g written; + the previous iterate when the split is shifted
         tensors = 3 + (1 if getattr(w, "gamma", 0.0) else 0)
     scan_note = None
-    if w.block == "rnn_tanh" and w.dtype == "f32" and kk > 1 and os.environ.get("HBP_SCAN_OPERAND", "1") != "0":
-        # every scan but the last reads u and tanh' and writes the two terms of the next VJP's operand instead of g
+    if (w.block == "rnn_tanh" and w.dtype == "f32" and kk > 1 and os.environ.get("HBP_GEMM_PAIR", "1") == "0"
+            and os.environ.get("HBP_SCAN_OPERAND", "1") != "0"):
+        # without CTA pairs every scan but the last reads u and tanh' and writes the two terms of the next VJP's operand
         tensors = (4 * (kk - 1) + 2) / kk
         scan_note = f"{kk - 1} of {kk} scans write the next VJP's split operand (4 tensors), the last writes g (2)"
     scan_bytes = tensors * w.steps * w.tokens * w.d * es

@@ -258,10 +258,11 @@ int64_t hbp_launch_count(const hbp_ctx* ctx);
 /* How often since creation a call of this context has taken a form among several that would serve it: a recurrence as one
  * launch (clusters of cell_cluster.cu; those of rnn_cluster.cu; clusters of 16 CTAs with four rows each, rnn_persistent.cu)
  * or step by step (counted per step); a float product on the tensor cores, or a product on the CUDA cores.  GEMM_PARTS: those of
- * GEMM_F32 whose operands lie in the workspace already split (gemm_parts.cu); the others split theirs inside the kernel. */
+ * GEMM_F32 whose operands lie in the workspace already split (gemm_parts.cu); the others split theirs inside the kernel.  GEMM_CELL:
+ * all-step products of a float recurrent kind that form their left operand while they load it (gemm_cell.cu). */
 typedef enum {
   HBP_FORM_CELL_CLUSTER = 0, HBP_FORM_RNN_CLUSTER = 1, HBP_FORM_RNN_FOUR_ROWS = 2, HBP_FORM_STEP = 3, HBP_FORM_GEMM_F32 = 4,
-  HBP_FORM_GEMM_SIMT = 5, HBP_FORM_GEMM_PARTS = 6, HBP_FORM_COUNT = 7
+  HBP_FORM_GEMM_SIMT = 5, HBP_FORM_GEMM_PARTS = 6, HBP_FORM_GEMM_CELL = 7, HBP_FORM_COUNT = 8
 } hbp_form;
 int64_t hbp_form_count(const hbp_ctx* ctx, int32_t form);
 
@@ -270,7 +271,8 @@ int64_t hbp_form_count(const hbp_ctx* ctx, int32_t form);
  * bit 1 = the tensor-core GEMM pairs CTAs (tcgen05 cta_group::2, 256 x 256 tiles): the default; HBP_GEMM_PAIR=0
  * keeps single CTAs (128 x 256 tiles; float MLP stacks then have their operands split inside the kernel, which needs no
  * clusters: what also runs where the device refuses a launch in clusters),
- * bit 2 = on the float tanh RNN the reverse scan between two all-step VJPs (Eq. 9 followed by Eq. 8) also writes
+ * bit 2 = on the float tanh RNN, where the all-step products do not form that operand themselves (fewer than 32 units, single
+ * CTAs), the reverse scan between two all-step VJPs (Eq. 9 followed by Eq. 8) also writes
  * the next VJP's left operand g_{t+1} * tanh'(z_t), split for the tensor cores, instead of the intermediate
  * iterate: the default; HBP_SCAN_OPERAND=0 keeps the separate pass (same bits in every result, a cross-check).
  * HBP_LAYER_GROUP=n (no bit) caps the layers whose hidden-size scratch is held at once at n, where the stack's size asks for no

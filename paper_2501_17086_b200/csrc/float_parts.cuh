@@ -1,5 +1,7 @@
 // A float as three bf16 parts that add up to it: the form in which float operands reach the tensor cores.
 #pragma once
+#include <cuda.h>
+
 #include "hbp_internal.h"
 
 namespace hbp {
@@ -58,6 +60,12 @@ __device__ __forceinline__ void store_parts4(bf16* at, int64_t plane, const floa
   *reinterpret_cast<uint2*>(at + 2 * plane) = make_uint2(l0, l1);
 }
 
+namespace tc {
+// Tensor map of planes of a matrix with `cols` columns and `rows` rows per batch entry: boxes of box_c x box_r x one entry x all
+// parts (gemm_parts.cu).
+bool map_planes(CUtensorMap* tm, const Planes& P, int cols, int rows, int batch, int box_c, int box_r, CUtensorMapSwizzle swizzle);
+}  // namespace tc
+
 // D(m, n) = sum_k A(m, k) B(n, k) of operands held as planes (gemm_parts.cu).  a_mn / b_mn: the plane's columns are the
 // operand's rows (else they are k).  Epilogues as in GemmArgs, float: EPI_STORE, EPI_GELU_FWD (gelu(acc) to Dp, gelu'(acc) to D2),
 // EPI_MUL (acc * E to Dp), EPI_RESID (D, with relu the mask to D2).
@@ -83,5 +91,21 @@ bool gemm_parts(Launcher& lc, const PartsGemm& g, int* status_word);
 bool parts_fill(int M, int N, int batch);
 // src [rows][cols] (cols contiguous and a multiple of 4, any alignment) -> dst rows of the first batch entry on
 void split_parts(Launcher& lc, const float* src, const Planes& dst, int64_t rows, int cols);
+
+// The left operand of a recurrent kind's all-step products, formed while it is loaded (gemm_cell.cu): g = g_{t+1} of every step
+// (LSTM: rows of 2d), coef = the forward pass's coefficients (tanh', C4, C5), both 16-byte aligned; d = units, a multiple of 4.
+struct CellOperand {
+  const float* g = nullptr;
+  const float* coef = nullptr;
+  int64_t rows = 0;
+  int d = 0;
+};
+// out (rows ld apart) = operand times W, W's planes [1, 3 or 4 times d][d]; + delta (laid out like out) unless null.  LSTM: out and delta are
+// the hidden halves, and uc = fg g_h c_h (+ delta_c), the cell halves, rows of 2d.  false (of either): nothing was launched.
+bool cell_vjp(Launcher& lc, int kind, const CellOperand& o, const Planes& W, const float* delta, float* out, int64_t ld, const float* fg,
+              const float* delta_c, float* uc, int* status_word);
+// dW = operand^T H (rows of H ldh apart, 16-byte aligned), dU = operand^T X (X of any alignment, rows of `in`)
+bool cell_wgrad(Launcher& lc, int kind, const CellOperand& o, const float* H, int64_t ldh, const float* X, int in, float* dW, float* dU,
+                float* partial, size_t partial_floats, int* status_word);
 
 }  // namespace hbp

@@ -432,8 +432,9 @@ __global__ void split_parts_kernel(const float* __restrict__ src, Planes dst, in
   store_parts4(dst.p + row * dst.ld + c, dst.plane, v);
 }
 
-// planes of a matrix with `cols` columns and `rows` rows per batch entry: boxes of box_c x box_r x one entry x all parts
-bool map_planes(CUtensorMap* tm, const Planes& P, int cols, int rows, int batch, int box_c, int box_r, CUtensorMapSwizzle swizzle) {
+}  // namespace
+
+bool tc::map_planes(CUtensorMap* tm, const Planes& P, int cols, int rows, int batch, int box_c, int box_r, CUtensorMapSwizzle swizzle) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
   const cuuint64_t dims[4] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)batch, 3};
@@ -442,8 +443,6 @@ bool map_planes(CUtensorMap* tm, const Planes& P, int cols, int rows, int batch,
   return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, P.p, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
-
-}  // namespace
 
 void split_parts(Launcher& lc, const float* src, const Planes& dst, int64_t rows, int cols) {
   const int64_t n = rows * (cols / 4);

@@ -59,6 +59,10 @@ struct hbp_ctx {
   // h_0..h_{T-1} as [d][T*B], X* the inputs as [in][T*B], W* the recurrent matrix transposed
   float *Ahi = nullptr, *Alo = nullptr, *Hhi = nullptr, *Hlo = nullptr, *Xhi = nullptr, *Xlo = nullptr;
   float *Whi = nullptr, *Wlo = nullptr;
+  // Float recurrent kinds of 32 units and up instead of all of the above: W as three bf16 planes; the products form their left operand
+  // while they load it (gemm_cell.cu).  use_cell: until the device refuses such a launch.
+  Planes Wp;
+  bool use_cell = false;
   char* U = nullptr;       // [steps][N][d] block VJP outputs (dY before the LayerNorm finish)
   char* H1 = nullptr;      // [group][N][h] dZ
   // Float residual MLP stacks: the operands of every product as three bf16 planes (gemm_parts.cu).  OPp = what W1 is applied to
@@ -149,6 +153,22 @@ bool keeps_parts(const hbp_config& f) {
          f.tokens > 32 && f.d >= 64 && f.hidden >= 64;
 }
 
+// Whether a recurrent kind's all-step products form their operands as they load them (gemm_cell.cu).  Narrower cells than a
+// k-block of 32 channels would be mostly padding.
+bool forms_operands(const hbp_ctx* c) {
+  const hbp_config& f = c->cfg;
+  const bool recurrent = f.block == HBP_BLOCK_RNN_TANH || f.block == HBP_BLOCK_GRU || f.block == HBP_BLOCK_LSTM;
+  return recurrent && f.dtype == HBP_F32 && (f.block == HBP_BLOCK_LSTM ? f.d / 2 : f.d) >= 32 && c->gemm_pair && !c->force_simt;
+}
+
+// Rows of a plane start at 128 bytes (a pass over 112 to 1400 columns takes 1 to 6 % less so: 3 layers 356 (1196) x 127 rows 229 us
+// instead of 242, 5 layers 424 (932) x 1219 488 instead of 503) unless that adds more than a quarter of the memory, where it
+// gains nothing (96 (220) x 79 rows 301 instead of 294).
+size_t plane_cols(size_t cols) {
+  const size_t line = (cols + 63) / 64 * 64;
+  return 4 * line <= 5 * cols ? line : (cols + 15) / 16 * 16;
+}
+
 // Lays the workspace out, with planes for the weights of weight_layers layers (0: none at all); with base == nullptr only the
 // total size is computed.
 size_t carve(hbp_ctx* c, char* base, int weight_layers) {
@@ -158,6 +178,10 @@ size_t carve(hbp_ctx* c, char* base, int weight_layers) {
     char* p = base ? base + off : nullptr;
     off += align_up(bytes);
     return p;
+  };
+  auto take_planes = [&](Planes& P, size_t entries, size_t rows, size_t cols) {
+    P.ld = (int64_t)plane_cols(cols); P.sb = (int64_t)rows * P.ld; P.plane = (int64_t)entries * P.sb;
+    P.p = (bf16*)take(3 * (size_t)P.plane * 2);
   };
   const size_t es = f.dtype == HBP_F32 ? 4 : 2;
   const size_t N = (size_t)f.tokens, d = (size_t)f.d, h = (size_t)f.hidden;
@@ -173,6 +197,11 @@ size_t carve(hbp_ctx* c, char* base, int weight_layers) {
   const bool recurrent = f.block == HBP_BLOCK_RNN_TANH || f.block == HBP_BLOCK_GRU || f.block == HBP_BLOCK_LSTM;
   if (f.dtype == HBP_BF16 && !recurrent) c->xres = (float*)take(N * d * 4);
   c->partial_floats = (size_t)kGateBlocks * d;
+  const bool cell = forms_operands(c);
+  if (cell) {
+    const size_t u = f.block == HBP_BLOCK_LSTM ? d / 2 : d;
+    take_planes(c->Wp, 1, u * (f.block == HBP_BLOCK_LSTM ? 4 : f.block == HBP_BLOCK_GRU ? 3 : 1), u);
+  }
   if (recurrent) {
     size_t pb = cell_pack_bytes(f.block, f.block == HBP_BLOCK_LSTM ? f.d / 2 : f.d, f.in_dim);
     const size_t rb = f.block == HBP_BLOCK_RNN_TANH ? rnn_cluster_pack_bytes(f.d, f.in_dim) : 0;
@@ -185,7 +214,7 @@ size_t carve(hbp_ctx* c, char* base, int weight_layers) {
     c->C5 = take(rows * 5 * u * es);
     c->A4 = take(rows * 4 * u * es);
     c->hres = (double*)take(2 * N * d * 8);
-    if (f.dtype == HBP_F32) {
+    if (f.dtype == HBP_F32 && !cell) {
       c->Ahi = (float*)take(rows * 4 * u * 4); c->Alo = (float*)take(rows * 4 * u * 4);
       c->Hhi = (float*)take(rows * u * 4); c->Hlo = (float*)take(rows * u * 4);
       c->Xhi = (float*)take(rows * in * 4); c->Xlo = (float*)take(rows * in * 4);
@@ -201,7 +230,7 @@ size_t carve(hbp_ctx* c, char* base, int weight_layers) {
     c->C4 = take(steps * N * 4 * d * es);
     c->A4 = take(steps * N * 4 * d * es);
     c->hres = (double*)take(2 * N * d * 8);
-    if (f.dtype == HBP_F32) {
+    if (f.dtype == HBP_F32 && !cell) {
       c->Ahi = (float*)take(steps * N * 4 * d * 4); c->Alo = (float*)take(steps * N * 4 * d * 4);
       c->Hhi = (float*)take(steps * N * d * 4); c->Hlo = (float*)take(steps * N * d * 4);
       c->Xhi = (float*)take(steps * N * in * 4); c->Xlo = (float*)take(steps * N * in * 4);
@@ -218,7 +247,7 @@ size_t carve(hbp_ctx* c, char* base, int weight_layers) {
       const size_t pb = rnn_persistent_proj_bytes(f.L, f.tokens, f.d);
       if (pb) c->Pd = (double*)take(pb);
     }
-    if (f.dtype == HBP_F32) {
+    if (f.dtype == HBP_F32 && !cell) {
       c->Ahi = (float*)take(steps * N * d * 4); c->Alo = (float*)take(steps * N * d * 4);
       c->Hhi = (float*)take(steps * N * d * 4); c->Hlo = (float*)take(steps * N * d * 4);
       c->Xhi = (float*)take(steps * N * (size_t)f.in_dim * 4); c->Xlo = (float*)take(steps * N * (size_t)f.in_dim * 4);
@@ -247,17 +276,6 @@ size_t carve(hbp_ctx* c, char* base, int weight_layers) {
       c->CB = take(steps * N * d * es);
       c->rstd = (float*)take(steps * N * 4);
     }
-    // Rows of a plane start at 128 bytes (a pass over 112 to 1400 columns takes 1 to 6 % less so: 3 layers 356 (1196) x 127 rows 229 us
-    // instead of 242, 5 layers 424 (932) x 1219 488 instead of 503) unless that adds more than a quarter of the memory, where it
-    // gains nothing (96 (220) x 79 rows 301 instead of 294).
-    auto plane_cols = [](size_t cols) {
-      const size_t line = (cols + 63) / 64 * 64;
-      return 4 * line <= 5 * cols ? line : (cols + 15) / 16 * 16;
-    };
-    auto take_planes = [&](Planes& P, size_t entries, size_t rows, size_t cols) {
-      P.ld = (int64_t)plane_cols(cols); P.sb = (int64_t)rows * P.ld; P.plane = (int64_t)entries * P.sb;
-      P.p = (bf16*)take(3 * (size_t)P.plane * 2);
-    };
     const size_t layers = (size_t)c->layers;
     if (parts) {
       take_planes(c->OPp, layers, N, d);
@@ -580,6 +598,39 @@ struct Run {
     }
   }
 
+  // ---- all-step products of the float recurrent kinds, operands formed while they are loaded (gemm_cell.cu) ----------------
+  CellOperand cell_operand() const {
+    CellOperand o;
+    o.g = (const float*)at(g, state);
+    o.rows = (int64_t)c->cfg.L * N;
+    o.d = (int)(c->cfg.block == HBP_BLOCK_LSTM ? d / 2 : d);
+    o.coef = (const float*)(c->cfg.block == HBP_BLOCK_RNN_TANH ? c->C : c->cfg.block == HBP_BLOCK_GRU ? c->C4 : c->C5);
+    return o;
+  }
+  // false: this context's products are other kernels' from here on (a launch in clusters was refused)
+  bool cell_product(bool launched) {
+    if (launched) lc.ran(HBP_FORM_GEMM_CELL);
+    else c->use_cell = false;
+    return launched;
+  }
+  bool cell_vjp_all() {
+    if (!c->use_cell) return false;
+    const bool every = c->cfg.loss == HBP_LOSS_EVERY_STEP, lstm = c->cfg.block == HBP_BLOCK_LSTM;
+    const int64_t h0 = lstm ? d / 2 : 0;  // the hidden half of a state
+    const float* dl = every ? (const float*)delta : nullptr;
+    if (!cell_product(cell_vjp(lc, c->cfg.block, cell_operand(), c->Wp, dl ? dl + h0 : nullptr, (float*)c->U + h0, d, (const float*)c->Fg, dl,
+                               lstm ? (float*)c->U : nullptr, c->status)))
+      return false;
+    u_has_delta = every;
+    return true;
+  }
+  bool cell_wgrad_all(const hbp_grads* gr) {
+    if (!c->use_cell) return false;
+    const int64_t h0 = c->cfg.block == HBP_BLOCK_LSTM ? d / 2 : 0;
+    return cell_product(cell_wgrad(lc, c->cfg.block, cell_operand(), (const float*)x_all + h0, d, (const float*)inputs, c->cfg.in_dim, gr->dW,
+                                   gr->dU, c->partial, c->partial_floats, c->status));
+  }
+
   // ---- RNN ---------------------------------------------------------------------------------------
   // u_t = (g_{t+1} * tanh'(z_t)) W for every t at once (one GEMM over T*B rows)
   GemmArgs rnn_vjp_args() const {
@@ -599,6 +650,7 @@ struct Run {
     return a;
   }
   void rnn_vjp_all() {
+    if (cell_vjp_all()) return;
     const GemmArgs a = rnn_vjp_args();
     u_has_delta = a.epi == EPI_ADD;
     if (c->Ahi && !operand_ready)
@@ -618,6 +670,7 @@ struct Run {
     return rnn_tc == 1;
   }
   void rnn_wgrad(const hbp_grads* gr) {
+    if (cell_wgrad_all(gr)) return;
     const int T = c->cfg.L;
     const int64_t rows = (int64_t)T * N, in = c->cfg.in_dim;
     // float on the tensor cores: at most 512 rows (16 k-blocks) per split keeps each fp32 accumulation chain
@@ -646,6 +699,7 @@ struct Run {
   // ---- GRU ---------------------------------------------------------------------------------------
   // u_t = (g_{t+1} * [c_r | c_z | c_nr]_t) W for every t at once: one GEMM over T*B rows with K = 3d
   void gru_vjp_all() {
+    if (cell_vjp_all()) return;
     const int T = c->cfg.L;
     const int64_t rows = (int64_t)T * N;
     GemmArgs a = base_args();
@@ -673,6 +727,7 @@ struct Run {
   // dW = [dr|dz|d(W_n h)]^T H (H = states 0..T-1),  dU = [dr|dz|dn]^T X, with the pre-activation gradients
   // g * coefficients; dU is two products because its third row block uses another coefficient than dW's
   void gru_wgrad(const hbp_grads* gr) {
+    if (cell_wgrad_all(gr)) return;
     const int T = c->cfg.L;
     const int64_t rows = (int64_t)T * N, in = c->cfg.in_dim;
     int split = (int)(rows / (c->Ahi ? 512 : 2048));
@@ -711,6 +766,7 @@ struct Run {
   // ---- LSTM (u = d / 2 units; rows of g, U and the states are 2u wide) ------------------------------------
   // u_h = [t c_i | t c_f | t c_g | g_h c_o] W for every t at once (one GEMM, K = 4u); u_c elementwise beside it
   void lstm_vjp_all() {
+    if (cell_vjp_all()) return;
     const int T = c->cfg.L;
     const int64_t rows = (int64_t)T * N, u = d / 2;
     const bool every = c->cfg.loss == HBP_LOSS_EVERY_STEP;
@@ -740,6 +796,7 @@ struct Run {
   }
   // dW = [..]^T H (H = the h half of states 0..T-1), dU = [..]^T X with the same four-block operand
   void lstm_wgrad(const hbp_grads* gr) {
+    if (cell_wgrad_all(gr)) return;
     const int T = c->cfg.L;
     const int64_t rows = (int64_t)T * N, in = c->cfg.in_dim, u = d / 2;
     int split = (int)(rows / (c->Ahi ? 512 : 2048));
@@ -963,6 +1020,7 @@ hbp_status hbp_create(const hbp_config* cfg, void* workspace, size_t workspace_b
   c->ws = (char*)workspace;
   c->ws_bytes = workspace_bytes;
   c->use_parts = c->weight_layers > 0;
+  c->use_cell = forms_operands(c);
   const char* lg = std::getenv("HBP_LAYER_GROUP");
   const int cap = lg ? std::atoi(lg) : 0;
   if (cap > 0 && cap < c->group) c->group = cap;  // (the scratch is carved for the larger group)
@@ -1104,6 +1162,7 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
                         r.at(ctx->Fg, (int64_t)t * state), r.at(ctx->C5, (int64_t)t * N * 5 * u),
                         r.at(xa, (int64_t)(t + 1) * state), (int)N, (int)u, f.in_dim);
     }
+    if (ctx->use_cell) split_parts(r.lc, (const float*)params->W, ctx->Wp, 4 * u, (int)u);
     if (ctx->Ahi) {
       split_tf32_transposed(r.lc, (const float*)xa + u, nullptr, ctx->Hhi, ctx->Hlo, (int64_t)T * N, (int)u, d);
       split_tf32_transposed(r.lc, (const float*)inputs, nullptr, ctx->Xhi, ctx->Xlo, (int64_t)T * N, f.in_dim);
@@ -1122,6 +1181,7 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
                        r.at(ctx->Zc, (int64_t)t * state), r.at(ctx->C4, (int64_t)t * 4 * state),
                        r.at(xa, (int64_t)(t + 1) * state), (int)N, (int)d, f.in_dim);
     }
+    if (ctx->use_cell) split_parts(r.lc, (const float*)params->W, ctx->Wp, 3 * d, (int)d);
     if (ctx->Ahi) {
       split_tf32_transposed(r.lc, (const float*)xa, nullptr, ctx->Hhi, ctx->Hlo, (int64_t)T * N, (int)d);
       split_tf32_transposed(r.lc, (const float*)inputs, nullptr, ctx->Xhi, ctx->Xlo, (int64_t)T * N, f.in_dim);
@@ -1155,6 +1215,7 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
                          f.in_dim);
       }
     }
+    if (ctx->use_cell) split_parts(r.lc, (const float*)params->W, ctx->Wp, d, (int)d);
     if (ctx->Ahi) {  // operand splits that do not change between backward calls
       split_tf32_transposed(r.lc, (const float*)xa, nullptr, ctx->Hhi, ctx->Hlo, (int64_t)T * N, (int)d);
       split_tf32_transposed(r.lc, (const float*)inputs, nullptr, ctx->Xhi, ctx->Xlo, (int64_t)T * N, f.in_dim);
