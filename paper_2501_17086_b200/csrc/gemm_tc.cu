@@ -3,8 +3,10 @@
 //
 //   D(m, n) = sum_k A(m, k) B(n, k), fp32 accumulate, batched (one launch covers all layers of a group).
 //
-// Persistent kernel, one CTA per SM, 320 threads:
-//   warp 0      TMA producer (one lane): fills a ring of {A 128x64, B 128x64 (pairs) or 256x64} bf16 tiles
+// Persistent kernel, one CTA per SM, 384 threads:
+//   warps 0, 10 TMA producers of A and of B (one lane each): fill a ring of {A 128x64, B 128x64 (pairs) or 256x64} bf16 tiles.  (One
+//               producer of both held the narrow tiles back, and MN-major operands, which come as two copies a stage: 2664 x 512 x
+//               2048 16.4 -> 15.8 us, in tiles of 128 columns 15.7 -> 14.5; 8192 x 1024 x 4096 50.4 -> 48.8)
 //   warp 1      MMA issuer (one lane): 4 x tcgen05.mma of 16 of K per stage; owns the TMEM allocation
 //   warps 2..9  epilogue: two warps per 32-lane TMEM quarter, 128 accumulator columns each; each warp
 //               stages 32-row chunks through private 4 KB swizzled buffers, so every global access of
@@ -36,12 +38,12 @@ constexpr int A_BYTES = BM * BK * 2;
 constexpr int PAIR_STAGE_BYTES = A_BYTES + 128 * BK * 2;
 template <bool kPair, bool kTf32>
 struct Mode {
-  static constexpr int kBRows = kPair ? 128 : 256;
   static constexpr int kTileM = kPair ? 256 : 128;
   static constexpr int kEpiBufs = kPair && !kTf32 ? 2 : 1;  // staging buffers per epilogue warp
   static constexpr int kRingBytes = (kEpiBufs == 2 ? 5 : 6) * PAIR_STAGE_BYTES;  // single CTAs: 4, 6 or 8 stages
 };
-constexpr int EPI_WARPS = 8, THREADS = 64 + 32 * EPI_WARPS;
+constexpr int MAX_STAGES = 8;
+constexpr int EPI_WARPS = 8, kProducerB = 2 + EPI_WARPS, THREADS = 64 + 32 * EPI_WARPS + 64;
 constexpr uint32_t TMEM_COLS = 512;
 constexpr int EPI_BUF_BYTES = 4096;  // 32 rows x 128 bytes
 constexpr int SMEM_BYTES = Mode<true, false>::kRingBytes + 2 * EPI_WARPS * EPI_BUF_BYTES + 1024 /*alignment slack*/ + 512 /*barriers*/;
@@ -52,8 +54,10 @@ struct TcParams {
   int m_tiles, n_tiles, num_tiles, k_blocks;
   int a_mn, b_mn;  // 1: the operand is MN-major
   int tf32;        // operands are float, multiplied as tf32 (else bf16)
-  int n_mma;       // columns one MMA covers: 256, or 64 / 128 for a narrow single-CTA product (N <= 128), whose B tiles,
-                   // instructions and epilogue then leave the padding columns out
+  int n_mma;       // columns of a tile (and of one MMA): 64, 128, 192 (pairs only) or 256
+  int b_rows;      // rows of B that a CTA stages: half of them (pairs) or all
+  int stages;
+  uint32_t stage_bytes;
   int segs;        // K segments, each with its own pair of operand maps (3 for the split-float product)
   int splits, kb_per_split;  // split-K: tile z index = split * batch + b; each split covers kb_per_split k-blocks
   int epi, d_f32;
@@ -62,7 +66,7 @@ struct TcParams {
   const void* E; int64_t lde, e_sb;
   const void* gate; int64_t gate_sb;
   float* R;
-  float2* stats; int64_t stats_sb;
+  float2* stats; int64_t stats_sb; int slots;
   int* status;
   uint64_t wait_limit_ns;  // limit of every barrier wait
   int stall;               // self-test of the bounded waits only: the producer arms its first stage and copies nothing
@@ -151,20 +155,21 @@ __device__ __forceinline__ void residual_chunk(const TcParams& p, int b, int row
 }
 
 // ------------------------------------------------------------------------------------------- kernel
-template <bool kPair, bool kTf32>
+// kNarrow: tiles of p.n_mma columns; else of 256, whose constants the compiler folds (a run-time width costs the large products 2 to 4 %)
+template <bool kPair, bool kTf32, bool kNarrow>
 __global__ void __launch_bounds__(THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmB1,
                const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
                const __grid_constant__ CUtensorMap tmD, const __grid_constant__ CUtensorMap tmD2,
                const __grid_constant__ CUtensorMap tmE, const TcParams p) {
-  // single CTAs size their stages by the B tile they load (a narrow product: 64 or 128 rows instead of 256), so the
-  // same 192 KB ring is 4, 6 or 8 stages deep: the bytes in flight, not the stage count, hide the load latency
-  constexpr int MAX_STAGES = 8;
-  const int STAGE_BYTES = kPair ? PAIR_STAGE_BYTES : A_BYTES + p.n_mma * 128;
+  constexpr int kFullB = kPair ? BN / 2 : BN, kFullStage = A_BYTES + kFullB * 128;
+  const int STAGE_BYTES = kNarrow ? (int)p.stage_bytes : kFullStage;
+  const int STAGES = kNarrow ? p.stages : Mode<kPair, kTf32>::kRingBytes / kFullStage;
+  const int b_rows = kNarrow ? p.b_rows : kFullB;
   constexpr int RING_BYTES = Mode<kPair, kTf32>::kRingBytes, EPI_BUFS = Mode<kPair, kTf32>::kEpiBufs;
-  const int STAGES = RING_BYTES / STAGE_BYTES;
-  constexpr int B_ROWS = Mode<kPair, kTf32>::kBRows, TILE_M = Mode<kPair, kTf32>::kTileM;
+  constexpr int TILE_M = Mode<kPair, kTf32>::kTileM;
+  const int tile_n = kNarrow ? p.n_mma : BN;
   // pair mode: rank of this CTA in its pair; the even CTA (leader) owns the pipeline's full barriers and
   // issues the MMAs, its peer's tile loads signal the leader's barriers
   const uint32_t rank = kPair ? cluster_ctarank() : 0u;
@@ -231,8 +236,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const int row_elems = kTf32 ? 32 : 64;
   const uint32_t mn_block = kTf32 ? 4096u : 8192u;
 
-  if (warp == 0) {
-    // ------------------------------------------------------------------ TMA producer
+  if (warp == 0 || warp == kProducerB) {
+    // ------------------------------------------------------------------ TMA producers: of A, and of B
+    const bool of_a = warp == 0;
     if (lane == 0) {
       int stage = 0;
       uint32_t phase = 0;
@@ -242,7 +248,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const int zc = tile / tiles_per_batch, r = tile % tiles_per_batch;
         const int b = zc % p.batch, split = zc / p.batch;
         // n fastest: a wave shares few A row-panels.  This CTA's rows of A and (pair) its half of B's columns
-        const int m0 = (r / p.n_tiles) * TILE_M + (int)rank * BM, n0 = (r % p.n_tiles) * BN + (int)rank * (BN - B_ROWS);
+        const int m0 = (r / p.n_tiles) * TILE_M + (int)rank * BM, n0 = (r % p.n_tiles) * tile_n + (kPair ? (int)rank * b_rows : 0);
         const int kb_lo = split * p.kb_per_split, kb_hi = min(p.k_blocks, kb_lo + p.kb_per_split);
         for (int seg = 0; seg < p.segs && ok; ++seg) {
           const CUtensorMap* mA = seg == 0 ? &tmA : (seg == 1 ? &tmA1 : &tmA2);
@@ -252,30 +258,33 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             const uint32_t sA = base + stage * STAGE_BYTES, sB = sA + A_BYTES;
             // pair: all four tile loads of a stage (two per CTA) complete on the leader's barrier
             const uint32_t fb = kPair ? map_to_cta(full_bar(stage), 0) : full_bar(stage);
-            if (leader) mbar_expect_tx(full_bar(stage), kPair ? 2 * STAGE_BYTES : A_BYTES + p.n_mma * 128);
-            issued_mask |= 1u << stage;
-            issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
+            if (of_a) {
+              if (leader) mbar_expect_tx(full_bar(stage), kPair ? 2 * STAGE_BYTES : STAGE_BYTES);
+              issued_mask |= 1u << stage;
+              issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
+            }
             if (p.stall) { ok = false; break; }  // self-test: bytes are expected that nobody sends
             const int k0 = kb * row_elems;
             auto load = [&](uint32_t dst, const CUtensorMap* tm, int c0, int c1) {
               if (kPair) tma_load_3d_pair(dst, tm, fb, c0, c1, b);
               else tma_load_3d(dst, tm, fb, c0, c1, b);
             };
-            if (p.a_mn) {
+            if (!of_a) {
+              if (p.b_mn) {
+                for (int i = 0; i * row_elems < b_rows; ++i) load(sB + i * mn_block, mB, n0 + row_elems * i, k0);
+              } else {
+                load(sB, mB, k0, n0);
+              }
+            } else if (p.a_mn) {
               for (int i = 0; i < BM / row_elems; ++i) load(sA + i * mn_block, mA, m0 + row_elems * i, k0);
             } else {
               load(sA, mA, k0, m0);
-            }
-            if (p.b_mn) {
-              for (int i = 0; i < (kPair ? B_ROWS : p.n_mma) / row_elems; ++i) load(sB + i * mn_block, mB, n0 + row_elems * i, k0);
-            } else {
-              load(sB, mB, k0, n0);
             }
             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
           }
         }
       }
-      if (!ok && leader) {
+      if (!ok && leader && of_a) {
         // leave no copy of ours in flight: wait (bounded) for every stage armed last
         for (int s = 0; s < STAGES; ++s)
           if (issued_mask & (1u << s)) {
@@ -296,7 +305,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       const bool issuer = elected != 0;
       const uint32_t fmt = kTf32 ? 2u : 1u;  // operand format: tf32 or bf16
       const uint32_t idesc = (1u << 4) /*fp32 accumulate*/ | (fmt << 7) | (fmt << 10) | ((uint32_t)p.a_mn << 15) |
-                             ((uint32_t)p.b_mn << 16) | ((uint32_t)((kPair ? BN : p.n_mma) >> 3) << 17) | ((uint32_t)(TILE_M >> 4) << 24);
+                             ((uint32_t)p.b_mn << 16) | ((uint32_t)(tile_n >> 3) << 17) | ((uint32_t)(TILE_M >> 4) << 24);
       // one instruction consumes 32 bytes of K: 32 bytes along a K-major row, or 16 rows of an MN-major bf16 block.
       // Descriptors differ between stages and k-steps only in their start address (bits 0..13, in 16-byte units):
       // they are formed once and advanced by adding to the low word.
@@ -369,7 +378,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
       }
     }
-  } else {
+  } else if (warp < kProducerB) {
     // ------------------------------------------------------------------ epilogue
     const int quarter = warp & 3, half = (warp - 2) >> 2, ew = warp - 2;
     const uint32_t buf0 = epi_base + ew * EPI_BUFS * EPI_BUF_BYTES;
@@ -381,8 +390,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const bool staged = p.epi != EPI_RESID;
     const bool has_e = p.epi == EPI_MUL || p.epi == EPI_STORE_LN || p.epi == EPI_ADD;
     const int cw = p.d_f32 ? 32 : 64;      // accumulator columns per staged chunk (128 bytes of output per row)
-    // columns of this warp's half that the MMAs write: a narrow product leaves the rest of the tile out
-    const int my_cols = min(128, max(0, (kPair ? BN : p.n_mma) - half * 128));
+    // columns of this warp's half (the first has the odd 64)
+    const int half_cols = (tile_n + 127) / 128 * 64, my_cols = half ? tile_n - half_cols : half_cols;
     const int nchunks = (my_cols + cw - 1) / cw;
     const uint32_t acce_target[2] = {kPair ? map_to_cta(acce_bar(0), 0) : acce_bar(0),
                                      kPair ? map_to_cta(acce_bar(1), 0) : acce_bar(1)};
@@ -393,8 +402,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     for (int tile = first_tile; tile < p.num_tiles; tile += tile_step) {
       // b indexes the outputs: with split-K it is split * batch + batch entry (partial sums [split][batch][M][N])
       const int b = tile / tiles_per_batch, r = tile % tiles_per_batch;
-      const int m0 = (r / p.n_tiles) * TILE_M + (int)rank * BM, n0 = (r % p.n_tiles) * BN;  // this CTA's 128 rows
-      const int row0 = m0 + quarter * 32, colw = n0 + half * 128;
+      const int m0 = (r / p.n_tiles) * TILE_M + (int)rank * BM, n0 = (r % p.n_tiles) * tile_n;  // this CTA's 128 rows
+      const int row0 = m0 + quarter * 32, colw = n0 + half * half_cols;
       // chunk c of E goes through buffer c % EPI_BUFS, where the result replaces it
       auto load_e = [&](int c) {
         const uint32_t i = c % EPI_BUFS;
@@ -409,8 +418,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       }
       if (!mbar_wait(accf_bar(acc), acc_phase, abort_flag, p.status, p.wait_limit_ns)) break;
       tc_fence_after();
-      const uint32_t tsrc = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN + half * 128);
-      if (nchunks == 0) {  // nothing of a narrow product in this half: only hand the accumulator back
+      const uint32_t tsrc = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN + half * half_cols);
+      if (nchunks == 0) {  // nothing of a narrow tile in this half: only hand the accumulator back
         tc_fence_before();
         __syncwarp();
         if (lane == 0) release_acc(acc);
@@ -478,9 +487,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             }
           }
           if (p.epi == EPI_STORE_LN) {  // one slot of row sums per 64 columns
-            if (row0 + lane < p.M)
-              p.stats[(int64_t)b * p.stats_sb + (int64_t)(row0 + lane) * (4 * p.n_tiles) + 4 * (n0 / BN) + 2 * half + c] =
-                  make_float2(s1, s2);
+            const int slot = colw / 64 + c;
+            if (row0 + lane < p.M && slot < p.slots) p.stats[(int64_t)b * p.stats_sb + (int64_t)(row0 + lane) * p.slots + slot] = make_float2(s1, s2);
             s1 = s2 = 0.0f;
           }
           if (p.d_f32) {
@@ -569,6 +577,28 @@ bool make_map(CUtensorMap* tm, const void* base, int extent_mn, int K, int batch
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Width of the tiles of a product on CTA pairs: 256 columns, or fewer where that fills the pairs better or shortens the last epilogue:
+// one layer's product on 10 row blocks of 256 is 20 tiles of 256 for 74 pairs.  Clocks: a k-block takes some 512 whatever the width
+// (256 columns: its instructions; fewer: copies from L2), an epilogue 8 to 24 per column, under the next tile's products where there is
+// one.  In tiles of 256 / 128 columns: 2664 x 512 x 2048 15.8 / 14.5 us, 2664 x 512 x 1536 13.5 / 12.2, 1000 x 768 x 3072 20.0 / 18.7; but
+// 2664 x 2048 x 512 11.9 / 13.5 and 8192 x 1024 x 4096 48.8 / 79, where there are enough.
+int pair_tile_width(const GemmArgs& g, int k_blocks, int pairs) {
+  const int per_col = g.epi == EPI_GELU_FWD ? 24 : g.epi == EPI_MUL || g.epi == EPI_STORE_LN || g.epi == EPI_ACCUM ? 14 : 8;
+  const int64_t rows = (int64_t)((g.M + 255) / 256) * g.batch;
+  int64_t best = 0;
+  int width = BN;
+  for (int w = BN; w >= 64; w -= 64) {
+    const int64_t waves = (rows * ((g.N + w - 1) / w) + pairs - 1) / pairs;
+    const int64_t products = (int64_t)k_blocks * 512, epilogue = (int64_t)w * per_col;
+    const int64_t cost = waves * (products > epilogue ? products : epilogue) + epilogue + 2000;
+    if (best == 0 || 100 * cost < 93 * best) {
+      best = cost;
+      width = w;
+    }
+  }
+  return width;
+}
+
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 // An operand qualifies if one of its two strides is 1 and the others keep every row 16-byte aligned.
@@ -619,7 +649,7 @@ int sm_count() {
 
 }  // namespace tc
 
-int gemm_tc_stats_slots(int N) { return 4 * ((N + BN - 1) / BN); }
+int gemm_tc_stats_slots(int N) { return (N + 63) / 64; }
 
 bool gemm_tc(Launcher& lc, const GemmArgs& g, int* status_word) {
   if (!status_word) return false;
@@ -671,8 +701,10 @@ bool gemm_tc(Launcher& lc, const GemmArgs& g, int* status_word) {
   // not padding (64-wide recurrent states).  The LayerNorm row sums keep the full tile: their slots are per 64 columns.
   const bool narrow = g.N <= 128 && g.epi != EPI_STORE_LN;
   const bool pair = lc.gemm_pair && sms >= 2 && g.M > BM && !narrow;
-  const int n_mma = !narrow ? BN : (g.N <= 64 ? 64 : 128);
-  const int b_rows = pair ? Mode<true, false>::kBRows : n_mma;
+  const int row_elems = f32 ? 32 : 64;
+  const int k_blocks = (g.K + row_elems - 1) / row_elems;
+  const int n_mma = narrow ? (g.N <= 64 ? 64 : 128) : pair && !f32 ? pair_tile_width(g, k_blocks, sms / 2) : BN;
+  const int b_rows = pair ? n_mma / 2 : n_mma;
   CUtensorMap tmA, tmB;
   if (!make_map(&tmA, A0, g.M, g.K, g.batch, a_sm, a_sk, g.a_sb, a_mn, BM, f32)) return false;
   if (!make_map(&tmB, B0, g.N, g.K, g.batch, b_sn, b_sk, g.b_sb, b_mn, b_rows, f32)) return false;
@@ -687,8 +719,6 @@ bool gemm_tc(Launcher& lc, const GemmArgs& g, int* status_word) {
     tmA1 = a_lo; tmB1 = tmB;     // segment 1: lo x hi
     tmB = b_lo;                  // segment 0: hi x lo (tmA stays A_hi)
   }
-  const int row_elems = f32 ? 32 : 64;
-  const int k_blocks = (g.K + row_elems - 1) / row_elems;
   int splits = g.splitk > 1 ? g.splitk : 1;
   if (splits > k_blocks) splits = k_blocks;
   const int kb_per_split = (k_blocks + splits - 1) / splits;
@@ -710,10 +740,12 @@ bool gemm_tc(Launcher& lc, const GemmArgs& g, int* status_word) {
   static PerDevice<bool> attr_done;  // the shared-memory opt-in is a per-device attribute of the kernel
   bool& attr_set = attr_done.here();
   if (!attr_set) {
-    if (cudaFuncSetAttribute(gemm_tc_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(gemm_tc_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(gemm_tc_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(gemm_tc_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) != cudaSuccess) {
+    bool ok = true;
+    for (auto kernel : {gemm_tc_kernel<false, false, false>, gemm_tc_kernel<false, false, true>, gemm_tc_kernel<false, true, false>,
+                        gemm_tc_kernel<false, true, true>, gemm_tc_kernel<true, false, false>, gemm_tc_kernel<true, false, true>,
+                        gemm_tc_kernel<true, true, false>})
+      ok = ok && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) == cudaSuccess;
+    if (!ok) {
       cudaGetLastError();
       return false;
     }
@@ -722,12 +754,19 @@ bool gemm_tc(Launcher& lc, const GemmArgs& g, int* status_word) {
   TcParams p;
   p.M = g.M; p.N = g.N; p.K = g.K; p.batch = g.batch;
   p.m_tiles = pair ? (g.M + 255) / 256 : (g.M + BM - 1) / BM;
-  p.n_tiles = (g.N + BN - 1) / BN;
+  p.n_tiles = (g.N + n_mma - 1) / n_mma;
   p.num_tiles = p.m_tiles * p.n_tiles * g.batch * splits;
   p.k_blocks = k_blocks;
   p.a_mn = a_mn; p.b_mn = b_mn;
   p.tf32 = f32; p.segs = f32 ? 3 : 1;
   p.n_mma = n_mma;
+  p.b_rows = b_rows;
+  // stages sized by the B tile that a CTA loads (in blocks of 64 columns where it is MN-major): a narrow tile's ring is deeper, as the
+  // bytes in flight, not the stage count, hide the load latency
+  p.stage_bytes = A_BYTES + (b_mn ? (b_rows + 63) / 64 * 64 : b_rows) * 128;
+  const int ring = f32 ? (pair ? Mode<true, true>::kRingBytes : Mode<false, true>::kRingBytes) : (pair ? Mode<true, false>::kRingBytes : Mode<false, false>::kRingBytes);
+  p.stages = ring / (int)p.stage_bytes < MAX_STAGES ? ring / (int)p.stage_bytes : MAX_STAGES;
+  p.slots = gemm_tc_stats_slots(g.N);
   p.splits = splits; p.kb_per_split = kb_per_split;
   p.epi = g.epi; p.d_f32 = out_f32;
   p.D = g.D; p.ldd = g.ldd; p.d_sb = g.d_sb;
@@ -739,15 +778,13 @@ bool gemm_tc(Launcher& lc, const GemmArgs& g, int* status_word) {
   p.status = status_word;
   p.wait_limit_ns = g.wait_limit_ns ? g.wait_limit_ns : WAIT_LIMIT_NS;
   p.stall = g.test_stall;
-  if (pair) {
-    const int pairs = p.num_tiles < sms / 2 ? p.num_tiles : sms / 2;
-    launch_chained(lc, f32 ? gemm_tc_kernel<true, true> : gemm_tc_kernel<true, false>, dim3(2 * pairs), THREADS, SMEM_BYTES, 2, tmA, tmB,
-                   tmA1, tmB1, tmA2, tmB2, tmD, tmD2, tmE, p);
-  } else {
-    const int grid = p.num_tiles < sms ? p.num_tiles : sms;
-    launch_chained(lc, f32 ? gemm_tc_kernel<false, true> : gemm_tc_kernel<false, false>, dim3(grid), THREADS, SMEM_BYTES, 1, tmA, tmB, tmA1,
-                   tmB1, tmA2, tmB2, tmD, tmD2, tmE, p);
-  }
+  const bool full = n_mma == BN;
+  const int workers = pair ? sms / 2 : sms;
+  auto kernel = pair ? (f32 ? gemm_tc_kernel<true, true, false> : full ? gemm_tc_kernel<true, false, false> : gemm_tc_kernel<true, false, true>)
+                     : (f32 ? (full ? gemm_tc_kernel<false, true, false> : gemm_tc_kernel<false, true, true>)
+                            : (full ? gemm_tc_kernel<false, false, false> : gemm_tc_kernel<false, false, true>));
+  launch_chained(lc, kernel, dim3((pair ? 2 : 1) * (p.num_tiles < workers ? p.num_tiles : workers)), THREADS, SMEM_BYTES, pair ? 2 : 1, tmA, tmB,
+                 tmA1, tmB1, tmA2, tmB2, tmD, tmD2, tmE, p);
   if (splits > 1) reduce_splitk(lc, g.partial, (float*)g.D, splits, (int64_t)g.batch * g.M * g.N);
   return true;
 }
