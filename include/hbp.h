@@ -259,10 +259,12 @@ int64_t hbp_launch_count(const hbp_ctx* ctx);
  * launch (clusters of cell_cluster.cu; those of rnn_cluster.cu; clusters of 16 CTAs with four rows each, rnn_persistent.cu)
  * or step by step (counted per step); a float product on the tensor cores, or a product on the CUDA cores.  GEMM_PARTS: those of
  * GEMM_F32 whose operands lie in the workspace already split (gemm_parts.cu); the others split theirs inside the kernel.  GEMM_CELL:
- * all-step products of a float recurrent kind that form their left operand while they load it (gemm_cell.cu). */
+ * all-step products of a float recurrent kind that form their left operand while they load it (gemm_cell.cu).  FEW_ROWS: a forward
+ * pass, or the iterations of a backward pass, of a float MLP stack as one launch (few_rows.cu). */
 typedef enum {
   HBP_FORM_CELL_CLUSTER = 0, HBP_FORM_RNN_CLUSTER = 1, HBP_FORM_RNN_FOUR_ROWS = 2, HBP_FORM_STEP = 3, HBP_FORM_GEMM_F32 = 4,
-  HBP_FORM_GEMM_SIMT = 5, HBP_FORM_GEMM_PARTS = 6, HBP_FORM_GEMM_CELL = 7, HBP_FORM_COUNT = 8
+  HBP_FORM_GEMM_SIMT = 5, HBP_FORM_GEMM_PARTS = 6, HBP_FORM_GEMM_CELL = 7, HBP_FORM_FEW_ROWS = 8,
+  HBP_FORM_COUNT = 9
 } hbp_form;
 int64_t hbp_form_count(const hbp_ctx* ctx, int32_t form);
 

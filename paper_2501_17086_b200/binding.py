@@ -18,7 +18,7 @@ HBP_F32, HBP_BF16 = 0, 1
 BLOCKS = {"mlp": 0, "preln_mlp": 1, "rnn_tanh": 2, "preln_transformer": 3, "gru": 4, "lstm": 5, "relu_mlp": 6, "postln_mlp": 7}
 GATE_ONE, GATE_CHANNEL_SHARED, GATE_CHANNEL_PER_STEP = 0, 1, 2
 LOSS_FINAL, LOSS_EVERY_STEP = 0, 1
-FORMS = ("cell_cluster", "rnn_cluster", "rnn_four_rows", "step", "gemm_f32", "gemm_simt", "gemm_parts", "gemm_cell")
+FORMS = ("cell_cluster", "rnn_cluster", "rnn_four_rows", "step", "gemm_f32", "gemm_simt", "gemm_parts", "gemm_cell", "few_rows")
 
 EXPORTS = ["hbp_workspace_bytes", "hbp_create", "hbp_forward", "hbp_backward", "hbp_exact",
            "hbp_cumsumprod_scratch_bytes", "hbp_cumsumprod", "hbp_cumsumprod_status", "hbp_sync_status", "hbp_launch_count", "hbp_form_count",

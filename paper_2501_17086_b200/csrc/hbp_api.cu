@@ -7,6 +7,7 @@
 #include <new>
 #include <vector>
 
+#include "few_rows.cuh"
 #include "float_parts.cuh"
 #include "hbp_internal.h"
 
@@ -598,6 +599,33 @@ struct Run {
     }
   }
 
+  // ---- float MLP stacks of few rows (few_rows.cu) -------------------------------------------------
+  bool few_rows() const {
+    const hbp_config& f = c->cfg;
+    return f.dtype == HBP_F32 && (f.block == HBP_BLOCK_MLP || f.block == HBP_BLOCK_PRELN_MLP) && !lc.force_simt && lc.gemm_pair && !c->use_parts &&
+           few_rows_take(N, f.d, f.hidden);
+  }
+  FewRows few_rows_args() const {
+    const hbp_config& f = c->cfg;
+    FewRows a;
+    a.L = f.L; a.d = f.d; a.h = f.hidden; a.N = N;
+    a.preln = c->preln; a.eps = f.ln_eps;
+    a.W1 = (const float*)p->W1; a.W2 = (const float*)p->W2; a.a = (const float*)p->a; a.gate = f.gate;
+    a.Y = (float*)c->Y; a.rstd = c->rstd; a.ACT = (float*)c->ACT; a.DACT = (float*)c->DACT;
+    return a;
+  }
+  // All iterations from the initial estimate on; with dz the parameter pass's dZ of all layers as well.
+  bool few_rows_iterations(int iters, bool dz) {
+    if (!few_rows() || shifted || (dz && c->group < c->layers)) return false;
+    FewRows a = few_rows_args();
+    a.k = iters;
+    a.every = c->cfg.loss == HBP_LOSS_EVERY_STEP;
+    a.delta = (const float*)delta;
+    a.g_all = (float*)g;
+    if (dz) a.dZ = (float*)c->H1;
+    return few_rows_backward(lc, a);
+  }
+
   // ---- all-step products of the float recurrent kinds, operands formed while they are loaded (gemm_cell.cu) ----------------
   CellOperand cell_operand() const {
     CellOperand o;
@@ -1144,6 +1172,15 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
   r.x_all = (const char*)x_all;
   char* xa = (char*)x_all;
   const int64_t N = r.N, d = r.d, h = r.h, state = r.state;
+  if (r.few_rows()) {
+    FewRows a = r.few_rows_args();
+    a.x0 = (const float*)x0;
+    a.x_all = (float*)x_all;
+    if (few_rows_forward(r.lc, a)) {
+      ctx->forward_done = true;
+      return r.result();
+    }
+  }
   copy_state(r.lc, f.dtype, xa, x0, state);
   if (ctx->xres) convert_to_f32(r.lc, f.dtype, x0, ctx->xres, state);
 
@@ -1355,13 +1392,28 @@ static hbp_status backward_common(hbp_ctx* ctx, const hbp_params* params, int32_
   const int steps = ctx->steps;
   const bool tr = f.block == HBP_BLOCK_PRELN_TRANSFORMER, rnn = f.block == HBP_BLOCK_RNN_TANH;
   const bool gru = f.block == HBP_BLOCK_GRU;
+  if (!exact) {
+    r.shifted = f.gamma != 0.0f;
+    bool done;
+    {
+      PhaseScope ph(r, HBP_PHASE_VJP);
+      done = r.few_rows_iterations(k < steps ? k : steps, grads != nullptr);
+    }
+    if (done) {
+      if (grads) {
+        PhaseScope ph(r, HBP_PHASE_WGRAD);
+        r.mlp_wgrad(0, ctx->layers, grads);
+        r.gate_grads(grads);
+      }
+      return r.result();
+    }
+  }
   {
     PhaseScope ph(r, HBP_PHASE_OTHER);
     r.set_last_state();
   }
 
   if (!exact) {
-    r.shifted = f.gamma != 0.0f;
     // g^0 = CumSumProd(delta, K) (Eq. 10), then k iterations of {all-step VJP (Eq. 8); reverse scan (Eq. 9, 11)}
     const int iters = k < steps ? k : steps;
     {

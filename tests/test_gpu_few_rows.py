@@ -1,0 +1,52 @@
+"""Float MLP stacks of few rows as one launch a pass: rows that fill a cluster's four in part, hidden units that leave CTAs without any,
+more layers than CTAs, widths at both ends of the rule, every gate and loss."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("block", ["mlp", "preln_mlp"])
+@pytest.mark.parametrize("L,d,h,rows", [(1, 4, 4, 1), (8, 64, 256, 32), (3, 12, 20, 5), (17, 100, 36, 31), (9, 256, 256, 6), (2, 516, 124, 3), (20, 32, 2048, 4)])
+def test_few_rows_match_the_oracle(block, L, d, h, rows):
+    from oracle import run as orun
+    from paper_2501_17086_b200.workloads import Workload, make_inputs
+    from test_gpu_parity import compare, run_gpu
+    w = Workload("t", block, "f32", L=L, d=d, hidden=h, tokens=rows, batch=1, seq=1, seed=9800 + d, loss="final_mse")
+    inp = make_inputs(w, "cuda")
+    gpu = run_gpu(w, inp, (0, 1, 3))
+    assert gpu["ctx"].forms["few_rows"] == 4   # the forward pass and three backward passes
+    compare(w, gpu, orun.run(w, inp, ks=(0, 1, 3), grads_for=("exact", 3)), (0, 1, 3), ("exact", 3))
+
+
+@pytest.mark.parametrize("gate", ["one", "shared", "per_step"])
+@pytest.mark.parametrize("every", [False, True])
+@pytest.mark.parametrize("block,L,d,h,rows", [("mlp", 5, 36, 100, 7), ("preln_mlp", 19, 64, 96, 30)])
+def test_few_rows_agree_with_a_launch_per_product(gate, every, block, L, d, h, rows, monkeypatch):
+    from paper_2501_17086_b200 import binding as B
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(d + rows)
+    rand = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    params = {"W1": rand(L, h, d) / d ** 0.5, "W2": rand(L, d, h) * (0.5 / h ** 0.5)}
+    if gate != "one":
+        params["a"] = 0.7 + 0.3 * torch.rand((d,) if gate == "shared" else (L, d), generator=gen, device="cuda")
+    x0, delta = rand(rows, d), rand(L + 1, rows, d) if every else rand(rows, d)
+    cfg = B.make_config(block, "f32", L, d, rows, hidden=h, gate={"one": B.GATE_ONE, "shared": B.GATE_CHANNEL_SHARED, "per_step": B.GATE_CHANNEL_PER_STEP}[gate],
+                        loss=B.LOSS_EVERY_STEP if every else B.LOSS_FINAL)
+    outs = []
+    for simt in ("0", "1"):
+        monkeypatch.setenv("HBP_FORCE_SIMT", simt)
+        ctx = B.Context(cfg)
+        got = {"x": ctx.forward(params, x0)}
+        for k in (1, 2):
+            grads = ctx.new_grads(with_gate=True)
+            got[k] = ctx.backward(params, k, delta, got["x"], grads=grads)
+            got.update({(k, n): t for n, t in grads.items()})
+        got["without"] = ctx.backward(params, 2, delta, got["x"])   # no parameter gradients asked for
+        ctx.sync_status()
+        assert ctx.forms["few_rows"] == (0 if simt == "1" else 4)
+        outs.append(got)
+    assert torch.equal(outs[0]["without"], outs[0][2])
+    for key, value in outs[0].items():  # each within some 5e-7 of the sums in 64 bits
+        ref = outs[1][key]
+        assert float((value - ref).norm() / ref.norm()) < 2e-6, key
