@@ -19,6 +19,7 @@ struct FewRows {
   bool every = false;  // delta [L+1][N][d], else [N][d]
   const float* delta = nullptr;
   float* g_all = nullptr;
+  bool resident = false;  // (few_rows_backward's: weights and gelu' stay in shared memory)
   float* dZ = nullptr;  // [L][N][h], or null: no parameter gradients follow
 };
 // Whether a stack is one that these serve faster than a launch per product.
@@ -26,5 +27,9 @@ bool few_rows_take(int64_t N, int d, int h);
 // false (of either): nothing was launched (unaligned weights, more layers than fit shared memory, launches in clusters refused).
 bool few_rows_forward(Launcher& lc, const FewRows& a);
 bool few_rows_backward(Launcher& lc, const FewRows& a);
+
+// Parameter gradients from the states g [L+1][N][d], what W1 was applied to y [L][N][d] (16-byte aligned) and the dZ of
+// few_rows_backward; dW1, dW2 of any alignment.
+void few_rows_wgrad(Launcher& lc, const FewRows& a, const float* g, const float* y, float* dW1, float* dW2);
 
 }  // namespace hbp

@@ -1402,7 +1402,9 @@ static hbp_status backward_common(hbp_ctx* ctx, const hbp_params* params, int32_
     if (done) {
       if (grads) {
         PhaseScope ph(r, HBP_PHASE_WGRAD);
-        r.mlp_wgrad(0, ctx->layers, grads);
+        FewRows a = r.few_rows_args();
+        a.dZ = (float*)ctx->H1;
+        few_rows_wgrad(r.lc, a, (const float*)g_all, (const float*)r.mlp_operand(0), grads->dW1, grads->dW2);
         r.gate_grads(grads);
       }
       return r.result();

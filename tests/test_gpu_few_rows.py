@@ -7,7 +7,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("block", ["mlp", "preln_mlp"])
-@pytest.mark.parametrize("L,d,h,rows", [(1, 4, 4, 1), (8, 64, 256, 32), (3, 12, 20, 5), (17, 100, 36, 31), (9, 256, 256, 6), (2, 516, 124, 3), (20, 32, 2048, 4)])
+@pytest.mark.parametrize("L,d,h,rows", [(1, 4, 4, 1), (8, 64, 256, 32), (3, 12, 20, 5), (17, 100, 36, 31), (9, 256, 256, 6), (2, 388, 124, 3), (20, 32, 2048, 4)])
 def test_few_rows_match_the_oracle(block, L, d, h, rows):
     from oracle import run as orun
     from paper_2501_17086_b200.workloads import Workload, make_inputs
