@@ -1,13 +1,13 @@
 // Flash-style causal attention backward on the tensor cores (bf16, head dimension 64).
 //
 // The S x S score matrix is never stored: each CTA recomputes the blocks it needs from Q, K and the
-// forward's log-sum-exp.  Two kernels, so that every output is owned by exactly one CTA (no atomics, runs
-// are bitwise reproducible):
-//   attn_dkv_kernel  one CTA per 128 keys; loops over blocks of 64 queries that can see them:
+// forward's log-sum-exp.  Two kinds of block, so that every output is owned by exactly one CTA (no atomics,
+// runs are bitwise reproducible):
+//   dK, dV           one CTA per 128 keys; loops over blocks of 64 queries that can see them:
 //                       S^T = K Q^T, dP^T = V dO^T            (tcgen05.mma 128x64x16, accumulators in TMEM)
 //                       P^T = exp(S^T/sqrt(dh) - lse), dS^T = P^T * (dP^T - D)   (8 warps, one key row per lane, 32 query columns per thread)
 //                       dV += P^T dO,  dK += dS^T Q           (P^T, dS^T go back through shared memory as bf16)
-//   attn_dq_kernel   one CTA per 128 queries; loops over blocks of 64 keys up to the diagonal:
+//   dQ               one CTA per 128 queries; loops over blocks of 64 keys up to the diagonal:
 //                       S = Q K^T, dP = dO V^T, dS = P * (dP - D),  dQ += dS K
 // with D_i = sum(dO_i * O_i).  All tiles are moved by TMA (128-byte swizzle); the same shared-memory tile
 // serves as a K-major operand (contraction over the head dimension) and as an MN-major operand (contraction
@@ -79,11 +79,9 @@ __device__ __forceinline__ uint64_t desc_add(uint64_t d, uint32_t bytes) { retur
 __device__ __forceinline__ uint32_t bar_at(uint32_t bars, int i) { return bars + 8u * i; }
 
 template <bool kDKV>
-__global__ void __launch_bounds__(THREADS, 2)
-attn_bwd_tc_kernel(const __grid_constant__ CUtensorMap tmBig0, const __grid_constant__ CUtensorMap tmBig1,
-                   const __grid_constant__ CUtensorMap tmSmall0, const __grid_constant__ CUtensorMap tmSmall1,
-                   const __grid_constant__ CUtensorMap tmOut0, const __grid_constant__ CUtensorMap tmOut1,
-                   const AttnTcParams p) {
+__device__ __forceinline__ void attn_bwd_body(const CUtensorMap& tmBig0, const CUtensorMap& tmBig1, const CUtensorMap& tmSmall0,
+                                              const CUtensorMap& tmSmall1, const CUtensorMap& tmOut0, const CUtensorMap& tmOut1, const AttnTcParams& p,
+                                              const int blk, const int h, const int b) {
   // kDKV: big tiles = K, V (rows = keys), small tiles = Q, dO (rows = queries), outputs dK (Out0), dV (Out1).
   // else: big tiles = Q, dO (rows = queries), small tiles = K, V (rows = keys), output dQ (Out0).
   extern __shared__ uint8_t smem_raw[];
@@ -105,7 +103,6 @@ attn_bwd_tc_kernel(const __grid_constant__ CUtensorMap tmBig0, const __grid_cons
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int blk = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
   const int big0 = blk * BIG;  // first key (dkv) or first query (dq) of this CTA
   // inner blocks: dkv: queries from big0 on; dq: keys up to the last query of the block
   const int n_small = (p.S + SMALL - 1) / SMALL;
@@ -138,6 +135,8 @@ attn_bwd_tc_kernel(const __grid_constant__ CUtensorMap tmBig0, const __grid_cons
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  chain_next();
+  chain_wait();
   const uint32_t tmem = *tmem_slot;
   // TMEM columns: scores [0,64), dP [64,128), accumulator 0 [128,192), accumulator 1 [192,256)
   const uint32_t tS = tmem, tDP = tmem + 64, tAcc0 = tmem + 128, tAcc1 = tmem + 192;
@@ -351,6 +350,20 @@ attn_bwd_tc_kernel(const __grid_constant__ CUtensorMap tmBig0, const __grid_cons
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
   }
+}
+
+// Both in one launch, the dK/dV blocks first (they have a product more): the dQ blocks fill the SMs that these leave.  A launch each
+// before, plainly one after the other: 64 (batch entry, head) pairs of 333 rows 15.5 + 10.2 us and two gaps of 2 -> 18; exact pass of 2
+// layers, 24 pairs of 1024 rows, 272 -> 224, 96 pairs 574 -> 525; 768 pairs of 1024 rows 642 -> 641.  (Loading the first tiles before
+// the tensor memory is there made blocks of large batches a quarter slower.)
+__global__ void __launch_bounds__(THREADS, 2)
+attn_bwd_tc_kernel(const __grid_constant__ CUtensorMap kB, const __grid_constant__ CUtensorMap vB, const __grid_constant__ CUtensorMap qS,
+                   const __grid_constant__ CUtensorMap oS, const __grid_constant__ CUtensorMap dK, const __grid_constant__ CUtensorMap dV,
+                   const __grid_constant__ CUtensorMap qB, const __grid_constant__ CUtensorMap oB, const __grid_constant__ CUtensorMap kS,
+                   const __grid_constant__ CUtensorMap vS, const __grid_constant__ CUtensorMap dQ, const AttnTcParams p) {
+  const int blocks = (p.S + BIG - 1) / BIG, blk = (int)(blockIdx.x % blocks), pairs = p.B * p.H, pair = (int)(blockIdx.x / blocks);
+  if (pair < pairs) attn_bwd_body<true>(kB, vB, qS, oS, dK, dV, p, blk, pair % p.H, pair / p.H);
+  else attn_bwd_body<false>(qB, oB, kS, vS, dQ, dQ, p, blocks - 1 - blk, (pair - pairs) % p.H, (pair - pairs) / p.H);  // (the long ones first here too)
 }
 
 // ------------------------------------------------------------------------------------------- forward
@@ -612,8 +625,7 @@ bool attention_bwd_tc(Launcher& lc, const AttnArgs& a, int* status_word) {
   static PerDevice<bool> attr_done;  // per-device kernel attribute
   bool& attr_set = attr_done.here();
   if (!attr_set) {
-    if (cudaFuncSetAttribute(attn_bwd_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) != cudaSuccess ||
-        cudaFuncSetAttribute(attn_bwd_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) != cudaSuccess) {
+    if (cudaFuncSetAttribute(attn_bwd_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) != cudaSuccess) {
       cudaGetLastError();
       return false;
     }
@@ -631,13 +643,9 @@ bool attention_bwd_tc(Launcher& lc, const AttnArgs& a, int* status_word) {
   }
   p.scale = 1.0f / sqrtf((float)DH);
   p.status = status_word;
-  dim3 grid((a.seq + BIG - 1) / BIG, a.heads, a.batch);
-  // dK, dV: big tiles K, V; small tiles Q, dO
-  attn_bwd_tc_kernel<true><<<grid, THREADS, SMEM_BYTES, lc.stream>>>(kB, vB, qS, oS, dk, dv, p);
-  // dQ: big tiles Q, dO; small tiles K, V
-  attn_bwd_tc_kernel<false><<<grid, THREADS, SMEM_BYTES, lc.stream>>>(qB, oB, kS, vS, dq, dq, p);
-  lc.count(2);
-  lc.check();
+  const int64_t grid = 2 * (int64_t)((a.seq + BIG - 1) / BIG) * a.heads * a.batch;
+  if (grid > INT32_MAX) return false;
+  launch_chained(lc, attn_bwd_tc_kernel, dim3((unsigned)grid), THREADS, SMEM_BYTES, 1, kB, vB, qS, oS, dk, dv, qB, oB, kS, vS, dq, p);
   return true;
 }
 
@@ -669,6 +677,8 @@ bool attention_fwd_tc(Launcher& lc, const AttnArgs& a, int* status_word) {
   p.scale = 1.0f / sqrtf((float)DH);
   p.status = status_word;
   dim3 grid((a.seq + BIG - 1) / BIG, a.heads, a.batch);
+  // (not chained to the product before: its blocks would gather three to an SM on the first SMs that come free, forward pass of 2 layers, 16
+  // heads of 2000 rows, 460 -> 504 us)
   attn_fwd_tc_kernel<<<grid, THREADS, FWD_SMEM_BYTES, lc.stream>>>(q, k, v, o, a.lse, p);
   lc.count();
   lc.check();
