@@ -788,13 +788,11 @@ __global__ void __launch_bounds__(256) reduce_both_kernel(const float* __restric
                                                           int M, int d, int in, int gru) {
   chain_next();
   chain_wait();
-  const int64_t elems = (int64_t)M * (d + in), i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= elems) return;
+  const int64_t elems = (int64_t)M * (d + in), i = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
+  const double s = reduce_eighths(partial + i, i < elems, splits, elems);
+  if (threadIdx.x >= 32 || i >= elems) return;
   const int m = (int)(i / (d + in)), n = (int)(i % (d + in)), q = m / d;
   if (gru && q == (n < d ? 3 : 2)) return;
-  double s = 0.0;
-#pragma unroll 8
-  for (int k = 0; k < splits; ++k) s += (double)partial[k * elems + i];
   if (n < d) dW[(int64_t)m * d + n] = (float)s;
   else dU[(int64_t)(gru && q == 3 ? m - d : m) * in + n - d] = (float)s;
 }
@@ -870,14 +868,14 @@ bool cell_wgrad(Launcher& lc, int kind, const CellOperand& o, const float* H, in
   }
   if (o.rows > (int64_t)1 << 30) return false;
   p.k_blocks = (int)((o.rows + BK - 1) / BK);
-  // As many splits of the rows as give the shortest longest queue of a CTA pair, four k-blocks at least in each (of equal ones the
-  // fewest: every split is a set of partial sums).  A wide tile costs more than a narrow one only where the tensor core bounds it.
+  // As many splits of the rows as give the shortest longest queue of a CTA pair, four k-blocks at least in each (of those within
+  // 5 % the fewest: every split is a set of partial sums).  A wide tile costs more than a narrow one only where the tensor core bounds it.
   const int64_t outputs = (int64_t)p.M * (o.d + in);
   const int pairs = sm_count() / 2;
   int64_t best = 0;
   for (int s = 1; s <= pairs && s * outputs <= (int64_t)partial_floats && (s == 1 || s * 4 <= p.k_blocks); ++s) {
     const int64_t per = (p.k_blocks + s - 1) / s, cost = ((int64_t)p.tiles * s + pairs - 1) / pairs * (per + 4);
-    if (best == 0 || cost < best) {
+    if (best == 0 || 100 * cost < 95 * best) {
       best = cost;
       p.splits = s;
     }
@@ -889,7 +887,7 @@ bool cell_wgrad(Launcher& lc, int kind, const CellOperand& o, const float* H, in
   if (!make_map_epi(&tmD0, partial, true, p.M, n0, p.splits, n0, (int64_t)p.M * n0)) return false;
   if (p.both) {
     if (!launch_kind<true>(lc, p.tiles * p.splits, tmD0, tmD0, tmD0, tmD0, p)) return false;
-    launch_chained(lc, reduce_both_kernel, dim3((unsigned)((outputs + 255) / 256)), 256, 0, 1, (const float*)partial, dW, dU, p.splits, p.M, o.d, in,
+    launch_chained(lc, reduce_both_kernel, dim3((unsigned)((outputs + 31) / 32)), 256, 0, 1, (const float*)partial, dW, dU, p.splits, p.M, o.d, in,
                    (int)(kind == HBP_BLOCK_GRU));
     return true;
   }

@@ -105,7 +105,7 @@ struct hbp_ctx {
 namespace {
 
 constexpr size_t kAlign = 256;
-constexpr int kGateBlocks = 256;
+constexpr int kGateBlocks = 592;
 constexpr int kMaxSplit = 256;
 
 inline size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }

@@ -343,6 +343,24 @@ bool attention_bwd_tc(Launcher& lc, const AttnArgs& a, int* status_word);
 bool attention_fwd_tc(Launcher& lc, const AttnArgs& a, int* status_word);
 
 // ---------------------------------------------------------------- device math
+// Sum over `splits` partial sums, `stride` apart from p on, of one element per lane of a block of 256: each warp adds an eighth of them
+// in double, the first one the eighths (all in fixed order).  The sum is that warp's.  From kManySplits on this is faster than a thread
+// for each element.
+constexpr int kManySplits = 16;
+__device__ __forceinline__ double reduce_eighths(const float* __restrict__ p, bool in, int splits, int64_t stride) {
+  __shared__ double eighths[8][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, per = (splits + 7) / 8, end = min(splits, (warp + 1) * per);
+  double s = 0.0;
+  if (in) {
+#pragma unroll 8
+    for (int k = warp * per; k < end; ++k) s += (double)p[k * stride];
+  }
+  eighths[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0)
+    for (int w = 1; w < 8; ++w) s += eighths[w][lane];
+  return s;
+}
 __device__ __forceinline__ float gelu_f(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752440f)); }
 __device__ __forceinline__ float gelu_prime_f(float z) {
   return 0.5f * (1.0f + erff(z * 0.70710678118654752440f)) + z * expf(-0.5f * z * z) * 0.39894228040143267794f;

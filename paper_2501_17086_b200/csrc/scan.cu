@@ -589,24 +589,62 @@ __global__ void __launch_bounds__(1024) postln_prepass_kernel(const T* __restric
 template <typename T>
 __global__ void __launch_bounds__(256) gate_grad_kernel(const T* __restrict__ g, const T* __restrict__ x,
                                                         int64_t rows, int d, float* __restrict__ partial) {
+  constexpr int V = Vec<T>::N;
+  __shared__ float red[256 * V];
   const int64_t per = (rows + gridDim.x - 1) / gridDim.x;
   const int64_t r0 = (int64_t)blockIdx.x * per, r1 = min(rows, r0 + per);
-  for (int c = threadIdx.x; c < d; c += blockDim.x) {
-    // four running sums over interleaved rows: eight loads in flight per thread instead of two, fixed order
-    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    int64_t r = r0;
-    for (; r + 4 <= r1; r += 4) {
-      float gv[4], xv[4];
+  // 16 bytes per load; where a row has fewer of them than the block threads, several rows at a time
+  const int vecs = d / V, cols = min(vecs, 256), groups = 256 / cols, group = threadIdx.x / cols, col = threadIdx.x % cols;
+  for (int c0 = 0; c0 < vecs; c0 += cols) {
+    const int c = (c0 + col) * V;
+    float sum[V];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        gv[i] = to_f(g[(r + i) * d + c]);
-        xv[i] = to_f(x[(r + i) * d + c]);
+    for (int i = 0; i < V; ++i) sum[i] = 0.0f;
+    if (group < groups && c < d) {
+      // four running sums over interleaved rows: eight loads in flight per thread, fixed order
+      float acc[4][V];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int i = 0; i < V; ++i) acc[k][i] = 0.0f;
+      int64_t r = r0 + group;
+      for (; r + 3 * groups < r1; r += 4 * groups) {
+        Vec<T> gv[4], xv[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          gv[k] = ldv_stream<T>(g + (r + k * groups) * d + c);
+          xv[k] = ldv_stream<T>(x + (r + k * groups) * d + c);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          float a[V], b[V];
+          gv[k].get(a);
+          xv[k].get(b);
+#pragma unroll
+          for (int i = 0; i < V; ++i) acc[k][i] = fmaf(a[i], b[i], acc[k][i]);
+        }
+      }
+      for (; r < r1; r += groups) {
+        float a[V], b[V];
+        ldv_stream<T>(g + r * d + c).get(a);
+        ldv_stream<T>(x + r * d + c).get(b);
+#pragma unroll
+        for (int i = 0; i < V; ++i) acc[0][i] = fmaf(a[i], b[i], acc[0][i]);
       }
 #pragma unroll
-      for (int i = 0; i < 4; ++i) acc[i] = fmaf(gv[i], xv[i], acc[i]);
+      for (int i = 0; i < V; ++i) sum[i] = (acc[0][i] + acc[1][i]) + (acc[2][i] + acc[3][i]);
     }
-    for (; r < r1; ++r) acc[0] = fmaf(to_f(g[r * d + c]), to_f(x[r * d + c]), acc[0]);
-    partial[(int64_t)blockIdx.x * d + c] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+#pragma unroll
+    for (int i = 0; i < V; ++i) red[threadIdx.x * V + i] = sum[i];
+    __syncthreads();
+    if (group == 0 && c < d)
+#pragma unroll
+      for (int i = 0; i < V; ++i) {
+        float s = sum[i];
+        for (int q = 1; q < groups; ++q) s += red[(q * cols + col) * V + i];
+        partial[(int64_t)blockIdx.x * d + c + i] = s;
+      }
+    __syncthreads();
   }
 }
 
