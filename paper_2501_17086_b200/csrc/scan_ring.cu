@@ -1,6 +1,6 @@
-// Reverse scan over time for problems with few channels (Eq. 9 / Eq. 12 with diagonal K; the recurrent
-// workloads: hundreds to thousands of steps, 10^4..10^5 channels).  There are too few independent recurrences
-// to hide memory latency with threads, so each block hides it with a deep ring of TMA loads instead: a block
+// Reverse scan over time (Eq. 9 / Eq. 12 with diagonal K), from 32 steps on.  Made for few channels (the recurrent workloads: hundreds to
+// thousands of steps, 10^4..10^5 channels), where there are too few independent recurrences to hide memory latency with threads: each
+// block hides it with a deep ring of TMA loads instead, which is as good for many channels (scan_reverse has the times): a block
 // owns 512 bytes of channels (128 floats / 256 bf16) and walks all steps serially, one 32-bit word of channels
 // per lane; a producer warp keeps the ring of {8..64 steps x 512 bytes} boxes full per input stream (u, a
 // separately given delta, an element-wise gate), and four consumer warps - one per scheduler, so that the
@@ -89,13 +89,15 @@ struct RingMaps {
 // g_l * coef_{l-1}, split into its two tf32 terms: the operand never makes a round trip through g.  Four further
 // warps - again one per scheduler - turn a stage the consumers have finished into operand rows, in place over g_l
 // and the coefficients; g itself is then stored only on request (by the consumers' own stores).
-template <typename T, int NS, bool kElemGate, bool kOp>
+// kWideSum: two float streams are added up in double, as the serial scan of short sequences does (scan.cu).
+template <typename T, int NS, bool kElemGate, bool kOp, bool kWideSum>
 __global__ void __launch_bounds__((kConsumerWarps * (kOp ? 2 : 1) + 1) * 32) scan_ring_kernel(const ScanArgs s,
                                                                                             const __grid_constant__ RingMaps m,
                                                                                             int nstages, int rows_ps) {
   typedef typename RingAcc<T>::type A;
   constexpr int EPT = 4 / (int)sizeof(T);  // channels per lane: one 32-bit word
   static_assert(!kOp || EPT == 1, "the operand by-product is a float path");
+  static_assert(!kWideSum || (EPT == 1 && NS == 2), "two float streams");
   constexpr int STREAMS = NS + (kElemGate ? 1 : 0) + (kOp ? 1 : 0);
   constexpr int OP_STREAM = STREAMS - 1;
   const int kRows = rows_ps;                       // steps per ring stage
@@ -285,10 +287,15 @@ __global__ void __launch_bounds__((kConsumerWarps * (kOp ? 2 : 1) + 1) * 32) sca
       if (NS >= 2) {
         unpack_word<T>(w[NS - 1][r], t);
 #pragma unroll
-        for (int e = 0; e < EPT; ++e) f[e] += t[e];
+        for (int e = 0; e < EPT && !kWideSum; ++e) f[e] += t[e];
       }
 #pragma unroll
       for (int e = 0; e < EPT; ++e) widen(f[e], uu[r][e]);
+      if (kWideSum) {
+        A more;
+        widen(t[0], more);
+        uu[r][0] += more;
+      }
     }
     if (kElemGate) {
       unpack_word<T>(w[RAW - 1][r], f);
@@ -397,27 +404,34 @@ bool make_map2(CUtensorMap* tm, const void* base, bool f32, int64_t steps, int64
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <typename T, int NS, bool kElemGate, bool kOp>
+template <typename T, int NS, bool kElemGate, bool kOp, bool kWideSum = false>
 void launch_ring(Launcher& lc, const ScanArgs& s, const RingMaps& m, unsigned grid, int nstages, int rows_ps, size_t smem) {
   static PerDevice<size_t> configured_on;  // per-device kernel attribute
   size_t& configured = configured_on.here();
   if (smem > configured) {
-    cudaFuncSetAttribute(scan_ring_kernel<T, NS, kElemGate, kOp>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(scan_ring_kernel<T, NS, kElemGate, kOp, kWideSum>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     configured = smem;
   }
-  scan_ring_kernel<T, NS, kElemGate, kOp>
+  scan_ring_kernel<T, NS, kElemGate, kOp, kWideSum>
       <<<grid, (kConsumerWarps * (kOp ? 2 : 1) + 1) * 32, smem, lc.stream>>>(s, m, nstages, rows_ps);
   lc.count();
   lc.check();
 }
 
 template <typename T>
-void dispatch_ring(Launcher& lc, const ScanArgs& s, int ns, bool eg, bool op, const RingMaps& m, unsigned grid, int nstages,
+void dispatch_ring(Launcher& lc, const ScanArgs& s, int ns, bool eg, bool op, bool wide_sum, const RingMaps& m, unsigned grid, int nstages,
                    int rows_ps, size_t smem) {
   if constexpr (std::is_same<T, float>::value) {
     if (op) {  // never together with an element gate (see scan_ring)
       if (ns == 1) launch_ring<T, 1, false, true>(lc, s, m, grid, nstages, rows_ps, smem);
       else launch_ring<T, 2, false, true>(lc, s, m, grid, nstages, rows_ps, smem);
+      return;
+    }
+  }
+  if constexpr (std::is_same<T, float>::value) {
+    if (ns == 2 && wide_sum) {
+      if (eg) launch_ring<T, 2, true, false, true>(lc, s, m, grid, nstages, rows_ps, smem);
+      else launch_ring<T, 2, false, false, true>(lc, s, m, grid, nstages, rows_ps, smem);
       return;
     }
   }
@@ -433,7 +447,7 @@ void dispatch_ring(Launcher& lc, const ScanArgs& s, int ns, bool eg, bool op, co
 
 }  // namespace
 
-bool scan_ring(Launcher& lc, const ScanArgs& s) {
+bool scan_ring(Launcher& lc, const ScanArgs& s, bool wide_sum) {
   if (s.xhat || s.keep != 1.0f || s.gamma != 0.0f) return false;
   if (s.gate == HBP_GATE_CHANNEL_PER_STEP && s.a) return false;  // a small [steps][d] table: not a stream of this shape
   const bool f32 = s.dtype == HBP_F32;
@@ -486,8 +500,8 @@ bool scan_ring(Launcher& lc, const ScanArgs& s) {
     return false;
   if (!op) m.oh = m.ol = m.og;
   const size_t smem = (size_t)nstages * nstreams * rows_ps * kRowBytes + (size_t)nstages * (op ? 16 + 8 * kConsumerWarps : 16) + 16 + 128;
-  if (f32) dispatch_ring<float>(lc, s, ns, eg, op, m, grid, nstages, rows_ps, smem);
-  else dispatch_ring<bf16>(lc, s, ns, eg, false, m, grid, nstages, rows_ps, smem);
+  if (f32) dispatch_ring<float>(lc, s, ns, eg, op, wide_sum, m, grid, nstages, rows_ps, smem);
+  else dispatch_ring<bf16>(lc, s, ns, eg, false, false, m, grid, nstages, rows_ps, smem);
   if (op && s.op_done) *s.op_done = true;
   return true;
 }
