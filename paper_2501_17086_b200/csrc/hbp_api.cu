@@ -904,10 +904,16 @@ struct Run {
 
   // Reverse scan over steps [lo, hi) that adds the block VJPs in U (finishing LayerNorm-backward on the way).
   void scan_with_u(int lo, int hi) {
-    if (c->preln && c->lnpart && stats_ok)
+    const bool sums = c->preln && c->lnpart && stats_ok, alone = sums && hi - lo == 1 && !shifted;
+    if (sums && !alone)
       ln_stats_finish(lc, c->lnpart + (int64_t)lo * N * c->ln_slots, c->ln_slots, c->rstd + (int64_t)lo * N,
                       c->lnstat + (int64_t)lo * N, (int64_t)(hi - lo) * N, (int)d);
-    scan_reverse(lc, scan_args(lo, hi, true));
+    ScanArgs s = scan_args(lo, hi, true);
+    if (alone) {
+      s.lnpart = c->lnpart;
+      s.ln_slots = c->ln_slots;
+    }
+    scan_reverse(lc, s);
     stats_ok = true;
   }
   ScanArgs scan_args(int lo, int hi, bool with_u) const {

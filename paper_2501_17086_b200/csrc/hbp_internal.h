@@ -181,6 +181,9 @@ struct ScanArgs {
   // If set, [L][rows] of {rstd, mean(dy), mean(dy*xhat), 0} prepared by ln_stats_finish: the kernel then
   // needs no reduction of its own and streams like the plain scan.
   const float4* lnstat = nullptr;
+  // If set (bf16, one step, no shifted split): the partial sums [L][rows][ln_slots] that lnstat is made from; the kernel makes it itself.
+  const float2* lnpart = nullptr;
+  int ln_slots = 0;
   void* scratch = nullptr;  // time-chunked variant only
   size_t scratch_bytes = 0;
   int* status = nullptr;  // device status word for bounded waits (may be null)

@@ -228,6 +228,64 @@ __global__ void __launch_bounds__(256) scan_depth_lnstat_kernel(const ScanArgs s
   }
 }
 
+// One step of it (the exact pass goes step by step), with the row statistics formed here from the GEMM's partial sums, in ln_stats_finish's
+// order, while the step's operands are on their way: a launch of 2 us less in a chain of 10 a layer.
+__global__ void __launch_bounds__(256) scan_one_lnstat_kernel(const ScanArgs s) {
+  chain_next();
+  chain_wait();
+  constexpr int V = Vec<bf16>::N;
+  __shared__ float4 stat[256 + 2];  // of the rows that the block's groups of channels lie in (d is a multiple of V)
+  const int l = s.l_lo;
+  const int64_t state_elems = s.rows * s.d, off = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * V;
+  const bool in = off < state_elems;
+  const int64_t row = off / s.d, row0 = (int64_t)blockIdx.x * blockDim.x * V / s.d;
+  const int ch = (int)(off - row * s.d);
+  const int64_t at = (int64_t)l * state_elems + off;
+  bf16* g = (bf16*)s.g;
+  Vec<bf16> carry, dy, xh, gate, delta;
+  const bf16 *gp = gate_at<bf16>(s, l, state_elems, off, ch), *dp = delta_at<bf16>(s, l, state_elems);
+  if (in) {
+    carry = ldv<bf16>(g + at + state_elems);
+    dy = ldv_stream<bf16>((const bf16*)s.u + at);
+    xh = ldv_stream<bf16>((const bf16*)s.xhat + at);
+    if (gp) gate = ldv<bf16>(gp);
+    if (dp) delta = ldv_stream<bf16>(dp + off);
+  }
+  const int64_t last = min(s.rows - 1, (((int64_t)blockIdx.x + 1) * blockDim.x * V - 1) / s.d);
+  for (int r = threadIdx.x; r <= (int)(last - row0); r += blockDim.x) {
+    const float2* part = s.lnpart + ((int64_t)l * s.rows + row0 + r) * s.ln_slots;
+    float s1 = 0.0f, s2 = 0.0f;
+#pragma unroll 8
+    for (int k = 0; k < s.ln_slots; ++k) {
+      const float2 t = part[k];
+      s1 += t.x;
+      s2 += t.y;
+    }
+    const float inv_d = 1.0f / (float)s.d;
+    stat[r] = make_float4(s.rstd[(int64_t)l * s.rows + row0 + r], s1 * inv_d, s2 * inv_d, 0.0f);
+  }
+  __syncthreads();
+  if (!in) return;
+  const float4 st = stat[row - row0];
+  float c[V], y[V], x[V], val[V], more[V];
+  carry.get(c);
+  dy.get(y);
+  xh.get(x);
+  if (gp) gate.get(more);
+#pragma unroll
+  for (int i = 0; i < V; ++i) val[i] = (gp ? more[i] : s.keep) * c[i];
+#pragma unroll
+  for (int i = 0; i < V; ++i) val[i] += st.x * (y[i] - st.y - x[i] * st.z);
+  if (dp) {
+    delta.get(more);
+#pragma unroll
+    for (int i = 0; i < V; ++i) val[i] += more[i];
+  }
+  Vec<bf16> out;
+  out.set(val);
+  stv<bf16>(g + at, out);
+}
+
 __global__ void ln_stats_finish_kernel(const float2* __restrict__ stats, int slots, const float* __restrict__ rstd,
                                        float4* __restrict__ lnstat, int64_t count, float inv_d) {
   chain_next();
@@ -704,6 +762,10 @@ void scan_reverse(Launcher& lc, const ScanArgs& s) {
   if (s.l_hi <= s.l_lo || s.rows <= 0) return;
   const int V = s.dtype == HBP_F32 ? 4 : 8;
   const int64_t nvec = s.rows * s.d / V;
+  if (s.xhat && s.lnpart) {
+    launch_chained(lc, scan_one_lnstat_kernel, dim3((unsigned)((nvec + 255) / 256)), 256, 0, 1, s);
+    return;
+  }
   if (s.xhat && s.lnstat) {
     const unsigned grid = (unsigned)((nvec + 255) / 256);
     const bool shift = s.gamma != 0.0f;
