@@ -33,21 +33,21 @@ constexpr int A_BYTES = BM * BK * 2;
 // CTA pair (two CTAs of a cluster on one 256 x 256 tile, tcgen05 cta_group::2): each CTA stages its own 128 rows of A
 // and its own 128 of the 256 columns of B, so a stage is 32 KB instead of 48 KB for the same flops per SM: five stages
 // and two staging buffers per epilogue warp fit (six stages and one buffer: the same main loop, 16384 x 8192 x 2048 x 4
-// 1115 -> 1174 TFLOP/s, but an epilogue that waits for each of its copies).  Single CTAs and float operands, whose main loop
-// moves three times the bytes per flop and whose epilogue only stores, keep the deeper ring.
+// 1115 -> 1174 TFLOP/s, but an epilogue that waits for each of its copies).  Float operands run on single CTAs only: the float
+// products of 32 units and more that pairs would take are the bf16 kernels' (gemm_parts.cu, gemm_cell.cu).
 constexpr int PAIR_STAGE_BYTES = A_BYTES + 128 * BK * 2;
-template <bool kPair, bool kTf32>
+template <bool kPair>
 struct Mode {
   static constexpr int kTileM = kPair ? 256 : 128;
-  static constexpr int kEpiBufs = kPair && !kTf32 ? 2 : 1;  // staging buffers per epilogue warp
+  static constexpr int kEpiBufs = kPair ? 2 : 1;  // staging buffers per epilogue warp
   static constexpr int kRingBytes = (kEpiBufs == 2 ? 5 : 6) * PAIR_STAGE_BYTES;  // single CTAs: 4, 6 or 8 stages
 };
 constexpr int MAX_STAGES = 8;
 constexpr int EPI_WARPS = 8, kProducerB = 2 + EPI_WARPS, THREADS = 64 + 32 * EPI_WARPS + 64;
 constexpr uint32_t TMEM_COLS = 512;
 constexpr int EPI_BUF_BYTES = 4096;  // 32 rows x 128 bytes
-constexpr int SMEM_BYTES = Mode<true, false>::kRingBytes + 2 * EPI_WARPS * EPI_BUF_BYTES + 1024 /*alignment slack*/ + 512 /*barriers*/;
-static_assert(Mode<false, false>::kRingBytes + EPI_WARPS * EPI_BUF_BYTES == Mode<true, false>::kRingBytes + 2 * EPI_WARPS * EPI_BUF_BYTES, "one size");
+constexpr int SMEM_BYTES = Mode<true>::kRingBytes + 2 * EPI_WARPS * EPI_BUF_BYTES + 1024 /*alignment slack*/ + 512 /*barriers*/;
+static_assert(Mode<false>::kRingBytes + EPI_WARPS * EPI_BUF_BYTES == Mode<true>::kRingBytes + 2 * EPI_WARPS * EPI_BUF_BYTES, "one size");
 
 struct TcParams {
   int M, N, K, batch;
@@ -165,10 +165,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                const __grid_constant__ CUtensorMap tmE, const TcParams p) {
   constexpr int kFullB = kPair ? BN / 2 : BN, kFullStage = A_BYTES + kFullB * 128;
   const int STAGE_BYTES = kNarrow ? (int)p.stage_bytes : kFullStage;
-  const int STAGES = kNarrow ? p.stages : Mode<kPair, kTf32>::kRingBytes / kFullStage;
+  const int STAGES = kNarrow ? p.stages : Mode<kPair>::kRingBytes / kFullStage;
   const int b_rows = kNarrow ? p.b_rows : kFullB;
-  constexpr int RING_BYTES = Mode<kPair, kTf32>::kRingBytes, EPI_BUFS = Mode<kPair, kTf32>::kEpiBufs;
-  constexpr int TILE_M = Mode<kPair, kTf32>::kTileM;
+  constexpr int RING_BYTES = Mode<kPair>::kRingBytes, EPI_BUFS = Mode<kPair>::kEpiBufs;
+  constexpr int TILE_M = Mode<kPair>::kTileM;
   const int tile_n = kNarrow ? p.n_mma : BN;
   // pair mode: rank of this CTA in its pair; the even CTA (leader) owns the pipeline's full barriers and
   // issues the MMAs, its peer's tile loads signal the leader's barriers
@@ -343,13 +343,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             for (int k = 0; k < 4; ++k) {
               const uint64_t adk = ad + (uint64_t)(k * a_step16), bdk = bd + (uint64_t)(k * b_step16);
               const uint32_t acc_k = k == 0 ? accum : 1u;
-              if (kPair) {
-                if (kTf32) tc_mma_tf32_pair(tmem_d, adk, bdk, idesc, acc_k);
-                else tc_mma_pair(tmem_d, adk, bdk, idesc, acc_k);
-              } else {
-                if (kTf32) tc_mma_tf32(tmem_d, adk, bdk, idesc, acc_k);
-                else tc_mma(tmem_d, adk, bdk, idesc, acc_k);
-              }
+              if (kPair) tc_mma_pair(tmem_d, adk, bdk, idesc, acc_k);
+              else if (kTf32) tc_mma_tf32(tmem_d, adk, bdk, idesc, acc_k);
+              else tc_mma(tmem_d, adk, bdk, idesc, acc_k);
             }
             // frees the stage (in both CTAs of a pair) once these MMAs have read it
             if (kPair) tc_commit_pair(empty_bar(stage));
@@ -697,16 +693,16 @@ bool gemm_tc(Launcher& lc, const GemmArgs& g, int* status_word) {
   if (g.epi == EPI_RESID && !g.R && !g.E) return false;
 
   // CTA pairs wherever there are at least two 128-row blocks (unless the context asks for single CTAs): a stage is
-  // 32 KB instead of 48 KB for the same flops per SM: five stages beside two staging buffers per epilogue warp (float operands
-  // six and one) where single CTAs have four, and a third less is drawn from L2
+  // 32 KB instead of 48 KB for the same flops per SM: five stages beside two staging buffers per epilogue warp where single
+  // CTAs have four, and a third less is drawn from L2
   const int sms = sm_count();
   // A product at most 128 columns wide runs on single CTAs with MMAs of 64 or 128 columns, so that most of the tile is
   // not padding (64-wide recurrent states).  The LayerNorm row sums keep the full tile: their slots are per 64 columns.
   const bool narrow = g.N <= 128 && g.epi != EPI_STORE_LN;
-  const bool pair = lc.gemm_pair && sms >= 2 && g.M > BM && !narrow;
+  const bool pair = lc.gemm_pair && sms >= 2 && g.M > BM && !narrow && !f32;
   const int row_elems = f32 ? 32 : 64;
   const int k_blocks = (g.K + row_elems - 1) / row_elems;
-  const int n_mma = narrow ? (g.N <= 64 ? 64 : 128) : pair && !f32 ? pair_tile_width(g, k_blocks, sms / 2) : BN;
+  const int n_mma = narrow ? (g.N <= 64 ? 64 : 128) : pair ? pair_tile_width(g, k_blocks, sms / 2) : BN;
   const int b_rows = pair ? n_mma / 2 : n_mma;
   CUtensorMap tmA, tmB;
   if (!make_map(&tmA, A0, g.M, g.K, g.batch, a_sm, a_sk, g.a_sb, a_mn, BM, f32)) return false;
@@ -745,8 +741,7 @@ bool gemm_tc(Launcher& lc, const GemmArgs& g, int* status_word) {
   if (!attr_set) {
     bool ok = true;
     for (auto kernel : {gemm_tc_kernel<false, false, false>, gemm_tc_kernel<false, false, true>, gemm_tc_kernel<false, true, false>,
-                        gemm_tc_kernel<false, true, true>, gemm_tc_kernel<true, false, false>, gemm_tc_kernel<true, false, true>,
-                        gemm_tc_kernel<true, true, false>})
+                        gemm_tc_kernel<false, true, true>, gemm_tc_kernel<true, false, false>, gemm_tc_kernel<true, false, true>})
       ok = ok && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) == cudaSuccess;
     if (!ok) {
       cudaGetLastError();
@@ -767,7 +762,7 @@ bool gemm_tc(Launcher& lc, const GemmArgs& g, int* status_word) {
   // stages sized by the B tile that a CTA loads (in blocks of 64 columns where it is MN-major): a narrow tile's ring is deeper, as the
   // bytes in flight, not the stage count, hide the load latency
   p.stage_bytes = A_BYTES + (b_mn ? (b_rows + 63) / 64 * 64 : b_rows) * 128;
-  const int ring = f32 ? (pair ? Mode<true, true>::kRingBytes : Mode<false, true>::kRingBytes) : (pair ? Mode<true, false>::kRingBytes : Mode<false, false>::kRingBytes);
+  const int ring = pair ? Mode<true>::kRingBytes : Mode<false>::kRingBytes;
   p.stages = ring / (int)p.stage_bytes < MAX_STAGES ? ring / (int)p.stage_bytes : MAX_STAGES;
   p.slots = gemm_tc_stats_slots(g.N);
   p.splits = splits; p.kb_per_split = kb_per_split;
@@ -783,7 +778,7 @@ bool gemm_tc(Launcher& lc, const GemmArgs& g, int* status_word) {
   p.stall = g.test_stall;
   const bool full = n_mma == BN;
   const int workers = pair ? sms / 2 : sms;
-  auto kernel = pair ? (f32 ? gemm_tc_kernel<true, true, false> : full ? gemm_tc_kernel<true, false, false> : gemm_tc_kernel<true, false, true>)
+  auto kernel = pair ? (full ? gemm_tc_kernel<true, false, false> : gemm_tc_kernel<true, false, true>)
                      : (f32 ? (full ? gemm_tc_kernel<false, true, false> : gemm_tc_kernel<false, true, true>)
                             : (full ? gemm_tc_kernel<false, false, false> : gemm_tc_kernel<false, false, true>));
   launch_chained(lc, kernel, dim3((pair ? 2 : 1) * (p.num_tiles < workers ? p.num_tiles : workers)), THREADS, SMEM_BYTES, pair ? 2 : 1, tmA, tmB,
