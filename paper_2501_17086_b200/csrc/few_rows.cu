@@ -6,6 +6,7 @@
 //             then its part of the block's output for all channels, which it writes to all CTAs; each adds the parts in rank order.
 //   backward  the layers are split over the cluster: every CTA forms the vector-Jacobian products of its layers from the iterate it
 //             holds for them and writes them to all CTAs; each then scans all layers for itself and keeps the iterates it needs.
+//   exact     the same split with one layer at a time: its CTA forms the product, all add it to the running gradient.
 // Weights lie in shared memory: forward two layers' at a time (the next layer's are copied while one is worked on), backward those of the
 // CTA's layers for all iterations where they fit.  Bound by latency and shared-memory bandwidth (a 16-byte broadcast takes four clocks:
 // a thread forms four neighbouring outputs of all rows).  Results that go to memory are stored after the barrier, not before: a
@@ -213,7 +214,7 @@ __device__ __host__ inline Share share_of(int width) {
 }
 __device__ __host__ inline int share_floats(int width) { return share_of(width).groups * kRows * 4 * share_of(width).quads; }
 
-// k iterations from g^0, all states of the last estimate to g_all; with dZ also gelu'(Z) times what the block is differentiated against in
+// k iterations from g^0 (or exact backpropagation), all states of the last estimate to g_all; with dZ also gelu'(Z) times what the block is differentiated against in
 // the last estimate, the parameter gradients' operand.
 __global__ void __launch_bounds__(kThreads, 1) few_rows_backward_kernel(const FewRows a) {
   extern __shared__ __align__(16) float smem[];
@@ -222,8 +223,8 @@ __global__ void __launch_bounds__(kThreads, 1) few_rows_backward_kernel(const Fe
   const int64_t row0 = (int64_t)(blockIdx.x / kCluster) * kRows, state = a.N * d;
   const int rows = (int)min((int64_t)kRows, a.N - row0);
   float* G = smem;                     // [slots][kRows][d]: g_{l+1} of this CTA's layers l = slot * kCluster + rank
-  float* U = G + slots * rd;           // [2][L][kRows][d]: all layers' vector-Jacobian products, of alternating iterations
-  float* dz = U + 2 * L * rd;          // [kRows][h]
+  float* U = G + (a.exact ? 0 : slots * rd);  // [2][L][kRows][d]: all layers' vector-Jacobian products, of alternating iterations
+  float* dz = U + 2 * (a.exact ? 1 : L) * rd; // [kRows][h]  (exact: no G, and two layers' products in turn)
   float* y = dz + kRows * h;           // [kRows][d]: a layer's product before its LayerNorm
   float* last_delta = y + rd;          // [kRows][d]: delta of the last state
   float* red = last_delta + rd;        // [groups][kRows][columns of a pass]
@@ -304,48 +305,73 @@ __global__ void __launch_bounds__(kThreads, 1) few_rows_backward_kernel(const Fe
       __syncthreads();
     }
   };
-  auto vjp = [&](float* u, bool to_memory) {
-    for (int s = 0; s < slots; ++s) {
-      const int l = s * kCluster + rank;
-      if (l >= L) break;
-      const float *W2 = a.W2 + (int64_t)l * d * h, *W1 = a.W1 + (int64_t)l * h * d, *prime = a.DACT + ((int64_t)l * a.N + row0) * h;
-      if (a.resident) {
-        W2 = kept + s * per_slot;
-        W1 = W2 + d * h;
-        prime = W1 + d * h;
-      }
-      product(W2, h, G + s * rd, d, d, [&](int r, int i, float v) {
-        v = r < rows ? v * prime[r * h + i] : 0.0f;
-        dz[r * h + i] = v;
-        if (to_memory && r < rows) a.dZ[((int64_t)l * a.N + row0 + r) * h + i] = v;
-      });
-      if (to_memory) continue;
-      const uint32_t to = smem_u32(u + l * rd);
-      if (!a.preln) {
-        product(W1, d, dz, h, h, [&](int r, int c, float v) {
-#pragma unroll
-          for (int j = 0; j < kCluster; ++j) st_peer(to + 4u * (r * d + c), j, v);
-        });
-        continue;
-      }
-      product(W1, d, dz, h, h, [&](int r, int c, float v) { y[r * d + c] = v; });
-      if (warp < kRows) {  // through the LayerNorm: rstd (dy - mean dy - xhat mean(dy xhat))
-        const bool in = warp < rows;
-        const float *xh = a.Y + l * state + (row0 + warp) * d, *dy = y + warp * d;
-        float s1 = 0.0f, s2 = 0.0f;
-        for (int c = lane; c < d; c += 32) {
-          s1 += dy[c];
-          s2 = fmaf(dy[c], in ? xh[c] : 0.0f, s2);
-        }
-        const float m1 = warp_sum(s1) / (float)d, m2 = warp_sum(s2) / (float)d, r = in ? a.rstd[l * a.N + row0 + warp] : 0.0f;
-        for (int c = lane; c < d; c += 32) {
-          const float v = r * (dy[c] - m1 - (in ? xh[c] : 0.0f) * m2);
-#pragma unroll
-          for (int j = 0; j < kCluster; ++j) st_peer(to + 4u * (warp * d + c), j, v);
-        }
-      }
-      // (y is written again only after the next product's barriers)
+  auto layer = [&](int s, const float* x, float* u, bool to_memory) {
+    const int l = s * kCluster + rank;
+    const float *W2 = a.W2 + (int64_t)l * d * h, *W1 = a.W1 + (int64_t)l * h * d, *prime = a.DACT + ((int64_t)l * a.N + row0) * h;
+    if (a.resident) {
+      W2 = kept + s * per_slot;
+      W1 = W2 + d * h;
+      prime = W1 + d * h;
     }
+    product(W2, h, x, d, d, [&](int r, int i, float v) {
+      v = r < rows ? v * prime[r * h + i] : 0.0f;
+      dz[r * h + i] = v;
+      if (to_memory && r < rows) a.dZ[((int64_t)l * a.N + row0 + r) * h + i] = v;
+    });
+    if (to_memory) return;
+    const uint32_t to = smem_u32(u + l * rd);
+    if (!a.preln) {
+      product(W1, d, dz, h, h, [&](int r, int c, float v) {
+#pragma unroll
+        for (int j = 0; j < kCluster; ++j) st_peer(to + 4u * (r * d + c), j, v);
+      });
+      return;
+    }
+    product(W1, d, dz, h, h, [&](int r, int c, float v) { y[r * d + c] = v; });
+    if (warp < kRows) {  // through the LayerNorm: rstd (dy - mean dy - xhat mean(dy xhat))
+      const bool in = warp < rows;
+      const float *xh = a.Y + l * state + (row0 + warp) * d, *dy = y + warp * d;
+      float s1 = 0.0f, s2 = 0.0f;
+      for (int c = lane; c < d; c += 32) {
+        s1 += dy[c];
+        s2 = fmaf(dy[c], in ? xh[c] : 0.0f, s2);
+      }
+      const float m1 = warp_sum(s1) / (float)d, m2 = warp_sum(s2) / (float)d, r = in ? a.rstd[l * a.N + row0 + warp] : 0.0f;
+      for (int c = lane; c < d; c += 32) {
+        const float v = r * (dy[c] - m1 - (in ? xh[c] : 0.0f) * m2);
+#pragma unroll
+        for (int j = 0; j < kCluster; ++j) st_peer(to + 4u * (warp * d + c), j, v);
+      }
+    }
+    // (y is written again only after the next product's barriers)
+  };
+  if (a.exact) {  // step by step: one CTA forms a layer's product, all add it to the running gradient (in place of last_delta)
+    for (int e = tid; e < rows * d; e += kThreads)
+      if (L % kCluster == rank) a.g_all[L * state + row0 * d + e] = last_delta[e];
+    copy_wait<0>();
+    cluster_sync();  // every CTA's shared memory may be written from here on
+    for (int l = L - 1; l >= 0; --l) {
+      const bool own = l % kCluster == rank;
+      const float* u = U + (l & 1) * rd;
+      if (own) layer(l / kCluster, last_delta, U + ((l & 1) - l) * rd, false);
+      cluster_sync();
+      for (int e = tid; e < rd; e += kThreads) {
+        const bool in = e < rows * d;
+        const int64_t at = l * state + row0 * d + e;
+        float g = a.gate == HBP_GATE_ONE ? last_delta[e] : gate_of(a, l)[e % d] * last_delta[e];
+        g += u[e];
+        if (a.every && in) g += a.delta[at];
+        last_delta[e] = g;
+        if (own && in) a.g_all[at] = g;
+      }
+      if (own && a.dZ)
+        for (int e = tid; e < rows * h; e += kThreads) a.dZ[((int64_t)l * a.N + row0) * h + e] = dz[e];
+      __syncthreads();
+    }
+    return;
+  }
+  auto vjp = [&](float* u, bool to_memory) {
+    for (int s = 0; s * kCluster + rank < L; ++s) layer(s, G + s * rd, u, to_memory);
   };
   scan(nullptr, a.k == 0);
   copy_wait<0>();
@@ -424,7 +450,8 @@ size_t forward_smem(const FewRows& a) {
 }
 size_t backward_smem(const FewRows& a) {
   const int slots = (a.L + kCluster - 1) / kCluster, red_d = share_floats(a.d), red_h = share_floats(a.h);
-  return (size_t)4 * (kRows * (slots * a.d + 2 * a.L * a.d + a.h + 2 * a.d) + (red_d > red_h ? red_d : red_h) + (a.resident ? slots * (2 * a.d * a.h + kRows * a.h) : 0));
+  const int states = a.exact ? 2 : slots + 2 * a.L;
+  return (size_t)4 * (kRows * (states * a.d + a.h + 2 * a.d) + (red_d > red_h ? red_d : red_h) + (a.resident ? slots * (2 * a.d * a.h + kRows * a.h) : 0));
 }
 
 bool launch(Launcher& lc, void (*kernel)(const FewRows), size_t smem, const FewRows& a) {
@@ -444,7 +471,7 @@ bool aligned(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 // 32 rows, forward / backward(1) / backward(4) with gradients in us, here and with a launch per product: 8 layers 64 (256) 22, 18, 29 and
 // 133, 46, 107; 128 (512) 37, 31, 73 and 166, 54, 134; 256 (256) pre-LN 49, 31, 76 and 152, 54, 127; 2 layers 64 (128) 9, 13, 15 and 31, 41,
-// 58; 64 layers 64 (256) 162, 78, 200 and 1050, 95, 252; 64 layers 128 (512) 278, 158, 401 and 1313, 156, 397.  Beyond 64 K weights a matrix
+// 58 (exact pass 38 and 163, 107 and 207, pre-LN 109 and 167, 18 and 48); 64 layers 64 (256) 162, 78, 200 and 1050, 95, 252; 64 layers 128 (512) 278, 158, 401 and 1313, 156, 397 (exact 337 and 1197, 1285 and 1595).  Beyond 64 K weights a matrix
 // the forward pass's two layers no longer fit shared memory, and backward passes gain less (8 layers 256 (1024) 79, 200 and 82, 214).
 bool few_rows_take(int64_t N, int d, int h) { return N <= 32 && (int64_t)d * h <= 64 * 1024; }
 

@@ -16,6 +16,7 @@ struct FewRows {
   float *x_all = nullptr, *Y = nullptr, *rstd = nullptr, *ACT = nullptr, *DACT = nullptr;
   // backward
   int k = 0;
+  bool exact = false;  // (then k is not read)
   bool every = false;  // delta [L+1][N][d], else [N][d]
   const float* delta = nullptr;
   float* g_all = nullptr;

@@ -614,10 +614,11 @@ struct Run {
     a.Y = (float*)c->Y; a.rstd = c->rstd; a.ACT = (float*)c->ACT; a.DACT = (float*)c->DACT;
     return a;
   }
-  // All iterations from the initial estimate on; with dz the parameter pass's dZ of all layers as well.
-  bool few_rows_iterations(int iters, bool dz) {
+  // All iterations from the initial estimate on, or exact backpropagation; with dz the parameter pass's dZ of all layers as well.
+  bool few_rows_iterations(bool exact, int iters, bool dz) {
     if (!few_rows() || shifted || (dz && c->group < c->layers)) return false;
     FewRows a = few_rows_args();
+    a.exact = exact;
     a.k = iters;
     a.every = c->cfg.loss == HBP_LOSS_EVERY_STEP;
     a.delta = (const float*)delta;
@@ -1398,23 +1399,21 @@ static hbp_status backward_common(hbp_ctx* ctx, const hbp_params* params, int32_
   const int steps = ctx->steps;
   const bool tr = f.block == HBP_BLOCK_PRELN_TRANSFORMER, rnn = f.block == HBP_BLOCK_RNN_TANH;
   const bool gru = f.block == HBP_BLOCK_GRU;
-  if (!exact) {
-    r.shifted = f.gamma != 0.0f;
-    bool done;
-    {
-      PhaseScope ph(r, HBP_PHASE_VJP);
-      done = r.few_rows_iterations(k < steps ? k : steps, grads != nullptr);
+  r.shifted = !exact && f.gamma != 0.0f;
+  bool done;
+  {
+    PhaseScope ph(r, exact ? HBP_PHASE_OTHER : HBP_PHASE_VJP);
+    done = r.few_rows_iterations(exact, k < steps ? k : steps, grads != nullptr);
+  }
+  if (done) {
+    if (grads) {
+      PhaseScope ph(r, HBP_PHASE_WGRAD);
+      FewRows a = r.few_rows_args();
+      a.dZ = (float*)ctx->H1;
+      few_rows_wgrad(r.lc, a, (const float*)g_all, (const float*)r.mlp_operand(0), grads->dW1, grads->dW2);
+      r.gate_grads(grads);
     }
-    if (done) {
-      if (grads) {
-        PhaseScope ph(r, HBP_PHASE_WGRAD);
-        FewRows a = r.few_rows_args();
-        a.dZ = (float*)ctx->H1;
-        few_rows_wgrad(r.lc, a, (const float*)g_all, (const float*)r.mlp_operand(0), grads->dW1, grads->dW2);
-        r.gate_grads(grads);
-      }
-      return r.result();
-    }
+    return r.result();
   }
   {
     PhaseScope ph(r, HBP_PHASE_OTHER);

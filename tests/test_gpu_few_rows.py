@@ -15,7 +15,7 @@ def test_few_rows_match_the_oracle(block, L, d, h, rows):
     w = Workload("t", block, "f32", L=L, d=d, hidden=h, tokens=rows, batch=1, seq=1, seed=9800 + d, loss="final_mse")
     inp = make_inputs(w, "cuda")
     gpu = run_gpu(w, inp, (0, 1, 3))
-    assert gpu["ctx"].forms["few_rows"] == 4   # the forward pass and three backward passes
+    assert gpu["ctx"].forms["few_rows"] == 5   # the forward pass, three backward passes and the exact one
     compare(w, gpu, orun.run(w, inp, ks=(0, 1, 3), grads_for=("exact", 3)), (0, 1, 3), ("exact", 3))
 
 
@@ -42,11 +42,38 @@ def test_few_rows_agree_with_a_launch_per_product(gate, every, block, L, d, h, r
             grads = ctx.new_grads(with_gate=True)
             got[k] = ctx.backward(params, k, delta, got["x"], grads=grads)
             got.update({(k, n): t for n, t in grads.items()})
+        grads = ctx.new_grads(with_gate=True)
+        got["exact"] = ctx.exact(params, delta, got["x"], grads=grads)
+        got.update({("exact", n): t for n, t in grads.items()})
         got["without"] = ctx.backward(params, 2, delta, got["x"])   # no parameter gradients asked for
+        got["exact without"] = ctx.exact(params, delta, got["x"])
         ctx.sync_status()
-        assert ctx.forms["few_rows"] == (0 if simt == "1" else 4)
+        assert ctx.forms["few_rows"] == (0 if simt == "1" else 6)
         outs.append(got)
-    assert torch.equal(outs[0]["without"], outs[0][2])
+    assert torch.equal(outs[0]["without"], outs[0][2]) and torch.equal(outs[0]["exact without"], outs[0]["exact"])
     for key, value in outs[0].items():  # each within some 5e-7 of the sums in 64 bits
         ref = outs[1][key]
         assert float((value - ref).norm() / ref.norm()) < 2e-6, key
+
+
+@pytest.mark.parametrize("block", ["mlp", "preln_mlp"])
+def test_more_layers_than_the_iterations_have_memory_for_are_exact_in_one_launch(block):
+    """The exact pass keeps two layers' products, the iterations all layers'; as many iterations as layers give the same gradients."""
+    from paper_2501_17086_b200 import harness
+    from paper_2501_17086_b200.workloads import Workload, make_inputs
+    w = Workload("t", block, "f32", L=40, d=256, hidden=64, tokens=2, batch=1, seq=1, seed=9899, loss="final_mse")
+    inp = make_inputs(w, "cuda")
+    params = harness.params_for(w, inp)
+    ctx = harness.make_context(w)
+    x = ctx.forward(params, inp["x0"])
+    delta = harness.loss_delta(w, x, inp)
+    exact, all_of_them = ctx.new_grads(), ctx.new_grads()
+    g = ctx.exact(params, delta, x, grads=exact)
+    assert ctx.forms["few_rows"] == 2
+    other = ctx.backward(params, 40, delta, x, grads=all_of_them)
+    ctx.sync_status()
+    assert ctx.forms["few_rows"] == 2
+    bound = 40 * 2 * 2.0 ** -24  # two roundings a layer
+    assert float((g - other).norm() / other.norm()) < bound
+    for n in exact:
+        assert float((exact[n] - all_of_them[n]).norm() / all_of_them[n].norm()) < bound, n
