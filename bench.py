@@ -58,30 +58,28 @@ def config_of(w, k, touched_bytes=None):
 # profiles/.  An entry is used only while the kernel's sources still hash to the value recorded with the capture and
 # the workload has the captured shapes; otherwise the bench line carries "traffic": null.
 TRAFFIC = {
-    # gemm_tc_kernel, VJP pair (dA + dY): c5_small (4 layers x 16384 tokens): 2036.314 + 1054.398 and 3038.729 + 279.232 MB;
-    # c2_small (8 layers x 8192 tokens): 738.478 + 504.902 and 790.265 + 129.146 MB
+    # gemm_tc_kernel, VJP pair (dA + dY): c5_small (4 layers x 16384 tokens): 2155.041 + 1054.668 and 2384.491 + 278.565 MB;
+    # c2_small (8 layers x 8192 tokens): 738.780 + 504.475 and 791.784 + 127.636 MB
     "gemm_vjp": [
-        {"sources": ("gemm_tc.cu", "tc_common.cuh"), "sha256": "5ddffe2221713528", "shape": ("preln_mlp", "bf16", 2048, 8192),
-         "bytes_per_token_layer": (2036.314e6 + 1054.398e6 + 3038.729e6 + 279.232e6) / (4 * 16384),
+        {"sources": ("gemm_tc.cu", "tc_common.cuh"), "sha256": "458482f102991da5", "shape": ("preln_mlp", "bf16", 2048, 8192),
+         "bytes_per_token_layer": (2155.041e6 + 1054.668e6 + 2384.491e6 + 278.565e6) / (4 * 16384),
          "profile": "profiles/gemm_tc_kernel_c5_small.md"},
-        {"sources": ("gemm_tc.cu", "tc_common.cuh"), "sha256": "5ddffe2221713528", "shape": ("preln_mlp", "bf16", 1024, 4096),
-         "bytes_per_token_layer": (738.478e6 + 504.902e6 + 790.265e6 + 129.146e6) / (8 * 8192),
+        {"sources": ("gemm_tc.cu", "tc_common.cuh"), "sha256": "458482f102991da5", "shape": ("preln_mlp", "bf16", 1024, 4096),
+         "bytes_per_token_layer": (738.780e6 + 504.475e6 + 791.784e6 + 127.636e6) / (8 * 8192),
          "profile": "profiles/gemm_tc_kernel_c2_small.md"}],
-    # scan_depth_lnstat_kernel: c5_small 605.051 MB read + 213.533 MB written for 4 steps x 16384 x 2048 elements; c2_small
-    # 286.285 + 80.494 MB for 8 x 8192 x 1024 (the writes still in L2 when such a small launch ends are not in the counter)
+    # scan_depth_lnstat_kernel: c5_small 605.050 MB read + 213.970 MB written for 4 steps x 16384 x 2048 elements; c2_small
+    # 286.283 + 80.576 MB for 8 x 8192 x 1024 (the writes still in L2 when such a small launch ends are not in the counter)
     "scan_lnstat": [
-        {"sources": ("scan.cu",), "sha256": "0f92d71cff018e9f", "shape": ("preln_mlp", "bf16", 2048, 8192),
-         "bytes_per_state_element_step": (605.051e6 + 213.533e6) / (4 * 16384 * 2048),
+        {"sources": ("scan.cu",), "sha256": "655dd8f4f6b9a76c", "shape": ("preln_mlp", "bf16", 2048, 8192),
+         "bytes_per_state_element_step": (605.050e6 + 213.970e6) / (4 * 16384 * 2048),
          "profile": "profiles/scan_depth_lnstat_kernel_c5_small.md"},
-        {"sources": ("scan.cu",), "sha256": "0f92d71cff018e9f", "shape": ("preln_mlp", "bf16", 1024, 4096),
-         "bytes_per_state_element_step": (286.285e6 + 80.494e6) / (8 * 8192 * 1024),
+        {"sources": ("scan.cu",), "sha256": "655dd8f4f6b9a76c", "shape": ("preln_mlp", "bf16", 1024, 4096),
+         "bytes_per_state_element_step": (286.283e6 + 80.576e6) / (8 * 8192 * 1024),
          "profile": "profiles/scan_depth_lnstat_kernel_c2_small.md"}],
-    # scan_ring_kernel on c3 (dram__bytes.sum.per_second x gpu__time_duration of the capture): the scan that writes the
-    # next VJP's split operand 6.046 TB/s x 169.0 us, the plain one 5.680 TB/s x 84.7 us
+    # scan_ring_kernel on c3: 268.531 MB read + 213.144 MB written, the mean of five scans
     "scan_ring": [
-        {"sources": ("scan_ring.cu", "tc_common.cuh"), "sha256": "926e6b3b23b4c4d9", "shape": ("rnn_tanh", "f32", 512, 0),
-         "bytes_per_state_element_step": 5.680e12 * 84.7e-6 / (4096 * 32 * 512),
-         "bytes_per_state_element_step_operand": 6.046e12 * 169.0e-6 / (4096 * 32 * 512),
+        {"sources": ("scan_ring.cu", "tc_common.cuh"), "sha256": "d2b53992756ec04d", "shape": ("rnn_tanh", "f32", 512, 0),
+         "bytes_per_state_element_step": (268.531e6 + 213.144e6) / (4096 * 32 * 512),
          "profile": "profiles/scan_ring_kernel_c3.md"}],
 }
 
@@ -408,12 +406,9 @@ def measure(env, wname, k, steps, warmup, headline, detail):
         scan_roof["traffic"] = t["bytes_per_state_element_step"] * w.steps * w.tokens * w.d
         scan_roof["traffic_source"] = t["profile"] + " (scaled by steps)"
     t = measured_traffic("scan_ring", w)
-    if t:
+    if t and not scan_note:
         scan_roof["kernel"] = "scan_ring_kernel"
-        per = t["bytes_per_state_element_step"]
-        if scan_note:  # the average over the phase's scans, like bytes_per_scan
-            per = ((kk - 1) * t["bytes_per_state_element_step_operand"] + per) / kk
-        scan_roof["traffic"] = per * w.steps * w.tokens * w.d
+        scan_roof["traffic"] = t["bytes_per_state_element_step"] * w.steps * w.tokens * w.d
         scan_roof["traffic_source"] = t["profile"]
 
     phases = {"vjp": vjp_ms / steps, "scan": scan_ms / steps, "wgrad": wg_ms / steps}
