@@ -2,6 +2,7 @@
 // hbp_forward / hbp_backward / hbp_exact.  No device memory is allocated here; every buffer is either
 // the caller's or a slice of the caller's workspace.
 #include <cstdint>
+#include <algorithm>
 #include <cstdlib>
 #include <cstring>
 #include <new>
@@ -105,7 +106,9 @@ struct hbp_ctx {
 namespace {
 
 constexpr size_t kAlign = 256;
-constexpr int kGateBlocks = 592;
+// Blocks of a gate gradient: four to an SM where the partial sums' buffer, sized for the recurrent kinds' products, holds that many
+// (131072 x 512: 132 us with 256, 85 with 592); what is carved for every kind holds the first.
+constexpr int kGateBlocks = 256, kMostGateBlocks = 592;
 constexpr int kMaxSplit = 256;
 
 inline size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
@@ -894,12 +897,13 @@ struct Run {
 
   void gate_grads(const hbp_grads* gr) {
     if (!gr->da || c->cfg.gate == HBP_GATE_ONE) return;
+    const int blocks = (int)std::min<size_t>(kMostGateBlocks, c->partial_floats / d);
     if (c->cfg.gate == HBP_GATE_CHANNEL_SHARED) {
-      gate_grad(lc, c->cfg.dtype, at(g, state), x_all, (int64_t)c->steps * N, (int)d, gr->da, c->partial, kGateBlocks);
+      gate_grad(lc, c->cfg.dtype, at(g, state), x_all, (int64_t)c->steps * N, (int)d, gr->da, c->partial, blocks);
     } else {
       for (int l = 0; l < c->steps; ++l)
         gate_grad(lc, c->cfg.dtype, at(g, (int64_t)(l + 1) * state), at(x_all, (int64_t)l * state), N, (int)d,
-                  gr->da + (int64_t)l * d, c->partial, kGateBlocks);
+                  gr->da + (int64_t)l * d, c->partial, blocks);
     }
   }
 
