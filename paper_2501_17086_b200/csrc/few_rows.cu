@@ -247,14 +247,15 @@ __global__ void __launch_bounds__(kThreads, 1) few_rows_backward_kernel(const Fe
     copy_group();
   }
   for (int e = tid; e < rd; e += kThreads) last_delta[e] = e < rows * d ? a.delta[(a.every ? L * state : 0) + row0 * d + e] : 0.0f;  // (each its own)
-  // Every CTA walks the layers down for all elements: g_l = delta_l + a_l g_{l+1} (+ u_l), and keeps the iterates of its own.
+  // Every CTA walks the layers down for all elements: g_l = delta_l + a_l g_{l+1} (+ u_l), and keeps the iterates of its own.  The running
+  // value is a double, as in the scans of scan.cu: a state is rounded where it is stored, not on the way to the next one.
   auto scan = [&](const float* u, bool last) {
     for (int e = tid; e < rd; e += kThreads) {
       const int c = e % d;
       const bool in = e < rows * d;
       const int64_t at = row0 * d + e;
-      float g = last_delta[e];
-      if (last && in && L % kCluster == rank) a.g_all[L * state + at] = g;
+      double g = last_delta[e];
+      if (last && in && L % kCluster == rank) a.g_all[L * state + at] = (float)g;
       for (int top = L - 1; top >= 0; top -= kCluster) {  // eight layers' operands at a time, then their chain
         float ul[kCluster], dl[kCluster], gt[kCluster];
 #pragma unroll
@@ -271,10 +272,10 @@ __global__ void __launch_bounds__(kThreads, 1) few_rows_backward_kernel(const Fe
         for (int j = 0; j < kCluster; ++j) {
           const int l = top - j;
           if (l < 0) continue;
-          if (l % kCluster == rank) G[l / kCluster * rd + e] = g;
+          if (l % kCluster == rank) G[l / kCluster * rd + e] = (float)g;
           g = gt[j] * g + ul[j];
           g += dl[j];
-          if (last && in && l % kCluster == rank) a.g_all[l * state + at] = g;
+          if (last && in && l % kCluster == rank) a.g_all[l * state + at] = (float)g;
         }
       }
     }
@@ -358,9 +359,11 @@ __global__ void __launch_bounds__(kThreads, 1) few_rows_backward_kernel(const Fe
       for (int e = tid; e < rd; e += kThreads) {
         const bool in = e < rows * d;
         const int64_t at = l * state + row0 * d + e;
-        float g = a.gate == HBP_GATE_ONE ? last_delta[e] : gate_of(a, l)[e % d] * last_delta[e];
-        g += u[e];
-        if (a.every && in) g += a.delta[at];
+        double sum = last_delta[e];  // (rounded once a layer)
+        if (a.gate != HBP_GATE_ONE) sum *= gate_of(a, l)[e % d];
+        sum += u[e];
+        if (a.every && in) sum += a.delta[at];
+        const float g = (float)sum;
         last_delta[e] = g;
         if (own && in) a.g_all[at] = g;
       }

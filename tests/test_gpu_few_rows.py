@@ -1,4 +1,4 @@
-"""Float MLP stacks of few rows as one launch a pass: rows that fill a cluster's four in part, hidden units that leave CTAs without any,
+"""Float MLP stacks of few rows as one launch a pass: rows that fill a cluster's three in part, hidden units that leave CTAs without any,
 more layers than CTAs, widths at both ends of the rule, every gate and loss."""
 import pytest
 import torch
@@ -54,6 +54,37 @@ def test_few_rows_agree_with_a_launch_per_product(gate, every, block, L, d, h, r
     for key, value in outs[0].items():  # each within some 5e-7 of the sums in 64 bits
         ref = outs[1][key]
         assert float((value - ref).norm() / ref.norm()) < 2e-6, key
+
+
+@pytest.mark.parametrize("gate", ["one", "shared", "per_step"])
+@pytest.mark.parametrize("block", ["mlp", "preln_mlp"])
+def test_scans_round_a_state_only_where_it_is_stored(block, gate):
+    """Blocks that add nothing (W2 = 0) leave the recurrence g_l = delta_l + a_l g_{l+1}: the truncated pass's states are those of the
+    recurrence in 64 bits, each rounded once; the exact pass goes from one stored state to the next with one rounding each."""
+    from paper_2501_17086_b200 import binding as B
+    L, d, h, rows = 100, 32, 64, 32
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(77)
+    rand = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    params = {"W1": rand(L, h, d) / d ** 0.5, "W2": torch.zeros((L, d, h), device="cuda")}
+    a = torch.ones((L, d), device="cuda")
+    if gate != "one":
+        params["a"] = 0.9 + 0.1 * torch.rand((d,) if gate == "shared" else (L, d), generator=gen, device="cuda")
+        a = params["a"].expand(L, d)
+    delta = rand(L + 1, rows, d)
+    ctx = B.Context(B.make_config(block, "f32", L, d, rows, hidden=h, loss=B.LOSS_EVERY_STEP,
+                                  gate={"one": B.GATE_ONE, "shared": B.GATE_CHANNEL_SHARED, "per_step": B.GATE_CHANNEL_PER_STEP}[gate]))
+    x = ctx.forward(params, rand(rows, d))
+    truncated = [ctx.backward(params, k, delta, x) for k in (0, 1)]
+    exact = ctx.exact(params, delta, x)
+    ctx.sync_status()
+    assert ctx.forms["few_rows"] == 4
+    ref = delta.double()
+    for l in range(L - 1, -1, -1):
+        ref[l] += a[l].double() * ref[l + 1]
+    for g in truncated:  # half a unit in the last place, and what the sums in 64 bits themselves are off by
+        assert bool(((g.double() - ref).abs() <= 2.0 ** -24 * ref.abs() + 2.0 ** -45 * ref.abs().max()).all())
+    assert torch.equal(exact[:-1], (a[:, None].double() * exact[1:].double() + delta[:-1].double()).float())
 
 
 @pytest.mark.parametrize("block", ["mlp", "preln_mlp"])
