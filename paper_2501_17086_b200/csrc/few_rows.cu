@@ -457,11 +457,17 @@ size_t backward_smem(const FewRows& a) {
   return (size_t)4 * (kRows * (states * a.d + a.h + 2 * a.d) + (red_d > red_h ? red_d : red_h) + (a.resident ? slots * (2 * a.d * a.h + kRows * a.h) : 0));
 }
 
-bool launch(Launcher& lc, void (*kernel)(const FewRows), size_t smem, const FewRows& a) {
+// The kernel's limit is set once per device and for any size: one set for a call could be lowered by another thread's before the launch.
+template <void (*kernel)(const FewRows)>
+bool launch(Launcher& lc, size_t smem, const FewRows& a) {
   if (smem > kMostSmem) return false;
-  if (smem > (48 << 10) && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
+  static PerDevice<bool> attr_done;
+  if (!attr_done.here()) {
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMostSmem) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    attr_done.here() = true;
   }
   const unsigned clusters = (unsigned)((a.N + kRows - 1) / kRows);
   if (try_launch_chained(lc, kernel, dim3(clusters * kCluster), kThreads, smem, kCluster, a) != cudaSuccess) return false;
@@ -480,14 +486,14 @@ bool few_rows_take(int64_t N, int d, int h) { return N <= 32 && (int64_t)d * h <
 
 bool few_rows_forward(Launcher& lc, const FewRows& a) {
   if (!aligned(a.W1) || !aligned(a.W2)) return false;
-  return launch(lc, few_rows_forward_kernel, forward_smem(a), a);
+  return launch<few_rows_forward_kernel>(lc, forward_smem(a), a);
 }
 bool few_rows_backward(Launcher& lc, const FewRows& args) {
   FewRows a = args;
   if (!aligned(a.W1) || !aligned(a.W2)) return false;
   a.resident = true;
   if (backward_smem(a) > kMostSmem) a.resident = false;
-  return launch(lc, few_rows_backward_kernel, backward_smem(a), a);
+  return launch<few_rows_backward_kernel>(lc, backward_smem(a), a);
 }
 
 void few_rows_wgrad(Launcher& lc, const FewRows& a, const float* g, const float* y, float* dW1, float* dW2) {

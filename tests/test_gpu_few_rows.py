@@ -108,3 +108,52 @@ def test_more_layers_than_the_iterations_have_memory_for_are_exact_in_one_launch
     assert float((g - other).norm() / other.norm()) < bound
     for n in exact:
         assert float((exact[n] - all_of_them[n]).norm() / all_of_them[n].norm()) < bound, n
+
+
+LOWERED = r"""
+#define _GNU_SOURCE
+#include <dlfcn.h>
+#include <cuda_runtime_api.h>
+int lowered = 0, limits = 0;
+static struct { const void* f; int bytes; } seen[256];
+cudaError_t cudaFuncSetAttribute(const void* f, enum cudaFuncAttribute attr, int value) {
+  if (attr == cudaFuncAttributeMaxDynamicSharedMemorySize) {
+    int i = 0;
+    while (i < limits && seen[i].f != f) ++i;
+    if (i == limits && limits < 256) seen[limits++].f = f;
+    if (value < seen[i].bytes) ++lowered;
+    seen[i].bytes = value;
+  }
+  typedef cudaError_t (*Fn)(const void*, enum cudaFuncAttribute, int);
+  static Fn real = 0;
+  if (!real) real = (Fn)dlsym(RTLD_NEXT, "cudaFuncSetAttribute");
+  if (!real) real = (Fn)dlsym(dlopen("libcudart.so.12", RTLD_NOW | RTLD_NOLOAD), "cudaFuncSetAttribute");
+  return real(f, attr, value);
+}
+"""
+
+TWO_SIZES = r"""
+import ctypes, os
+import torch
+from paper_2501_17086_b200 import binding as B
+stand_in = ctypes.CDLL(os.environ["LD_PRELOAD"])
+read = lambda name: ctypes.c_int.in_dll(stand_in, name).value
+rand = lambda *s: torch.randn(s, device="cuda")
+for L, d, sizes in ((8, 64, (256, 128)), (2, 128, (512, 256))):   # backward 164 and 97 KB a CTA; forward 160 and 94
+    for h, rows in zip(sizes, (32, 3)):
+        ctx = B.Context(B.make_config("mlp", "f32", L, d, rows, hidden=h))
+        params = {"W1": rand(L, h, d) / d ** 0.5, "W2": rand(L, d, h) / h ** 0.5}
+        x = ctx.forward(params, rand(rows, d))
+        ctx.backward(params, 1, rand(rows, d), x)
+        ctx.sync_status()
+        assert ctx.forms["few_rows"] == 2
+assert read("limits") >= 2 and read("lowered") == 0, (read("limits"), read("lowered"))
+print("REFUSED 0")
+"""
+
+
+def test_a_small_stack_does_not_lower_the_memory_limit_of_a_large_one(tmp_path):
+    """A kernel's limit of dynamic shared memory belongs to the kernel, whatever thread sets it: a call that set its own size could lower
+    it between another thread's set-up and launch, which would then fail.  A stand-in for the runtime's call sees every value set."""
+    from test_gpu_refused_clusters import _run_refused
+    _run_refused(tmp_path, TWO_SIZES, LOWERED)

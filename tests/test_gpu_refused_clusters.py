@@ -100,9 +100,9 @@ print("REFUSED", refused.value)
 """
 
 
-def _run_refused(tmp_path, child):
+def _run_refused(tmp_path, child, stand_in=REFUSE):
     src, lib = tmp_path / "refuse.c", tmp_path / "librefuse.so"
-    src.write_text(REFUSE)
+    src.write_text(stand_in)
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     subprocess.check_call(["gcc", "-shared", "-fPIC", "-I" + os.path.join(cuda, "include"), str(src), "-o", str(lib), "-ldl"])
     env = dict(os.environ, LD_PRELOAD=str(lib), PYTHONPATH=ROOT)
