@@ -393,10 +393,11 @@ __global__ void __launch_bounds__(kThreads, 1) few_rows_backward_kernel(const Fe
 constexpr int kTile = 64, kMostRows = 32;
 __global__ void __launch_bounds__(kThreads, 1) few_rows_wgrad_kernel(const FewRows a, const float* g, const float* y, float* dW1, float* dW2) {
   __shared__ __align__(16) float sa[kMostRows][kTile], sb[kMostRows][kTile];
-  const int tid = threadIdx.x, l = blockIdx.z >> 1, d = a.d, h = a.h, N = (int)a.N;
-  const bool first = blockIdx.z & 1;  // dW1 [h][d], else dW2 [d][h]
-  const int M = first ? h : d, K = first ? d : h, m0 = blockIdx.y * kTile, n0 = blockIdx.x * kTile;
-  if (m0 >= M || n0 >= K) return;
+  const int tid = threadIdx.x, d = a.d, h = a.h, N = (int)a.N;
+  const int dt = (d + kTile - 1) / kTile, ht = (h + kTile - 1) / kTile;  // as many blocks for either product
+  const int block = (int)(blockIdx.x % (dt * ht)), product = (int)(blockIdx.x / (dt * ht)), l = product >> 1;
+  const bool first = product & 1;  // dW1 [h][d], else dW2 [d][h]
+  const int M = first ? h : d, K = first ? d : h, across = first ? dt : ht, m0 = block / across * kTile, n0 = block % across * kTile;
   chain_next();
   chain_wait();
   const float* A = first ? a.dZ + (int64_t)l * N * h : g + (int64_t)(l + 1) * N * d;
@@ -497,9 +498,8 @@ bool few_rows_backward(Launcher& lc, const FewRows& args) {
 }
 
 void few_rows_wgrad(Launcher& lc, const FewRows& a, const float* g, const float* y, float* dW1, float* dW2) {
-  // (blocks of the wider of the two shapes' grids that the other does not have end at once)
-  const unsigned dt = (unsigned)((a.d + kTile - 1) / kTile), ht = (unsigned)((a.h + kTile - 1) / kTile), most = dt > ht ? dt : ht;
-  launch_chained(lc, few_rows_wgrad_kernel, dim3(most, most, 2 * a.L), kThreads, 0, 1, a, g, y, dW1, dW2);
+  const unsigned dt = (unsigned)((a.d + kTile - 1) / kTile), ht = (unsigned)((a.h + kTile - 1) / kTile);
+  launch_chained(lc, few_rows_wgrad_kernel, dim3(dt * ht * 2 * (unsigned)a.L), kThreads, 0, 1, a, g, y, dW1, dW2);
 }
 
 }  // namespace hbp

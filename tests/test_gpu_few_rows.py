@@ -110,6 +110,28 @@ def test_more_layers_than_the_iterations_have_memory_for_are_exact_in_one_launch
         assert float((exact[n] - all_of_them[n]).norm() / all_of_them[n].norm()) < bound, n
 
 
+def test_weight_gradients_of_more_layers_than_a_grid_is_deep():
+    """The exact pass of any number of layers is one launch; so are its weight gradients, here of 2 x 32769 products (a grid has 65535
+    blocks in its third dimension).  Against 64 bits from the pass's own states: sums of two rows and of four units."""
+    from paper_2501_17086_b200 import binding as B
+    L, d, h, rows = 32769, 4, 4, 2
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(79)
+    rand = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    params = {"W1": rand(L, h, d) / 2, "W2": rand(L, d, h) * (0.5 / L ** 0.5)}
+    ctx = B.Context(B.make_config("mlp", "f32", L, d, rows, hidden=h))
+    x = ctx.forward(params, rand(rows, d))
+    grads = ctx.new_grads()
+    g = ctx.exact(params, rand(rows, d), x, grads=grads)
+    ctx.sync_status()
+    assert ctx.forms["few_rows"] == 2
+    z = (x[:-1].double() @ params["W1"].double().mT).requires_grad_()
+    act = torch.nn.functional.gelu(z)
+    dz, = torch.autograd.grad(act, z, g[1:].double() @ params["W2"].double())
+    for got, ref in ((grads["dW1"], dz.mT @ x[:-1].double()), (grads["dW2"], g[1:].double().mT @ act.detach())):
+        assert float((got - ref).norm() / ref.norm()) < 8 * 2.0 ** -24
+
+
 LOWERED = r"""
 #define _GNU_SOURCE
 #include <dlfcn.h>
