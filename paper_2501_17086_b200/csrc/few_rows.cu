@@ -479,19 +479,36 @@ bool aligned(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 }  // namespace
 
-// 32 rows, forward / backward(1) / backward(4) with gradients in us, here and with a launch per product: 8 layers 64 (256) 22, 18, 29 and
-// 133, 46, 107; 128 (512) 37, 31, 73 and 166, 54, 134; 256 (256) pre-LN 49, 31, 76 and 152, 54, 127; 2 layers 64 (128) 9, 13, 15 and 31, 41,
-// 58 (exact pass 38 and 163, 107 and 207, pre-LN 109 and 167, 18 and 48); 64 layers 64 (256) 162, 78, 200 and 1050, 95, 252; 64 layers 128 (512) 278, 158, 401 and 1313, 156, 397 (exact 337 and 1197, 1285 and 1595).  Beyond 64 K weights a matrix
-// the forward pass's two layers no longer fit shared memory, and backward passes gain less (8 layers 256 (1024) 79, 200 and 82, 214).
+// 32 rows, forward pass in us here and with a launch per product: 8 layers 64 (256) 22 and 133, 128 (512) 37 and 166, 256 (256) 43 and 159, 2
+// layers 64 (128) 9 and 31, 64 layers 64 (256) 162 and 1050, 64 layers 128 (512) 278 and 1313.  Beyond 64 K weights a matrix its two layers
+// no longer fit shared memory, and backward passes gain less (8 layers 256 (1024) 79, 200 and 82, 214).
 bool few_rows_take(int64_t N, int d, int h) { return N <= 32 && (int64_t)d * h <= 64 * 1024; }
 
 bool few_rows_forward(Launcher& lc, const FewRows& a) {
   if (!aligned(a.W1) || !aligned(a.W2)) return false;
   return launch<few_rows_forward_kernel>(lc, forward_smem(a), a);
 }
+// Which backward passes gain.  A CTA works its layers off one by one, every 8 layers take an iteration 4 to 13 us more, where the batched
+// products of all layers hardly take longer for more of them (and from 32 layers on their scan runs in the ring).  Backward(1) and (4)
+// without gradients in us here and with a launch per product, 32 rows: 64 (256) 8 layers 10, 22 and 29, 91; 24 layers 21, 69 and 40, 126; 32
+// layers 27, 89 and 34, 95; 64 layers 48, 168 and 44, 118; 200 layers 32 (128) 91, 321 and 78, 164.  Matrices of more than 32 K weights, as
+// long as neither side makes the batched products long too (64 (1024), 24 layers 45, 163 and 59, 203), break even at one layer a CTA: 256
+// (256) 8 layers 20, 63 and 29, 97; 9 layers 32, 109 and 29, 97, of which the gradient pass makes 48, 125 and 57, 126 (pre-LN 49, 131
+// and 55, 121); 512 (128) pre-LN, 9 layers 43, 141 and 32, 106, with gradients 57, 155 and 64, 138.
+// The exact pass always gains (32 rows 8 layers 64 (256) 38 and 163, 64 layers 337 and 1197, with gradients) until the weights of such
+// matrices, read from L2 by a CTA at a time, and the gradients written no longer fit there: 256 (256), 3 rows with gradients 64 layers
+// (34 + 34 MB) 957 and 1452, 100 layers 2213 and 2283, pre-LN 2311 and 2073, 400 layers 9069 and 9006, 9482 and 8197; with more
+// clusters to wait for them 9 rows 200 layers 4208 and 4834, 32 rows 4132 and 4628, but pre-LN 4334 and 4227.
+static bool backward_gains(const FewRows& a) {
+  const int64_t weights = (int64_t)a.d * a.h;
+  const bool heavy = weights > 32 * 1024 && a.d < 1024 && a.h < 1024;
+  if (a.exact) return !heavy || 8 * a.L * weights * (a.dZ ? 2 : 1) <= (72 << 20) || (!a.preln && a.N > 8);
+  if (a.L <= kCluster) return true;
+  return heavy ? a.L <= 2 * kCluster && a.dZ && a.d <= 256 && a.k <= 3 : a.L <= 3 * kCluster;
+}
 bool few_rows_backward(Launcher& lc, const FewRows& args) {
   FewRows a = args;
-  if (!aligned(a.W1) || !aligned(a.W2)) return false;
+  if (!aligned(a.W1) || !aligned(a.W2) || !backward_gains(a)) return false;
   a.resident = true;
   if (backward_smem(a) > kMostSmem) a.resident = false;
   return launch<few_rows_backward_kernel>(lc, backward_smem(a), a);

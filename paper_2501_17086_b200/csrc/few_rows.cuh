@@ -25,7 +25,8 @@ struct FewRows {
 };
 // Whether a stack is one that these serve faster than a launch per product.
 bool few_rows_take(int64_t N, int d, int h);
-// false (of either): nothing was launched (unaligned weights, more layers than fit shared memory, launches in clusters refused).
+// false (of either): nothing was launched (unaligned weights, more layers than fit shared memory or than gain, launches in clusters
+// refused).
 bool few_rows_forward(Launcher& lc, const FewRows& a);
 bool few_rows_backward(Launcher& lc, const FewRows& a);
 

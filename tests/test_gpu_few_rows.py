@@ -62,7 +62,7 @@ def test_scans_round_a_state_only_where_it_is_stored(block, gate):
     """Blocks that add nothing (W2 = 0) leave the recurrence g_l = delta_l + a_l g_{l+1}: the truncated pass's states are those of the
     recurrence in 64 bits, each rounded once; the exact pass goes from one stored state to the next with one rounding each."""
     from paper_2501_17086_b200 import binding as B
-    L, d, h, rows = 100, 32, 64, 32
+    L, d, h, rows = 24, 32, 64, 32
     gen = torch.Generator(device="cuda")
     gen.manual_seed(77)
     rand = lambda *s: torch.randn(s, generator=gen, device="cuda")
@@ -108,6 +108,32 @@ def test_more_layers_than_the_iterations_have_memory_for_are_exact_in_one_launch
     assert float((g - other).norm() / other.norm()) < bound
     for n in exact:
         assert float((exact[n] - all_of_them[n]).norm() / all_of_them[n].norm()) < bound, n
+
+
+# layers, width, hidden units, block, and whether the iterations of backward(1), backward(4), both with gradients, and the exact pass
+# without and with gradients are one launch: the last number of layers that gains by it, and the next
+@pytest.mark.parametrize("L,d,h,rows,block,taken", [
+    (24, 64, 256, 32, "mlp", "yyyyyy"), (25, 64, 256, 32, "mlp", "nnnnyy"), (24, 64, 1024, 32, "preln_mlp", "yyyyyy"), (25, 64, 1024, 1, "mlp", "nnnnyy"),
+    (8, 256, 256, 3, "preln_mlp", "yyyyyy"), (9, 256, 256, 3, "mlp", "nnynyy"), (16, 128, 512, 3, "mlp", "nnynyy"), (17, 128, 512, 3, "mlp", "nnnnyy"),
+    (9, 512, 128, 3, "mlp", "nnnnyy"), (73, 256, 256, 3, "mlp", "nnnnyn"), (145, 256, 256, 8, "mlp", "nnnnnn"), (145, 256, 256, 9, "mlp", "nnnnyy"),
+    (145, 256, 256, 9, "preln_mlp", "nnnnnn")])
+def test_backward_passes_of_deep_stacks_are_one_launch_only_where_that_gains(L, d, h, rows, block, taken):
+    from paper_2501_17086_b200 import binding as B
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(81)
+    rand = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    params = {"W1": rand(L, h, d) / d ** 0.5, "W2": rand(L, d, h) * (0.5 / (L * h) ** 0.5)}
+    ctx = B.Context(B.make_config(block, "f32", L, d, rows, hidden=h))
+    x, delta, g = ctx.forward(params, rand(rows, d)), rand(rows, d), ctx.new_states()
+    calls = [lambda gr: ctx.backward(params, 1, delta, x, g_all=g, grads=gr), lambda gr: ctx.backward(params, 4, delta, x, g_all=g, grads=gr)] * 2
+    calls += [lambda gr: ctx.exact(params, delta, x, g_all=g, grads=gr)] * 2
+    got = ""
+    for call, with_grads in zip(calls, (0, 0, 1, 1, 0, 1)):
+        before = ctx.forms["few_rows"]
+        call(ctx.new_grads() if with_grads else None)
+        got += "y" if ctx.forms["few_rows"] > before else "n"
+    ctx.sync_status()
+    assert got == taken
 
 
 def test_weight_gradients_of_more_layers_than_a_grid_is_deep():
