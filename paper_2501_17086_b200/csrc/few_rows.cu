@@ -460,8 +460,9 @@ size_t backward_smem(const FewRows& a) {
 
 // The kernel's limit is set once per device and for any size: one set for a call could be lowered by another thread's before the launch.
 template <void (*kernel)(const FewRows)>
-bool launch(Launcher& lc, size_t smem, const FewRows& a) {
+bool launch(Launcher& lc, size_t smem, const FewRows& a, bool* refused) {
   if (smem > kMostSmem) return false;
+  *refused = true;
   static PerDevice<bool> attr_done;
   if (!attr_done.here()) {
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMostSmem) != cudaSuccess) {
@@ -472,6 +473,7 @@ bool launch(Launcher& lc, size_t smem, const FewRows& a) {
   }
   const unsigned clusters = (unsigned)((a.N + kRows - 1) / kRows);
   if (try_launch_chained(lc, kernel, dim3(clusters * kCluster), kThreads, smem, kCluster, a) != cudaSuccess) return false;
+  *refused = false;
   lc.ran(HBP_FORM_FEW_ROWS);
   return true;
 }
@@ -484,9 +486,9 @@ bool aligned(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 // no longer fit shared memory, and backward passes gain less (8 layers 256 (1024) 79, 200 and 82, 214).
 bool few_rows_take(int64_t N, int d, int h) { return N <= 32 && (int64_t)d * h <= 64 * 1024; }
 
-bool few_rows_forward(Launcher& lc, const FewRows& a) {
+bool few_rows_forward(Launcher& lc, const FewRows& a, bool* refused) {
   if (!aligned(a.W1) || !aligned(a.W2)) return false;
-  return launch<few_rows_forward_kernel>(lc, forward_smem(a), a);
+  return launch<few_rows_forward_kernel>(lc, forward_smem(a), a, refused);
 }
 // Which backward passes gain.  A CTA works its layers off one by one, every 8 layers take an iteration 4 to 13 us more, where the batched
 // products of all layers hardly take longer for more of them (and from 32 layers on their scan runs in the ring).  Backward(1) and (4)
@@ -506,12 +508,12 @@ static bool backward_gains(const FewRows& a) {
   if (a.L <= kCluster) return true;
   return heavy ? a.L <= 2 * kCluster && a.dZ && a.d <= 256 && a.k <= 3 : a.L <= 3 * kCluster;
 }
-bool few_rows_backward(Launcher& lc, const FewRows& args) {
+bool few_rows_backward(Launcher& lc, const FewRows& args, bool* refused) {
   FewRows a = args;
   if (!aligned(a.W1) || !aligned(a.W2) || !backward_gains(a)) return false;
   a.resident = true;
   if (backward_smem(a) > kMostSmem) a.resident = false;
-  return launch<few_rows_backward_kernel>(lc, backward_smem(a), a);
+  return launch<few_rows_backward_kernel>(lc, backward_smem(a), a, refused);
 }
 
 void few_rows_wgrad(Launcher& lc, const FewRows& a, const float* g, const float* y, float* dW1, float* dW2) {

@@ -25,10 +25,10 @@ struct FewRows {
 };
 // Whether a stack is one that these serve faster than a launch per product.
 bool few_rows_take(int64_t N, int d, int h);
-// false (of either): nothing was launched (unaligned weights, more layers than fit shared memory or than gain, launches in clusters
-// refused).
-bool few_rows_forward(Launcher& lc, const FewRows& a);
-bool few_rows_backward(Launcher& lc, const FewRows& a);
+// false (of either): nothing was launched (unaligned weights, more layers than fit shared memory or than gain); with *refused, because the
+// device refuses the launch.
+bool few_rows_forward(Launcher& lc, const FewRows& a, bool* refused);
+bool few_rows_backward(Launcher& lc, const FewRows& a, bool* refused);
 
 // Parameter gradients from the states g [L+1][N][d], what W1 was applied to y [L][N][d] (16-byte aligned) and the dZ of
 // few_rows_backward; dW1, dW2 of any alignment.

@@ -65,6 +65,7 @@ struct hbp_ctx {
   // while they load it (gemm_cell.cu).  use_cell: until the device refuses such a launch.
   Planes Wp;
   bool use_cell = false;
+  bool few_refused = false;  // few_rows.cu: the device has refused such a launch, none is asked for again
   char* U = nullptr;       // [steps][N][d] block VJP outputs (dY before the LayerNorm finish)
   char* H1 = nullptr;      // [group][N][h] dZ
   // Float residual MLP stacks: the operands of every product as three bf16 planes (gemm_parts.cu).  OPp = what W1 is applied to
@@ -606,7 +607,7 @@ struct Run {
   bool few_rows() const {
     const hbp_config& f = c->cfg;
     return f.dtype == HBP_F32 && (f.block == HBP_BLOCK_MLP || f.block == HBP_BLOCK_PRELN_MLP) && !lc.force_simt && lc.gemm_pair && !c->use_parts &&
-           few_rows_take(N, f.d, f.hidden);
+           !c->few_refused && few_rows_take(N, f.d, f.hidden);
   }
   FewRows few_rows_args() const {
     const hbp_config& f = c->cfg;
@@ -627,7 +628,7 @@ struct Run {
     a.delta = (const float*)delta;
     a.g_all = (float*)g;
     if (dz) a.dZ = (float*)c->H1;
-    return few_rows_backward(lc, a);
+    return few_rows_backward(lc, a, &c->few_refused);
   }
 
   // ---- all-step products of the float recurrent kinds, operands formed while they are loaded (gemm_cell.cu) ----------------
@@ -1187,7 +1188,7 @@ hbp_status hbp_forward(hbp_ctx* ctx, const hbp_params* params, const void* x0, c
     FewRows a = r.few_rows_args();
     a.x0 = (const float*)x0;
     a.x_all = (float*)x_all;
-    if (few_rows_forward(r.lc, a)) {
+    if (few_rows_forward(r.lc, a, &ctx->few_refused)) {
       ctx->forward_done = true;
       return r.result();
     }

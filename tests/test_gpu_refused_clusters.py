@@ -100,6 +100,42 @@ print("REFUSED", refused.value)
 """
 
 
+FEW_ROWS = r"""
+import ctypes, os
+import torch
+from paper_2501_17086_b200 import harness
+from paper_2501_17086_b200.workloads import Workload, make_inputs
+
+refused = ctypes.c_int.in_dll(ctypes.CDLL(os.environ["LD_PRELOAD"]), "refused_launches")
+for block in ("mlp", "preln_mlp"):
+    w = Workload("t", block, "f32", L=5, d=64, hidden=96, tokens=20, batch=1, seq=1, seed=9060)
+    inp = make_inputs(w, "cuda")
+    params = harness.params_for(w, inp)
+    outs = []
+    for single in (False, True):
+        if single:
+            os.environ["HBP_GEMM_PAIR"] = "0"
+        ctx = harness.make_context(w)
+        os.environ.pop("HBP_GEMM_PAIR", None)
+        before, got = refused.value, []
+        for again in range(2):
+            x = ctx.forward(params, inp["x0"])
+            delta = harness.loss_delta(w, x, inp)
+            got.append(x)
+            for exact in (False, True):
+                grads = ctx.new_grads()
+                got.append(ctx.exact(params, delta, x, grads=grads) if exact else ctx.backward(params, 2, delta, x, grads=grads))
+                got += [grads[n] for n in sorted(grads)]
+        ctx.sync_status()
+        assert ctx.forms["few_rows"] == 0
+        # the first pass asks once, and no pass asks again; by request none is asked for
+        assert refused.value - before == (0 if single else 1), (block, single, refused.value - before)
+        outs.append(got)
+    assert all(torch.equal(a, b) for a, b in zip(*outs)), block
+print("REFUSED", refused.value)
+"""
+
+
 def _run_refused(tmp_path, child, stand_in=REFUSE):
     src, lib = tmp_path / "refuse.c", tmp_path / "librefuse.so"
     src.write_text(stand_in)
@@ -119,3 +155,7 @@ def test_refused_cluster_launches_fall_back_to_one_launch_per_step(tmp_path):
 
 def test_float_stacks_need_no_clusters(tmp_path):
     _run_refused(tmp_path, STACKS)
+
+
+def test_float_stacks_of_few_rows_take_a_launch_per_product(tmp_path):
+    _run_refused(tmp_path, FEW_ROWS)
