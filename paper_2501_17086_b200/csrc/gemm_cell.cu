@@ -8,12 +8,18 @@
 // steps of 32), persistent, 512 threads:
 //   warp 0       VJP: TMA producer of W's planes
 //   warp 1       MMA issuer (one lane of the even CTA): 12 x tcgen05.mma 256 x n_tile x 16 per 32 of K, the product of the high parts
-//                into one accumulator, the five small ones into another, so that only every sixth addition is made at full
-//                magnitude, where the tensor core's truncation counts
+//                into one accumulator, the five small ones into another (FINE: all into one), so that only every sixth addition is
+//                made at full magnitude, where the tensor core's truncation counts
 //   warps 4..7   epilogue: the two accumulators added, delta added (VJP), out by TMA tile copies
 //   warps 8..15  load g and the coefficients (16 bytes per lane, the next blocks' loads in flight while one is worked on), multiply,
 //                split and store the parts: K-major rows of 64 bytes for the VJP; MN-major rows of 128 bytes for the weight gradients,
 //                whose right operand (states, inputs) they split likewise, so that nothing is ever written transposed
+// FINE, the weight gradients of T * B rows that are no multiple of 4: they have always been sums of floats, 3e-8 to 1.2e-7 from 64 bits
+// (tanh RNN 1.5e-7 to 7e-7), and stay so.  One accumulator per 32 rows, the small terms first, and the epilogue adds it, rounded and
+// its truncation made good (float_parts.cuh), to sums kept in tensor memory; every 512 rows these go out as a set of partial
+// sums, which are added in double.  Weight gradients in us as float sums before / as the other form / so: GRU 32385 x 512 1590 / 330 / 750
+// (errors 7e-8 / 1.1e-6 / 7e-8), 131967 x 64 550 / 70 / 105, LSTM 32385 x 512 1720 / 500 / 1190, tanh RNN 135135 x 512 10400 / 525 / 1140 (2e-7 /
+// 1.3e-6 / 7e-8).  Tiles of 96 columns 980, of 256, whose one set of accumulators holds up the products, 840 (GRU 32385 x 512).
 // Nothing of the operand goes through memory.  Before, it was written as two tf32 parts by a pass (the tanh RNN's by the scan before)
 // and read back by gemm_tc.cu, for the gradients transposed, their partial sums written every 512 rows.  One VJP with its pass and
 // scan, before / now: tanh RNN 131072 x 512 446 / 404 us, GRU 32768 x 512 345 / 250, GRU 131072 x 64 138 / 72; the weight
@@ -48,9 +54,13 @@ constexpr int SMEM_BYTES = kStages * (int)kStageBytes + kEpiWarps * kEpiBufs * (
 // The operand is multiplied by this on the way in and the sums divided by it: the low part of any normal float is then a normal
 // bf16, also of gradients below 1e-34, which long recurrences have (values from 2^103 on overflow: refine).
 constexpr float kScale = 16777216.0f, kUnscale = 1.0f / 16777216.0f;
-// Weight gradients: rows that add up in the tensor core (64 additions at full magnitude) before the sum is added, rounded, to the
-// split's partial sums.
-constexpr int kDrainBlocks = 1024 / BK;
+// Weight gradients: rows that add up in the tensor core (32 additions at full magnitude, each of which truncates) before the sum is
+// added, rounded, to the split's partial sums.  With 1024 rows (as once here) a pass takes 0.5 to 2 %
+// less (GRU 32768 x 512 5339 for 5367 us, tanh RNN 131072 x 512 2715 for 2768) and is twice as far from 64 bits: dW, dU of the tanh RNN 32768 x 512 1.3e-6, 1.7e-6 (as three tf32 products 1.2e-6, 1.6e-6) and
+// 5.9e-7, 7.8e-7 with 512, of the GRU 1.1e-6 (1.2e-6) and 5.4e-7.  That the sums of a split are added in float adds 2e-9 to that.
+constexpr int kDrainBlocks = 512 / BK;
+// FINE: rows from which on the tensor core is used (as in gemm_f32.cu), k-blocks of a set of partial sums, most sets asked for, and the widest tile that leaves two accumulators room beside the sums
+constexpr int kFewProducts = 17, kFineSet = 512 / BK, kMostFineSets = 256, kFineTileN = 160;
 
 struct Params {
   CellOperand o;
@@ -71,6 +81,7 @@ struct Params {
     int N, n_tile, m_tiles, n_tiles, vec;
   } seg[2];
   int M, tiles, splits, k_blocks, per_split, both;
+  int group, merge, sets_per_split;  // k-blocks added up in the tensor core; such sums in a set of partial sums; sets of a split
   int* status;
 };
 
@@ -132,6 +143,20 @@ __device__ __forceinline__ void refine_grad(const Params& p, int segment, int m,
   }
 }
 
+// 32 columns of this thread's TMEM lane; tc_st_wait() before they are read back
+__device__ __forceinline__ void tc_st32(uint32_t taddr, const float* v) {
+  const uint32_t* r = reinterpret_cast<const uint32_t*>(v);
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31};"
+      ::"r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]),
+      "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]),
+      "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]),
+      "r"(r[31]), "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void tc_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 // Two neighbouring floats in one register pair, for the packed float instructions.
 typedef unsigned long long f2;
 __device__ __forceinline__ f2 mul2(f2 a, f2 b) {
@@ -213,7 +238,7 @@ __device__ __forceinline__ Unit unit_of(const Params& p, int unit) {
   return u;
 }
 
-template <int KIND, bool GRAD>
+template <int KIND, bool GRAD, bool FINE>
 __global__ void __launch_bounds__(THREADS, 1)
 gemm_cell_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmD, const __grid_constant__ CUtensorMap tmD1,
                  const __grid_constant__ CUtensorMap tmE, const __grid_constant__ Params p) {
@@ -264,10 +289,11 @@ gemm_cell_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
   chain_next();
   chain_wait();
 
-  // accumulators: `sets` pairs of n_tile columns (the widest tiles fill the tensor memory with one)
+  // accumulators: `sets` pairs of n_tile columns (the widest tiles fill the tensor memory with one); FINE: single ones, the sums behind
   auto item_n_tile = [&](int item) { return GRAD ? p.seg[unit_of(p, item).segment].n_tile : p.n_tile; };
   const int widest = GRAD ? max(p.seg[0].n_tile, p.seg[1].n_tile) : p.n_tile;
-  const int sets = 4 * widest <= (int)TMEM_COLS ? 2 : 1;
+  constexpr int kAccs = FINE ? 1 : 2;  // accumulators of a set
+  const int sets = (2 * kAccs + (FINE ? 1 : 0)) * widest <= (int)TMEM_COLS ? 2 : 1;
 
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsFew));
@@ -324,12 +350,12 @@ gemm_cell_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         if (GRAD) {
           const Unit u = unit_of(p, item);
           n_kb = u.kb_hi - u.kb_lo;
-          group = kDrainBlocks;
+          group = p.group;
         }
         for (int kb = 0; kb < n_kb && ok; kb += group) {
           if (!mbar_wait(acce_bar(set), set_phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
           const int end = min(n_kb, kb + group);
-          const uint32_t d_high = tmem_base + (uint32_t)(set * 2 * widest), d_small = d_high + (uint32_t)n_tile;
+          const uint32_t d_high = tmem_base + (uint32_t)(set * kAccs * widest), d_small = FINE ? d_high : d_high + (uint32_t)n_tile;
           for (int i = kb; i < end; ++i) {
             if (!stage_ready && !mbar_wait(full_bar(stage), phase, abort_flag, p.status)) { ok = false; break; }
             tc_fence_after();
@@ -345,7 +371,7 @@ gemm_cell_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
 #pragma unroll
                 for (int k = 0; k < 2; ++k)
                   tc_mma_pair(q < 5 ? d_small : d_high, ad + (uint64_t)(qa[q] * a_part + k * a_k), bd + (uint64_t)(qb[q] * b_part + k * b_k), idesc,
-                              i > kb || k > 0 || (q > 0 && q < 5));
+                              i > kb || k > 0 || (q > 0 && (FINE || q < 5)));
               tc_commit_pair(empty_bar(stage));
               if (i + 1 == end) tc_commit_pair(accf_bar(set));
             }
@@ -382,7 +408,7 @@ gemm_cell_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
       if (GRAD) {
         u = unit_of(p, item);
         n_kb = u.kb_hi - u.kb_lo;
-        group = kDrainBlocks;
+        group = p.group;
         n_tile = p.seg[u.segment].n_tile;
         N = p.seg[u.segment].N;
       } else {
@@ -397,6 +423,7 @@ gemm_cell_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
       const int row0 = u.m0 + (int)rank * BM + ew * 32;
       const int chunks = min(n_tile, (N - u.n0 + 31) / 32 * 32) / 32;
       const CUtensorMap* out = GRAD && u.segment ? &tmD1 : &tmD;
+      int set_z = GRAD ? u.split * p.sets_per_split : 0, in_set = 0;  // the set of partial sums, and how many sums it has
       for (int kb = 0; kb < n_kb && ok; kb += group) {
         auto load_e = [&](int c, int to) {  // lane 0
           mbar_expect_tx(epi_bar(ew, to), kFloatBuf);
@@ -404,7 +431,7 @@ gemm_cell_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
           e_flight |= 1u << to;
         };
         if (lane == 0) {
-          if (GRAD) tma_store_wait_all();  // the group before has been added to the partial sums
+          if (GRAD && !FINE) tma_store_wait_all();  // the sums that these are added to have been written
           else tma_store_wait_read();
           if (!GRAD && p.has_e) {  // (tiles of 256 columns hold up the products until the epilogue has read them)
             for (int c = kEpiBufs - 1; c < chunks; ++c) tma_prefetch_3d(&tmE, u.n0 + c * 32, row0, 0);
@@ -414,40 +441,65 @@ gemm_cell_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         __syncwarp();
         if (!mbar_wait(accf_bar(set), set_phase, abort_flag, p.status)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t tsrc = tmem_base + ((uint32_t)(ew * 32) << 16) + (uint32_t)(set * 2 * widest);
+        const uint32_t tsrc = tmem_base + ((uint32_t)(ew * 32) << 16) + (uint32_t)(set * kAccs * widest);
         float v[2][32], w[2][32];
+        // the second accumulator, or what the set's sums are so far
+        const uint32_t tmore = FINE ? tmem_base + ((uint32_t)(ew * 32) << 16) + (uint32_t)(sets * widest) : tsrc + n_tile;
+        const bool keep = FINE && in_set + 1 < p.merge && kb + group < n_kb;  // the set goes on
         tc_ld32_async(tsrc, v[0]);
-        tc_ld32_async(tsrc + n_tile, w[0]);
+        if (!FINE || in_set > 0) tc_ld32_async(tmore, w[0]);
         auto chunk = [&](int c, float (&s)[32], float (&t)[32], float (&s_next)[32], float (&t_next)[32]) {
           tc_ld_wait();
           if (c + 1 < chunks) {
             tc_ld32_async(tsrc + (c + 1) * 32, s_next);
-            tc_ld32_async(tsrc + n_tile + (c + 1) * 32, t_next);
+            if (!FINE || in_set > 0) tc_ld32_async(tmore + (c + 1) * 32, t_next);
           }
           const int col = u.n0 + c * 32;
+          auto release = [&]() {  // the accumulators, before the last chunk goes out
+            if (c + 1 < chunks) return;
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(map_to_cta(acce_bar(set), 0));
+          };
+          if (FINE) {
+            const float factor = ((3 * kb + lane) & 7) < 3 ? kUnscale * kOneUp : kUnscale;
+#pragma unroll
+            for (int i = 0; i < 32; ++i) s[i] = fmaf(s[i], factor, in_set > 0 ? t[i] : 0.0f);
+            if (keep) {
+              release();
+              tc_st32(tmore + c * 32, s);
+              return;
+            }
+            // sums of a few products, where a truncation or a part left out counts as much as a rounding: as plain float sums (refine)
+            if (p.o.rows < kFewProducts)
+#pragma unroll
+              for (int i = 0; i < 32; ++i) s[i] = __uint_as_float(0x7fffffffu);
+          }
           f2 all = 0;  // not finite if one of the sums is not
 #pragma unroll
           for (int i = 0; i < 32; i += 2) {
-            const f2 one = mul2(add2(pack2(__float_as_uint(s[i]), __float_as_uint(s[i + 1])), pack2(__float_as_uint(t[i]), __float_as_uint(t[i + 1]))),
-                                pack2(__float_as_uint(kUnscale), __float_as_uint(kUnscale)));
+            f2 one = pack2(__float_as_uint(s[i]), __float_as_uint(s[i + 1]));
+            if (!FINE) {
+              one = mul2(add2(one, pack2(__float_as_uint(t[i]), __float_as_uint(t[i + 1]))), pack2(__float_as_uint(kUnscale), __float_as_uint(kUnscale)));
+              s[i] = __uint_as_float((uint32_t)one);
+              s[i + 1] = __uint_as_float((uint32_t)(one >> 32));
+            }
             all = add2(all, one);
-            s[i] = __uint_as_float((uint32_t)one);
-            s[i + 1] = __uint_as_float((uint32_t)(one >> 32));
           }
           const bool doubt = !(fabsf(__uint_as_float((uint32_t)all) + __uint_as_float((uint32_t)(all >> 32))) < __uint_as_float(0x7f800000u));
           if (__any_sync(0xffffffffu, doubt)) {
             tc_ld_wait();
-            if (GRAD) refine_grad<KIND>(p, u.segment, row0 + lane, col, (u.kb_lo + kb) * BK, min((int)p.o.rows, min(u.kb_hi, u.kb_lo + kb + group) * BK), s);
-            else refine_vjp<KIND>(p, row0 + lane, col, s);
+            if (GRAD) {
+              const int first = u.kb_lo + (FINE ? kb - in_set * group : kb);  // (the whole set's, where it is one sum)
+              refine_grad<KIND>(p, u.segment, row0 + lane, col, first * BK, min((int)p.o.rows, min(u.kb_hi, u.kb_lo + kb + group) * BK), s);
+            } else {
+              refine_vjp<KIND>(p, row0 + lane, col, s);
+            }
             const int again = min(c + 1, chunks - 1) * 32;  // (so that the next chunk need not be held in registers meanwhile)
             tc_ld32(tsrc + again, s_next);
-            tc_ld32(tsrc + n_tile + again, t_next);
+            if (!FINE || in_set > 0) tc_ld32(tmore + again, t_next);
           }
-          if (c + 1 == chunks) {
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(map_to_cta(acce_bar(set), 0));  // handed back before the last chunk goes out
-          }
+          release();
           const uint32_t at = buf0 + buf * kFloatBuf;
           if (!GRAD && p.has_e) {
             if (!mbar_wait(epi_bar(ew, buf), (e_phase >> buf) & 1u, abort_flag, p.status)) { ok = false; return; }
@@ -469,8 +521,8 @@ gemm_cell_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
           fence_async_smem();
           __syncwarp();
           if (lane == 0) {
-            if (GRAD && kb > 0) tma_add_3d(out, at, col, row0, u.split);
-            else tma_store_3d(out, at, col, row0, u.split);
+            if (GRAD && !FINE && in_set > 0) tma_add_3d(out, at, col, row0, set_z);
+            else tma_store_3d(out, at, col, row0, set_z);
             if (!GRAD && p.has_e && c + kEpiBufs - 1 < chunks) {  // into the buffer that the chunk before this one went out from
               tma_store_wait_read<1>();
               load_e(c + kEpiBufs - 1, buf == 0 ? kEpiBufs - 1 : buf - 1);
@@ -484,6 +536,8 @@ gemm_cell_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
           chunk(c, v[0], w[0], v[1], w[1]);
           if (ok && c + 1 < chunks) chunk(c + 1, v[1], w[1], v[0], w[0]);
         }
+        if (keep) tc_st_wait();
+        if (GRAD && ++in_set == p.merge) { in_set = 0; ++set_z; }
         if (++set == sets) { set = 0; set_phase ^= 1u; }
       }
     }
@@ -763,7 +817,6 @@ gemm_cell_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
 
 // An even split of n columns into `tiles` tiles, a multiple of 32 wide.
 int even_width(int n, int tiles) { return ((n + tiles - 1) / tiles + 31) / 32 * 32; }
-int tile_width(int n) { return even_width(n, (n + kMaxTileN - 1) / kMaxTileN); }
 // Width of the VJP's tiles: the least time over the waves of CTA pairs.  A k-block takes 2400 clocks at 256 columns and 1380 at 128,
 // where forming the operand bounds it, so that narrower ones gain nothing (131072 x 512 x 512 in tiles of 256 and 128: 322 and 368 us;
 // 32768 x 512 x 1536, 4 waves and 7: 219 and 208).
@@ -797,26 +850,30 @@ __global__ void __launch_bounds__(256) reduce_both_kernel(const float* __restric
   else dU[(int64_t)(gru && q == 3 ? m - d : m) * in + n - d] = (float)s;
 }
 
-template <int KIND, bool GRAD>
+template <int KIND, bool GRAD, bool FINE>
 bool launch(Launcher& lc, int items, const CUtensorMap& w, const CUtensorMap& d0, const CUtensorMap& d1, const CUtensorMap& e, const Params& p) {
   static PerDevice<bool> attr_done;
   if (!attr_done.here()) {
-    if (cudaFuncSetAttribute(gemm_cell_kernel<KIND, GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) != cudaSuccess) {
+    if (cudaFuncSetAttribute(gemm_cell_kernel<KIND, GRAD, FINE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) != cudaSuccess) {
       cudaGetLastError();
       return false;
     }
     attr_done.here() = true;
   }
   const int pairs = sm_count() / 2;
-  return try_launch_chained(lc, gemm_cell_kernel<KIND, GRAD>, dim3(2 * (items < pairs ? items : pairs)), THREADS, SMEM_BYTES, 2, w, d0, d1, e, p) ==
+  return try_launch_chained(lc, gemm_cell_kernel<KIND, GRAD, FINE>, dim3(2 * (items < pairs ? items : pairs)), THREADS, SMEM_BYTES, 2, w, d0, d1, e, p) ==
          cudaSuccess;
 }
-template <bool GRAD>
+template <bool GRAD, bool FINE>
 bool launch_kind(Launcher& lc, int items, const CUtensorMap& w, const CUtensorMap& d0, const CUtensorMap& d1, const CUtensorMap& e, const Params& p) {
-  if (p.kind == HBP_BLOCK_RNN_TANH) return launch<HBP_BLOCK_RNN_TANH, GRAD>(lc, items, w, d0, d1, e, p);
-  if (p.kind == HBP_BLOCK_GRU) return launch<HBP_BLOCK_GRU, GRAD>(lc, items, w, d0, d1, e, p);
-  return launch<HBP_BLOCK_LSTM, GRAD>(lc, items, w, d0, d1, e, p);
+  if (p.kind == HBP_BLOCK_RNN_TANH) return launch<HBP_BLOCK_RNN_TANH, GRAD, FINE>(lc, items, w, d0, d1, e, p);
+  if (p.kind == HBP_BLOCK_GRU) return launch<HBP_BLOCK_GRU, GRAD, FINE>(lc, items, w, d0, d1, e, p);
+  return launch<HBP_BLOCK_LSTM, GRAD, FINE>(lc, items, w, d0, d1, e, p);
 }
+// Rows of the operand whose sums stay as exact as sums of floats are (see the FINE form of the kernel).
+bool fine_sums(int64_t rows) { return rows % 4 != 0; }
+// Where states and inputs fit one tile's columns the operand is loaded and split once for both: the GRU's of four blocks then.
+bool both_at_once(int d, int in) { return d + in <= kMaxTileN; }
 int blocks_of(int kind) { return kind == HBP_BLOCK_RNN_TANH ? 1 : kind == HBP_BLOCK_GRU ? 3 : 4; }
 
 }  // namespace
@@ -845,7 +902,13 @@ bool cell_vjp(Launcher& lc, int kind, const CellOperand& o, const Planes& W, con
   if (!make_map_epi(&tmD, out, true, (int)o.rows, o.d, 1, ld, 0)) return false;
   tmE = tmD;
   if (delta && !make_map_epi(&tmE, delta, true, (int)o.rows, o.d, 1, ld, 0)) return false;
-  return launch_kind<false>(lc, p.num_tiles, tmW, tmD, tmD, tmE, p);
+  return launch_kind<false, false>(lc, p.num_tiles, tmW, tmD, tmD, tmE, p);
+}
+
+size_t cell_partial_floats(int kind, int64_t rows, int d, int in) {
+  if (!fine_sums(rows)) return 0;
+  const int64_t sets = (rows + kFineSet * BK - 1) / (kFineSet * BK), blocks = kind == HBP_BLOCK_GRU && both_at_once(d, in) ? 4 : blocks_of(kind);
+  return (size_t)((sets < kMostFineSets ? sets : kMostFineSets) * blocks * d * (d + in));
 }
 
 bool cell_wgrad(Launcher& lc, int kind, const CellOperand& o, const float* H, int64_t ldh, const float* X, int in, float* dW, float* dU,
@@ -854,8 +917,10 @@ bool cell_wgrad(Launcher& lc, int kind, const CellOperand& o, const float* H, in
   p.o = o;
   p.kind = kind;
   p.blocks = blocks_of(kind);
-  // Where states and inputs fit one tile's columns the operand is loaded and split once for both.
-  p.both = o.d + in <= kMaxTileN;
+  p.both = both_at_once(o.d, in);
+  const bool fine = fine_sums(o.rows);
+  const int widest = fine ? kFineTileN : kMaxTileN;
+  auto tile_width = [&](int n) { return even_width(n, (n + widest - 1) / widest); };
   p.M = (p.both && kind == HBP_BLOCK_GRU ? 4 : p.blocks) * o.d;
   p.status = status_word;
   const int m_tiles = (p.M + TILE_M - 1) / TILE_M, n0 = p.both ? o.d + in : o.d;
@@ -881,21 +946,32 @@ bool cell_wgrad(Launcher& lc, int kind, const CellOperand& o, const float* H, in
     }
   }
   if (best == 0) return false;
-  p.per_split = (p.k_blocks + p.splits - 1) / p.splits;
+  const int per = (p.k_blocks + p.splits - 1) / p.splits, chain = fine ? 1 : kDrainBlocks, groups = (per + chain - 1) / chain;
+  p.sets_per_split = fine ? (per + kFineSet - 1) / kFineSet : 1;
+  while (p.sets_per_split > 1 && p.splits * p.sets_per_split * outputs > (int64_t)partial_floats) --p.sets_per_split;
+  p.merge = (groups + p.sets_per_split - 1) / p.sets_per_split;
+  p.group = (per + groups - 1) / groups;
+  p.per_split = p.sets_per_split * p.merge * p.group;
   p.splits = (p.k_blocks + p.per_split - 1) / p.per_split;
+  const int set_blocks = p.merge * p.group, last = p.k_blocks - (p.splits - 1) * p.per_split;
+  const int sets = (p.splits - 1) * p.sets_per_split + (last + set_blocks - 1) / set_blocks;
   CUtensorMap tmD0, tmD1;
-  if (!make_map_epi(&tmD0, partial, true, p.M, n0, p.splits, n0, (int64_t)p.M * n0)) return false;
+  if (!make_map_epi(&tmD0, partial, true, p.M, n0, sets, n0, (int64_t)p.M * n0)) return false;
   if (p.both) {
-    if (!launch_kind<true>(lc, p.tiles * p.splits, tmD0, tmD0, tmD0, tmD0, p)) return false;
-    launch_chained(lc, reduce_both_kernel, dim3((unsigned)((outputs + 31) / 32)), 256, 0, 1, (const float*)partial, dW, dU, p.splits, p.M, o.d, in,
+    if (!(fine ? launch_kind<true, true>(lc, p.tiles * p.splits, tmD0, tmD0, tmD0, tmD0, p)
+               : launch_kind<true, false>(lc, p.tiles * p.splits, tmD0, tmD0, tmD0, tmD0, p)))
+      return false;
+    launch_chained(lc, reduce_both_kernel, dim3((unsigned)((outputs + 31) / 32)), 256, 0, 1, (const float*)partial, dW, dU, sets, p.M, o.d, in,
                    (int)(kind == HBP_BLOCK_GRU));
     return true;
   }
-  float* part1 = partial + (int64_t)p.splits * p.M * o.d;
-  if (!make_map_epi(&tmD1, part1, true, p.M, in, p.splits, in, (int64_t)p.M * in)) return false;
-  if (!launch_kind<true>(lc, p.tiles * p.splits, tmD0, tmD0, tmD1, tmD0, p)) return false;
-  reduce_splitk(lc, partial, dW, p.splits, (int64_t)p.M * o.d);
-  reduce_splitk(lc, part1, dU, p.splits, (int64_t)p.M * in);
+  float* part1 = partial + (int64_t)sets * p.M * o.d;
+  if (!make_map_epi(&tmD1, part1, true, p.M, in, sets, in, (int64_t)p.M * in)) return false;
+  if (!(fine ? launch_kind<true, true>(lc, p.tiles * p.splits, tmD0, tmD0, tmD1, tmD0, p)
+             : launch_kind<true, false>(lc, p.tiles * p.splits, tmD0, tmD0, tmD1, tmD0, p)))
+    return false;
+  reduce_splitk(lc, partial, dW, sets, (int64_t)p.M * o.d);
+  reduce_splitk(lc, part1, dU, sets, (int64_t)p.M * in);
   return true;
 }
 

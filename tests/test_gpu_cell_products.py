@@ -95,3 +95,43 @@ def test_cell_products_carry_what_is_not_finite(block, value):
     assert not torch.isfinite(d1["dW"]).all() and not torch.isfinite(d1["dU"]).all()
     rows = torch.isfinite(d1["dU"]).all(dim=1)   # operand channels that the element does not reach
     assert torch.allclose(d0["dU"][rows], d1["dU"][rows], rtol=1e-5, atol=1e-6 * float(d0["dU"].abs().max()))
+
+
+def _step(block, x, xt, W, U, a):
+    """One step's next state, in 64 bits (`xt` the inputs of the same rows)."""
+    if block == "rnn_tanh":
+        return a * x + torch.tanh(x @ W.T + xt @ U.T)
+    if block == "gru":
+        (ur, uz, un), (wr, wz, wn) = (xt @ U.T).chunk(3, -1), (x @ W.T).chunk(3, -1)
+        z = torch.sigmoid(uz + wz)
+        return z * x + (1 - z) * torch.tanh(un + torch.sigmoid(ur + wr) * wn)
+    c, h = x.chunk(2, -1)
+    i, f, g, o = (xt @ U.T + h @ W.T).chunk(4, -1)
+    c = torch.sigmoid(f) * c + torch.sigmoid(i) * torch.tanh(g)
+    return torch.cat([c, torch.sigmoid(o) * torch.tanh(c)], -1)
+
+
+# Rows of the product a multiple of 4: 32 additions a chain in the tensor core, each of which loses up to 2^-23 of a partial sum, that is on
+# average half as large as the whole: 32 * 2^-23 / 4.  Else sums of floats: 16 rounded additions a set, at random, 4 * 2^-24.
+@pytest.mark.parametrize("T,B", [(500, 132), (499, 131), (499, 130), (33, 3), (17, 1), (5, 3)])
+@pytest.mark.parametrize("units,in_dim", [(64, 12), (96, 100), (164, 128)])   # one tile for states and inputs together, two, one each
+@pytest.mark.parametrize("block", ["rnn_tanh", "gru", "lstm"])
+def test_weight_gradients_are_as_exact_as_their_rows_allow(block, units, in_dim, T, B):
+    """Against 64 bits from the pass's own states and iterate, so that nothing but the products' sums is compared."""
+    from paper_2501_17086_b200 import harness
+    from paper_2501_17086_b200.workloads import make_inputs
+    w = _workload(block, units, in_dim, T, B)
+    inp = make_inputs(w, "cuda")
+    ctx, params, X = harness.make_context(w), harness.params_for(w, inp), harness.rnn_inputs(w, inp)
+    x = ctx.forward(params, inp["x0"], X)
+    delta = harness.loss_delta(w, x, inp)
+    grads = ctx.new_grads()
+    g = ctx.backward(params, 1, delta, x, X, grads=grads)
+    ctx.sync_status()
+    assert ctx.forms["gemm_cell"] == 2
+    W, U = (params[n].double().requires_grad_() for n in ("W", "U"))
+    rows = lambda t: t.reshape(T * B, -1).double()
+    out = _step(block, rows(x[:-1]), rows(X), W, U, params["a"].double() if "a" in params else None)
+    for name, ref in zip(("dW", "dU"), torch.autograd.grad(out, (W, U), rows(g[1:]))):
+        bound = 32 * 2.0 ** -23 / 4 if T * B % 4 == 0 else 4 * 2.0 ** -24
+        assert float((grads[name] - ref).norm() / ref.norm()) < bound, name
