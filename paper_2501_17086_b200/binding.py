@@ -193,7 +193,7 @@ class Context:
         self._keep = None
 
     def selftest_wait_timeout(self, limit_ns=1_000_000):
-        """Enqueues a GEMM tile whose pipeline stalls on purpose with every wait limited to ``limit_ns``; the next
+        """Enqueues two GEMM tiles whose pipelines stall on purpose with every wait limited to ``limit_ns``; the next
         sync_status() raises HbpError(8)."""
         scratch = torch.empty((128 << 10) + 256, dtype=torch.uint8, device=self.device)
         base = (scratch.data_ptr() + 255) // 256 * 256

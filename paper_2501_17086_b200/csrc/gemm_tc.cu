@@ -19,6 +19,7 @@
 // Every wait on an mbarrier is bounded: after ~4 s it raises a shared abort flag, records
 // HBP_ERR_TIMEOUT in the status word, and all roles drain and leave through the common exit that
 // frees the tensor memory.
+#include "ring_drain.cuh"
 #include "tc_common.cuh"
 
 namespace hbp {
@@ -69,7 +70,7 @@ struct TcParams {
   float2* stats; int64_t stats_sb; int slots;
   int* status;
   uint64_t wait_limit_ns;  // limit of every barrier wait
-  int stall;               // self-test of the bounded waits only: the producer arms its first stage and copies nothing
+  int stall;               // self-test of the bounded waits only.  1: the first stage is armed and nothing copied; 2: B copied, nothing armed
 };
 
 // ------------------------------------------------------------------------------------------- epilogue math
@@ -193,6 +194,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   auto epi_bar = [&](int w, int i) { return bar0 + 8u * (2 * MAX_STAGES + 5 + 2 * w + i); };
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * MAX_STAGES + 5 + 2 * EPI_WARPS);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  RingReport* report = reinterpret_cast<RingReport*>(tmem_slot + 2);  // (the owner's counts)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -236,14 +238,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const int row_elems = kTf32 ? 32 : 64;
   const uint32_t mn_block = kTf32 ? 4096u : 8192u;
 
+  bool ok = true;  // until one of this thread's waits gives up
+  uint32_t filled = 0, stalled = 0;  // stages that this producer has issued its copies into; and armed without (self-test)
   if (warp == 0 || warp == kProducerB) {
     // ------------------------------------------------------------------ TMA producers: of A, and of B
     const bool of_a = warp == 0;
     if (lane == 0) {
       int stage = 0;
       uint32_t phase = 0;
-      uint32_t issued_mask = 0, issued_parity = 0;
-      bool ok = true;
       for (int tile = first_tile; tile < p.num_tiles && ok; tile += tile_step) {
         const int zc = tile / tiles_per_batch, r = tile % tiles_per_batch;
         const int b = zc % p.batch, split = zc / p.batch;
@@ -258,12 +260,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             const uint32_t sA = base + stage * STAGE_BYTES, sB = sA + A_BYTES;
             // pair: all four tile loads of a stage (two per CTA) complete on the leader's barrier
             const uint32_t fb = kPair ? map_to_cta(full_bar(stage), 0) : full_bar(stage);
-            if (of_a) {
-              if (leader) mbar_expect_tx(full_bar(stage), kPair ? 2 * STAGE_BYTES : STAGE_BYTES);
-              issued_mask |= 1u << stage;
-              issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
+            if (p.stall && (of_a || p.stall == 1)) {  // self-test: bytes are expected that nobody sends, or come that nobody expects
+              if (of_a && p.stall == 1) {
+                mbar_expect_tx(full_bar(stage), STAGE_BYTES);
+                stalled = 1;
+              }
+              ok = false;
+              break;
             }
-            if (p.stall) { ok = false; break; }  // self-test: bytes are expected that nobody sends
+            if (of_a && leader) mbar_expect_tx(full_bar(stage), kPair ? 2 * STAGE_BYTES : STAGE_BYTES);
             const int k0 = kb * row_elems;
             auto load = [&](uint32_t dst, const CUtensorMap* tm, int c0, int c1) {
               if (kPair) tma_load_3d_pair(dst, tm, fb, c0, c1, b);
@@ -280,19 +285,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             } else {
               load(sA, mA, k0, m0);
             }
+            ++filled;
             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
           }
         }
-      }
-      if (!ok && leader && of_a) {
-        // leave no copy of ours in flight: wait (bounded) for every stage armed last
-        for (int s = 0; s < STAGES; ++s)
-          if (issued_mask & (1u << s)) {
-            uint64_t t0 = global_ns();
-            const uint64_t lim = p.wait_limit_ns < 100000000ull ? p.wait_limit_ns : 100000000ull;
-            while (!mbar_try_wait(full_bar(s), (issued_parity >> s) & 1u) && global_ns() - t0 < lim) {
-            }
-          }
       }
     }
   } else if (warp == 1) {
@@ -315,7 +311,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       const uint32_t kStage16 = (uint32_t)STAGE_BYTES >> 4;
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0;
-      bool ok = true;
       // The tensor core idles whenever this thread takes longer between two MMAs than one MMA runs, so nothing that
       // has to wait for an answer sits between them: the barrier of the NEXT stage (and of the next tile's
       // accumulator) is only tested, without blocking, before the current stage's MMAs go out, and the answer is
@@ -412,7 +407,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         load_e(0);
         if (EPI_BUFS > 1 && nchunks > 1) load_e(1);
       }
-      if (!mbar_wait(accf_bar(acc), acc_phase, abort_flag, p.status, p.wait_limit_ns)) break;
+      if (!mbar_wait(accf_bar(acc), acc_phase, abort_flag, p.status, p.wait_limit_ns)) { ok = false; break; }
       tc_fence_after();
       const uint32_t tsrc = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN + half * half_cols);
       if (nchunks == 0) {  // nothing of a narrow tile in this half: only hand the accumulator back
@@ -430,7 +425,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         __syncwarp();
         if (lane == 0) release_acc(acc);
       } else {
-        bool ok = true;
         float s1 = 0.0f, s2 = 0.0f;  // EPI_STORE_LN: row sums of acc and acc * E over the current 64 columns
 #pragma unroll 1
         for (int c = 0; c < nchunks; ++c) {
@@ -539,9 +533,22 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
   }
 
-  tc_fence_before();
-  __syncthreads();
-  if (kPair) cluster_sync();  // neither CTA leaves (or frees) while its peer may still read its tiles or signal its barriers
+  if (roles_gave_up<kPair>(abort_flag, ok)) {
+    if (lane == 0 && (warp == 0 || warp == kProducerB)) {
+      const uint32_t mine = smem_u32(&report->filled[2 * rank + (warp == 0 ? 0 : 1)]);
+      st_cluster(kPair ? map_to_cta(mine, 0) : mine, filled);
+      if (leader && warp == 0) report->armed = filled + stalled;
+    }
+    __syncthreads();
+    if (kPair) cluster_sync();
+    if (leader && threadIdx.x == 0) {
+      const uint32_t a = A_BYTES, b = (uint32_t)STAGE_BYTES - A_BYTES;
+      auto none = [](uint32_t, uint32_t) {};
+      if (kPair) drain_ring<4>(full_bar(0), STAGES, report, {a, b, a, b}, none);
+      else drain_ring<2>(full_bar(0), STAGES, report, {a, b}, none);
+    }
+    if (kPair) cluster_sync();
+  }
   if (warp == 1) {
     tc_fence_after();
     if (kPair) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
@@ -697,7 +704,7 @@ bool gemm_tc(Launcher& lc, const GemmArgs& g, int* status_word) {
   // CTAs have four, and a third less is drawn from L2
   const int sms = sm_count();
   // A product at most 128 columns wide runs on single CTAs with MMAs of 64 or 128 columns, so that most of the tile is
-  // not padding (64-wide recurrent states).  The LayerNorm row sums keep the full tile: their slots are per 64 columns.
+  // not padding (64-wide recurrent states).  Those with LayerNorm row sums stay on pairs, whose tiles may be as narrow (pair_tile_width).
   const bool narrow = g.N <= 128 && g.epi != EPI_STORE_LN;
   const bool pair = lc.gemm_pair && sms >= 2 && g.M > BM && !narrow && !f32;
   const int row_elems = f32 ? 32 : 64;

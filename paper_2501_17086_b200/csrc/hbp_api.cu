@@ -1160,8 +1160,8 @@ hbp_status hbp_selftest_wait_timeout(hbp_ctx* ctx, void* scratch, size_t scratch
   Launcher lc;
   lc.stream = (cudaStream_t)cuda_stream;
   lc.launches = &ctx->launches;
-  // one 128 x 256 x 64 bf16 tile; the producer arms the first pipeline stage and issues no copy, so the MMA role's
-  // wait for it runs out after limit_ns
+  // one 128 x 256 x 64 bf16 tile, twice: the producers arm the first pipeline stage and issue no copy, then copy one operand into a stage
+  // that is not armed; either way the MMA role's wait for it runs out after limit_ns
   char* base = (char*)scratch;
   GemmArgs g;
   g.in_dtype = HBP_BF16;
@@ -1171,8 +1171,8 @@ hbp_status hbp_selftest_wait_timeout(hbp_ctx* ctx, void* scratch, size_t scratch
   g.epi = EPI_STORE;
   g.D = base + (48 << 10); g.ldd = 256;
   g.wait_limit_ns = limit_ns;
-  g.test_stall = 1;
-  if (!gemm_tc(lc, g, ctx->status)) return HBP_ERR_UNSUPPORTED;
+  for (g.test_stall = 1; g.test_stall <= 2; ++g.test_stall)
+    if (!gemm_tc(lc, g, ctx->status)) return HBP_ERR_UNSUPPORTED;
   return lc.err == cudaSuccess ? HBP_OK : HBP_ERR_CUDA;
 }
 

@@ -58,7 +58,7 @@ struct GemmArgs {
   int splitk = 1;      // > 1: partial sums to `partial` [splitk][batch][M][N], reduced in fixed order
   float* partial = nullptr;
   // self-test of the tensor-core kernel's bounded waits (hbp_selftest_wait_timeout): a wait limit other than the
-  // default, and a producer that arms its first pipeline stage without issuing the copies
+  // default, and producers that arm the first pipeline stage without issuing the copies (1) or copy B without arming it (2)
   uint64_t wait_limit_ns = 0;
   int test_stall = 0;
   bool dry_run = false;  // gemm_tc only: answer whether it would take this product, launch nothing

@@ -255,6 +255,23 @@ def test_a_bounded_wait_that_runs_out_is_reported_and_the_context_stays_usable()
         assert rel(np64(g[l]), ref["hbp"][2][l]) < 2e-2, l
 
 
+def test_a_kernel_whose_wait_ran_out_waits_for_the_copies_it_asked_for_and_no_others():
+    """The self-test's two tiles, one with a pipeline stage that expects bytes nobody sends, one with a copy that no stage expects, end
+    when their waits do: bytes that were never asked for are not waited for, and those that were have come by then."""
+    import time
+    from paper_2501_17086_b200 import binding as B, harness
+    from paper_2501_17086_b200.workloads import WORKLOADS
+    ctx = harness.make_context(WORKLOADS["c2_twin"])
+    for limit in (0.001, 0.2):   # (the first call also loads the kernels)
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        ctx.selftest_wait_timeout(limit_ns=int(limit * 1e9))
+        with pytest.raises(B.HbpError):
+            ctx.sync_status()
+        elapsed = time.perf_counter() - t0
+    assert 2 * limit <= elapsed < 2 * limit + 0.1   # one more wait: 0.1 s for a stage, or the limit
+
+
 def test_kernel_modes_belong_to_the_context(monkeypatch):
     """Two contexts created under different settings keep their own modes, and a call through either launches its own
     kind of kernels however the calls are interleaved: the modes read back as created, the CUDA-core context
