@@ -33,6 +33,7 @@
 #include <type_traits>
 
 #include "float_parts.cuh"
+#include "ring_drain.cuh"
 #include "tc_common.cuh"
 
 namespace hbp {
@@ -303,7 +304,7 @@ gemm_cell_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         const int half_n = p.n_tile / 2;
         const uint32_t b_bytes = (half_n > 64 ? 2 : 1) * kMnBlock;
         int stage = 0;
-        uint32_t phase = 0, issued_mask = 0, issued_parity = 0;
+        uint32_t phase = 0;
         bool ok = true;
         for (int item = first_item; item < items && ok; item += item_step) {
           const int n0 = (item % p.n_tiles) * p.n_tile + (int)rank * half_n;
@@ -312,22 +313,13 @@ gemm_cell_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
               if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
               const uint32_t sB = base + stage * kStageBytes + kABytes, fb = map_to_cta(full_bar(stage), 0);
               if (leader) mbar_expect_tx(full_bar(stage), 2 * b_bytes);
-              issued_mask |= 1u << stage;
-              issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
               const int k0 = q * p.o.d + c * BK;
               tma_load_4d_pair(sB, &tmW, fb, n0, k0, 0, 0);
               if (half_n > 64) tma_load_4d_pair(sB + kMnBlock, &tmW, fb, n0 + 64, k0, 0, 0);
               if (++stage == kStages) { stage = 0; phase ^= 1u; }
             }
         }
-        if (!ok && leader) {  // leave no copy in flight: wait (bounded) for every stage armed last
-          for (int s = 0; s < kStages; ++s)
-            if (issued_mask & (1u << s)) {
-              const uint64_t t0 = global_ns();
-              while (!mbar_try_wait(full_bar(s), (issued_parity >> s) & 1u) && global_ns() - t0 < 100000000ull) {
-              }
-            }
-        }
+        if (!ok) tell_peer(abort_flag);
       }
     } else if (warp == 1 && leader) {
       // ---------------------------------------------------------------- MMA issuer (the warp converged, one elected lane issues)
@@ -386,6 +378,7 @@ gemm_cell_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         const uint64_t t0 = global_ns();
         while (!mbar_try_wait(drain_bar, 0) && global_ns() - t0 < 100000000ull) {
         }
+        tell_peer(abort_flag);
       }
     }
   } else if (warp < 8) {
@@ -550,6 +543,7 @@ gemm_cell_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
           }
         }
     }
+    if (!ok) tell_peer(abort_flag);
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsLoad));
     // ------------------------------------------------------------------ operands
@@ -804,11 +798,10 @@ gemm_cell_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         }
       }
     }
+    if (!ok) tell_peer(abort_flag);
   }
 
-  tc_fence_before();
-  __syncthreads();
-  cluster_sync();  // neither CTA leaves (or frees) while its peer may still read its tiles or signal its barriers
+  if (roles_gave_up<true>(abort_flag, true) && !GRAD) outlast_copies();
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");

@@ -23,6 +23,7 @@
 #include <type_traits>
 
 #include "float_parts.cuh"
+#include "ring_drain.cuh"
 #include "tc_common.cuh"
 
 namespace hbp {
@@ -133,7 +134,7 @@ gemm_parts_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       // ---------------------------------------------------------------- TMA producers
       if (lane == 0) {
         int stage = 0;
-        uint32_t phase = 0, issued_mask = 0, issued_parity = 0;
+        uint32_t phase = 0;
         bool ok = true;
         for (int tile = first_tile; tile < p.num_tiles && ok; tile += tile_step) {
           const int b = tile / tiles_per_batch, r = tile % tiles_per_batch;
@@ -144,8 +145,6 @@ gemm_parts_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             const int k0 = kb * BK;
             if (warp == 0) {
               if (leader) mbar_expect_tx(full_bar(stage), 2 * stage_bytes);
-              issued_mask |= 1u << stage;
-              issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
               if (g.a_mn) {
                 tma_load_4d_pair(sA, &tmA, fb, m0, k0, b, 0);
                 tma_load_4d_pair(sA + kMnBlock, &tmA, fb, m0 + 64, k0, b, 0);
@@ -161,14 +160,7 @@ gemm_parts_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             if (++stage == stages) { stage = 0; phase ^= 1u; }
           }
         }
-        if (!ok && leader && warp == 0) {  // leave no copy in flight: wait (bounded) for every stage armed last
-          for (int s = 0; s < stages; ++s)
-            if (issued_mask & (1u << s)) {
-              const uint64_t t0 = global_ns();
-              while (!mbar_try_wait(full_bar(s), (issued_parity >> s) & 1u) && global_ns() - t0 < 100000000ull) {
-              }
-            }
-        }
+        if (!ok) tell_peer(abort_flag);
       }
     } else if (warp == 1 && leader) {
       // ---------------------------------------------------------------- MMA issuer (the warp converged, one elected lane issues)
@@ -217,6 +209,7 @@ gemm_parts_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         const uint64_t t0 = global_ns();
         while (!mbar_try_wait(drain_bar, 0) && global_ns() - t0 < 100000000ull) {
         }
+        tell_peer(abort_flag);
       }
     }
   } else {
@@ -407,11 +400,10 @@ gemm_parts_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         }
       }
     }
+    if (!ok) tell_peer(abort_flag);
   }
 
-  tc_fence_before();
-  __syncthreads();
-  cluster_sync();  // neither CTA leaves (or frees) while its peer may still read its tiles or signal its barriers
+  if (roles_gave_up<true>(abort_flag, true)) outlast_copies();
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");

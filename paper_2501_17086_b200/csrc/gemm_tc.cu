@@ -543,9 +543,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     if (kPair) cluster_sync();
     if (leader && threadIdx.x == 0) {
       const uint32_t a = A_BYTES, b = (uint32_t)STAGE_BYTES - A_BYTES;
-      auto none = [](uint32_t, uint32_t) {};
-      if (kPair) drain_ring<4>(full_bar(0), STAGES, report, {a, b, a, b}, none);
-      else drain_ring<2>(full_bar(0), STAGES, report, {a, b}, none);
+      if (kPair) drain_ring<4>(full_bar(0), STAGES, report, {a, b, a, b});
+      else drain_ring<2>(full_bar(0), STAGES, report, {a, b});
     }
     if (kPair) cluster_sync();
   }
