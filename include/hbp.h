@@ -273,7 +273,9 @@ int64_t hbp_form_count(const hbp_ctx* ctx, int32_t form);
  * bit 0 = HBP_FORCE_SIMT=1 (every contraction on the CUDA-core kernels, a cross-check of the tensor-core ones),
  * bit 1 = the tensor-core GEMM pairs CTAs (tcgen05 cta_group::2, 256 x 256 tiles): the default; HBP_GEMM_PAIR=0
  * keeps single CTAs (128 x 256 tiles; float MLP stacks then have their operands split inside the kernel, which needs no
- * clusters: what also runs where the device refuses a launch in clusters),
+ * clusters: what also runs where the device refuses a launch in clusters; float recurrent kinds of 32 units and more then
+ * have their operands split by passes of their own, with workspace for them: a context made without it on a device that
+ * refuses clusters computes its all-step products on the CUDA cores or, GRU and LSTM, split inside the kernel),
  * bit 2 = on the float tanh RNN, where the all-step products do not form that operand themselves (fewer than 32 units, single
  * CTAs), the reverse scan between two all-step VJPs (Eq. 9 followed by Eq. 8) also writes
  * the next VJP's left operand g_{t+1} * tanh'(z_t), split for the tensor cores, instead of the intermediate

@@ -303,8 +303,9 @@ def test_kernel_modes_belong_to_the_context(monkeypatch):
         assert float((o - outs[0]).norm() / outs[0].norm()) < 2e-2
 
 
-@pytest.mark.parametrize("T,d,batch", [(200, 128, 6), (70, 256, 3), (129, 64, 5)])
-def test_scan_that_writes_the_next_vjp_operand_changes_no_bit(monkeypatch, T, d, batch):
+# where the products do not form that operand themselves: single CTAs, and below 32 units
+@pytest.mark.parametrize("T,d,batch,pair", [(200, 128, 6, "0"), (70, 256, 3, "0"), (129, 64, 5, "0"), (150, 28, 6, "1"), (66, 4, 9, "1")])
+def test_scan_that_writes_the_next_vjp_operand_changes_no_bit(monkeypatch, T, d, batch, pair):
     """Float tanh RNN: between two all-step VJPs the time scan writes g_{t+1} * tanh'(z_t), split for the tensor
     cores, instead of the intermediate iterate.  It forms that product from the very float it would have stored, so
     every k gives the same bits as a context that keeps the separate pass (HBP_SCAN_OPERAND=0), parameter gradients
@@ -314,6 +315,7 @@ def test_scan_that_writes_the_next_vjp_operand_changes_no_bit(monkeypatch, T, d,
     from paper_2501_17086_b200.workloads import WORKLOADS, make_inputs
     w = dataclasses.replace(WORKLOADS["c3_twin"], L=T, d=d, batch=batch, tokens=batch, in_dim=32)
     inp = make_inputs(w, "cuda")
+    monkeypatch.setenv("HBP_GEMM_PAIR", pair)
     fused = harness.make_context(w)
     monkeypatch.setenv("HBP_SCAN_OPERAND", "0")
     plain = harness.make_context(w)
@@ -322,14 +324,18 @@ def test_scan_that_writes_the_next_vjp_operand_changes_no_bit(monkeypatch, T, d,
     params = harness.params_for(w, inp)
     X = harness.rnn_inputs(w, inp)
     for k in (1, 2, 5):
-        got = []
+        got, launches = [], []
         for ctx in (fused, plain):
             x_all = ctx.forward(params, inp["x0"], X)
             delta = harness.loss_delta(w, x_all, inp)
             grads = ctx.new_grads(with_gate=True)
+            before = ctx.launches
             g = ctx.backward(params, k, delta, x_all, X, grads=grads)
+            launches.append(ctx.launches - before)
             ctx.sync_status()
             got.append((g.clone(), {n: t.clone() for n, t in grads.items()}))
+        # the scan of every estimate that a VJP follows has written that VJP's operand: a pass less each
+        assert launches[0] == launches[1] - k and not fused.forms["gemm_cell"]
         assert torch.equal(got[0][0], got[1][0])
         for n in got[0][1]:
             assert torch.equal(got[0][1][n], got[1][1][n]), n

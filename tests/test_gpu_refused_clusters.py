@@ -136,6 +136,48 @@ print("REFUSED", refused.value)
 """
 
 
+CELL_PRODUCTS = r"""
+import ctypes, os
+import torch
+from paper_2501_17086_b200 import harness
+from paper_2501_17086_b200.workloads import Workload, make_inputs
+
+refused = ctypes.c_int.in_dll(ctypes.CDLL(os.environ["LD_PRELOAD"]), "refused_launches")
+for block, u in (("gru", 64), ("lstm", 40), ("rnn_tanh", 100)):
+    for T, B, first in ((7, 40, True), (9, 39, False)):
+        w = Workload("t", block, "f32", L=T, d=2 * u if block == "lstm" else u, hidden=u if block == "lstm" else 0, in_dim=16,
+                     batch=B, tokens=B, seed=9100 + u, loss="every_mse")
+        inp = make_inputs(w, "cuda")
+        params, xin = harness.params_for(w, inp), harness.rnn_inputs(w, inp)
+        outs = []
+        for mode in (None, "HBP_GEMM_PAIR", "HBP_FORCE_SIMT"):
+            if mode:
+                os.environ[mode] = "0" if mode == "HBP_GEMM_PAIR" else "1"
+            ctx = harness.make_context(w)
+            if mode:
+                os.environ.pop(mode)
+            x = ctx.forward(params, inp["x0"], xin)
+            delta = harness.loss_delta(w, x, inp)
+            got, asked = [x], []
+            if not first:   # the gradients of the exact pass are the first such product
+                grads = ctx.new_grads()
+                got += [ctx.exact(params, delta, x, xin, grads=grads)] + [grads[n] for n in sorted(grads)]
+            for k in (2, 3, 2):
+                before, grads = refused.value, ctx.new_grads()
+                got += [ctx.backward(params, k, delta, x, xin, grads=grads)] + [grads[n] for n in sorted(grads)]
+                asked.append(refused.value - before)
+            ctx.sync_status()
+            # the first product is refused, and none is asked for again
+            assert asked == ([1, 0, 0] if first and not mode else [0, 0, 0]), (block, T, mode, asked)
+            assert ctx.forms["gemm_cell"] == 0
+            outs.append(got)
+        for other in outs[:2]:   # single CTAs' tf32 products are 1.2e-6 from 64 bits, float sums in any order less
+            for a, b in zip(other, outs[2]):
+                assert float((a - b).norm() / b.norm()) < 5e-6, (block, T)
+print("REFUSED", refused.value)
+"""
+
+
 def _run_refused(tmp_path, child, stand_in=REFUSE):
     src, lib = tmp_path / "refuse.c", tmp_path / "librefuse.so"
     src.write_text(stand_in)
@@ -159,3 +201,7 @@ def test_float_stacks_need_no_clusters(tmp_path):
 
 def test_float_stacks_of_few_rows_take_a_launch_per_product(tmp_path):
     _run_refused(tmp_path, FEW_ROWS)
+
+
+def test_cell_products_need_no_clusters(tmp_path):
+    _run_refused(tmp_path, CELL_PRODUCTS)
