@@ -58,14 +58,14 @@ def config_of(w, k, touched_bytes=None):
 # profiles/.  An entry is used only while the kernel's sources still hash to the value recorded with the capture and
 # the workload has the captured shapes; otherwise the bench line carries "traffic": null.
 TRAFFIC = {
-    # gemm_tc_kernel, VJP pair (dA + dY): c5_small (4 layers x 16384 tokens): 2176.996 + 1055.083 and 2517.696 + 278.793 MB;
-    # c2_small (8 layers x 8192 tokens): 739.093 + 504.293 and 794.887 + 128.236 MB
+    # gemm_tc_kernel, VJP pair (dA + dY): c5_small (4 layers x 16384 tokens): 2121.899 + 1054.033 and 2438.503 + 279.543 MB;
+    # c2_small (8 layers x 8192 tokens): 738.675 + 505.052 and 796.289 + 128.911 MB
     "gemm_vjp": [
-        {"sources": ("gemm_tc.cu", "tc_common.cuh"), "sha256": "b5fe2a008fda27bc", "shape": ("preln_mlp", "bf16", 2048, 8192),
-         "bytes_per_token_layer": (2176.996e6 + 1055.083e6 + 2517.696e6 + 278.793e6) / (4 * 16384),
+        {"sources": ("gemm_tc.cu", "tc_common.cuh"), "sha256": "48e1ccd304ba5914", "shape": ("preln_mlp", "bf16", 2048, 8192),
+         "bytes_per_token_layer": (2121.899e6 + 1054.033e6 + 2438.503e6 + 279.543e6) / (4 * 16384),
          "profile": "profiles/gemm_tc_kernel_c5_small.md"},
-        {"sources": ("gemm_tc.cu", "tc_common.cuh"), "sha256": "b5fe2a008fda27bc", "shape": ("preln_mlp", "bf16", 1024, 4096),
-         "bytes_per_token_layer": (739.093e6 + 504.293e6 + 794.887e6 + 128.236e6) / (8 * 8192),
+        {"sources": ("gemm_tc.cu", "tc_common.cuh"), "sha256": "48e1ccd304ba5914", "shape": ("preln_mlp", "bf16", 1024, 4096),
+         "bytes_per_token_layer": (738.675e6 + 505.052e6 + 796.289e6 + 128.911e6) / (8 * 8192),
          "profile": "profiles/gemm_tc_kernel_c2_small.md"}],
     # scan_depth_lnstat_kernel: c5_small 605.050 MB read + 213.970 MB written for 4 steps x 16384 x 2048 elements; c2_small
     # 286.283 + 80.576 MB for 8 x 8192 x 1024 (the writes still in L2 when such a small launch ends are not in the counter)

@@ -238,8 +238,8 @@ hbp_status hbp_sync_status(hbp_ctx* ctx, void* cuda_stream);
  * Enqueues two tiles of the GEMM kernel, one whose copy role expects bytes that it never requests, then one that requests
  * bytes it does not expect, with every wait limited
  * to limit_ns (1 us .. 1 s) instead of the usual 4 s: the wait runs out, the kernel records HBP_ERR_TIMEOUT in the
- * context's status word, all of its roles leave, what copies were requested are waited for, the tensor memory is freed and the
- * kernel ends.  The next hbp_sync_status returns HBP_ERR_TIMEOUT.  scratch: device memory, 256-byte aligned, >= 128 KiB (contents
+ * context's status word, all of its roles leave, the tensor memory is freed and, 0.1 s later, when any copy
+ * is over, the kernel ends.  The next hbp_sync_status returns HBP_ERR_TIMEOUT.  scratch: device memory, 256-byte aligned, >= 128 KiB (contents
  * irrelevant, may be overwritten).  Nothing waits without a limit at any point. */
 hbp_status hbp_selftest_wait_timeout(hbp_ctx* ctx, void* scratch, size_t scratch_bytes, uint64_t limit_ns,
                                      void* cuda_stream);

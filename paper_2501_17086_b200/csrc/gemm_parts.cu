@@ -403,10 +403,13 @@ gemm_parts_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     if (!ok) tell_peer(abort_flag);
   }
 
-  if (roles_gave_up<true>(abort_flag, true)) outlast_copies();
+  tc_fence_before();
+  cluster_sync();  // neither CTA leaves (or frees) while its peer may still read its tiles or signal its barriers
   if (warp == 1) {
+    const int gave_up = *abort_flag;
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
+    if (gave_up) outlast_copies();
   }
 }
 

@@ -194,7 +194,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   auto epi_bar = [&](int w, int i) { return bar0 + 8u * (2 * MAX_STAGES + 5 + 2 * w + i); };
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * MAX_STAGES + 5 + 2 * EPI_WARPS);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  RingReport* report = reinterpret_cast<RingReport*>(tmem_slot + 2);  // (the owner's counts)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -239,7 +238,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const uint32_t mn_block = kTf32 ? 4096u : 8192u;
 
   bool ok = true;  // until one of this thread's waits gives up
-  uint32_t filled = 0, stalled = 0;  // stages that this producer has issued its copies into; and armed without (self-test)
   if (warp == 0 || warp == kProducerB) {
     // ------------------------------------------------------------------ TMA producers: of A, and of B
     const bool of_a = warp == 0;
@@ -261,10 +259,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             // pair: all four tile loads of a stage (two per CTA) complete on the leader's barrier
             const uint32_t fb = kPair ? map_to_cta(full_bar(stage), 0) : full_bar(stage);
             if (p.stall && (of_a || p.stall == 1)) {  // self-test: bytes are expected that nobody sends, or come that nobody expects
-              if (of_a && p.stall == 1) {
-                mbar_expect_tx(full_bar(stage), STAGE_BYTES);
-                stalled = 1;
-              }
+              if (of_a && p.stall == 1) mbar_expect_tx(full_bar(stage), STAGE_BYTES);
               ok = false;
               break;
             }
@@ -285,7 +280,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             } else {
               load(sA, mA, k0, m0);
             }
-            ++filled;
             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
           }
         }
@@ -533,25 +527,20 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
   }
 
-  if (roles_gave_up<kPair>(abort_flag, ok)) {
-    if (lane == 0 && (warp == 0 || warp == kProducerB)) {
-      const uint32_t mine = smem_u32(&report->filled[2 * rank + (warp == 0 ? 0 : 1)]);
-      st_cluster(kPair ? map_to_cta(mine, 0) : mine, filled);
-      if (leader && warp == 0) report->armed = filled + stalled;
-    }
+  tc_fence_before();
+  if (kPair) {
+    if (!ok) tell_peer(abort_flag);
+    __syncwarp();
+    cluster_sync();  // neither CTA leaves (or frees) while its peer may still read its tiles or signal its barriers
+  } else {
     __syncthreads();
-    if (kPair) cluster_sync();
-    if (leader && threadIdx.x == 0) {
-      const uint32_t a = A_BYTES, b = (uint32_t)STAGE_BYTES - A_BYTES;
-      if (kPair) drain_ring<4>(full_bar(0), STAGES, report, {a, b, a, b});
-      else drain_ring<2>(full_bar(0), STAGES, report, {a, b});
-    }
-    if (kPair) cluster_sync();
   }
   if (warp == 1) {
+    const int gave_up = *abort_flag;
     tc_fence_after();
     if (kPair) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
     else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
+    if (gave_up) outlast_copies();
   }
 }
 

