@@ -942,12 +942,12 @@ bool cell_wgrad(Launcher& lc, int kind, const CellOperand& o, const float* H, in
     }
   }
   if (best == 0) return false;
-  const int per = (p.k_blocks + p.splits - 1) / p.splits, chain = fine ? 1 : kDrainBlocks, groups = (per + chain - 1) / chain;
+  p.group = fine ? 1 : kDrainBlocks;
+  const int per = (p.k_blocks + p.splits - 1) / p.splits, groups = (per + p.group - 1) / p.group;
   p.sets_per_split = fine ? (per + kFineSet - 1) / kFineSet : 1;
   while (p.sets_per_split > 1 && p.splits * p.sets_per_split * outputs > (int64_t)partial_floats) --p.sets_per_split;
   p.merge = (groups + p.sets_per_split - 1) / p.sets_per_split;
-  p.group = (per + groups - 1) / groups;
-  p.per_split = p.sets_per_split * p.merge * p.group;
+  p.per_split = fine ? p.sets_per_split * p.merge : per;
   p.splits = (p.k_blocks + p.per_split - 1) / p.per_split;
   const int set_blocks = p.merge * p.group, last = p.k_blocks - (p.splits - 1) * p.per_split;
   const int sets = (p.splits - 1) * p.sets_per_split + (last + set_blocks - 1) / set_blocks;

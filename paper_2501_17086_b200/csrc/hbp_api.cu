@@ -158,8 +158,12 @@ bool keeps_parts(const hbp_config& f) {
          f.tokens > 32 && f.d >= 64 && f.hidden >= 64;
 }
 
-// Whether a recurrent kind's all-step products form their operands as they load them (gemm_cell.cu).  Narrower cells than a
-// k-block of 32 channels would be mostly padding.
+// Whether a recurrent kind's all-step products form their operands as they load them (gemm_cell.cu), for any number of rows: backward(1),
+// backward(4) and the latter with gradients in us, split by passes of their own before / so, 32 units: tanh RNN 4 x 2 rows 35, -, 58
+// with gradients of (1) / 29, -, 45; GRU 128 x 32 rows 29, -, 88 / 24, -, 36; 512 units LSTM 4 x 2 rows 78, -, 97 / 56, -, 75.  Below 32 units,
+// where a k-block of 32 channels is in part padding, the passes were kept; measured since, they lose there too: 1024 x 128 rows, GRU
+// 28 units 150, 490, 632 / 95, 268, 330, 16 units 112, 335, 453 / 102, 298, 355, 4 units 101, 295, 400 / 101, 295, 349; tanh RNN 4 units
+// 94, 296, 385 / 66, 187, 253; LSTM 8 units 161, 530, 616 / 129, 407, 482.
 bool forms_operands(const hbp_ctx* c) {
   const hbp_config& f = c->cfg;
   const bool recurrent = f.block == HBP_BLOCK_RNN_TANH || f.block == HBP_BLOCK_GRU || f.block == HBP_BLOCK_LSTM;

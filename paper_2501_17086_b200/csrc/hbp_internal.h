@@ -103,7 +103,7 @@ struct Launcher {
 // (chain_wait) for it to be over and its writes seen before they touch memory.  A kernel that calls chain_wait before any access
 // to global memory may be launched this way after anything.  Exact pass of a 6-layer decoder 512 wide, 2664 rows, 67 launches: 883 ->
 // 742 us; float stack of 12 layers 520 wide 2746 -> 2668.  Not for the CUDA-core kernels: launched like this 34 of them of 4 to 8 us
-// each (8 layers 64 wide, 32 rows) are bound by the launching thread, 246 -> 315 us.  (The ring scan and the recurrences: not tried.)
+// each (8 layers 64 wide, 32 rows, a launch per product) are bound by the launching thread, 246 -> 315 us.  (The ring scan and the recurrences: not tried.)
 template <typename... P, typename... A>
 cudaError_t try_launch_chained(Launcher& lc, void (*kernel)(P...), dim3 grid, int threads, size_t smem, int cluster, A&&... args) {
   cudaLaunchConfig_t cfg = {};
