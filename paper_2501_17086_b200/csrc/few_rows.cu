@@ -482,8 +482,9 @@ bool aligned(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 }  // namespace
 
 // 32 rows, forward pass in us here and with a launch per product: 8 layers 64 (256) 22 and 133, 128 (512) 37 and 166, 256 (256) 43 and 159, 2
-// layers 64 (128) 9 and 31, 64 layers 64 (256) 162 and 1050, 64 layers 128 (512) 278 and 1313.  Beyond 64 K weights a matrix its two layers
-// no longer fit shared memory, and backward passes gain less (8 layers 256 (1024) 79, 200 and 82, 214).
+// layers 64 (128) 9 and 31, 64 layers 64 (256) 162 and 1050, 64 layers 128 (512) 278 and 1313; 1 row, 8 layers 64 (256) 20 and 101.  Beyond 64 K
+// weights a matrix its two layers no longer fit shared memory, and backward passes gain less (8 layers 256 (1024) 79, 200 and 82, 214).
+// 32 rows are where the products move to the tensor cores (hbp_api.cu, keeps_parts), not where these kernels stop gaining.
 bool few_rows_take(int64_t N, int d, int h) { return N <= 32 && (int64_t)d * h <= 64 * 1024; }
 
 bool few_rows_forward(Launcher& lc, const FewRows& a, bool* refused) {

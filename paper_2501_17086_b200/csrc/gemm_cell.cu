@@ -60,7 +60,9 @@ constexpr float kScale = 16777216.0f, kUnscale = 1.0f / 16777216.0f;
 // less (GRU 32768 x 512 5339 for 5367 us, tanh RNN 131072 x 512 2715 for 2768) and is twice as far from 64 bits: dW, dU of the tanh RNN 32768 x 512 1.3e-6, 1.7e-6 (as three tf32 products 1.2e-6, 1.6e-6) and
 // 5.9e-7, 7.8e-7 with 512, of the GRU 1.1e-6 (1.2e-6) and 5.4e-7.  That the sums of a split are added in float adds 2e-9 to that.
 constexpr int kDrainBlocks = 512 / BK;
-// FINE: rows from which on the tensor core is used (as in gemm_f32.cu), k-blocks of a set of partial sums, most sets asked for, and the widest tile that leaves two accumulators room beside the sums
+// FINE: rows from which on the tensor core is used (as in gemm_f32.cu), k-blocks of a set of partial sums, most sets asked for, and the
+// widest tile that leaves two accumulators room beside the sums (three and four of them, on tiles of 128 and 96 columns, gain nothing: a
+// k-block takes the loading warps as long for any width)
 constexpr int kFewProducts = 17, kFineSet = 512 / BK, kMostFineSets = 256, kFineTileN = 160;
 
 struct Params {
