@@ -112,12 +112,14 @@ def _step(block, x, xt, W, U, a):
 
 
 # Rows of the product a multiple of 4: 32 additions a chain in the tensor core, each of which loses up to 2^-23 of a partial sum, that is on
-# average half as large as the whole: 32 * 2^-23 / 4.  Else sums of floats: 16 rounded additions a set, at random, 4 * 2^-24.
+# average half as large as the whole: 32 * 2^-23 / 4.  Else sums of floats: 16 rounded additions a set, at random, 4 * 2^-24.  The tanh RNN's
+# coefficients 1 - tanh^2 were formed from states not yet rounded to floats, which here they are: 2 |tanh| |W row| |x| 2^-25, 4 * 2^-24 at most.
 @pytest.mark.parametrize("T,B", [(500, 132), (499, 131), (499, 130), (33, 3), (17, 1), (5, 3)])
-@pytest.mark.parametrize("units,in_dim", [(64, 12), (96, 100), (164, 128)])   # one tile for states and inputs together, two, one each
+# states and inputs in one tile together, in two, in one and more each, the last of them with columns past their end
+@pytest.mark.parametrize("units,in_dim", [(64, 12), (96, 100), (164, 128), (256, 8), (300, 40), (452, 180)])
 @pytest.mark.parametrize("block", ["rnn_tanh", "gru", "lstm"])
 def test_weight_gradients_are_as_exact_as_their_rows_allow(block, units, in_dim, T, B):
-    """Against 64 bits from the pass's own states and iterate, so that nothing but the products' sums is compared."""
+    """Against 64 bits from the pass's own states and iterate, so that little but the products' sums is compared."""
     from paper_2501_17086_b200 import harness
     from paper_2501_17086_b200.workloads import make_inputs
     w = _workload(block, units, in_dim, T, B)
@@ -133,5 +135,5 @@ def test_weight_gradients_are_as_exact_as_their_rows_allow(block, units, in_dim,
     rows = lambda t: t.reshape(T * B, -1).double()
     out = _step(block, rows(x[:-1]), rows(X), W, U, params["a"].double() if "a" in params else None)
     for name, ref in zip(("dW", "dU"), torch.autograd.grad(out, (W, U), rows(g[1:]))):
-        bound = 32 * 2.0 ** -23 / 4 if T * B % 4 == 0 else 4 * 2.0 ** -24
+        bound = (32 * 2.0 ** -23 / 4 if T * B % 4 == 0 else 4 * 2.0 ** -24) + (4 * 2.0 ** -24 if block == "rnn_tanh" else 0)
         assert float((grads[name] - ref).norm() / ref.norm()) < bound, name
