@@ -530,7 +530,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   tc_fence_before();
   if (kPair) {
     if (!ok) tell_peer(abort_flag);
-    __syncwarp();
     cluster_sync();  // neither CTA leaves (or frees) while its peer may still read its tiles or signal its barriers
   } else {
     __syncthreads();

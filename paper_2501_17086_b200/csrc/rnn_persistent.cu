@@ -51,6 +51,7 @@ __device__ __forceinline__ void send_peer(uint32_t addr, double v, uint32_t bar)
                : "memory");
 }
 __device__ __forceinline__ void cluster_barrier() {
+  __syncwarp();  // (the .aligned forms are for whole warps)
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ uint64_t now_ns() {
