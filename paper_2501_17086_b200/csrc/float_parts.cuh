@@ -104,8 +104,6 @@ struct CellOperand {
 // the hidden halves, and uc = fg g_h c_h (+ delta_c), the cell halves, rows of 2d.  false (of either): nothing was launched.
 bool cell_vjp(Launcher& lc, int kind, const CellOperand& o, const Planes& W, const float* delta, float* out, int64_t ld, const float* fg,
               const float* delta_c, float* uc, int* status_word);
-// Floats of partial sums that the weight gradients of so many rows want (they take fewer).
-size_t cell_partial_floats(int kind, int64_t rows, int d, int in);
 // dW = operand^T H (rows of H ldh apart, 16-byte aligned), dU = operand^T X (X of any alignment, rows of `in`)
 bool cell_wgrad(Launcher& lc, int kind, const CellOperand& o, const float* H, int64_t ldh, const float* X, int in, float* dW, float* dU,
                 float* partial, size_t partial_floats, int* status_word);

@@ -18,7 +18,7 @@
 // (tanh RNN 1.5e-7 to 7e-7), and stay so.  One accumulator per 32 rows, the small terms first, and the epilogue adds it, rounded and
 // its truncation made good (float_parts.cuh), to sums kept in tensor memory; every 512 rows these go out as a set of partial
 // sums, which are added in double.  Weight gradients in us as float sums before / as the other form / so: GRU 32385 x 512 1590 / 330 / 750
-// (errors 7e-8 / 1.1e-6 / 7e-8), 131967 x 64 550 / 70 / 105, LSTM 32385 x 512 1720 / 500 / 1190, tanh RNN 135135 x 512 10400 / 525 / 1140 (2e-7 /
+// (errors 7e-8 / 1.1e-6 / 7e-8), 131967 x 64 550 / 70 / 100, LSTM 32385 x 512 1720 / 500 / 1190, tanh RNN 135135 x 512 10400 / 525 / 1140 (2e-7 /
 // 1.3e-6 / 7e-8).  Tiles of 96 columns 980, of 256, whose one set of accumulators holds up the products, 840 (GRU 32385 x 512).
 // Nothing of the operand goes through memory.  Before, it was written as two tf32 parts by a pass (the tanh RNN's by the scan before)
 // and read back by gemm_tc.cu, for the gradients transposed, their partial sums written every 512 rows.  One VJP with its pass and
@@ -55,15 +55,17 @@ constexpr int SMEM_BYTES = kStages * (int)kStageBytes + kEpiWarps * kEpiBufs * (
 // The operand is multiplied by this on the way in and the sums divided by it: the low part of any normal float is then a normal
 // bf16, also of gradients below 1e-34, which long recurrences have (values from 2^103 on overflow: refine).
 constexpr float kScale = 16777216.0f, kUnscale = 1.0f / 16777216.0f;
-// Weight gradients: rows that add up in the tensor core (32 additions at full magnitude, each of which truncates) before the sum is
-// added, rounded, to the split's partial sums.  With 1024 rows (as once here) a pass takes 0.5 to 2 %
-// less (GRU 32768 x 512 5339 for 5367 us, tanh RNN 131072 x 512 2715 for 2768) and is twice as far from 64 bits: dW, dU of the tanh RNN 32768 x 512 1.3e-6, 1.7e-6 (as three tf32 products 1.2e-6, 1.6e-6) and
-// 5.9e-7, 7.8e-7 with 512, of the GRU 1.1e-6 (1.2e-6) and 5.4e-7.  That the sums of a split are added in float adds 2e-9 to that.
+// Weight gradients: rows that add up in the tensor core (32 additions at full magnitude, each of which truncates) before the sum is added,
+// rounded, to the split's partial sums.  With 1024 rows (as once here) a pass takes 0.5 to 2 % less (GRU 32768 x 512 5339 for 5367 us, tanh
+// RNN 131072 x 512 2715 for 2768) and is twice as far from 64 bits: dW, dU of the tanh RNN 32768 x 512 1.3e-6, 1.7e-6 (as three tf32
+// products 1.2e-6, 1.6e-6) and 5.9e-7, 7.8e-7 with 512, of the GRU 1.1e-6 (1.2e-6) and 5.4e-7.  That the sums of a split are added in
+// float adds 2e-9 to that.
 constexpr int kDrainBlocks = 512 / BK;
-// FINE: rows from which on the tensor core is used (as in gemm_f32.cu), k-blocks of a set of partial sums, most sets asked for, and the
-// widest tile that leaves two accumulators room beside the sums (three and four of them, on tiles of 128 and 96 columns, gain nothing: a
-// k-block takes the loading warps as long for any width)
-constexpr int kFewProducts = 17, kFineSet = 512 / BK, kMostFineSets = 256, kFineTileN = 160;
+// FINE: rows from which on the tensor core is used (as in gemm_f32.cu); k-blocks of a set of partial sums, more where the workspace, which
+// is that of the splits, has no room for so many sets (GRU of 131967 rows, 64 units and inputs: 57 k-blocks, 3.1e-8 -> 3.7e-8 from 64 bits;
+// 512 and 512: 30, 5.0e-8 -> 5.8e-8, and 4250 -> 3780 us); the widest tile that leaves two accumulators room beside the sums (three
+// and four of them, on tiles of 128 and 96 columns, gain nothing: a k-block takes the loading warps as long for any width)
+constexpr int kFewProducts = 17, kFineSet = 512 / BK, kFineTileN = 160;
 
 struct Params {
   CellOperand o;
@@ -901,12 +903,6 @@ bool cell_vjp(Launcher& lc, int kind, const CellOperand& o, const Planes& W, con
   tmE = tmD;
   if (delta && !make_map_epi(&tmE, delta, true, (int)o.rows, o.d, 1, ld, 0)) return false;
   return launch_kind<false, false>(lc, p.num_tiles, tmW, tmD, tmD, tmE, p);
-}
-
-size_t cell_partial_floats(int kind, int64_t rows, int d, int in) {
-  if (!fine_sums(rows)) return 0;
-  const int64_t sets = (rows + kFineSet * BK - 1) / (kFineSet * BK), blocks = kind == HBP_BLOCK_GRU && both_at_once(d, in) ? 4 : blocks_of(kind);
-  return (size_t)((sets < kMostFineSets ? sets : kMostFineSets) * blocks * d * (d + in));
 }
 
 bool cell_wgrad(Launcher& lc, int kind, const CellOperand& o, const float* H, int64_t ldh, const float* X, int in, float* dW, float* dU,

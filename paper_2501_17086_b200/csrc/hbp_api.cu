@@ -319,10 +319,6 @@ size_t carve(hbp_ctx* c, char* base, int weight_layers) {
       c->dopart = (float2*)take(Lb * N * c->do_slots * sizeof(float2));
     }
   }
-  if (cell) {
-    const size_t pf = cell_partial_floats(f.block, (int64_t)f.L * f.tokens, f.block == HBP_BLOCK_LSTM ? f.d / 2 : f.d, f.in_dim);
-    if (pf > c->partial_floats) c->partial_floats = pf;
-  }
   c->partial = (float*)take(c->partial_floats * 4);
   return off;
 }

@@ -59,6 +59,16 @@ def test_workspace_sizes_and_config_errors(B):
     assert e.value.code == 6
 
 
+@pytest.mark.parametrize("units,in_dim", [(64, 12), (64, 64), (512, 512)])
+@pytest.mark.parametrize("block", ["rnn_tanh", "gru", "lstm"])
+def test_workspace_of_odd_row_counts_is_that_of_even_ones(B, block, units, in_dim):
+    """How the weight gradients of T * B rows that are no multiple of 4 are added up asks for no memory of its own."""
+    lstm = block == "lstm"
+    need = [B.workspace_bytes(B.make_config(block, "f32", T, units * (2 if lstm else 1), 129, hidden=units if lstm else 0, in_dim=in_dim, batch=129,
+                                            gate=B.GATE_CHANNEL_SHARED if block == "rnn_tanh" else B.GATE_ONE)) for T in (1023, 1024)]
+    assert need[0] < need[1]
+
+
 def test_argument_errors_before_any_cuda_call(B):
     lib = B.lib
     n = C.c_size_t()
