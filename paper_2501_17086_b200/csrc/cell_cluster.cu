@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(max_threads(MT, EX), 1) cell_forward_kernel(co
       cst[o] = o_live[it] ? (double)to_f(((const T*)p.x0)[(int64_t)(row0 + o_row[it]) * S + o_unit[it]]) : 0.0;
   }
   __syncthreads();
-  tc::cluster_sync();  // every CTA of the cluster has started: barriers and buffers exist
+  tc::cluster_sync_whole_warps();  // every CTA of the cluster has started: barriers and buffers exist
 
   bool ok = true;
   for (int t = 0; t < p.T; ++t) {
@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(max_threads(MT, EX), 1) cell_backward_kernel(c
     }
   }
   __syncthreads();
-  tc::cluster_sync();
+  tc::cluster_sync_whole_warps();
 
   bool ok = true;
   for (int s = 0; s < p.T; ++s) {
@@ -713,7 +713,7 @@ __global__ void __launch_bounds__(max_threads(MT, EX), 1) cell_backward_kernel(c
     }
   }
   if (__syncthreads_or(!ok)) after_timeout(p.status);
-  tc::cluster_sync();
+  tc::cluster_sync_whole_warps();
 }
 
 // the functions of the gates on their own: out[i] = {e^-|v|, 1 / (1 + e^-|v|), sigmoid(v), 1 - sigmoid(v), tanh(v), 1 - tanh(v)^2}

@@ -73,10 +73,14 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
-// (The .aligned forms are for whole warps, and lanes come here from roles and loops that they left one by one.)
+// (The .aligned forms are for whole warps.)
+__device__ __forceinline__ void cluster_sync_whole_warps() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// ... for lanes that come from roles and loops that they left one by one
 __device__ __forceinline__ void cluster_sync() {
   __syncwarp();
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  cluster_sync_whole_warps();
 }
 // shared::cluster address of `addr` (a shared::cta address of this CTA) in the CTA of rank `rank`
 __device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank) {
