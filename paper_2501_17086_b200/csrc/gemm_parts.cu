@@ -160,7 +160,6 @@ gemm_parts_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             if (++stage == stages) { stage = 0; phase ^= 1u; }
           }
         }
-        if (!ok) tell_peer(abort_flag);
       }
     } else if (warp == 1 && leader) {
       // ---------------------------------------------------------------- MMA issuer (the warp converged, one elected lane issues)
@@ -209,7 +208,6 @@ gemm_parts_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         const uint64_t t0 = global_ns();
         while (!mbar_try_wait(drain_bar, 0) && global_ns() - t0 < 100000000ull) {
         }
-        tell_peer(abort_flag);
       }
     }
   } else {
@@ -400,16 +398,14 @@ gemm_parts_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         }
       }
     }
-    if (!ok) tell_peer(abort_flag);
   }
 
   tc_fence_before();
-  cluster_sync();  // neither CTA leaves (or frees) while its peer may still read its tiles or signal its barriers
+  leave_together(abort_flag);  // neither CTA leaves (or frees) while its peer may still read its tiles or signal its barriers
   if (warp == 1) {
-    const int gave_up = *abort_flag;
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
-    if (gave_up) outlast_copies();
+    if (*abort_flag) outlast_copies();
   }
 }
 

@@ -237,13 +237,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const int row_elems = kTf32 ? 32 : 64;
   const uint32_t mn_block = kTf32 ? 4096u : 8192u;
 
-  bool ok = true;  // until one of this thread's waits gives up
   if (warp == 0 || warp == kProducerB) {
     // ------------------------------------------------------------------ TMA producers: of A, and of B
     const bool of_a = warp == 0;
     if (lane == 0) {
       int stage = 0;
       uint32_t phase = 0;
+      bool ok = true;
       for (int tile = first_tile; tile < p.num_tiles && ok; tile += tile_step) {
         const int zc = tile / tiles_per_batch, r = tile % tiles_per_batch;
         const int b = zc % p.batch, split = zc / p.batch;
@@ -305,6 +305,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       const uint32_t kStage16 = (uint32_t)STAGE_BYTES >> 4;
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0;
+      bool ok = true;
       // The tensor core idles whenever this thread takes longer between two MMAs than one MMA runs, so nothing that
       // has to wait for an answer sits between them: the barrier of the NEXT stage (and of the next tile's
       // accumulator) is only tested, without blocking, before the current stage's MMAs go out, and the answer is
@@ -401,7 +402,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         load_e(0);
         if (EPI_BUFS > 1 && nchunks > 1) load_e(1);
       }
-      if (!mbar_wait(accf_bar(acc), acc_phase, abort_flag, p.status, p.wait_limit_ns)) { ok = false; break; }
+      if (!mbar_wait(accf_bar(acc), acc_phase, abort_flag, p.status, p.wait_limit_ns)) break;
       tc_fence_after();
       const uint32_t tsrc = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN + half * half_cols);
       if (nchunks == 0) {  // nothing of a narrow tile in this half: only hand the accumulator back
@@ -419,6 +420,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         __syncwarp();
         if (lane == 0) release_acc(acc);
       } else {
+        bool ok = true;
         float s1 = 0.0f, s2 = 0.0f;  // EPI_STORE_LN: row sums of acc and acc * E over the current 64 columns
 #pragma unroll 1
         for (int c = 0; c < nchunks; ++c) {
@@ -528,18 +530,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   }
 
   tc_fence_before();
-  if (kPair) {
-    if (!ok) tell_peer(abort_flag);
-    cluster_sync();  // neither CTA leaves (or frees) while its peer may still read its tiles or signal its barriers
-  } else {
-    __syncthreads();
-  }
+  if (kPair) leave_together(abort_flag);  // neither CTA leaves (or frees) while its peer may still read its tiles or signal its barriers
+  else __syncthreads();
   if (warp == 1) {
-    const int gave_up = *abort_flag;
     tc_fence_after();
     if (kPair) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
     else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
-    if (gave_up) outlast_copies();
+    if (*abort_flag) outlast_copies();
   }
 }
 
