@@ -58,14 +58,14 @@ def config_of(w, k, touched_bytes=None):
 # profiles/.  An entry is used only while the kernel's sources still hash to the value recorded with the capture and
 # the workload has the captured shapes; otherwise the bench line carries "traffic": null.
 TRAFFIC = {
-    # gemm_tc_kernel, VJP pair (dA + dY): c5_small (4 layers x 16384 tokens): 2121.899 + 1054.033 and 2438.503 + 279.543 MB;
-    # c2_small (8 layers x 8192 tokens): 738.675 + 505.052 and 796.289 + 128.911 MB
+    # gemm_tc_kernel, VJP pair (dA + dY): c5_small (4 layers x 16384 tokens): 2506.604 + 1049.792 and 3870.687 + 281.069 MB;
+    # c2_small (8 layers x 8192 tokens): 741.680 + 503.876 and 799.564 + 130.955 MB
     "gemm_vjp": [
-        {"sources": ("gemm_tc.cu", "tc_common.cuh"), "sha256": "48e1ccd304ba5914", "shape": ("preln_mlp", "bf16", 2048, 8192),
-         "bytes_per_token_layer": (2121.899e6 + 1054.033e6 + 2438.503e6 + 279.543e6) / (4 * 16384),
+        {"sources": ("gemm_tc.cu", "tc_common.cuh"), "sha256": "440ccffdad2a0b67", "shape": ("preln_mlp", "bf16", 2048, 8192),
+         "bytes_per_token_layer": (2506.604e6 + 1049.792e6 + 3870.687e6 + 281.069e6) / (4 * 16384),
          "profile": "profiles/gemm_tc_kernel_c5_small.md"},
-        {"sources": ("gemm_tc.cu", "tc_common.cuh"), "sha256": "48e1ccd304ba5914", "shape": ("preln_mlp", "bf16", 1024, 4096),
-         "bytes_per_token_layer": (738.675e6 + 505.052e6 + 796.289e6 + 128.911e6) / (8 * 8192),
+        {"sources": ("gemm_tc.cu", "tc_common.cuh"), "sha256": "440ccffdad2a0b67", "shape": ("preln_mlp", "bf16", 1024, 4096),
+         "bytes_per_token_layer": (741.680e6 + 503.876e6 + 799.564e6 + 130.955e6) / (8 * 8192),
          "profile": "profiles/gemm_tc_kernel_c2_small.md"}],
     # scan_depth_lnstat_kernel: c5_small 605.050 MB read + 213.970 MB written for 4 steps x 16384 x 2048 elements; c2_small
     # 286.283 + 80.576 MB for 8 x 8192 x 1024 (the writes still in L2 when such a small launch ends are not in the counter)
@@ -76,10 +76,10 @@ TRAFFIC = {
         {"sources": ("scan.cu",), "sha256": "655dd8f4f6b9a76c", "shape": ("preln_mlp", "bf16", 1024, 4096),
          "bytes_per_state_element_step": (286.283e6 + 80.576e6) / (8 * 8192 * 1024),
          "profile": "profiles/scan_depth_lnstat_kernel_c2_small.md"}],
-    # scan_ring_kernel on c3: 268.531 MB read + 213.144 MB written, the mean of five scans
+    # scan_ring_kernel on c3: 268.554 MB read + 212.822 MB written, the mean of five scans
     "scan_ring": [
-        {"sources": ("scan_ring.cu", "tc_common.cuh"), "sha256": "d2b53992756ec04d", "shape": ("rnn_tanh", "f32", 512, 0),
-         "bytes_per_state_element_step": (268.531e6 + 213.144e6) / (4096 * 32 * 512),
+        {"sources": ("scan_ring.cu", "tc_common.cuh"), "sha256": "d043b5e0fd774dfa", "shape": ("rnn_tanh", "f32", 512, 0),
+         "bytes_per_state_element_step": (268.554e6 + 212.822e6) / (4096 * 32 * 512),
          "profile": "profiles/scan_ring_kernel_c3.md"}],
 }
 
